@@ -197,3 +197,78 @@ def tolerance(case):
     if case["path"] in ("apply", "apply_pca"):
         return {"rel": 1e-6, "max": 1e-5, "differ": 2e-5}
     return {"rel": 1e-5, "max": 1e-4, "differ": 1e-4}
+
+
+# ---------------------------------------------------------------- the same in fp64
+
+def _nearest64(X, C):
+    """Index of the nearest row of C for every row of X (both fp64)."""
+    lab = torch.empty(X.shape[0], dtype=torch.int64, device=X.device)
+    c2 = (C * C).sum(1)
+    for r in range(0, X.shape[0], 65_536):
+        lab[r:r + 65_536] = torch.argmin(c2 - 2.0 * (X[r:r + 65_536] @ C.t()), dim=1)
+    return lab
+
+
+def _kmeans64(X, k, iters):
+    """Lloyd rounds from the first k rows; the centroids are fp32 between rounds, as the interface
+    hands them out."""
+    C = X[:k].clone()
+    for _ in range(iters):
+        one = torch.nn.functional.one_hot(_nearest64(X, C), k).double()
+        n = one.sum(0)[:, None]
+        C = torch.where(n > 0, (one.t() @ X) / n.clamp(min=1.0), C).float().double()
+    return C, _nearest64(X, C)
+
+
+def _closed_form64(Yq, Yfp, lab, k):
+    one = torch.nn.functional.one_hot(lab, k).double()
+    n = one.sum(0)[:, None]
+    d = n.clamp(min=1.0)
+    q, f = Yq.double(), Yfp.double()
+    muq, muf = (one.t() @ q) / d, (one.t() @ f) / d
+    q, f = q - muq[lab], f - muf[lab]
+    g = ((one.t() @ (q * f)) / d) / ((one.t() @ (q * q)) / d).clamp(min=1e-8)
+    g = torch.where(n > 0, g, torch.ones_like(g))
+    return g, torch.where(n > 0, muf - g * muq, torch.zeros_like(g))
+
+
+def _pca64(Yq, p):
+    mean = Yq.double().mean(0)
+    X = Yq.double() - mean
+    _, vec = torch.linalg.eigh(X.t() @ X)
+    comps = vec[:, -p:].t().flip(0)
+    top = torch.gather(comps, 1, comps.abs().argmax(1, keepdim=True))
+    return mean, comps * torch.sign(top)
+
+
+def exact(case, seed):
+    """`run`'s outputs in fp64 (what the interface hands on as fp32 in between -- centroids, mean,
+    components, projected rows -- is rounded to fp32 there); None for the largest."""
+    path, k = case["path"], case["k"]
+    if case["rows"] * case["cols"] > 1_100_000_000:
+        return None
+    st = prepare(case, seed)
+    if path in ("fit", "fit_pca"):
+        if path == "fit":
+            C, lab = _kmeans64(st["Yq"].double(), k, case["iters"])
+            g, b = _closed_form64(st["Yq"], st["Yfp"], lab, k)
+            return C, g, b, lab.int()
+        mean, comps = _pca64(st["Yq"], case["p"])
+        Z = ((st["Yq"].double() - mean.float().double()) @ comps.float().double().t()).float()
+        C, lab = _kmeans64(Z.double(), k, case["iters"])
+        g, b = _closed_form64(st["Yq"], st["Yfp"], lab, k)
+        return dict(mean=mean, comps=comps, centroids=C, gamma=g, beta=b, labels=lab.int())
+    Y = st["Y"]
+    out = torch.empty(Y.shape, dtype=torch.float64, device=DEV)
+    lab = torch.empty(Y.shape[0], dtype=torch.int32, device=DEV)
+    a = case.get("alpha", 1.0)
+    for r in range(0, Y.shape[0], 65_536):
+        y = Y[r:r + 65_536].double()
+        x = y
+        if path == "apply_pca":
+            x = ((y - st["mean"].double()) @ st["comps"].double().t()).float().double()
+        lb = _nearest64(x, st["C"].double())
+        out[r:r + 65_536] = y + a * (st["G"].double()[lb] * y + st["B"].double()[lb] - y)
+        lab[r:r + 65_536] = lb.int()
+    return out, lab
