@@ -297,8 +297,8 @@ cat_status_t cat_solve_gamma_beta(const double *sumQ, const double *sumF,
  * the projection on the LQ outputs of the fit set, Algorithm 2 step 1 applies it at inference.
  *
  * cat_pca_fit: column means of Yq [N, D] -> mean_out [D]; covariance of the centred rows in fp64
- * (1 / (N - 1)); its eigen-decomposition by one-sided Jacobi rotations in fp64 on the device; the p
- * directions of largest variance -> components_out [p, D] (rows, unit length, decreasing variance;
+ * (1 / (N - 1)); its largest eigenpairs in fp64 on the device (tridiagonal reduction, bisection, inverse iteration);
+ * the p directions of largest variance -> components_out [p, D] (rows, unit length, decreasing variance;
  * the sign of a row is fixed so that its entry of largest magnitude is positive); their variances
  * -> eigenvalues_out [p] double, may be NULL.  Deterministic.  N >= 2, 1 <= p <= D,
  * D <= CAT_PCA_MAX_D, p <= CAT_PCA_MAX_P.  Directions whose variances coincide are determined

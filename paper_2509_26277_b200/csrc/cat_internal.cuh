@@ -259,4 +259,11 @@ cudaError_t launch_fit_diag_round(const float *Y, int64_t N, int D, int K, const
                                   cat_fit_diag_t *diag, int slot, int recorded, cudaStream_t s);
 cudaError_t launch_reset_control(Control *ctl, cudaStream_t s);
 
+// The p largest eigenpairs of the symmetric positive semi-definite matrix A [D, D] (full, fp64; overwritten),
+// whose diagonal is also given: unit vectors -> comps [p, D] (fp32 rows, decreasing eigenvalue, entry of largest
+// magnitude positive), eigenvalues -> eig_out [p] (may be null).  refl: [D, D] scratch.  D <= CAT_PCA_MAX_D.
+size_t sym_eig_workspace_bytes(int D, int p);
+cudaError_t launch_sym_eig(double *A, const double *diag, double *refl, int D, int p, float *comps, double *eig_out,
+                           Control *ctl, void *workspace, cudaStream_t s);
+
 }  // namespace cat

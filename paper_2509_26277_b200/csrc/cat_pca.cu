@@ -4,12 +4,9 @@
 //   column means            fp64 partial sums per row chunk, added in a fixed order
 //   covariance              D x D, fp64 FMA on 64 x 64 register-tiled CTAs over the centred rows
 //                           (upper-triangular tiles, mirrored); 1 / (N - 1) normalisation
-//   eigen-decomposition     one-sided Jacobi (Hestenes) in fp64 on the device: plane rotations
-//                           orthogonalise the columns of G = Sigma V, all D / 2 disjoint column
-//                           pairs of a round-robin step in one launch; a sweep that rotates
-//                           nothing ends the iteration (later launches return at once)
-//   components              the p columns of V with the largest ||g||, sign fixed so that the entry
-//                           of largest magnitude is positive, stored as fp32 rows
+//   eigen-decomposition     the p largest pairs by tridiagonal reduction, bisection and inverse
+//                           iteration in fp64 (cat_eig.cu); a component's sign is fixed so that its
+//                           entry of largest magnitude is positive, stored as fp32 rows
 //   projection              Z = (Y - mean) V_p^T, fp64 accumulation, fp32 result
 //   affine with labels      out_i = gamma_l * y_i + beta_l for given cluster ids (Algorithm 2 steps 4-8)
 //
@@ -17,7 +14,6 @@
 #include "cat_internal.cuh"
 
 #include <cuda_bf16.h>
-#include <math_constants.h>
 
 namespace cat {
 
@@ -27,14 +23,6 @@ constexpr int PT = 64;          // tile edge of the fp64 contractions
 constexpr int PK = 16;          // depth of a shared-memory step
 constexpr int P_THREADS = 256;  // 16 x 16 threads, 4 x 4 outputs each
 constexpr int MEAN_CHUNKS = 64;
-constexpr int JACOBI_MAX_SWEEPS = 30;
-
-struct PcaCtl {
-    int done;       // 1 once a whole sweep has rotated nothing
-    int rotated;    // rotations of the current sweep
-    int sweeps;     // sweeps carried out
-    int pad;
-};
 
 // ---------------------------------------------------------------- column means
 __global__ void __launch_bounds__(128) col_partial_kernel(const float *__restrict__ Y, int64_t N, int D,
@@ -118,190 +106,19 @@ __global__ void __launch_bounds__(P_THREADS) cov_kernel(const float *__restrict_
         }
 }
 
-// G = (sum of the splits' upper triangles, mirrored) / (N - 1); V = identity
+// G = (sum of the splits' upper triangles, mirrored) / (N - 1), and its diagonal once more
 __global__ void cov_finish_kernel(const double *__restrict__ part, int splits, int D, int64_t N,
-                                  double *__restrict__ G, double *__restrict__ V, PcaCtl *ctl)
+                                  double *__restrict__ G, double *__restrict__ diag)
 {
     const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e == 0) {
-        ctl->done = 0;
-        ctl->rotated = 0;
-        ctl->sweeps = 0;
-    }
     if (e >= (size_t)D * D) return;
     const int a = (int)(e / D), b = (int)(e % D);
     const int lo = a < b ? a : b, hi = a < b ? b : a;
     double s = 0.0;
     for (int z = 0; z < splits; ++z) s += part[(size_t)z * D * D + (size_t)lo * D + hi];
-    G[e] = s / (double)(N > 1 ? N - 1 : 1);
-    V[e] = (a == b) ? 1.0 : 0.0;
-}
-
-// ---------------------------------------------------------------- one-sided Jacobi
-// Column pairs of round-robin step `step` over n = D rounded up to even "players" (index D, if
-// present, is a dummy): pair 0 = (n - 1, step), pair k = ((step + k) mod (n - 1), (step - k) mod (n - 1)).
-// G and V are column-major (column c at c * D).  One CTA rotates one pair so that the two columns
-// of G become orthogonal; the same rotation goes into V.
-__global__ void __launch_bounds__(256) jacobi_step_kernel(double *__restrict__ G, double *__restrict__ V, int D, int n,
-                                                          int step, PcaCtl *ctl)
-{
-    if (ctl->done) return;
-    __shared__ double red[3][8];
-    __shared__ double cs[2];
-    const int k = blockIdx.x;
-    int i, j;
-    if (k == 0) {
-        i = n - 1;
-        j = step;
-    } else {
-        i = (step + k) % (n - 1);
-        j = (step - k + (n - 1)) % (n - 1);
-    }
-    if (i >= D || j >= D) return;
-    if (i > j) {
-        const int t = i;
-        i = j;
-        j = t;
-    }
-    double *gi = G + (size_t)i * D, *gj = G + (size_t)j * D;
-    double a = 0.0, b = 0.0, c = 0.0;
-    for (int r = threadIdx.x; r < D; r += 256) {
-        const double x = gi[r], y = gj[r];
-        a = fma(x, x, a);
-        b = fma(y, y, b);
-        c = fma(x, y, c);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_xor_sync(0xffffffffu, a, o);
-        b += __shfl_xor_sync(0xffffffffu, b, o);
-        c += __shfl_xor_sync(0xffffffffu, c, o);
-    }
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) {
-        red[0][w] = a;
-        red[1][w] = b;
-        red[2][w] = c;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double aa = 0.0, bb = 0.0, cc = 0.0;
-        for (int q = 0; q < 8; ++q) {
-            aa += red[0][q];
-            bb += red[1][q];
-            cc += red[2][q];
-        }
-        double cth = 1.0, sth = 0.0;
-        // rotate unless the two columns are orthogonal to working precision already
-        if (fabs(cc) > 1e-15 * sqrt(aa * bb) && cc != 0.0) {
-            const double zeta = (bb - aa) / (2.0 * cc);
-            const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-            cth = 1.0 / sqrt(1.0 + t * t);
-            sth = cth * t;
-            atomicAdd(&ctl->rotated, 1);
-        }
-        cs[0] = cth;
-        cs[1] = sth;
-    }
-    __syncthreads();
-    const double cth = cs[0], sth = cs[1];
-    if (sth == 0.0) return;
-    double *vi = V + (size_t)i * D, *vj = V + (size_t)j * D;
-    for (int r = threadIdx.x; r < D; r += 256) {
-        const double x = gi[r], y = gj[r];
-        gi[r] = cth * x - sth * y;
-        gj[r] = sth * x + cth * y;
-        const double p = vi[r], q = vj[r];
-        vi[r] = cth * p - sth * q;
-        vj[r] = sth * p + cth * q;
-    }
-}
-
-__global__ void jacobi_sweep_end_kernel(PcaCtl *ctl)
-{
-    if (threadIdx.x != 0 || blockIdx.x != 0 || ctl->done) return;
-    ctl->sweeps += 1;
-    if (ctl->rotated == 0) ctl->done = 1;
-    ctl->rotated = 0;
-}
-
-// eigenvalue of column c = ||g_c|| (Sigma is positive semi-definite)
-__global__ void __launch_bounds__(256) column_norms_kernel(const double *__restrict__ G, int D, double *__restrict__ lam)
-{
-    __shared__ double red[8];
-    const double *g = G + (size_t)blockIdx.x * D;
-    double a = 0.0;
-    for (int r = threadIdx.x; r < D; r += 256) a = fma(g[r], g[r], a);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = a;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int q = 0; q < 8; ++q) t += red[q];
-        lam[blockIdx.x] = sqrt(t);
-    }
-}
-
-// Column c of V becomes component rank(c) if that rank is below p: rank = number of columns with a
-// larger eigenvalue (lower index first among equals).  Sign: the entry of largest magnitude (lowest
-// index among equals) is made positive.
-__global__ void __launch_bounds__(256) select_components_kernel(const double *__restrict__ V, const double *__restrict__ lam,
-                                                                int D, int p, float *__restrict__ comps,
-                                                                double *__restrict__ eig_out)
-{
-    __shared__ int s_rank;
-    __shared__ double s_best[8];
-    __shared__ int s_idx[8];
-    const int c = blockIdx.x;
-    const double mine = lam[c];
-    int cnt = 0;
-    for (int j = threadIdx.x; j < D; j += 256) {
-        const double o = lam[j];
-        cnt += (o > mine || (o == mine && j < c)) ? 1 : 0;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-    if (threadIdx.x == 0) s_rank = 0;
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) atomicAdd(&s_rank, cnt);
-    __syncthreads();
-    const int rank = s_rank;
-    if (rank >= p) return;
-    const double *v = V + (size_t)c * D;
-    double best = -1.0;
-    int bi = D;
-    for (int r = threadIdx.x; r < D; r += 256) {
-        const double m = fabs(v[r]);
-        if (m > best) {
-            best = m;
-            bi = r;
-        }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ob > best || (ob == best && oi < bi)) {
-            best = ob;
-            bi = oi;
-        }
-    }
-    if ((threadIdx.x & 31) == 0) {
-        s_best[threadIdx.x >> 5] = best;
-        s_idx[threadIdx.x >> 5] = bi;
-    }
-    __syncthreads();
-    double b = s_best[0];
-    int ix = s_idx[0];
-    for (int q = 1; q < 8; ++q)
-        if (s_best[q] > b || (s_best[q] == b && s_idx[q] < ix)) {
-            b = s_best[q];
-            ix = s_idx[q];
-        }
-    const double sign = (ix < D && v[ix] < 0.0) ? -1.0 : 1.0;
-    for (int r = threadIdx.x; r < D; r += 256) comps[(size_t)rank * D + r] = (float)(sign * v[r]);
-    if (threadIdx.x == 0 && eig_out) eig_out[rank] = mine;
+    s /= (double)(N > 1 ? N - 1 : 1);
+    G[e] = s;
+    if (a == b) diag[a] = s;
 }
 
 // ---------------------------------------------------------------- projection
@@ -434,17 +251,18 @@ int cov_splits(int D)
 }
 
 struct PcaWs {
-    PcaCtl *ctl;
+    Control *ctl;        // (first: cat_workspace_report reads the status of the bounded waits here)
     double *mean_part;   // [MEAN_CHUNKS][D]
     double *mean64;      // [D]
-    double *lam;         // [D]
-    double *G;           // [D][D], column-major
-    double *V;           // [D][D], column-major
+    double *diag;        // [D]
+    double *G;           // [D][D] covariance
+    double *refl;        // [D][D] reflections of the tridiagonal reduction
     double *cov_part;    // [splits][D][D]
+    void *eig;
     size_t bytes;
 };
 
-PcaWs carve_pca(void *base, int D)
+PcaWs carve_pca(void *base, int D, int p)
 {
     unsigned char *b = reinterpret_cast<unsigned char *>(base);
     size_t off = 0;
@@ -456,13 +274,14 @@ PcaWs carve_pca(void *base, int D)
     };
     PcaWs w{};
     const size_t DD = (size_t)D * D;
-    w.ctl = (PcaCtl *)take(sizeof(PcaCtl));
+    w.ctl = (Control *)take(sizeof(Control));
     w.mean_part = (double *)take((size_t)MEAN_CHUNKS * D * sizeof(double));
     w.mean64 = (double *)take((size_t)D * sizeof(double));
-    w.lam = (double *)take((size_t)D * sizeof(double));
+    w.diag = (double *)take((size_t)D * sizeof(double));
     w.G = (double *)take(DD * sizeof(double));
-    w.V = (double *)take(DD * sizeof(double));
+    w.refl = (double *)take(DD * sizeof(double));
     w.cov_part = (double *)take((size_t)cov_splits(D) * DD * sizeof(double));
+    w.eig = take(sym_eig_workspace_bytes(D, p));
     w.bytes = align_up(off, 256);
     return w;
 }
@@ -504,7 +323,7 @@ extern "C" {
 size_t cat_pca_workspace_bytes(int64_t N, int32_t D, int32_t p)
 {
     if (pca_shape(N, D, p) != CAT_OK) return 0;
-    return carve_pca(nullptr, D).bytes;
+    return carve_pca(nullptr, D, p).bytes;
 }
 
 cat_status_t cat_pca_fit(const float *Yq, int64_t N, int32_t D, int32_t p, float *mean_out,
@@ -518,7 +337,8 @@ cat_status_t cat_pca_fit(const float *Yq, int64_t N, int32_t D, int32_t p, float
         return CAT_ERR_ALIGN;
     if (!workspace || !al16(workspace) || workspace_bytes < cat_pca_workspace_bytes(N, D, p)) return CAT_ERR_WORKSPACE;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    PcaWs w = carve_pca(workspace, D);
+    PcaWs w = carve_pca(workspace, D, p);
+    CAT_CUDA(launch_reset_control(w.ctl, s));
 
     int chunks = (int)(N < MEAN_CHUNKS ? N : MEAN_CHUNKS);
     col_partial_kernel<<<dim3((D + 127) / 128, chunks), 128, 0, s>>>(Yq, N, D, w.mean_part);
@@ -528,23 +348,10 @@ cat_status_t cat_pca_fit(const float *Yq, int64_t N, int32_t D, int32_t p, float
     if ((int64_t)splits > N) splits = (int)N;
     cov_kernel<<<dim3(T, T, splits), P_THREADS, 0, s>>>(Yq, N, D, w.mean64, w.cov_part);
     const size_t DD = (size_t)D * D;
-    cov_finish_kernel<<<(unsigned)((DD + 255) / 256), 256, 0, s>>>(w.cov_part, splits, D, N, w.G, w.V, w.ctl);
+    cov_finish_kernel<<<(unsigned)((DD + 255) / 256), 256, 0, s>>>(w.cov_part, splits, D, N, w.G, w.diag);
     count_launch(4);
     CAT_CUDA(cudaGetLastError());
-    if (D > 1) {
-        const int n = (D + 1) & ~1;
-        for (int sweep = 0; sweep < JACOBI_MAX_SWEEPS; ++sweep) {
-            for (int step = 0; step < n - 1; ++step)
-                jacobi_step_kernel<<<n / 2, 256, 0, s>>>(w.G, w.V, D, n, step, w.ctl);
-            jacobi_sweep_end_kernel<<<1, 32, 0, s>>>(w.ctl);
-            count_launch(n);
-        }
-        CAT_CUDA(cudaGetLastError());
-    }
-    column_norms_kernel<<<D, 256, 0, s>>>(w.G, D, w.lam);
-    select_components_kernel<<<D, 256, 0, s>>>(w.V, w.lam, D, p, components_out, eigenvalues_out);
-    count_launch(2);
-    CAT_CUDA(cudaGetLastError());
+    CAT_CUDA(launch_sym_eig(w.G, w.diag, w.refl, D, p, components_out, eigenvalues_out, w.ctl, w.eig, s));
     return CAT_OK;
 }
 

@@ -100,3 +100,39 @@ def test_fit_and_apply_with_pca_on_the_linear_head_configs(config, p):
     want2 = want if n_diff == 0 else O.affine_with_labels(Ya, host(alab), host(r["gamma"]), host(r["beta"]))
     np.testing.assert_array_equal(host(out), want2)
     print(f"config {config} p={p}: near-tie rows {n_near} (label differs on {n_diff})")
+
+
+@pytest.mark.parametrize("n,d,p,kind", [
+    (8, 1, 1, "full"), (9, 2, 2, "full"), (40, 3, 2, "full"),
+    (600, 255, 9, "full"), (600, 256, 9, "full"), (700, 513, 150, "full"),   # edges of the columns per thread; more pairs than CTAs
+    (400, 2100, 6, "full"),                                                  # rows of the matrix in global memory
+    (20, 300, 40, "full"),                                                   # more components than the rank
+    (256, 64, 64, "equal"),                                                  # one eigenvalue, 64 times
+    (512, 96, 50, "pairs"),                                                  # every eigenvalue twice, zero blocks
+    (50, 33, 7, "constant"),                                                 # all rows the same: the zero matrix
+])
+def test_leading_eigenpairs_of_special_spectra(n, d, p, kind):
+    rng = np.random.default_rng(n * d + p)
+    if kind == "full":
+        Y = rng.normal(size=(n, d)) * np.linspace(3.0, 1.0, d) + 5.0
+    elif kind == "constant":
+        Y = np.ones((n, d)) * rng.normal(size=d)
+    else:
+        # rows +-s_j e_j: the covariance is diagonal with entries proportional to s_j^2
+        s = np.ones(d) if kind == "equal" else np.repeat(np.arange(d // 2, 0, -1.0), 2)
+        Y = np.concatenate([np.diag(s), -np.diag(s)] * (n // (2 * d)))
+    Y = Y.astype(np.float32)
+    mean, comps, eig = B.cat_pca_fit(dev(Y), p, want_eigenvalues=True)
+    q = min(d, p + 1)
+    _, o_comps, o_eig = P.pca_fit(Y, q)
+    top = max(float(o_eig[0]), 1e-30)
+    # both sides are within a few D ulp of the largest eigenvalue
+    np.testing.assert_allclose(host(eig), o_eig[:p], rtol=1e-9, atol=8 * d * 2.3e-16 * top)
+    C = host(comps).astype(np.float64)
+    np.testing.assert_allclose(C @ C.T, np.eye(p), atol=1e-6)
+    # leading subspaces that the spectrum separates from the rest
+    for r in sorted({1, p // 2, p}):
+        if r >= 1 and r < q and o_eig[r - 1] - o_eig[r] > 1e-4 * top:
+            assert P.projector_distance(C[:r], o_comps[:r]) < 1e-5
+    again = B.cat_pca_fit(dev(Y), p)
+    assert torch.equal(again[1], comps)
