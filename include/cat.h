@@ -25,7 +25,7 @@
  *   - Inputs must be finite.  Non-finite values give unspecified labels but
  *     never an out-of-range label or an invalid memory access.
  *   - Limits: 1 <= K <= CAT_MAX_K, K <= N < 2^31 (cat_fit and the step-level sums:
- *     N < 2^30), 1 <= D <= CAT_MAX_D.  D % 4 != 0 is supported through scalar loads (slower).
+ *     N < 2^30), 1 <= D <= CAT_MAX_D.  D % 4 != 0 goes through padded copies or scalar loads (slower).
  */
 #ifndef CAT_H_
 #define CAT_H_
@@ -388,7 +388,8 @@ cat_status_t cat_selftest_wait_timeout(void *workspace, size_t workspace_bytes, 
 
 /* Kernel selection for the distance contraction.  With K >= min_k (and D % 4 == 0,
  * K <= 256) the scores are formed on the tensor cores (tcgen05, TF32 or fp16 operands, fp32
- * accumulation); below it on the fp32 pipes.  Either way undecided rows are settled in
+ * accumulation); below it on the fp32 pipes.  Rows with D % 4 != 0 are scored from a padded fp16 copy
+ * where K >= min_k / 4 and K * D >= 1024.  Either way undecided rows are settled in
  * fp64, so the labels are the same.  Default 8: measured at K = 8, 16 and 32 (rows of 1000
  * columns) a Lloyd round takes half the time on the tensor path and so does inference, except
  * where low-precision scores leave most rows undecided (unimodal data, K = 32: there the fp32

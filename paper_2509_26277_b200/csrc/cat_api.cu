@@ -27,7 +27,8 @@ struct Carver {
     }
 };
 
-static void carve_assign_into(Carver &c, AssignWs &w, int64_t N, int D, int K)
+// row_copy: room for an fp16 copy of the rows (assignments of rows that TMA cannot address)
+static void carve_assign_into(Carver &c, AssignWs &w, int64_t N, int D, int K, bool row_copy)
 {
     w.ctl = c.take<Control>(1);
     w.cnorm = c.take<float>((size_t)K);
@@ -38,15 +39,17 @@ static void carve_assign_into(Carver &c, AssignWs &w, int64_t N, int D, int K)
     w.ynorm2 = c.take<float>((size_t)N);
     w.cand_rows = c.take<int32_t>((size_t)N);
     w.cand_list = c.take<uint64_t>((size_t)N);
-    w.ch = c.take<uint16_t>((size_t)K * D);
-    w.hscale = c.take<float>(4);
+    w.cmax = c.take<float>((size_t)K);
+    w.ch = c.take<uint16_t>((size_t)K * half_ld(D));
+    w.hscale = c.take<float>(row_copy ? 4 + (size_t)N : 4);
+    w.yh = row_copy ? c.take<uint16_t>((size_t)N * half_ld(D)) : nullptr;
 }
 
 AssignWs carve_assign(void *base, int64_t N, int D, int K)
 {
     Carver c(base);
     AssignWs w{};
-    carve_assign_into(c, w, N, D, K);
+    carve_assign_into(c, w, N, D, K, D % 4 != 0 && D >= TC_HALF_MIN_D && K <= 256);
     w.bytes = align_up(c.off, 256);
     return w;
 }
@@ -55,7 +58,7 @@ FitWs carve_fit(void *base, int64_t N, int D, int K)
 {
     Carver c(base);
     FitWs w{};
-    carve_assign_into(c, w.a, N, D, K);
+    carve_assign_into(c, w.a, N, D, K, false);
     SegGeom g = seg_geometry(2 * N, D, 2 * K);   // delta mode is the larger of the two
     size_t KD = (size_t)K * D;
     w.blk_hist = c.take<uint32_t>((size_t)g.nblk * 2 * K);
@@ -70,8 +73,8 @@ FitWs carve_fit(void *base, int64_t N, int D, int K)
         const size_t a = (size_t)g.max_segs * 2, b = (size_t)gf.max_segs * 3;
         w.segpart = c.take<double>((a > b ? a : b) * D);
     }
-    w.yh = c.take<uint16_t>((size_t)N * D);
-    w.ch = c.take<uint16_t>(KD);
+    w.yh = c.take<uint16_t>((size_t)N * half_ld(D));
+    w.ch = c.take<uint16_t>((size_t)K * half_ld(D));
     w.hscale = c.take<float>(4 + (size_t)N);
     w.sumQ = c.take<double>(KD);
     w.sumF = c.take<double>(KD);
@@ -111,6 +114,17 @@ static bool use_tensor_path(int64_t N, int D, int K)
     return K >= g_tc_min_k.load(std::memory_order_relaxed) && tc_supported(N, D, K);
 }
 
+// Assignments on fp16 copies of rows and centroids.  Rows that need padding (D % 8 != 0) have to earn
+// the copy: measured over ten rounds, 100 000 x 10 with K = 16 takes 491 us with it and 443 without,
+// K = 128 takes 642 and 820, 20 000 x 33 with K = 64 457 and 469.  Where D % 4 != 0 the alternative is scalar
+// loads on the fp32 pipes, which loses from a quarter of the usual K on (49 999 x 1001, K = 3: 4.1 ms).
+static bool use_half_path(int64_t N, int D, int K)
+{
+    const int min_k = g_tc_min_k.load(std::memory_order_relaxed);
+    if (D % 8 != 0 && (int64_t)D * K < 1024) return false;
+    return K >= (D % 4 != 0 ? min_k / 4 + (min_k % 4 != 0) : min_k) && tc_half_supported(N, D, K);
+}
+
 // the persistent single-launch kernels take the small shapes they support, unless switched off
 static bool use_small_fit(int64_t N, int D, int K)
 {
@@ -136,22 +150,42 @@ static cat_status_t run_assign(const float *Y, int64_t N, int D, int K, const fl
         CAT_CUDA(launch_small_apply(Y, N, D, K, C, gamma, beta, out, labels, w.ctl, s));
         return CAT_OK;
     }
-    // centroids_ready: the centroid update that produced C has already left its norms, its fp16
-    // copy and empty exact-pass queues in the workspace
-    if (!centroids_ready) CAT_CUDA(launch_centroid_norms(C, D, K, w.cnorm, w.ctl, s, top_level));
-    if (out && use_tensor_path(N, D, K) && choose_apply_form(N, D, K) == 64) {
+    if (K == 1 && !fast) {   // one cluster: nothing to decide
+        if (top_level) CAT_CUDA(launch_reset_control(w.ctl, s));
+        CAT_CUDA(cudaMemsetAsync(labels, 0, (size_t)N * sizeof(int32_t), s));
+        if (out) CAT_CUDA(launch_affine_labels(Y, N, D, K, labels, gamma, beta, out, s));
+        return CAT_OK;
+    }
+    if (out && !fast && use_tensor_path(N, D, K) && choose_apply_form(N, D, K) == 64) {
         // inference on 64-row tiles: fp16 copy of the centroids (scaled by a power of two from
         // their largest magnitude), rows converted inside the kernel
-        CAT_CUDA(launch_absmax(C, (size_t)K * D, w.hscale, s));
-        CAT_CUDA(launch_half_scale(w.hscale, s));
-        CAT_CUDA(launch_to_half(C, (size_t)K * D, w.hscale, w.ch, s));
+        CAT_CUDA(launch_centroid_half(C, D, K, w.cnorm, w.cmax, w.hscale, w.ch, w.ctl, s, top_level));
         CAT_CUDA(launch_apply_h64(Y, N, D, K, w.ch, w.hscale, w.cnorm, labels, w.refine_rows, w.cand_rows, w.cand_list,
                                   w.ctl, gamma, beta, out, s));
         CAT_CUDA(launch_refine_both(Y, N, D, K, C, labels, w.cand_rows, w.cand_list, w.refine_rows, w.ctl, gamma,
                                     beta, out, s));
-    } else if (use_tensor_path(N, D, K)) {
+        return CAT_OK;
+    }
+    if (w.yh && !Yh && !fast && use_half_path(N, D, K)) {
+        // Rows whose length TMA cannot address (D % 4 != 0): scored from a padded fp16 copy, as in a fit,
+        // then corrected in a pass of their own -- 16 bytes of traffic per element against 8, but on the
+        // tensor cores (49 999 x 1001, K = 50: 233 us against 1546 us on the fp32 pipes, whose loads of
+        // such rows are scalar).
+        CAT_CUDA(launch_half_shadow(Y, N, D, w.ynorm2, w.hscale, w.yh, s, false));
+        CAT_CUDA(launch_centroid_half(C, D, K, w.cnorm, w.cmax, w.hscale, w.ch, w.ctl, s, top_level));
+        CAT_CUDA(launch_assign_tc(Y, N, D, K, C, w.cnorm, w.ynorm2, labels, w.refine_rows, w.cand_rows, w.cand_list, w.ctl,
+                                  nullptr, nullptr, nullptr, s, w.yh, w.ch, w.hscale));
+        CAT_CUDA(launch_refine_both(Y, N, D, K, C, labels, w.cand_rows, w.cand_list, w.refine_rows, w.ctl, nullptr,
+                                    nullptr, nullptr, s));
+        if (out) CAT_CUDA(launch_affine_labels(Y, N, D, K, labels, gamma, beta, out, s));
+        return CAT_OK;
+    }
+    // centroids_ready: the centroid update that produced C has already left its norms, its fp16
+    // copy and empty exact-pass queues in the workspace
+    if (!centroids_ready) CAT_CUDA(launch_centroid_norms(C, D, K, w.cnorm, w.ctl, s, top_level));
+    if (Yh || use_tensor_path(N, D, K)) {
         if (!out && !row_norms_ready) CAT_CUDA(launch_row_norms(Y, N, D, w.ynorm2, s));
-        if (Yh && !centroids_ready) CAT_CUDA(launch_to_half(C, (size_t)K * D, hscale, Ch, s));
+        if (Yh && !centroids_ready) CAT_CUDA(launch_to_half(C, D, K, hscale, Ch, s));
         CAT_CUDA(launch_assign_tc(Y, N, D, K, C, w.cnorm, w.ynorm2, labels, w.refine_rows, w.cand_rows,
                                   w.cand_list, w.ctl, gamma, beta, out, s, Yh, Ch, hscale, fast));
         CAT_CUDA(launch_refine_both(Y, N, D, K, C, labels, w.cand_rows, w.cand_list, w.refine_rows, w.ctl, gamma,
@@ -281,10 +315,7 @@ cat_status_t cat_apply_bf16(const float *Yq, int64_t N, int32_t D, int32_t K, co
     if (use_tensor_path(N, D, K) && apply_h64_supported(N, D, K)) {
         // fused: the 64-row-tile kernel writes bf16 with the fast labels; the exact pass settles the
         // undecided rows' labels, and those rows are written once more
-        CAT_CUDA(launch_centroid_norms(centroids, D, K, w.cnorm, w.ctl, s, true));
-        CAT_CUDA(launch_absmax(centroids, (size_t)K * D, w.hscale, s));
-        CAT_CUDA(launch_half_scale(w.hscale, s));
-        CAT_CUDA(launch_to_half(centroids, (size_t)K * D, w.hscale, w.ch, s));
+        CAT_CUDA(launch_centroid_half(centroids, D, K, w.cnorm, w.cmax, w.hscale, w.ch, w.ctl, s, true));
         CAT_CUDA(launch_apply_h64(Yq, N, D, K, w.ch, w.hscale, w.cnorm, labels, w.refine_rows, w.cand_rows, w.cand_list, w.ctl,
                                   gamma, beta, reinterpret_cast<float *>(Y_out_bf16), s, true));
         CAT_CUDA(launch_refine_both(Yq, N, D, K, centroids, labels, w.cand_rows, w.cand_list, w.refine_rows, w.ctl, nullptr,
@@ -330,13 +361,13 @@ cat_status_t cat_assign_scores(const float *Yq, int64_t N, int32_t D, int32_t K,
     }
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     if (flags & CAT_ASSIGN_FP16_OPERANDS) {
-        if (!tc_half_supported(N, D, K) || N >= ((int64_t)1 << 30)) return CAT_ERR_UNSUPPORTED;
+        if (!tc_half_supported(N, D, K) || D % 8 != 0 || N >= ((int64_t)1 << 30)) return CAT_ERR_UNSUPPORTED;
         if (!workspace || !aligned16(workspace) || workspace_bytes < cat_fit_workspace_bytes(N, D, K))
             return CAT_ERR_WORKSPACE;
         FitWs w = carve_fit(workspace, N, D, K);
         CAT_CUDA(launch_centroid_norms(centroids, D, K, w.a.cnorm, w.a.ctl, s, true));
         CAT_CUDA(launch_half_shadow(Yq, N, D, w.a.ynorm2, w.hscale, w.yh, s));
-        CAT_CUDA(launch_to_half(centroids, (size_t)K * D, w.hscale, w.ch, s));
+        CAT_CUDA(launch_to_half(centroids, D, K, w.hscale, w.ch, s));
         CAT_CUDA(launch_assign_tc(Yq, N, D, K, centroids, w.a.cnorm, w.a.ynorm2, labels_out, w.a.refine_rows,
                                   w.a.cand_rows, w.a.cand_list, w.a.ctl, nullptr, nullptr, nullptr, s, w.yh, w.ch,
                                   w.hscale, &fast));
@@ -390,12 +421,12 @@ cat_status_t cat_fit_from(const float *Yq, const float *Yfp, int64_t N, int32_t 
                                   w.counts, w.a.ctl, &bar_count, s));
     }
 
-    const bool tc = use_tensor_path(N, D, K);
     // Yq is fixed over the fit: its row norms, and where the shape allows an fp16 copy for the
     // tensor cores, are made once
     // (only with the default start: centroids that are rows or means of rows cannot exceed the
     // largest magnitude of Yq, which sets the fp16 scale; caller-provided ones could overflow it)
-    const bool half = tc && !init_centroids && tc_half_supported(N, D, K);
+    const bool half = !init_centroids && use_half_path(N, D, K);
+    const bool tc = half || use_tensor_path(N, D, K);
     const void *Yh = half ? w.yh : nullptr;
     if (small) {
     } else if (half) CAT_CUDA(launch_half_shadow(Yq, N, D, w.a.ynorm2, w.hscale, w.yh, s));
@@ -479,10 +510,9 @@ cat_status_t cat_fit_shard_begin(const float *Yq, int64_t N, int32_t D, int32_t 
     FitWs w = carve_fit(workspace, N, D, K);
     CAT_CUDA(launch_reset_control(w.a.ctl, s));
     CAT_CUDA(cudaMemsetAsync(w.hscale, 0, 4 * sizeof(float), s));
-    const bool tc = use_tensor_path(N, D, K);
-    if (tc && tc_half_supported(N, D, K))
+    if (use_half_path(N, D, K))
         CAT_CUDA(launch_half_shadow(Yq, N, D, w.a.ynorm2, w.hscale, w.yh, s, false));
-    else if (tc)
+    else if (use_tensor_path(N, D, K))
         CAT_CUDA(launch_row_norms(Yq, N, D, w.a.ynorm2, s));
     // (the bit pattern of a non-negative float is the float itself)
     CAT_CUDA(cudaMemcpyAsync(amax_out, w.hscale, sizeof(float), cudaMemcpyDeviceToDevice, s));
@@ -508,8 +538,8 @@ cat_status_t cat_fit_shard_round(const float *Yq, int64_t N, int32_t D, int32_t 
         return CAT_ERR_WORKSPACE;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     FitWs w = carve_fit(workspace, N, D, K);
-    const bool tc = use_tensor_path(N, D, K);
-    const bool half = tc && tc_half_supported(N, D, K);
+    const bool half = use_half_path(N, D, K);
+    const bool tc = half || use_tensor_path(N, D, K);
     // the two label buffers of the workspace alternate; round 0 reads the all -1 buffer cat_fit_shard_begin left
     int32_t *cur = (round & 1) ? w.labels_prev : w.a.labels;
     int32_t *prev = (round & 1) ? w.a.labels : w.labels_prev;

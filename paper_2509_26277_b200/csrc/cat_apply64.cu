@@ -550,38 +550,11 @@ apply_h64_kernel(const __grid_constant__ CUtensorMap mapY, const __grid_constant
     }
 }
 
-// largest magnitude of a matrix (float bits, atomicMax into *amax_bits, which starts at 0)
-__global__ void __launch_bounds__(256) absmax_kernel(const float4 *__restrict__ src, size_t n4, unsigned int *amax_bits)
-{
-    pdl_enter();
-    float m = 0.f;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
-        const float4 v = __ldg(src + i);
-        m = fmaxf(fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y))), fmaxf(fabsf(v.z), fabsf(v.w)));
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0 && m == m && m < CUDART_INF_F) atomicMax(amax_bits, __float_as_uint(m));
-}
-
 }  // namespace
 
 bool apply_h64_supported(int64_t N, int D, int K)
 {
     return tc_supported(N, D, K) && D >= 128 && (D % 8 == 0) && N > H_ROWS;
-}
-
-cudaError_t launch_absmax(const float *src, size_t n, float *scale, cudaStream_t s)
-{
-    cudaError_t e = cudaMemsetAsync(scale, 0, 4 * sizeof(float), s);
-    if (e != cudaSuccess) return e;
-    const size_t n4 = n / 4;
-    size_t cb = (n4 + 255) / 256;
-    if (cb > (size_t)tc_sm_count()) cb = (size_t)tc_sm_count();
-    if (cb < 1) cb = 1;
-    absmax_kernel<<<(unsigned)cb, 256, 0, s>>>(reinterpret_cast<const float4 *>(src), n4, reinterpret_cast<unsigned int *>(scale));
-    count_launch();
-    return cudaGetLastError();
 }
 
 cudaError_t launch_apply_h64(const float *Y, int64_t N, int D, int K, const void *Ch, const float *scale,

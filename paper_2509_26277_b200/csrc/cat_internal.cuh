@@ -94,8 +94,10 @@ struct AssignWs {          // what assign/apply need
     float *ynorm2;         // [N] squared row norms (tensor-core labels-only path)
     int32_t *cand_rows;    // [N] rows queued with candidates
     uint64_t *cand_list;   // [N] their candidates, 4 x 16 bit
-    void *ch;              // [K*D] fp16 copy of the centroids (inference on fp16 operands)
-    float *hscale;         // [4] scale of that copy: {s_c, -2 / s_c, 2^-25 / s_c, -}
+    float *cmax;           // [K] largest magnitude of each centroid
+    void *ch;              // [K][half_ld(D)] fp16 copy of the centroids (inference on fp16 operands)
+    float *hscale;         // [4] scale of that copy: {s_c, -2 / s_c, 2^-25 / s_c, -}; with yh followed by [N] inverse row scales
+    void *yh;              // [N][half_ld(D)] fp16 copy of the rows (inference with D % 4 != 0), else null
     size_t bytes;
 };
 AssignWs carve_assign(void *base, int64_t N, int D, int K);
@@ -110,8 +112,8 @@ struct FitWs {
     int32_t *order;        // [2N] row indices sorted by key (stable)
     int32_t *labels_prev;  // [N] labels of the previous Lloyd round
     double *segpart;       // [max_segs][2][D] per-segment partial sums
-    void *yh;              // [N*D] fp16 copy of Yq (tensor-core fits with D % 8 == 0)
-    void *ch;              // [K*D] fp16 copy of the centroids
+    void *yh;              // [N][half_ld(D)] fp16 copy of Yq (tensor-core fits)
+    void *ch;              // [K][half_ld(D)] fp16 copy of the centroids
     float *hscale;         // [4 + N] scale of the fp16 centroids, then the inverse row scales
     double *sumQ, *sumF, *var, *cov;   // [K*D] each
     double *meanQ, *meanF;             // [K*D] each
@@ -163,9 +165,8 @@ void set_apply_column_split(int cs);
 int get_apply_column_split();
 int choose_apply_form(int64_t N, int D, int K);   // 1, 2, 4 or 64 for this shape under the current setting
 // 64-row-tile inference kernel on fp16 operands (cat_apply64.cu).  Ch = fp16(C * scale[0]) and
-// scale = {s_c, -2 / s_c, 2^-25 / s_c, -} come from launch_absmax + launch_half_scale + launch_to_half.
+// scale = {s_c, -2 / s_c, 2^-25 / s_c, -} come from launch_centroid_half.
 bool apply_h64_supported(int64_t N, int D, int K);
-cudaError_t launch_absmax(const float *src, size_t n, float *scale, cudaStream_t s);   // scale[0] <- bits of max |src|
 cudaError_t launch_half_scale(float *scale, cudaStream_t s);                           // bits of the maximum -> the three scale words
 cudaError_t launch_apply_h64(const float *Y, int64_t N, int D, int K, const void *Ch, const float *scale,
                              const float *cnorm, int32_t *labels, int32_t *refine_rows, int32_t *cand_rows,
@@ -190,14 +191,22 @@ cudaError_t launch_wait_selftest(Control *ctl, int limit_ms, cudaStream_t s);
 
 // fp16 copy of a matrix for repeated assignments, made in one sweep: squared row norms, per-row
 // power-of-two scales, Yh[i] = fp16(Y[i] * scale_i), and scale[4 + N] = {centroid scale s_c from the
-// largest magnitude, -2 / s_c, 2^-25 / s_c, unused, then 1 / scale_i for every row}.  Needs D % 8 == 0.
+// largest magnitude, -2 / s_c, 2^-25 / s_c, unused, then 1 / scale_i for every row}.  Rows of the copies
+// (of the centroids too) are half_ld(D) elements apart, so that any row length suits the tensor maps.
+__host__ __device__ constexpr int half_ld(int D) { return (D + 7) & ~7; }
+constexpr int TC_HALF_MIN_D = 8;
 bool tc_half_supported(int64_t N, int D, int K);
 // finish_scale = false leaves the bits of the largest magnitude in scale[0] (launch_half_scale turns them
 // into the three scale words later, e.g. once the maximum over several shards is known).
 cudaError_t launch_half_shadow(const float *Y, int64_t N, int D, float *ynorm2, float *scale, void *Yh,
                                cudaStream_t s, bool finish_scale = true);
-// dst = fp16(src * scale[0]) for n elements (n % 4 == 0)
-cudaError_t launch_to_half(const float *src, size_t n, const float *scale, void *dst, cudaStream_t s);
+// Ch = fp16(C * scale[0])
+cudaError_t launch_to_half(const float *C, int D, int K, const float *scale, void *Ch, cudaStream_t s);
+// Everything an assignment on fp16 operands needs of the centroids: norms, the scale words from their
+// largest magnitude (cmax: [K] scratch), the fp16 copy; empties the exact-pass queues as
+// launch_centroid_norms does.
+cudaError_t launch_centroid_half(const float *C, int D, int K, float *cnorm, float *cmax, float *scale, void *Ch, Control *ctl,
+                                 cudaStream_t s, bool reset_all);
 
 // Exact fp64 decision among the listed candidates of each queued row; optional affine output.
 cudaError_t launch_refine_both(const float *Y, int64_t N, int D, int K, const float *C, int32_t *labels,
@@ -258,6 +267,10 @@ cudaError_t launch_fit_diag_round(const float *Y, int64_t N, int D, int K, const
                                   const int32_t *refine_rows, const int32_t *cand_rows, const Control *ctl,
                                   cat_fit_diag_t *diag, int slot, int recorded, cudaStream_t s);
 cudaError_t launch_reset_control(Control *ctl, cudaStream_t s);
+
+// Y_out_i = gamma_l * Y_i + beta_l, l = labels[i]; a label outside [0, K) copies the row
+cudaError_t launch_affine_labels(const float *Y, int64_t N, int D, int K, const int32_t *labels, const float *gamma,
+                                 const float *beta, float *out, cudaStream_t s);
 
 // The p largest eigenpairs of the symmetric positive semi-definite matrix A [D, D] (full, fp64; overwritten),
 // whose diagonal is also given: unit vectors -> comps [p, D] (fp32 rows, decreasing eigenvalue, entry of largest

@@ -159,14 +159,16 @@ __global__ void __launch_bounds__(P_THREADS) project_kernel(const float *__restr
 }
 
 // ---------------------------------------------------------------- affine map for given cluster ids
-// one warp per row: out = fma(gamma_l, y, beta_l); a label outside [0, K) leaves the row as it is
+// one warp per row: out = fma(gamma_l, y, beta_l); a label outside [0, K) leaves the row as it is.
+// All loads of a step (eight per lane and operand) are in flight together.
+template <int VEC>
 __global__ void __launch_bounds__(256) affine_labels_kernel(const float *__restrict__ Y, int64_t N, int D, int K,
                                                             const int32_t *__restrict__ labels,
                                                             const float *__restrict__ gamma, const float *__restrict__ beta,
                                                             float *__restrict__ out)
 {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
-    const bool vec4 = (D & 3) == 0;
     for (int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); row < N; row += (int64_t)gridDim.x * 8) {
         const int l = labels[row];
         const bool ok = l >= 0 && l < K;
@@ -174,20 +176,48 @@ __global__ void __launch_bounds__(256) affine_labels_kernel(const float *__restr
         const float *g = gamma + (size_t)(ok ? l : 0) * D;
         const float *b = beta + (size_t)(ok ? l : 0) * D;
         float *o = out + (size_t)row * D;
-        if (vec4) {
-            for (int j = lane; j < (D >> 2); j += 32) {
-                const float4 yv = __ldcs(reinterpret_cast<const float4 *>(y) + j);
-                float4 v = yv;
-                if (ok) {
-                    const float4 gv = __ldg(reinterpret_cast<const float4 *>(g) + j);
-                    const float4 bv = __ldg(reinterpret_cast<const float4 *>(b) + j);
-                    v = make_float4(fmaf(gv.x, yv.x, bv.x), fmaf(gv.y, yv.y, bv.y), fmaf(gv.z, yv.z, bv.z),
-                                    fmaf(gv.w, yv.w, bv.w));
+        if (VEC == 4) {
+            const int D4 = D >> 2;
+            for (int j0 = lane; j0 < D4; j0 += 128) {
+                float4 yv[4], gv[4], bv[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int j = j0 + 32 * u;
+                    if (j < D4) {
+                        yv[u] = __ldcs(reinterpret_cast<const float4 *>(y) + j);
+                        gv[u] = __ldg(reinterpret_cast<const float4 *>(g) + j);
+                        bv[u] = __ldg(reinterpret_cast<const float4 *>(b) + j);
+                    }
                 }
-                __stcs(reinterpret_cast<float4 *>(o) + j, v);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int j = j0 + 32 * u;
+                    if (j >= D4) continue;
+                    float4 v = yv[u];
+                    if (ok)
+                        v = make_float4(fmaf(gv[u].x, v.x, bv[u].x), fmaf(gv[u].y, v.y, bv[u].y), fmaf(gv[u].z, v.z, bv[u].z),
+                                        fmaf(gv[u].w, v.w, bv[u].w));
+                    __stcs(reinterpret_cast<float4 *>(o) + j, v);
+                }
             }
         } else {
-            for (int j = lane; j < D; j += 32) o[j] = ok ? fmaf(g[j], y[j], b[j]) : y[j];
+            for (int j0 = lane; j0 < D; j0 += 256) {
+                float yv[8], gv[8], bv[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int j = j0 + 32 * u;
+                    if (j < D) {
+                        yv[u] = __ldg(y + j);
+                        gv[u] = __ldg(g + j);
+                        bv[u] = __ldg(b + j);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int j = j0 + 32 * u;
+                    if (j < D) o[j] = ok ? fmaf(gv[u], yv[u], bv[u]) : yv[u];
+                }
+            }
         }
     }
 }
@@ -290,6 +320,17 @@ inline bool al16(const void *q) { return (reinterpret_cast<uintptr_t>(q) & 15u) 
 
 }  // namespace
 
+cudaError_t launch_affine_labels(const float *Y, int64_t N, int D, int K, const int32_t *labels, const float *gamma,
+                                 const float *beta, float *out, cudaStream_t s)
+{
+    int64_t blocks = (N + 7) / 8;
+    if (blocks > 148 * 16) blocks = 148 * 16;
+    const cudaError_t e = launch_pdl(D % 4 == 0 ? affine_labels_kernel<4> : affine_labels_kernel<1>, dim3((unsigned)blocks), dim3(256),
+                                     0, s, Y, N, D, K, labels, gamma, beta, out);
+    count_launch();
+    return e;
+}
+
 cudaError_t launch_affine_bf16(const float *Y, int64_t N, int D, int K, const int32_t *labels, const float *gamma,
                                const float *beta, void *out_bf16, const int32_t *refine_rows, const int32_t *cand_rows,
                                const Control *ctl, cudaStream_t s)
@@ -378,11 +419,7 @@ cat_status_t cat_affine_with_labels(const float *Yq, int64_t N, int32_t D, int32
     if (K > CAT_MAX_K || D > CAT_MAX_D || N >= ((int64_t)1 << 31)) return CAT_ERR_UNSUPPORTED;
     if (!al16(Yq) || !al16(labels) || !al16(gamma) || !al16(beta) || !al16(Y_out)) return CAT_ERR_ALIGN;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    int64_t blocks = (N + 7) / 8;
-    if (blocks > 148 * 16) blocks = 148 * 16;
-    affine_labels_kernel<<<(unsigned)blocks, 256, 0, s>>>(Yq, N, D, K, labels, gamma, beta, Y_out);
-    count_launch();
-    CAT_CUDA(cudaGetLastError());
+    CAT_CUDA(launch_affine_labels(Yq, N, D, K, labels, gamma, beta, Y_out, s));
     return CAT_OK;
 }
 

@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(1024) centroid_update_kernel(const double *__r
             C[e] = c;
         }
         nrm += (double)c * (double)c;
-        if (Ch) Ch[e] = __float2half_rn(c * sc);
+        if (Ch) Ch[(size_t)k * half_ld(D) + j] = __float2half_rn(c * sc);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, o);

@@ -878,19 +878,25 @@ __global__ void row_norms_kernel(const float *__restrict__ Y, int64_t N, int D, 
     }
 }
 
-// scale[0] = s_c, the power of two that brings the largest magnitude of the matrix (the bits
-// left in scale[0] by the shadow kernel) to [2^13, 2^14); scale[1] = -2 / s_c (times 1 / row scale
-// it turns the fp16 accumulator into -2 y.c); scale[2] = 2^-25 / s_c.
-__global__ void half_scale_kernel(float *scale)
+// the power of two that brings amax to [2^13, 2^14)
+__device__ __forceinline__ float half_scale_of(float amax)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    const float amax = __uint_as_float(reinterpret_cast<unsigned int *>(scale)[0]);
     int e = 0;
     if (amax > 0.f) frexpf(amax, &e);    // amax = f * 2^e, f in [0.5, 1)
     int sh = 14 - e;
     if (sh > 100) sh = 100;
     if (sh < -100) sh = -100;
-    const float sc = ldexpf(1.f, sh);
+    return ldexpf(1.f, sh);
+}
+
+// scale[0] = s_c, the power of two for the largest magnitude of the matrix (whose bits the shadow
+// kernel left in scale[0]); scale[1] = -2 / s_c (times 1 / row scale it turns the fp16 accumulator
+// into -2 y.c); scale[2] = 2^-25 / s_c.
+__global__ void half_scale_kernel(float *scale)
+{
+    pdl_enter();
+    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    const float sc = half_scale_of(__uint_as_float(reinterpret_cast<unsigned int *>(scale)[0]));
     scale[0] = sc;
     scale[1] = -2.f / sc;
     scale[2] = 2.9802322e-8f / sc;
@@ -898,14 +904,19 @@ __global__ void half_scale_kernel(float *scale)
 
 // One sweep over the rows: squared norm (slightly over-estimated), the row's own power-of-two
 // scale s_i (largest magnitude to [2^13, 2^14)), rinv[i] = 1 / s_i, Yh[i, :] = fp16(Y[i, :] * s_i)
-// rounded to nearest, and the largest magnitude of the matrix (float bits, one atomicMax per CTA).
-// A row is handled by G lanes and read twice; the second read comes out of L1/L2.
-__global__ void __launch_bounds__(256) half_shadow_kernel(const float *__restrict__ Y, int64_t N, int D, int G,
+// rounded to nearest (rows of Yh ld elements apart), and the largest magnitude of the matrix (float
+// bits, one atomicMax per CTA).  A row is handled by G lanes and read twice; the second read comes
+// out of L1/L2.  VEC4: 128-bit loads (D % 4 == 0); otherwise a lane takes pairs of columns with
+// scalar loads, whose warp-wide accesses still cover whole lines.
+template <bool VEC4>
+__global__ void __launch_bounds__(256) half_shadow_kernel(const float *__restrict__ Y, int64_t N, int D, int ld, int G,
                                                           float *__restrict__ ynorm2, float *__restrict__ rinv,
                                                           unsigned int *__restrict__ amax_bits, __half *__restrict__ Yh)
 {
+    pdl_enter();
     __shared__ float wmax[8];
-    const int D4 = D >> 2;
+    constexpr int V = VEC4 ? 4 : 2;
+    const int DV = (D + V - 1) / V;
     const int rows_per_cta = 256 / G;
     const int sub = threadIdx.x / G, c0 = threadIdx.x % G;
     float cta_max = 0.f;
@@ -914,23 +925,31 @@ __global__ void __launch_bounds__(256) half_shadow_kernel(const float *__restric
     for (int64_t base = (int64_t)blockIdx.x * rows_per_cta; base < N; base += (int64_t)gridDim.x * rows_per_cta) {
         const int64_t row = base + sub;
         const bool live = row < N;
-        const float4 *y4 = reinterpret_cast<const float4 *>(Y + (size_t)(live ? row : 0) * D);
+        const float *y = Y + (size_t)(live ? row : 0) * D;
         float s = 0.f, m = 0.f;
-        for (int c = c0; c < D4; c += 8 * G) {
-            float4 v[8];
+        for (int c = c0; c < DV; c += 8 * G) {
+            float v[8][V];
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const int cc = c + u * G;
-                v[u] = (live && cc < D4) ? __ldg(y4 + cc) : make_float4(0.f, 0.f, 0.f, 0.f);
+                if (VEC4) {
+                    const float4 t = (live && cc < DV) ? __ldg(reinterpret_cast<const float4 *>(y) + cc) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    v[u][0] = t.x;
+                    v[u][1] = t.y;
+                    v[u][V - 2] = t.z;
+                    v[u][V - 1] = t.w;
+                } else {
+                    v[u][0] = (live && cc < DV) ? __ldg(y + 2 * cc) : 0.f;
+                    v[u][1] = (live && 2 * cc + 1 < D) ? __ldg(y + 2 * cc + 1) : 0.f;
+                }
             }
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                s = fmaf(v[u].x, v[u].x, s);
-                s = fmaf(v[u].y, v[u].y, s);
-                s = fmaf(v[u].z, v[u].z, s);
-                s = fmaf(v[u].w, v[u].w, s);
-                m = fmaxf(fmaxf(m, fmaxf(fabsf(v[u].x), fabsf(v[u].y))), fmaxf(fabsf(v[u].z), fabsf(v[u].w)));
-            }
+            for (int u = 0; u < 8; ++u)
+#pragma unroll
+                for (int q = 0; q < V; ++q) {
+                    s = fmaf(v[u][q], v[u][q], s);
+                    m = fmaxf(m, fabsf(v[u][q]));
+                }
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -951,15 +970,22 @@ __global__ void __launch_bounds__(256) half_shadow_kernel(const float *__restric
             rinv[row] = ldexpf(1.f, -sh);
         }
         if (m == m && m < CUDART_INF_F) cta_max = fmaxf(cta_max, m);
-        uint2 *h4 = reinterpret_cast<uint2 *>(Yh + (size_t)row * D);
-        for (int c = c0; c < D4; c += G) {
-            const float4 v = __ldg(y4 + c);
-            const __half2 lo = __floats2half2_rn(v.x * sc, v.y * sc);
-            const __half2 hi = __floats2half2_rn(v.z * sc, v.w * sc);
-            uint2 o2;
-            o2.x = *reinterpret_cast<const unsigned int *>(&lo);
-            o2.y = *reinterpret_cast<const unsigned int *>(&hi);
-            h4[c] = o2;
+        __half *h = Yh + (size_t)row * ld;
+        if (VEC4) {
+            for (int c = c0; c < DV; c += G) {
+                const float4 v = __ldg(reinterpret_cast<const float4 *>(y) + c);
+                const __half2 lo = __floats2half2_rn(v.x * sc, v.y * sc);
+                const __half2 hi = __floats2half2_rn(v.z * sc, v.w * sc);
+                uint2 o2;
+                o2.x = *reinterpret_cast<const unsigned int *>(&lo);
+                o2.y = *reinterpret_cast<const unsigned int *>(&hi);
+                reinterpret_cast<uint2 *>(h)[c] = o2;
+            }
+        } else {
+#pragma unroll 4
+            for (int c = c0; c < DV; c += G)   // (ld is even and at least D: the pair fits)
+                reinterpret_cast<__half2 *>(h)[c] =
+                    __floats2half2_rn(__ldg(y + 2 * c) * sc, 2 * c + 1 < D ? __ldg(y + 2 * c + 1) * sc : 0.f);
         }
     }
 #pragma unroll
@@ -973,19 +999,82 @@ __global__ void __launch_bounds__(256) half_shadow_kernel(const float *__restric
     }
 }
 
-// dst = fp16(src * scale[0]), round to nearest; n4 = number of float4 groups
-__global__ void to_half_kernel(const float4 *__restrict__ src, size_t n4, const float *__restrict__ scale,
-                               uint2 *__restrict__ dst)
+// dst[k, :] = fp16(src[k, :] * scale[0]), round to nearest; one CTA per row, rows of dst ld apart.
+// With cmax (the rows' largest magnitudes) the scale words are made here first (as half_scale_kernel
+// does) and CTA 0 leaves them in `scale`.
+__global__ void __launch_bounds__(256) to_half_kernel(const float *__restrict__ src, int K, int D, int ld,
+                                                      const float *__restrict__ cmax, float *__restrict__ scale,
+                                                      __half *__restrict__ dst)
 {
-    const float sc = scale[0];
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
-        const float4 v = __ldcs(src + i);
-        const __half2 lo = __floats2half2_rn(v.x * sc, v.y * sc);
-        const __half2 hi = __floats2half2_rn(v.z * sc, v.w * sc);
-        uint2 o;
-        o.x = *reinterpret_cast<const unsigned int *>(&lo);
-        o.y = *reinterpret_cast<const unsigned int *>(&hi);
-        dst[i] = o;
+    pdl_enter();
+    __shared__ float wmax[8];
+    float sc;
+    if (cmax) {
+        float m = 0.f;
+        for (int k = threadIdx.x; k < K; k += 256) m = fmaxf(m, cmax[k]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < 8; ++w) m = fmaxf(m, wmax[w]);
+        sc = half_scale_of(m);
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            scale[0] = sc;
+            scale[1] = -2.f / sc;
+            scale[2] = 2.9802322e-8f / sc;
+        }
+    } else
+        sc = scale[0];
+    const float *c = src + (size_t)blockIdx.x * D;
+    __half *h = dst + (size_t)blockIdx.x * ld;
+#pragma unroll 4
+    for (int j = threadIdx.x; j < D; j += 256) h[j] = __float2half_rn(__ldg(c + j) * sc);
+}
+
+// Squared norms (fp64 sum, rounded up) and largest finite magnitudes of the centroids, one CTA each;
+// the exact-pass queues are emptied, with reset_all the status word and counters too.
+__global__ void __launch_bounds__(256) centroid_prep_kernel(const float *__restrict__ C, int D, float *__restrict__ cnorm,
+                                                            float *__restrict__ cmax, Control *ctl, int reset_all)
+{
+    pdl_enter();
+    __shared__ double wsum[8];
+    __shared__ float wmax[8];
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        ctl->refine_count = 0;
+        ctl->cand_count = 0;
+        if (reset_all) {
+            ctl->device_status = CAT_OK;
+            ctl->refined_total = 0;
+            ctl->refined_last = 0;
+        }
+    }
+    const float *c = C + (size_t)blockIdx.x * D;
+    double s = 0.0;
+    float m = 0.f;
+#pragma unroll 4
+    for (int j = threadIdx.x; j < D; j += 256) {
+        const float v = __ldg(c + j);
+        s = fma((double)v, (double)v, s);
+        if (fabsf(v) < CUDART_INF_F) m = fmaxf(m, fabsf(v));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        s += __shfl_xor_sync(0xffffffffu, s, o);
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        wsum[threadIdx.x >> 5] = s;
+        wmax[threadIdx.x >> 5] = m;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) {
+            s += wsum[w];
+            m = fmaxf(m, wmax[w]);
+        }
+        cnorm[blockIdx.x] = __double2float_ru(s);
+        cmax[blockIdx.x] = m;
     }
 }
 
@@ -1027,15 +1116,15 @@ EncodeTiledFn encode_fn()
     return fn;
 }
 
-// 2-D row-major [rows, D] of fp32 (or fp16) viewed in boxes of box_rows x 128 bytes, 128-byte
-// swizzle, zero fill outside the matrix.
+// 2-D row-major [rows, D] of fp32 (or fp16: rows half_ld(D) apart) viewed in boxes of box_rows x 128
+// bytes, 128-byte swizzle, zero fill outside the matrix.
 bool make_map(CUtensorMap *map, const void *base, bool half, int64_t rows, int D, int box_rows)
 {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
     const size_t esz = half ? 2 : 4;
     cuuint64_t dims[2] = {(cuuint64_t)D, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)D * esz};
+    cuuint64_t strides[1] = {(cuuint64_t)(half ? half_ld(D) : D) * esz};
     cuuint32_t box[2] = {(cuuint32_t)(TC_SLAB_BYTES / esz), (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
     CUresult r = fn(map, half ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
@@ -1109,24 +1198,35 @@ cudaError_t launch_half_shadow(const float *Y, int64_t N, int D, float *ynorm2, 
     int64_t blocks = (N + rows_per_cta - 1) / rows_per_cta;
     const int64_t cap = (int64_t)sm_count() * 8;
     if (blocks > cap) blocks = cap;
-    half_shadow_kernel<<<(unsigned)blocks, 256, 0, s>>>(Y, N, D, G, ynorm2, rinv, reinterpret_cast<unsigned int *>(scale),
-                                                        reinterpret_cast<__half *>(Yh));
-    if (finish_scale) half_scale_kernel<<<1, 32, 0, s>>>(scale);
-    count_launch(finish_scale ? 2 : 1);
-    return cudaGetLastError();
+    unsigned int *amax = reinterpret_cast<unsigned int *>(scale);
+    if (D % 4 == 0)
+        e = launch_pdl(half_shadow_kernel<true>, dim3((unsigned)blocks), dim3(256), 0, s, Y, N, D, half_ld(D), G, ynorm2, rinv,
+                       amax, reinterpret_cast<__half *>(Yh));
+    else
+        e = launch_pdl(half_shadow_kernel<false>, dim3((unsigned)blocks), dim3(256), 0, s, Y, N, D, half_ld(D), G, ynorm2, rinv,
+                       amax, reinterpret_cast<__half *>(Yh));
+    if (e != cudaSuccess) return e;
+    count_launch();
+    return finish_scale ? launch_half_scale(scale, s) : cudaGetLastError();
 }
 
-cudaError_t launch_to_half(const float *src, size_t n, const float *scale, void *dst, cudaStream_t s)
+cudaError_t launch_to_half(const float *C, int D, int K, const float *scale, void *Ch, cudaStream_t s)
 {
-    const int threads = 256;
-    const size_t n4 = n / 4;
-    size_t cb = (n4 + threads - 1) / threads;
-    if (cb > (size_t)sm_count() * 16) cb = (size_t)sm_count() * 16;
-    if (cb < 1) cb = 1;
-    to_half_kernel<<<(unsigned)cb, threads, 0, s>>>(reinterpret_cast<const float4 *>(src), n4, scale,
-                                                    reinterpret_cast<uint2 *>(dst));
+    const cudaError_t e = launch_pdl(to_half_kernel, dim3((unsigned)K), dim3(256), 0, s, C, K, D, half_ld(D), nullptr,
+                                     const_cast<float *>(scale), reinterpret_cast<__half *>(Ch));
     count_launch();
-    return cudaGetLastError();
+    return e;
+}
+
+cudaError_t launch_centroid_half(const float *C, int D, int K, float *cnorm, float *cmax, float *scale, void *Ch, Control *ctl,
+                                 cudaStream_t s, bool reset_all)
+{
+    cudaError_t e = launch_pdl(centroid_prep_kernel, dim3((unsigned)K), dim3(256), 0, s, C, D, cnorm, cmax, ctl, reset_all ? 1 : 0);
+    if (e != cudaSuccess) return e;
+    e = launch_pdl(to_half_kernel, dim3((unsigned)K), dim3(256), 0, s, C, K, D, half_ld(D), cmax, scale,
+                   reinterpret_cast<__half *>(Ch));
+    count_launch(2);
+    return e;
 }
 
 cudaError_t launch_wait_selftest(Control *ctl, int limit_ms, cudaStream_t s)
@@ -1246,14 +1346,15 @@ int choose_apply_form(int64_t N, int D, int K) { return choose_column_split(N, D
 
 cudaError_t launch_half_scale(float *scale, cudaStream_t s)
 {
-    half_scale_kernel<<<1, 32, 0, s>>>(scale);
+    const cudaError_t e = launch_pdl(half_scale_kernel, dim3(1), dim3(32), 0, s, scale);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 bool tc_half_supported(int64_t N, int D, int K)
 {
-    return tc_supported(N, D, K) && (D % 8 == 0);
+    // rows of the fp16 copies are padded to 16 bytes, so every length goes
+    return D >= TC_HALF_MIN_D && K <= 256 && N >= 1 && encode_fn() != nullptr;
 }
 
 cudaError_t launch_assign_tc(const float *Y, int64_t N, int D, int K, const float *C, const float *cnorm,

@@ -556,3 +556,38 @@ def test_bounded_device_wait_reports_a_timeout_and_leaves_the_context_usable():
     assert B.cat_workspace_report(ws)["device_status"] == 0
     lab, best, second = O.assign(host(Yq), host(C))
     labels_match(host(labels), lab, best, second, "labels after the self-test")
+
+
+@pytest.mark.parametrize("n,d,k,scale", [(65, 9, 8, 1.0), (300, 10, 64, 1.0), (513, 33, 8, 1.0), (129, 63, 40, 1.0),
+                                         (257, 65, 129, 1.0), (1000, 1001, 50, 1.0), (700, 2047, 256, 1.0),
+                                         (90, 1003, 9, 3.0e4), (600, 510, 100, 2.0e-7)])
+def test_rows_of_any_length_on_padded_fp16_copies(n, d, k, scale):
+    """Row lengths that no tensor map can address (D % 4 != 0) through inference (fp32 and bf16 output,
+    blended too), labels alone and fitting: the scores come from padded fp16 copies there."""
+    Yq = (_rand(n + d, n, d) * scale).astype(np.float32)
+    Yfp = (Yq * 0.9 + 0.05 * scale * _rand(n + d + 1, n, d)).astype(np.float32)
+    C = (_rand(k, k, d) * scale).astype(np.float32)
+    g, b = _rand(k + 1, k, d), (_rand(k + 2, k, d) * scale).astype(np.float32)
+    want, lab, best, second = O.apply(Yq, C, g, b)
+    out, glab = B.cat_apply(dev(Yq), dev(C), dev(g), dev(b), want_labels=True)
+    labels_match(host(glab), lab, best, second, "labels")
+    np.testing.assert_array_equal(host(out), O.affine_with_labels(Yq, host(glab), g, b))
+    assert torch.equal(B.cat_assign(dev(Yq), dev(C)), glab)
+    o16, l16 = B.cat_apply_bf16(dev(Yq), dev(C), dev(g), dev(b), want_labels=True)
+    assert torch.equal(l16, glab) and torch.equal(o16, out.to(torch.bfloat16))
+    half, lh = B.cat_apply_blend(dev(Yq), dev(C), dev(g), dev(b), 0.5, want_labels=True)
+    assert torch.equal(lh, glab)
+    wh = O.affine_with_labels(Yq, host(glab), g, b, 0.5)
+    bound = 1e-6 * scale + 1e-5 * np.abs(wh) + 2.0 ** -24 * (np.abs(g[lab] * Yq) + np.abs(b[lab]))   # as in test_alpha_blend
+    assert (np.abs(host(half) - wh) <= bound).all()
+    if n >= k:
+        Cg, Gg, Bg, lg = B.cat_fit(dev(Yq), dev(Yfp), k, 4)
+        lab2, best2, second2 = O.assign(Yq, host(Cg))
+        labels_match(host(lg), lab2, best2, second2, "fit labels")
+        g_want, b_want = O.solve_gamma_beta(Yq, Yfp, host(lg), k)
+        close(host(Gg), g_want, "gamma")
+        close(host(Bg) / scale, b_want / scale, "beta")
+        ora = O.fit(Yq, Yfp, k, 4, near_rel=1e-5)
+        if ora.near.sum() == 0:
+            assert np.array_equal(host(lg), ora.labels)
+            close(host(Cg) / scale, ora.centroids / scale, "centroids")
