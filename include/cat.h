@@ -404,7 +404,9 @@ int32_t cat_get_tensor_core_min_k(void);
  * rows; K >= the tensor-core threshold above) have persistent single-launch kernels: scores on the
  * tensor cores, undecided rows settled in fp64 inside the kernel, and for fitting the per-cluster
  * sums kept on chip and combined across the grid in a fixed order, all rounds in one launch.
- * mask bit 0: the whole of cat_apply (Algorithm 2) runs that way.  mask bit 1: so do the K-Means
+ * mask bit 0: the whole of cat_apply (Algorithm 2) runs that way; so it does for other shapes with
+ * K <= 128 (K >= a quarter of the threshold, rows up to about 3300 columns), in two launches that keep
+ * each row in shared memory.  mask bit 1: so do the K-Means
  * rounds and the final assignment of cat_fit / cat_fit_from (Algorithm 1, step 2; calls without
  * per-round diagnostics).  Default 3: both are the faster form where they apply.  Clearing a bit
  * sends these shapes down the general multi-launch path instead: same labels (rows on a bisector

@@ -27,9 +27,10 @@ struct Carver {
     }
 };
 
-// row_copy: room for an fp16 copy of the rows (assignments of rows that TMA cannot address)
-static void carve_assign_into(Carver &c, AssignWs &w, int64_t N, int D, int K, bool row_copy)
+// inference: room for what only inference needs (prepared centroids; an fp16 copy of rows that TMA cannot address)
+static void carve_assign_into(Carver &c, AssignWs &w, int64_t N, int D, int K, bool inference)
 {
+    const bool row_copy = inference && D % 4 != 0 && D >= TC_HALF_MIN_D && K <= 256;
     w.ctl = c.take<Control>(1);
     w.cnorm = c.take<float>((size_t)K);
     w.refine_rows = c.take<int32_t>((size_t)N);
@@ -42,6 +43,8 @@ static void carve_assign_into(Carver &c, AssignWs &w, int64_t N, int D, int K, b
     w.cmax = c.take<float>((size_t)K);
     w.ch = c.take<uint16_t>((size_t)K * half_ld(D));
     w.hscale = c.take<float>(row_copy ? 4 + (size_t)N : 4);
+    const size_t prep = inference ? apply_rows_prep_bytes(N, D, K) : 0;
+    w.prep = prep ? c.take<unsigned char>(prep) : nullptr;
     w.yh = row_copy ? c.take<uint16_t>((size_t)N * half_ld(D)) : nullptr;
 }
 
@@ -49,7 +52,7 @@ AssignWs carve_assign(void *base, int64_t N, int D, int K)
 {
     Carver c(base);
     AssignWs w{};
-    carve_assign_into(c, w, N, D, K, D % 4 != 0 && D >= TC_HALF_MIN_D && K <= 256);
+    carve_assign_into(c, w, N, D, K, true);
     w.bytes = align_up(c.off, 256);
     return w;
 }
@@ -135,6 +138,25 @@ static bool use_small_apply(int64_t N, int D, int K)
     return (g_small_kernels.load(std::memory_order_relaxed) & 1) && use_tensor_path(N, D, K) && small_apply_supported(N, D, K);
 }
 
+// The kernel that keeps rows in shared memory, where it is the faster one.
+//   K from a quarter of the tensor-core threshold on: the alternative there is the fp32 pipes (50 000 x 1000,
+//   K = 2: 107 us against 270).
+//   Large K * D: its contraction runs on mma.sync with little reuse of the centroids, so on data whose clusters
+//   are far apart the 64-row-tile kernel is ahead (131 072 rows of a mixture: D = 512, K = 64 178 us against 170,
+//   D = 768, K = 48 239 against 212, D = 1000, K = 32 264 against 262).  The other way round where that kernel does
+//   not go (D % 8 != 0), for batches that leave its tiles idle, and for rows above 1024 columns, whose exact pass
+//   outside costs more than anything (60 000 x 2048 logits, K = 24: 415 us against 1219).
+//   Short rows with many centroids: a group of eight rows is too little work (128 406 x 48, K = 106: 83 against 75).
+static bool use_apply_rows(int64_t N, int D, int K)
+{
+    const int min_k = g_tc_min_k.load(std::memory_order_relaxed);
+    if (!(g_small_kernels.load(std::memory_order_relaxed) & 1) || get_apply_column_split() != 0 ||
+        K < min_k / 4 + (min_k % 4 != 0) || !apply_rows_supported(N, D, K))
+        return false;
+    if (D < 64) return K <= 64;
+    return (int64_t)K * D <= 32768 || D % 8 != 0 || N < 4096 || D > 1024;
+}
+
 // norms -> fast assignment (tensor cores for large K, fp32 pipes otherwise) -> exact pass for
 // undecided rows.  row_norms_ready: w.ynorm2 already holds this Y's squared row norms.
 static cat_status_t run_assign(const float *Y, int64_t N, int D, int K, const float *C,
@@ -148,6 +170,12 @@ static cat_status_t run_assign(const float *Y, int64_t N, int D, int K, const fl
         // small problems: everything in one persistent launch (exact decisions included)
         CAT_CUDA(launch_reset_control(w.ctl, s));
         CAT_CUDA(launch_small_apply(Y, N, D, K, C, gamma, beta, out, labels, w.ctl, s));
+        return CAT_OK;
+    }
+    if (out && labels && top_level && !fast && use_apply_rows(N, D, K)) {
+        // rows kept in shared memory from the first read to the corrected store (behind the kernel above
+        // where both apply: 200 704 x 64, K = 64 takes 69 us here and 43 there)
+        CAT_CUDA(launch_apply_rows(Y, N, D, K, C, gamma, beta, out, false, labels, w.ctl, w.prep, s));
         return CAT_OK;
     }
     if (K == 1 && !fast) {   // one cluster: nothing to decide
@@ -312,6 +340,10 @@ cat_status_t cat_apply_bf16(const float *Yq, int64_t N, int32_t D, int32_t K, co
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     AssignWs w = carve_assign(workspace, N, D, K);
     int32_t *labels = labels_out ? labels_out : w.labels;
+    if (use_apply_rows(N, D, K)) {
+        CAT_CUDA(launch_apply_rows(Yq, N, D, K, centroids, gamma, beta, Y_out_bf16, true, labels, w.ctl, w.prep, s));
+        return CAT_OK;
+    }
     if (use_tensor_path(N, D, K) && apply_h64_supported(N, D, K)) {
         // fused: the 64-row-tile kernel writes bf16 with the fast labels; the exact pass settles the
         // undecided rows' labels, and those rows are written once more

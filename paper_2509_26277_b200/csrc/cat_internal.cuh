@@ -97,6 +97,7 @@ struct AssignWs {          // what assign/apply need
     float *cmax;           // [K] largest magnitude of each centroid
     void *ch;              // [K][half_ld(D)] fp16 copy of the centroids (inference on fp16 operands)
     float *hscale;         // [4] scale of that copy: {s_c, -2 / s_c, 2^-25 / s_c, -}; with yh followed by [N] inverse row scales
+    void *prep;            // prepared centroids of the inference kernel that keeps rows in shared memory (or null)
     void *yh;              // [N][half_ld(D)] fp16 copy of the rows (inference with D % 4 != 0), else null
     size_t bytes;
 };
@@ -155,6 +156,13 @@ cudaError_t launch_small_fit(const float *Y, int64_t N, int D, int K, float *C, 
                              Control *ctl, unsigned int *bar_count, cudaStream_t s);
 cudaError_t launch_small_apply(const float *Y, int64_t N, int D, int K, const float *C, const float *gamma,
                                const float *beta, float *out, int32_t *labels, Control *ctl, cudaStream_t s);
+
+// Inference on groups of eight rows held in shared memory, exact decisions included (cat_apply_rows.cu).
+// Resets ctl.  out_bf16: `out` is a [N, D] bf16 matrix; prep: apply_rows_prep_bytes of scratch.
+bool apply_rows_supported(int64_t N, int D, int K);
+size_t apply_rows_prep_bytes(int64_t N, int D, int K);
+cudaError_t launch_apply_rows(const float *Y, int64_t N, int D, int K, const float *C, const float *gamma, const float *beta,
+                              void *out, bool out_bf16, int32_t *labels, Control *ctl, void *prep, cudaStream_t s);
 
 // Tensor-core (tcgen05, TF32) variant of launch_assign; ynorm2 is needed when out == nullptr.
 bool tc_supported(int64_t N, int D, int K);

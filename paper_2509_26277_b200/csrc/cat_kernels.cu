@@ -1062,6 +1062,7 @@ cudaError_t launch_fit_diag_round(const float *Y, int64_t N, int D, int K, const
 
 __global__ void reset_control_kernel(Control *ctl)
 {
+    pdl_enter();
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         ctl->refine_count = 0;
         ctl->cand_count = 0;
@@ -1074,9 +1075,9 @@ __global__ void reset_control_kernel(Control *ctl)
 
 cudaError_t launch_reset_control(Control *ctl, cudaStream_t s)
 {
-    reset_control_kernel<<<1, 32, 0, s>>>(ctl);
+    const cudaError_t e = launch_pdl(reset_control_kernel, dim3(1), dim3(32), 0, s, ctl);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace cat

@@ -1,0 +1,70 @@
+"""The inference kernel that keeps groups of eight rows in shared memory (any row length), through the C ABI,
+against the CPU oracle: edges of the group, of the sixteen-column steps, of the parts a warp takes and of the
+groups of sixteen centroids; rows the fast scores cannot decide; ties; extreme magnitudes."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import cat_oracle as O
+from paper_2509_26277_b200 import binding as B
+from tests.parity import labels_match
+
+pytestmark = pytest.mark.gpu
+
+
+def dev(a):
+    return torch.as_tensor(np.ascontiguousarray(a)).cuda()
+
+
+def host(t):
+    return t.detach().cpu().numpy()
+
+
+def _check(Yq, C, g, b):
+    _, lab, best, second = O.apply(Yq, C, g, b)
+    ws = B.workspace("apply", *Yq.shape, C.shape[0], "cuda")
+    out, glab = B.cat_apply(dev(Yq), dev(C), dev(g), dev(b), want_labels=True, ws=ws)
+    report = B.cat_workspace_report(ws)
+    assert report["device_status"] == 0
+    labels_match(host(glab), lab, best, second, "labels")
+    # the corrected row is one fused multiply-add of the label's coefficients: the same bits
+    np.testing.assert_array_equal(host(out), O.affine_with_labels(Yq, host(glab), g, b))
+    o16, l16 = B.cat_apply_bf16(dev(Yq), dev(C), dev(g), dev(b), want_labels=True)
+    assert torch.equal(l16, glab) and torch.equal(o16, out.to(torch.bfloat16))
+    return host(glab), report["refined_rows_last"]
+
+
+SHAPES = [(1, 1000, 8), (7, 1001, 2), (8, 16, 3), (9, 17, 16), (65, 31, 17), (100, 128, 33), (301, 129, 48), (77, 144, 64),
+          (513, 256, 65), (200, 257, 128), (90, 512, 24), (130, 513, 24), (1187, 528, 9), (4000, 1000, 16), (333, 1001, 50),
+          (129, 1024, 32), (71, 1999, 5), (40, 2048, 16), (2500, 100, 100), (50, 3001, 4),
+          (1300, 10, 16), (333, 3, 2), (700, 1000, 64), (450, 1001, 128), (300, 1023, 33), (260, 2047, 64), (90, 2048, 20)]
+
+
+@pytest.mark.parametrize("n,d,k", SHAPES)
+@pytest.mark.parametrize("kind", ["spread", "close"])
+def test_rows_kernel_matches_the_oracle(n, d, k, kind):
+    rng = np.random.default_rng(n * 31 + d + k)
+    Yq = (rng.normal(size=(n, d)) + 2.0).astype(np.float32)
+    g, b = rng.normal(size=(k, d)).astype(np.float32), rng.normal(size=(k, d)).astype(np.float32)
+    if kind == "spread":
+        C = (rng.normal(size=(k, d)) + 2.0).astype(np.float32)
+    else:
+        # a tight bunch far from the origin, two of them equal (always left to the exact decision)
+        C = (2.0 + 2e-3 * rng.normal(size=(k, d))).astype(np.float32)
+        C[-1] = C[0]
+    lab, undecided = _check(Yq, C, g, b)
+    if kind == "close":
+        assert undecided >= (lab == 0).sum()
+        assert not (lab == k - 1).any()
+
+
+@pytest.mark.parametrize("d,k", [(1000, 16), (1001, 32), (60, 40)])
+@pytest.mark.parametrize("scale", [1e-25, 1e-12, 1e15])
+def test_rows_kernel_at_extreme_magnitudes(d, k, scale):
+    rng = np.random.default_rng(d + k)
+    Yq = (rng.normal(size=(200, d)) * scale).astype(np.float32)
+    Yq[3] *= 1e-6 if scale < 1 else 1e6                      # a row far off the others' magnitude
+    Yq[5, d // 2:] *= 1e4                                    # and one whose parts differ
+    C = Yq[rng.choice(np.arange(6, 200), size=k, replace=False)].copy()
+    g, b = rng.normal(size=(k, d)).astype(np.float32), (rng.normal(size=(k, d)) * scale).astype(np.float32)
+    _check(Yq, C, g, b)
