@@ -7,7 +7,7 @@
 // inverse iteration with orthogonalisation against all larger pairs, then the reflections are
 // applied to the p vectors.  (Golub & Van Loan, Matrix Computations, ch. 8.)  One-sided Jacobi
 // rotations over all pairs of columns, the earlier form, took 155 ms for D = 1000: about ten sweeps
-// of 999 dependent launches.  This takes 9.5 ms there with p = 50 (13 ms with p = 200).
+// of 999 dependent launches.  This takes 5.1 ms there with p = 50.
 //
 // Both kernels are cooperative launches; every wait is bounded by TC_TIMEOUT_NS and reports
 // CAT_ERR_DEVICE_TIMEOUT in the control block.  Every sum has a fixed order: results do not vary
@@ -54,18 +54,65 @@ __device__ __forceinline__ bool wait_flag(const uint32_t *flag, uint32_t value, 
     }
 }
 
-// Grid barrier number `value`: a flag per CTA instead of one counter, since 148 arrivals at one
-// address are serialised in L2 and every step of the reduction waits here.  The whole CTA calls it.
-__device__ __forceinline__ bool flag_barrier(uint32_t *flags, uint32_t value, Control *ctl)
+// Grid barrier: a counter that only grows, polled by one thread per CTA; the n-th barrier is over at
+// n * gridDim.x arrivals.  The whole CTA calls it.
+__device__ __forceinline__ bool grid_barrier(uint32_t *counter, uint32_t n, Control *ctl)
 {
     __syncthreads();
+    bool ok = true;
     if (threadIdx.x == 0) {
         __threadfence();
-        store_flag(flags + blockIdx.x, value);
+        atomicAdd(counter, 1u);
+        ok = wait_flag(counter, n * gridDim.x, ctl);
     }
-    bool ok = true;
-    for (int g = threadIdx.x; g < (int)gridDim.x; g += ET) ok = wait_flag(flags + g, value, ctl) && ok;
     return __syncthreads_and(ok);
+}
+
+// Values that pass between CTAs without a barrier: each is its own flag.  The buffers start as all ones,
+// every word is written once per launch, and a reader polls the word until it is something else -- 64-bit
+// accesses are whole, so no fence is needed.
+constexpr unsigned long long UNSET = ~0ull;
+__device__ __forceinline__ void publish(double *p, double v)
+{
+    unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    if (b == UNSET) b = 0x7FF8000000000000ull;   // (a NaN stays a NaN)
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(b) : "memory");
+}
+__device__ __forceinline__ unsigned long long peek(const double *p)
+{
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+// out[c] = p[k0 + c * ET] for the columns in [lo, D), 0 elsewhere; false when the time limit is over
+template <int C>
+__device__ __forceinline__ bool collect(const double *p, int lo, int D, double (&out)[C], Control *ctl)
+{
+    unsigned long long b[C];
+    uint64_t t0 = 0;
+    for (uint32_t it = 0;; ++it) {
+        bool all = true;
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const int k = threadIdx.x + c * ET;
+            b[c] = k >= lo && k < D ? peek(p + k) : 0ull;
+        }
+#pragma unroll
+        for (int c = 0; c < C; ++c) all = all && b[c] != UNSET;
+        if (all) break;
+        if ((it & 255u) == 255u) {
+            if (*(volatile int *)&ctl->device_status != (int)CAT_OK) return false;
+            const uint64_t now = global_timer();
+            if (t0 == 0) t0 = now;
+            else if (now - t0 > TC_TIMEOUT_NS) {
+                atomicExch(&ctl->device_status, (int)CAT_ERR_DEVICE_TIMEOUT);
+                return false;
+            }
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < C; ++c) out[c] = __longlong_as_double((long long)b[c]);
+    return true;
 }
 
 __device__ __forceinline__ double warp_sum(double v)
@@ -75,16 +122,27 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
+__device__ __forceinline__ double tree8(const double *r)
+{
+    static_assert(EW == 8, "sum of the warps' parts");
+    return ((r[0] + r[1]) + (r[2] + r[3])) + ((r[4] + r[5]) + (r[6] + r[7]));
+}
+
 // every thread gets the CTA's sum; `red` must not be in use from an earlier call (callers alternate two)
 __device__ __forceinline__ double block_sum(double v, double *red)
 {
     v = warp_sum(v);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
-    double s = 0.0;
-#pragma unroll
-    for (int w = 0; w < EW; ++w) s += red[w];
-    return s;
+    return tree8(red);
+}
+// the same; `ok` becomes false in every thread if it was in one
+__device__ __forceinline__ double block_sum(double v, double *red, bool &ok)
+{
+    v = warp_sum(v);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    ok = __syncthreads_and(ok);
+    return tree8(red);
 }
 
 // Sums of 8 values over the warp: each exchange halves how many values a lane still carries, 9
@@ -132,65 +190,81 @@ struct TridiagParams {
     const double *diag;   // [D] its diagonal
     double *refl;         // [D][D] reflection j: entries k > j of row j
     double *d, *e, *tau;  // [D]
-    double *pbuf;         // [2][D]
-    double *rowbuf;       // [2][D]
-    uint32_t *flags;      // [gridDim.x], zero at launch
+    double *prod;         // [D][D] row j: products of step j; all ones at launch
+    double *next;         // [D][D] row j: row j of the matrix after update j - 2; all ones at launch
     Control *ctl;
     int D;
-    int resident;         // the CTA's rows live in shared memory
+    int resident;         // (rows not in registers) the CTA's rows live in shared memory
 };
 
-// Householder reduction to tridiagonal form.  Row i of the matrix belongs to CTA i mod G and stays
-// in its shared memory (D = 1000: 8 MB over 125 CTAs), or in global memory where that is too small;
-// columns are dealt out over the threads, so a thread keeps its columns' part of the vectors in
-// registers.  Step j needs one grid barrier: every CTA forms reflection j from row j (which the
-// owner has published up to update j - 2) and the vectors v, w of update j - 1, applies that update
-// to its own rows and in the same sweep multiplies them with the new reflection; the products of all
-// CTAs meet after the barrier.
-//   bound: latency.  A step moves 8 D values between CTAs and does 6 (D - j)^2 / G operations per
-//   CTA (under 0.5 us); barrier, L2 round trips and three block-wide sums make it 7.5 us on average
-//   (D = 1000: 7.5 ms in all).
-template <int C>
+// Householder reduction to tridiagonal form.  A row of the matrix belongs to one CTA and stays with it: for
+// D <= 1024 in registers (REGS: rows 8 me ... 8 me + 7, column k with thread k mod 256; 8 MB over 125 SMs at
+// D = 1000; a CTA's products are one 64-byte store and it leaves when its rows are done), beyond that in
+// shared or global memory (rows me, me + G, ...: there the work per step counts).  Step j: every CTA forms reflection j from
+// row j (which its owner has published up to update j - 2) and the vectors v, w of update j - 1, applies
+// that update to its own rows and in the same sweep multiplies them with the new reflection; each CTA
+// publishes its products and collects everybody's, word by word, without a barrier.
+//   bound: latency.  A step moves 2 D values between CTAs and does 6 (D - j)^2 / G operations per CTA;
+//   the exchange, three block-wide sums and a square root and two divisions in fp64 make it 3.1 us (D = 1000).
+//   With a grid barrier (a flag per CTA, polled by all) in place of the self-validating words the exchange alone
+//   took 6 of 9 us.
+template <int C, bool REGS>
 __global__ void __launch_bounds__(ET) tridiag_kernel(TridiagParams P)
 {
     extern __shared__ double sm[];
     __shared__ double red[2][EW], red_rows[EW][MAX_ROWS], s_x1;
+    constexpr int RR = REGS ? 8 : 1;
     const int D = P.D, G = gridDim.x, me = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int R = (D - me + G - 1) / G;
+    const int R = REGS ? (D - me * 8 < 8 ? D - me * 8 : 8) : (D - me + G - 1) / G;
+    const int i0 = REGS ? me * 8 : me, di = REGS ? 1 : G;   // own rows: i0 + r di
     double *sv = sm, *sw = sm + D, *rows = sm + 2 * D;
     const double scale = diagonal_scale(P.diag, D, red[0]);
     for (int k = tid; k < 2 * D; k += ET) sm[k] = 0.0;
-    for (int r = 0; r < R; ++r) {
-        double *src = P.A + (size_t)(me + r * G) * D;
-        double *dst = P.resident ? rows + (size_t)r * D : src;
-        for (int k = tid; k < D; k += ET) {
-            const double a = src[k] * scale;
-            dst[k] = a;
-            if (me + r * G == 0) P.rowbuf[k] = a;
+    double ar[RR][C];
+    if (REGS) {
+#pragma unroll
+        for (int r = 0; r < RR; ++r)
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                const int i = i0 + r * di, k = tid + c * ET;
+                ar[r][c] = i < D && k < D ? P.A[(size_t)i * D + k] * scale : 0.0;
+                if (i == 0 && k < D) publish(P.next + k, ar[r][c]);
+            }
+    } else {
+        for (int r = 0; r < R; ++r) {
+            double *src = P.A + (size_t)(me + r * G) * D;
+            double *dst = P.resident ? rows + (size_t)r * D : src;
+            for (int k = tid; k < D; k += ET) {
+                const double a = src[k] * scale;
+                dst[k] = a;
+                if (me + r * G == 0) publish(P.next + k, a);
+            }
         }
     }
     double vo[C], wo[C];
 #pragma unroll
     for (int c = 0; c < C; ++c) vo[c] = wo[c] = 0.0;
     double v1 = 0.0, w1 = 0.0;   // the previous update's v, w at index j
-    uint32_t bar = 1;
-    if (!flag_barrier(P.flags, bar, P.ctl)) return;
+    __syncthreads();
 
     for (int j = 0; j < D; ++j) {
+        // the CTA of row j + 1 (or the last one) records step j; in registers' form a CTA leaves with its last row
+        const bool lead = REGS ? me == (j + 1 < D ? j + 1 : j) / 8 : me == j % G;
+        if (REGS && i0 + R <= j) break;
         // row j after update j - 1, and the sum of squares behind its first off-diagonal entry
         double x[C];
+        bool ok = collect<C>(P.next + (size_t)j * D, j, D, x, P.ctl);
         double ss = 0.0;
 #pragma unroll
         for (int c = 0; c < C; ++c) {
             const int k = tid + c * ET;
-            x[c] = 0.0;
-            if (k >= j && k < D) x[c] = __ldcg(P.rowbuf + (size_t)(j & 1) * D + k) - (v1 * wo[c] + w1 * vo[c]);
-            if (k == j && me == 0) P.d[j] = x[c];
+            x[c] = fma(-v1, wo[c], fma(-w1, vo[c], x[c]));   // (v, w are zero up to index j - 1)
+            if (k == j && lead) P.d[j] = x[c];
             if (k == j + 1) s_x1 = x[c];
             if (k > j + 1) ss = fma(x[c], x[c], ss);
         }
-        if (j == D - 1) break;
-        ss = block_sum(ss, red[0]);
+        ss = block_sum(ss, red[0], ok);
+        if (!ok || j == D - 1) break;
         const double x1 = s_x1;
         double tau = 0.0, inv = 0.0, off = x1;
         if (ss > 0.0) {
@@ -204,63 +278,85 @@ __global__ void __launch_bounds__(ET) tridiag_kernel(TridiagParams P)
         for (int c = 0; c < C; ++c) {
             const int k = tid + c * ET;
             vn[c] = k == j + 1 ? (ss > 0.0 ? 1.0 : 0.0) : (k > j + 1 ? x[c] * inv : 0.0);
-            if (me == j % G && k > j && k < D) P.refl[(size_t)j * D + k] = vn[c];
+            if (lead && k > j && k < D) P.refl[(size_t)j * D + k] = vn[c];
         }
-        if (me == 0 && tid == 0) {
+        if (lead && tid == 0) {
             P.e[j] = off;
             P.tau[j] = tau;
         }
         // update j - 1 of the own rows and their products with the new reflection
-        const int r_first = j + 1 <= me ? 0 : (j + 1 - me + G - 1) / G;   // first own row with index > j
-        for (int r0 = r_first; r0 < R; r0 += 8) {
+        const int r_first = j + 1 <= i0 ? 0 : (j + 1 - i0 + di - 1) / di;   // first own row with index > j
+        if (REGS) {
             double acc[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                acc[u] = 0.0;
-                const int r = r0 + u, i = me + r * G;
-                if (r < R) {
-                    double *a_row = P.resident ? rows + (size_t)r * D : P.A + (size_t)i * D;
-                    const double vi = sv[i], wi = sw[i];
-                    const bool publish = i == j + 1;
+            for (int r = 0; r < RR; ++r) {
+                acc[r] = 0.0;
+                const int i = i0 + r;
+                if (i > j && i < D) {
+                    const double vi = -sv[i], wi = -sw[i];
 #pragma unroll
-                    for (int c = 0; c < C; ++c) {
-                        const int k = tid + c * ET;
-                        if (k > j && k < D) {
-                            const double a = a_row[k] - (vi * wo[c] + wi * vo[c]);
-                            a_row[k] = a;
-                            acc[u] = fma(a, vn[c], acc[u]);
-                            if (publish) P.rowbuf[(size_t)((j + 1) & 1) * D + k] = a;
+                    for (int c = 0; c < C; ++c)
+                        if (warp * 32 + 31 + c * ET > j) {   // (columns up to j are done with)
+                            ar[r][c] = fma(wi, vo[c], fma(vi, wo[c], ar[r][c]));
+                            acc[r] = fma(ar[r][c], vn[c], acc[r]);
+                        }
+                    if (i == j + 1) {
+#pragma unroll
+                        for (int c = 0; c < C; ++c) {
+                            const int k = tid + c * ET;
+                            if (k > j && k < D) publish(P.next + (size_t)(j + 1) * D + k, ar[r][c]);
                         }
                     }
                 }
             }
             const double s = warp_sum8(acc, lane);
-            if ((lane & 3) == 0) {
-                const int u = lane >> 2;
-                if (r0 + u < R) red_rows[warp][r0 + u] = s;
+            if ((lane & 3) == 0) red_rows[warp][lane >> 2] = s;
+        } else {
+            for (int r0 = r_first; r0 < R; r0 += 8) {
+                double acc[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    acc[u] = 0.0;
+                    const int r = r0 + u, i = i0 + r * di;
+                    if (r < R) {
+                        double *a_row = P.resident ? rows + (size_t)r * D : P.A + (size_t)i * D;
+                        const double vi = -sv[i], wi = -sw[i];
+#pragma unroll
+                        for (int c = 0; c < C; ++c) {
+                            const int k = tid + c * ET;
+                            if (k > j && k < D) {
+                                const double a = fma(wi, vo[c], fma(vi, wo[c], a_row[k]));
+                                a_row[k] = a;
+                                acc[u] = fma(a, vn[c], acc[u]);
+                                if (i == j + 1) publish(P.next + (size_t)(j + 1) * D + k, a);
+                            }
+                        }
+                    }
+                }
+                const double s = warp_sum8(acc, lane);
+                if ((lane & 3) == 0 && r0 + (lane >> 2) < R) red_rows[warp][r0 + (lane >> 2)] = s;
             }
         }
         __syncthreads();
-        for (int r = r_first + tid; r < R; r += 32)
-            if (tid < 32) {
-                double s = 0.0;
+        if (tid >= r_first && tid < R) {
+            double part[EW];
 #pragma unroll
-                for (int w = 0; w < EW; ++w) s += red_rows[w][r];
-                P.pbuf[(size_t)(j & 1) * D + me + r * G] = s;
-            }
-        if (!flag_barrier(P.flags, ++bar, P.ctl)) return;
+            for (int w = 0; w < EW; ++w) part[w] = red_rows[w][tid];
+            publish(P.prod + (size_t)j * D + i0 + tid * di, tree8(part));
+        }
         // w = tau A v - (tau / 2)(tau v'Av) v
+        ok = collect<C>(P.prod + (size_t)j * D, j + 1, D, wo, P.ctl);
         double pv = 0.0;
 #pragma unroll
         for (int c = 0; c < C; ++c) {
-            const int k = tid + c * ET;
-            wo[c] = k > j && k < D ? tau * __ldcg(P.pbuf + (size_t)(j & 1) * D + k) : 0.0;
+            wo[c] *= tau;
             pv = fma(wo[c], vn[c], pv);
+            if (tid + c * ET == j + 1) s_x1 = wo[c];
         }
-        const double p1 = tau * __ldcg(P.pbuf + (size_t)(j & 1) * D + j + 1);
-        const double half = 0.5 * tau * block_sum(pv, red[1]);
+        const double half = 0.5 * tau * block_sum(pv, red[1], ok);
+        if (!ok) break;
         v1 = ss > 0.0 ? 1.0 : 0.0;
-        w1 = p1 - half * v1;
+        w1 = s_x1 - half * v1;
 #pragma unroll
         for (int c = 0; c < C; ++c) {
             const int k = tid + c * ET;
@@ -278,7 +374,7 @@ struct EigvecParams {
     const double *diag;               // [D] diagonal of the unreduced matrix (for its scale)
     const double *d, *e, *tau, *refl;
     double *Z;                        // [p][D] vectors
-    uint32_t *flags;                  // [gridDim.x] barriers, then [p] published vectors; zero at launch
+    uint32_t *flags;                  // barrier counter, then [p] published vectors; zero at launch
     float *comps;                     // [p][D] out
     double *eig_out;                  // [p] out or null
     Control *ctl;
@@ -317,7 +413,7 @@ __global__ void __launch_bounds__(ET) eigvec_kernel(EigvecParams P)
     __shared__ int ok_flag;
     const int D = P.D, p = P.p, G = gridDim.x, me = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int NV = (p - me + G - 1) / G;
-    uint32_t *vec_flag = P.flags + G;
+    uint32_t *vec_flag = P.flags + 1;
     double *sd = sm, *u0 = sm + D, *u1 = sm + 2 * D, *u2 = sm + 3 * D, *l = sm + 4 * D;
     unsigned char *swapped = reinterpret_cast<unsigned char *>(sm + 5 * D);
     const double scale = diagonal_scale(P.diag, D, red[0]);
@@ -507,7 +603,7 @@ __global__ void __launch_bounds__(ET) eigvec_kernel(EigvecParams P)
                 }
             }
             // every CTA has read what this pass published before anything rewrites it
-            if (!flag_barrier(P.flags, gen, P.ctl)) return;
+            if (!grid_barrier(P.flags, gen, P.ctl)) return;
         }
     }
 
@@ -589,9 +685,8 @@ __global__ void __launch_bounds__(ET) eigvec_kernel(EigvecParams P)
 }
 
 struct EigWs {
-    double *Z, *d, *e, *tau, *pbuf, *rowbuf;
+    double *Z, *d, *e, *tau, *prod, *next;
     uint32_t *flags;
-    size_t flag_words;
     size_t bytes;
 };
 
@@ -611,10 +706,9 @@ EigWs carve_eig(void *base, int D, int p)
     w.d = (double *)take(row);
     w.e = (double *)take(row);
     w.tau = (double *)take(row);
-    w.pbuf = (double *)take(2 * row);
-    w.rowbuf = (double *)take(2 * row);
-    w.flag_words = 2 * 1024 + (size_t)p;
-    w.flags = (uint32_t *)take(w.flag_words * sizeof(uint32_t));
+    w.flags = (uint32_t *)take((size_t)(1 + p) * sizeof(uint32_t));
+    w.prod = (double *)take(2 * (size_t)D * row);
+    w.next = b ? w.prod + (size_t)D * D : nullptr;
     w.bytes = align_up(off, 256);
     return w;
 }
@@ -639,39 +733,36 @@ cudaError_t launch_sym_eig(double *A, const double *diag, double *refl, int D, i
                            Control *ctl, void *workspace, cudaStream_t s)
 {
     EigWs w = carve_eig(workspace, D, p);
-    cudaError_t err = cudaMemsetAsync(w.flags, 0, w.flag_words * sizeof(uint32_t), s);
+    cudaError_t err = cudaMemsetAsync(w.flags, 0, (size_t)(1 + p) * sizeof(uint32_t), s);
+    if (err == cudaSuccess) err = cudaMemsetAsync(w.prod, 0xFF, 2 * (size_t)D * D * sizeof(double), s);
     if (err != cudaSuccess) return err;
     int sms = 0, dev = 0;
     if ((err = cudaGetDevice(&dev)) != cudaSuccess) return err;
     if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return err;
-    if (sms > 1024) sms = 1024;
-    // at least eight rows per CTA: fewer CTAs meet at the barrier, and a row's sweep is short beside it
+    // eight rows per CTA (what a thread's registers hold for D <= 1024), more where the SMs run out
     int G = (D + 7) / 8;
     if (G > sms) G = sms;
     const int R = (D + G - 1) / G;
     if (R > MAX_ROWS || (p + sms - 1) / sms > MAX_VECS) return cudaErrorInvalidValue;
-    TridiagParams T{A, diag, refl, w.d, w.e, w.tau, w.pbuf, w.rowbuf, w.flags, ctl, D, 0};
+    TridiagParams T{A, diag, refl, w.d, w.e, w.tau, w.prod, w.next, ctl, D, 0};
+    const bool regs = D <= 1024 && R <= 8;
     size_t smem = (size_t)(2 + R) * D * sizeof(double);
-    T.resident = smem <= DYN_SMEM_LIMIT;   // D up to about 1850
+    T.resident = !regs && smem <= DYN_SMEM_LIMIT;   // D up to about 1850
     if (!T.resident) smem = (size_t)2 * D * sizeof(double);
-    EigvecParams V{diag, w.d, w.e, w.tau, refl, w.Z, w.flags + 1024, comps, eig_out, ctl, D, p};
+    const int C = (D + ET - 1) / ET;
+    if (regs && C <= 1) err = launch_coop(tridiag_kernel<1, true>, G, smem, T, s);
+    else if (regs && C <= 2) err = launch_coop(tridiag_kernel<2, true>, G, smem, T, s);
+    else if (regs) err = launch_coop(tridiag_kernel<4, true>, G, smem, T, s);
+    else if (C <= 8) err = launch_coop(tridiag_kernel<8, false>, G, smem, T, s);
+    else err = launch_coop(tridiag_kernel<16, false>, G, smem, T, s);
+    if (err != cudaSuccess) return err;
+    EigvecParams V{diag, w.d, w.e, w.tau, refl, w.Z, w.flags, comps, eig_out, ctl, D, p};
     const int GV = p < sms ? p : sms;
     const size_t smem_v = (size_t)5 * D * sizeof(double) + (size_t)D;
-    const int C = (D + ET - 1) / ET;
-    if (C <= 1) {
-        err = launch_coop(tridiag_kernel<1>, G, smem, T, s);
-        return err != cudaSuccess ? err : launch_coop(eigvec_kernel<1>, GV, smem_v, V, s);
-    }
-    if (C <= 2) {
-        err = launch_coop(tridiag_kernel<2>, G, smem, T, s);
-        return err != cudaSuccess ? err : launch_coop(eigvec_kernel<2>, GV, smem_v, V, s);
-    }
-    if (C <= 4) {
-        err = launch_coop(tridiag_kernel<4>, G, smem, T, s);
-        return err != cudaSuccess ? err : launch_coop(eigvec_kernel<4>, GV, smem_v, V, s);
-    }
-    err = launch_coop(tridiag_kernel<16>, G, smem, T, s);
-    return err != cudaSuccess ? err : launch_coop(eigvec_kernel<16>, GV, smem_v, V, s);
+    if (C <= 1) return launch_coop(eigvec_kernel<1>, GV, smem_v, V, s);
+    if (C <= 2) return launch_coop(eigvec_kernel<2>, GV, smem_v, V, s);
+    if (C <= 4) return launch_coop(eigvec_kernel<4>, GV, smem_v, V, s);
+    return launch_coop(eigvec_kernel<16>, GV, smem_v, V, s);
 }
 
 }  // namespace cat

@@ -2,7 +2,7 @@
 // "PCA is only used to obtain clusters"; Algorithm 1 step 1, Algorithm 2 step 1).
 //
 //   column means            fp64 partial sums per row chunk, added in a fixed order
-//   covariance              D x D, fp64 FMA on 64 x 64 register-tiled CTAs over the centred rows
+//   covariance              D x D, fp64 mma on 64 x 64 tiles over the centred rows
 //                           (upper-triangular tiles, mirrored); 1 / (N - 1) normalisation
 //   eigen-decomposition     the p largest pairs by tridiagonal reduction, bisection and inverse
 //                           iteration in fp64 (cat_eig.cu); a component's sign is fixed so that its
@@ -21,7 +21,7 @@ namespace {
 
 constexpr int PT = 64;          // tile edge of the fp64 contractions
 constexpr int PK = 16;          // depth of a shared-memory step
-constexpr int P_THREADS = 256;  // 16 x 16 threads, 4 x 4 outputs each
+constexpr int P_THREADS = 128;  // 2 x 2 warps, 32 x 32 outputs each
 constexpr int MEAN_CHUNKS = 64;
 
 // ---------------------------------------------------------------- column means
@@ -51,59 +51,86 @@ __global__ void col_mean_kernel(const double *__restrict__ part, int chunks, int
 }
 
 // ---------------------------------------------------------------- 64 x 64 fp64 tile product
-// acc[u][v] += sum_k As[k][ty * 4 + u] * Bs[k][tx * 4 + v] over one shared-memory step
-__device__ __forceinline__ void tile_step(const double (*As)[PT], const double (*Bs)[PT], int ty, int tx,
-                                          double (&acc)[4][4])
+// Four warps, 32 x 32 each, as 4 x 4 tiles of mma.m8n8k4 in fp64: 16 multiply-adds per operand element
+// read from shared memory, where the 4 x 4 register tiles of scalar FMAs this replaces had two.  Operands
+// sit in shared memory with strides of 4 mod 16 doubles, which spreads a fragment's half-warp reads over
+// all banks.
+__device__ __forceinline__ void mma_f64(double (&c)[2], double a, double b)
 {
-#pragma unroll
-    for (int k = 0; k < PK; ++k) {
-        double a[4], b[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) a[u] = As[k][ty * 4 + u];
-#pragma unroll
-        for (int v = 0; v < 4; ++v) b[v] = Bs[k][tx * 4 + v];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) acc[u][v] = fma(a[u], b[v], acc[u][v]);
-    }
+    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
+                 : "+d"(c[0]), "+d"(c[1])
+                 : "d"(a), "d"(b));
 }
 
 // Covariance tile (bi, bj), bj >= bi, over the rows of split blockIdx.z:
 // part[z][a][b] = sum_i (y_ia - mean_a)(y_ib - mean_b)
+//   bound: fp64 multiply-adds (4096 x 1000: 2.2 GFMA over the upper tiles, 0.13 ms at 64 per clock and SM).
 __global__ void __launch_bounds__(P_THREADS) cov_kernel(const float *__restrict__ Y, int64_t N, int D,
                                                         const double *__restrict__ mean, double *__restrict__ part)
 {
-    __shared__ double As[PK][PT], Bs[PK][PT];
+    constexpr int LD = PT + 4;
+    __shared__ double As[2][PK][LD], Bs[2][PK][LD];
     const int bi = blockIdx.y, bj = blockIdx.x;
     if (bj < bi) return;
-    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int m0 = (warp >> 1) * 32, n0 = (warp & 1) * 32, g = lane >> 2, t = lane & 3;
     const int64_t per = (N + gridDim.z - 1) / gridDim.z;
     const int64_t r0 = (int64_t)blockIdx.z * per;
     const int64_t r1 = r0 + per < N ? r0 + per : N;
-    double acc[4][4] = {};
-    for (int64_t r = r0; r < r1; r += PK) {
-        // 16 rows x 64 columns per operand: 1024 elements, 4 per thread
+    // a thread always fetches the same column of each operand, rows k0, k0 + 2, ...
+    const int c = tid & 63, k0 = tid >> 6;
+    const int ca = bi * PT + c, cb = bj * PT + c;
+    const double ma = ca < D ? mean[ca] : 0.0, mb = cb < D ? mean[cb] : 0.0;
+    float fa[PK / 2], fb[PK / 2];
+    auto fetch = [&](int64_t r) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int e = tid + q * P_THREADS, k = e >> 6, c = e & 63;
-            const int64_t row = r + k;
-            const int ca = bi * PT + c, cb = bj * PT + c;
-            As[k][c] = (row < r1 && ca < D) ? (double)Y[(size_t)row * D + ca] - mean[ca] : 0.0;
-            Bs[k][c] = (row < r1 && cb < D) ? (double)Y[(size_t)row * D + cb] - mean[cb] : 0.0;
+        for (int q = 0; q < PK / 2; ++q) {
+            const int64_t row = r + k0 + 2 * q;
+            fa[q] = row < r1 && ca < D ? __ldg(Y + (size_t)row * D + ca) : 0.f;
+            fb[q] = row < r1 && cb < D ? __ldg(Y + (size_t)row * D + cb) : 0.f;
         }
+    };
+    auto put = [&](int64_t r, int buf) {
+#pragma unroll
+        for (int q = 0; q < PK / 2; ++q) {
+            const bool in = r + k0 + 2 * q < r1;
+            As[buf][k0 + 2 * q][c] = in && ca < D ? (double)fa[q] - ma : 0.0;
+            Bs[buf][k0 + 2 * q][c] = in && cb < D ? (double)fb[q] - mb : 0.0;
+        }
+    };
+    double acc[4][4][2] = {};
+    fetch(r0);
+    put(r0, 0);
+    int buf = 0;
+    for (int64_t r = r0; r < r1; r += PK, buf ^= 1) {
         __syncthreads();
-        tile_step(As, Bs, ty, tx, acc);
-        __syncthreads();
+        const bool more = r + PK < r1;
+        if (more) fetch(r + PK);
+#pragma unroll
+        for (int k = 0; k < PK; k += 4) {
+            double a[4], b[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                a[i] = As[buf][k + t][m0 + 8 * i + g];
+                b[i] = Bs[buf][k + t][n0 + 8 * i + g];
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) mma_f64(acc[i][j], a[i], b[j]);
+        }
+        if (more) put(r + PK, buf ^ 1);
     }
     double *out = part + (size_t)blockIdx.z * D * D;
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const int a = bi * PT + ty * 4 + u, b = bj * PT + tx * 4 + v;
-            if (a < D && b < D) out[(size_t)a * D + b] = acc[u][v];
-        }
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int a = bi * PT + m0 + 8 * i + g, b = bj * PT + n0 + 8 * j + 2 * t + q;
+                if (a < D && b < D) out[(size_t)a * D + b] = acc[i][j][q];
+            }
 }
 
 // G = (sum of the splits' upper triangles, mirrored) / (N - 1), and its diagonal once more
@@ -123,39 +150,75 @@ __global__ void cov_finish_kernel(const double *__restrict__ part, int splits, i
 
 // ---------------------------------------------------------------- projection
 // Z[i, r] = sum_j (Y[i, j] - mean[j]) * comps[r, j], fp64 accumulation: one CTA per 64 rows x 64 components.
+//   bound: fp64 multiply-adds (50 000 x 1000, p = 50: 2.8 GFMA with p rounded up to 56, 0.15 ms at 64 per clock and SM).
 __global__ void __launch_bounds__(P_THREADS) project_kernel(const float *__restrict__ Y, int64_t N, int D, int p,
                                                             const float *__restrict__ mean, const float *__restrict__ comps,
                                                             float *__restrict__ Z)
 {
-    __shared__ double As[PK][PT], Bs[PK][PT];
-    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+    pdl_enter();
+    constexpr int LD = PK + 4;
+    __shared__ double As[2][PT][LD], Bs[2][PT][LD];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int m0 = (warp >> 1) * 32, n0 = (warp & 1) * 32, g = lane >> 2, t = lane & 3;
     const int64_t row0 = (int64_t)blockIdx.x * PT;
     const int c0 = blockIdx.y * PT;
-    double acc[4][4] = {};
-    for (int j0 = 0; j0 < D; j0 += PK) {
-        // operand element (m, k): 64 x 16 per operand, 4 per thread; k runs fastest so that a row's
-        // 16 columns are read together
+    const int tiles = p - c0 - n0 >= 32 ? 4 : (p - c0 - n0 + 7) / 8;   // component tiles of this warp that hold anything
+    // a thread always fetches the same column of a step, rows / components m, m + 8, ...
+    const int k = tid & 15, mb = tid >> 4;
+    float fa[8], fb[8], fm = 0.f;
+    auto fetch = [&](int j0) {
+        const int j = j0 + k;
+        fm = j < D ? __ldg(mean + j) : 0.f;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int e = tid + q * P_THREADS, m = e >> 4, k = e & 15;
-            const int j = j0 + k;
-            const int64_t row = row0 + m;
-            As[k][m] = (row < N && j < D) ? (double)Y[(size_t)row * D + j] - (double)mean[j] : 0.0;
-            const int r = c0 + m;
-            Bs[k][m] = (r < p && j < D) ? (double)comps[(size_t)r * D + j] : 0.0;
+        for (int q = 0; q < 8; ++q) {
+            const int64_t row = row0 + mb + 8 * q;
+            const int r = c0 + mb + 8 * q;
+            fa[q] = row < N && j < D ? __ldg(Y + (size_t)row * D + j) : 0.f;
+            fb[q] = r < p && j < D ? __ldg(comps + (size_t)r * D + j) : 0.f;
         }
+    };
+    auto put = [&](int j0, int buf) {
+        const bool in = j0 + k < D;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            As[buf][mb + 8 * q][k] = in ? (double)fa[q] - (double)fm : 0.0;
+            Bs[buf][mb + 8 * q][k] = (double)fb[q];
+        }
+    };
+    double acc[4][4][2] = {};
+    fetch(0);
+    put(0, 0);
+    int buf = 0;
+    for (int j0 = 0; j0 < D; j0 += PK, buf ^= 1) {
         __syncthreads();
-        tile_step(As, Bs, ty, tx, acc);
-        __syncthreads();
+        const bool more = j0 + PK < D;
+        if (more) fetch(j0 + PK);
+#pragma unroll
+        for (int kk = 0; kk < PK; kk += 4) {
+            double a[4], b[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                a[i] = As[buf][m0 + 8 * i + g][kk + t];
+                b[i] = Bs[buf][n0 + 8 * i + g][kk + t];
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (j < tiles)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) mma_f64(acc[i][j], a[i], b[j]);
+        }
+        if (more) put(j0 + PK, buf ^ 1);
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const int64_t row = row0 + ty * 4 + u;
-            const int r = c0 + tx * 4 + v;
-            if (row < N && r < p) Z[(size_t)row * p + r] = (float)acc[u][v];
-        }
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int64_t row = row0 + m0 + 8 * i + g;
+                const int r = c0 + n0 + 8 * j + 2 * t + q;
+                if (row < N && r < p) Z[(size_t)row * p + r] = (float)acc[i][j][q];
+            }
 }
 
 // ---------------------------------------------------------------- affine map for given cluster ids
@@ -271,13 +334,13 @@ __global__ void __launch_bounds__(256) affine_bf16_kernel(const float *__restric
     }
 }
 
+// row splits of the covariance: enough CTAs for four per SM
 int cov_splits(int D)
 {
     const int T = (D + PT - 1) / PT;
     const int tiles = T * (T + 1) / 2;
-    if (tiles >= 64) return 1;
-    int s = 128 / tiles;
-    return s < 1 ? 1 : (s > 32 ? 32 : s);
+    const int s = (4 * 148 + tiles - 1) / tiles;
+    return s > 32 ? 32 : s;
 }
 
 struct PcaWs {
@@ -404,10 +467,9 @@ cat_status_t cat_pca_project(const float *Y, int64_t N, int32_t D, int32_t p, co
     if (D > CAT_PCA_MAX_D || p > CAT_PCA_MAX_P || N >= ((int64_t)1 << 31)) return CAT_ERR_UNSUPPORTED;
     if (!al16(Y) || !al16(mean) || !al16(components) || !al16(Z_out)) return CAT_ERR_ALIGN;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    project_kernel<<<dim3((unsigned)((N + PT - 1) / PT), (p + PT - 1) / PT), P_THREADS, 0, s>>>(Y, N, D, p, mean, components,
-                                                                                             Z_out);
+    CAT_CUDA(launch_pdl(project_kernel, dim3((unsigned)((N + PT - 1) / PT), (p + PT - 1) / PT), dim3(P_THREADS), 0, s, Y, N, D, p, mean,
+                        components, Z_out));
     count_launch();
-    CAT_CUDA(cudaGetLastError());
     return CAT_OK;
 }
 
