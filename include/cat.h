@@ -408,8 +408,8 @@ int32_t cat_get_tensor_core_min_k(void);
  * K <= 128 (K >= a quarter of the threshold, rows up to about 3300 columns), in two launches that keep
  * each row in shared memory.  mask bit 1: so do the K-Means
  * rounds and the final assignment of cat_fit / cat_fit_from (Algorithm 1, step 2; calls without
- * per-round diagnostics).  Default 3: both are the faster form where they apply.  Clearing a bit
- * sends these shapes down the general multi-launch path instead: same labels (rows on a bisector
+ * per-round diagnostics), and of other sets of up to 8192 rows with moderate N * K * D.  Default 3:
+ * both are the faster form where they apply.  Clearing a bit sends these shapes down the general multi-launch path instead: same labels (rows on a bisector
  * apart, when a centroid differs in its last bit); sums that agree to fp64 rounding.  A PROCESS-WIDE
  * tuning and test hook like the one above. */
 void cat_set_small_problem_kernels(int32_t mask);

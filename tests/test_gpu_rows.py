@@ -7,7 +7,7 @@ import torch
 
 from oracle import cat_oracle as O
 from paper_2509_26277_b200 import binding as B
-from tests.parity import labels_match
+from tests.parity import close, labels_match
 
 pytestmark = pytest.mark.gpu
 
@@ -68,3 +68,35 @@ def test_rows_kernel_at_extreme_magnitudes(d, k, scale):
     C = Yq[rng.choice(np.arange(6, 200), size=k, replace=False)].copy()
     g, b = rng.normal(size=(k, d)).astype(np.float32), (rng.normal(size=(k, d)) * scale).astype(np.float32)
     _check(Yq, C, g, b)
+
+
+FITS = [(5, 4, 5), (600, 5, 2), (37, 1000, 16), (593, 1001, 7), (1024, 64, 64), (1500, 17, 300), (2300, 130, 33), (4100, 257, 24),
+        (8192, 50, 32), (300, 3000, 9), (148 * 4 + 1, 8, 3), (2000, 1999, 60)]
+
+
+@pytest.mark.parametrize("n,d,k", FITS)
+@pytest.mark.parametrize("kind", ["cloud", "repeated"])
+def test_fit_with_rows_in_shared_memory(n, d, k, kind):
+    """cat_fit on small sets (all rounds in one launch): labels, centroids and closed form against the oracle,
+    run-to-run repeatability, explicit start; a set with few distinct rows (zero distances, exact ties, empty
+    clusters, early fixed point)."""
+    rng = np.random.default_rng(n + 3 * d + k)
+    Yq = rng.normal(size=(n, d)).astype(np.float32)
+    if kind == "repeated":
+        Yq = Yq[rng.integers(0, max(2, min(n, k) // 2), size=n)].copy()
+    Yfp = (0.9 * Yq + 0.1 * rng.normal(size=(n, d))).astype(np.float32)
+    for init in (None, (Yq[rng.permutation(n)[:k]] + 0.25).astype(np.float32)):
+        ora = O.fit(Yq, Yfp, k, 6, init=init)
+        args = dict(init_centroids=None if init is None else dev(init))
+        C, G, Bt, lab = B.cat_fit(dev(Yq), dev(Yfp), k, 6, **args)
+        C2, G2, B2, lab2 = B.cat_fit(dev(Yq), dev(Yfp), k, 6, **args)
+        assert torch.equal(C, C2) and torch.equal(G, G2) and torch.equal(Bt, B2) and torch.equal(lab, lab2)
+        want, best, second = O.assign(Yq, host(C))
+        labels_match(host(lab), want, best, second, "labels")
+        if int(ora.near.sum()) == 0 or kind == "repeated":
+            close(host(C), ora.centroids, "centroids")
+            assert np.array_equal(host(lab), ora.labels)
+        g, b = O.solve_gamma_beta(Yq, Yfp, host(lab), k)
+        close(host(G), g, "gamma")
+        close(host(Bt), b, "beta")
+    assert B.cat_workspace_report(B.workspace("fit", n, d, k, "cuda"))["device_status"] == 0
