@@ -388,8 +388,8 @@ cat_status_t cat_selftest_wait_timeout(void *workspace, size_t workspace_bytes, 
 
 /* Kernel selection for the distance contraction.  With K >= min_k (and D % 4 == 0,
  * K <= 256) the scores are formed on the tensor cores (tcgen05, TF32 or fp16 operands, fp32
- * accumulation); below it on the fp32 pipes.  Rows with D % 4 != 0 are scored from a padded fp16 copy
- * where K >= min_k / 4 and K * D >= 1024.  Either way undecided rows are settled in
+ * accumulation); below it on the fp32 pipes.  Fits (and inference on rows with D % 4 != 0) use a padded
+ * fp16 copy of the rows from K >= min_k / 4 and K * D >= 1024 on, short rows excepted.  Either way undecided rows are settled in
  * fp64, so the labels are the same.  Default 8: measured at K = 8, 16 and 32 (rows of 1000
  * columns) a Lloyd round takes half the time on the tensor path and so does inference, except
  * where low-precision scores leave most rows undecided (unimodal data, K = 32: there the fp32

@@ -41,8 +41,10 @@ static void carve_assign_into(Carver &c, AssignWs &w, int64_t N, int D, int K, b
     w.cand_rows = c.take<int32_t>((size_t)N);
     w.cand_list = c.take<uint64_t>((size_t)N);
     w.cmax = c.take<float>((size_t)K);
+    w.cerr = c.take<float>((size_t)K);
+    w.mean = c.take<float>((size_t)D);
     w.ch = c.take<uint16_t>((size_t)K * half_ld(D));
-    w.hscale = c.take<float>(row_copy ? 4 + (size_t)N : 4);
+    w.hscale = c.take<float>(row_copy ? 4 + 2 * (size_t)N : 4);
     const size_t prep = inference ? apply_rows_prep_bytes(N, D, K) : 0;
     w.prep = prep ? c.take<unsigned char>(prep) : nullptr;
     w.yh = row_copy ? c.take<uint16_t>((size_t)N * half_ld(D)) : nullptr;
@@ -78,7 +80,7 @@ FitWs carve_fit(void *base, int64_t N, int D, int K)
     }
     w.yh = c.take<uint16_t>((size_t)N * half_ld(D));
     w.ch = c.take<uint16_t>((size_t)K * half_ld(D));
-    w.hscale = c.take<float>(4 + (size_t)N);
+    w.hscale = c.take<float>(4 + 2 * (size_t)N);
     w.sumQ = c.take<double>(KD);
     w.sumF = c.take<double>(KD);
     w.var = c.take<double>(KD);
@@ -86,6 +88,8 @@ FitWs carve_fit(void *base, int64_t N, int D, int K)
     w.meanQ = c.take<double>(KD);
     w.meanF = c.take<double>(KD);
     w.counts = c.take<int64_t>((size_t)K);
+    w.norm_part = c.take<unsigned char>(centroid_update_scratch_bytes(D, K));
+    w.arrivals = c.take<uint32_t>((size_t)K);
     if (small_fit_supported(N, D, K)) {
         // per-CTA partial sums and sizes of the persistent small-problem kernel
         w.small_part = c.take<double>(small_part_doubles(D, K));
@@ -117,15 +121,17 @@ static bool use_tensor_path(int64_t N, int D, int K)
     return K >= g_tc_min_k.load(std::memory_order_relaxed) && tc_supported(N, D, K);
 }
 
-// Assignments on fp16 copies of rows and centroids.  Rows that need padding (D % 8 != 0) have to earn
-// the copy: measured over ten rounds, 100 000 x 10 with K = 16 takes 491 us with it and 443 without,
-// K = 128 takes 642 and 820, 20 000 x 33 with K = 64 457 and 469.  Where D % 4 != 0 the alternative is scalar
-// loads on the fp32 pipes, which loses from a quarter of the usual K on (49 999 x 1001, K = 3: 4.1 ms).
+// Assignments on fp16 copies of rows and centroids, from the threshold on where rows need no padding.  Otherwise
+// the copy has to be earned: measured over ten rounds, 100 000 x 10 with K = 16 takes 491 us with it and 443 without,
+// K = 128 takes 642 and 820, 20 000 x 33 with K = 64 457 and 469; and a quarter of the threshold does, since the
+// fp32 pipes' tiles stay half empty there (a round on 33 805 x 1000, K = 2: 75 us against 111).
 static bool use_half_path(int64_t N, int D, int K)
 {
     const int min_k = g_tc_min_k.load(std::memory_order_relaxed);
-    if (D % 8 != 0 && (int64_t)D * K < 1024) return false;
-    return K >= (D % 4 != 0 ? min_k / 4 + (min_k % 4 != 0) : min_k) && tc_half_supported(N, D, K);
+    if (!tc_half_supported(N, D, K)) return false;
+    if (K >= min_k && D % 8 == 0) return true;
+    if (D % 4 == 0 && D < 256 && K < min_k) return false;   // (the pipes' tiles are short there: 100 000 x 200, K = 2: 93 us a round against 111)
+    return K >= min_k / 4 + (min_k % 4 != 0) && (int64_t)D * K >= 1024;
 }
 
 // the persistent single-launch kernels take the small shapes they support, unless switched off
@@ -171,7 +177,7 @@ static cat_status_t run_assign(const float *Y, int64_t N, int D, int K, const fl
                                int32_t *labels, const AssignWs &w, const float *gamma,
                                const float *beta, float *out, cudaStream_t s,
                                bool row_norms_ready = false, bool top_level = true,
-                               const void *Yh = nullptr, void *Ch = nullptr, const float *hscale = nullptr,
+                               const void *Yh = nullptr, void *Ch = nullptr, float *hscale = nullptr,
                                bool centroids_ready = false, const FastOut *fast = nullptr)
 {
     if (out && labels && top_level && !fast && use_small_apply(N, D, K)) {
@@ -195,7 +201,7 @@ static cat_status_t run_assign(const float *Y, int64_t N, int D, int K, const fl
     if (out && !fast && use_tensor_path(N, D, K) && choose_apply_form(N, D, K) == 64) {
         // inference on 64-row tiles: fp16 copy of the centroids (scaled by a power of two from
         // their largest magnitude), rows converted inside the kernel
-        CAT_CUDA(launch_centroid_half(C, D, K, w.cnorm, w.cmax, w.hscale, w.ch, w.ctl, s, top_level));
+        CAT_CUDA(launch_centroid_half(C, D, K, nullptr, w.cnorm, w.cmax, w.cerr, w.hscale, w.ch, w.ctl, s, top_level));
         CAT_CUDA(launch_apply_h64(Y, N, D, K, w.ch, w.hscale, w.cnorm, labels, w.refine_rows, w.cand_rows, w.cand_list,
                                   w.ctl, gamma, beta, out, s));
         CAT_CUDA(launch_refine_both(Y, N, D, K, C, labels, w.cand_rows, w.cand_list, w.refine_rows, w.ctl, gamma,
@@ -207,10 +213,11 @@ static cat_status_t run_assign(const float *Y, int64_t N, int D, int K, const fl
         // then corrected in a pass of their own -- 16 bytes of traffic per element against 8, but on the
         // tensor cores (49 999 x 1001, K = 50: 233 us against 1546 us on the fp32 pipes, whose loads of
         // such rows are scalar).
-        CAT_CUDA(launch_half_shadow(Y, N, D, w.ynorm2, w.hscale, w.yh, s, false));
-        CAT_CUDA(launch_centroid_half(C, D, K, w.cnorm, w.cmax, w.hscale, w.ch, w.ctl, s, top_level));
+        CAT_CUDA(launch_sample_mean(Y, N, D, w.mean, s));
+        CAT_CUDA(launch_half_shadow(Y, N, D, w.mean, w.ynorm2, w.hscale, w.yh, s, false));
+        CAT_CUDA(launch_centroid_half(C, D, K, w.mean, w.cnorm, w.cmax, w.cerr, w.hscale, w.ch, w.ctl, s, top_level));
         CAT_CUDA(launch_assign_tc(Y, N, D, K, C, w.cnorm, w.ynorm2, labels, w.refine_rows, w.cand_rows, w.cand_list, w.ctl,
-                                  nullptr, nullptr, nullptr, s, w.yh, w.ch, w.hscale));
+                                  nullptr, nullptr, nullptr, s, w.yh, w.ch, w.hscale, w.cerr));
         CAT_CUDA(launch_refine_both(Y, N, D, K, C, labels, w.cand_rows, w.cand_list, w.refine_rows, w.ctl, nullptr,
                                     nullptr, nullptr, s));
         if (out) CAT_CUDA(launch_affine_labels(Y, N, D, K, labels, gamma, beta, out, s));
@@ -218,12 +225,13 @@ static cat_status_t run_assign(const float *Y, int64_t N, int D, int K, const fl
     }
     // centroids_ready: the centroid update that produced C has already left its norms, its fp16
     // copy and empty exact-pass queues in the workspace
-    if (!centroids_ready) CAT_CUDA(launch_centroid_norms(C, D, K, w.cnorm, w.ctl, s, top_level));
+    if (!centroids_ready && !Yh) CAT_CUDA(launch_centroid_norms(C, D, K, w.cnorm, w.ctl, s, top_level));
     if (Yh || use_tensor_path(N, D, K)) {
         if (!out && !row_norms_ready) CAT_CUDA(launch_row_norms(Y, N, D, w.ynorm2, s));
-        if (Yh && !centroids_ready) CAT_CUDA(launch_to_half(C, D, K, hscale, Ch, s));
+        if (Yh && !centroids_ready)
+            CAT_CUDA(launch_centroid_half(C, D, K, w.mean, w.cnorm, w.cmax, w.cerr, hscale, Ch, w.ctl, s, top_level, false));
         CAT_CUDA(launch_assign_tc(Y, N, D, K, C, w.cnorm, w.ynorm2, labels, w.refine_rows, w.cand_rows,
-                                  w.cand_list, w.ctl, gamma, beta, out, s, Yh, Ch, hscale, fast));
+                                  w.cand_list, w.ctl, gamma, beta, out, s, Yh, Ch, hscale, w.cerr, fast));
         CAT_CUDA(launch_refine_both(Y, N, D, K, C, labels, w.cand_rows, w.cand_list, w.refine_rows, w.ctl, gamma,
                                     beta, out, s));
     } else {
@@ -266,7 +274,7 @@ static cat_status_t run_delta_update(const float *Yq, const int32_t *labels, con
     CAT_CUDA(launch_segment_sums(0, Yq, nullptr, w.order, w.cluster_start, w.seg_start, nullptr, nullptr, D,
                                  2 * K, g, w.segpart, s));
     CAT_CUDA(launch_centroid_update(w.segpart, w.seg_start, w.counts, D, K, w.sumQ, C, w.a.cnorm, w.hscale,
-                                    half ? w.ch : nullptr, w.a.ctl, s));
+                                    half ? w.ch : nullptr, half ? w.a.mean : nullptr, w.a.cerr, w.norm_part, w.arrivals, w.a.ctl, s));
     return CAT_OK;
 }
 
@@ -355,7 +363,7 @@ cat_status_t cat_apply_bf16(const float *Yq, int64_t N, int32_t D, int32_t K, co
     if (use_tensor_path(N, D, K) && apply_h64_supported(N, D, K)) {
         // fused: the 64-row-tile kernel writes bf16 with the fast labels; the exact pass settles the
         // undecided rows' labels, and those rows are written once more
-        CAT_CUDA(launch_centroid_half(centroids, D, K, w.cnorm, w.cmax, w.hscale, w.ch, w.ctl, s, true));
+        CAT_CUDA(launch_centroid_half(centroids, D, K, nullptr, w.cnorm, w.cmax, w.cerr, w.hscale, w.ch, w.ctl, s, true));
         CAT_CUDA(launch_apply_h64(Yq, N, D, K, w.ch, w.hscale, w.cnorm, labels, w.refine_rows, w.cand_rows, w.cand_list, w.ctl,
                                   gamma, beta, reinterpret_cast<float *>(Y_out_bf16), s, true));
         CAT_CUDA(launch_refine_both(Yq, N, D, K, centroids, labels, w.cand_rows, w.cand_list, w.refine_rows, w.ctl, nullptr,
@@ -405,12 +413,12 @@ cat_status_t cat_assign_scores(const float *Yq, int64_t N, int32_t D, int32_t K,
         if (!workspace || !aligned16(workspace) || workspace_bytes < cat_fit_workspace_bytes(N, D, K))
             return CAT_ERR_WORKSPACE;
         FitWs w = carve_fit(workspace, N, D, K);
-        CAT_CUDA(launch_centroid_norms(centroids, D, K, w.a.cnorm, w.a.ctl, s, true));
-        CAT_CUDA(launch_half_shadow(Yq, N, D, w.a.ynorm2, w.hscale, w.yh, s));
-        CAT_CUDA(launch_to_half(centroids, D, K, w.hscale, w.ch, s));
+        // (relative to the origin here: the scores handed out are those of the rows as they are)
+        CAT_CUDA(launch_half_shadow(Yq, N, D, nullptr, w.a.ynorm2, w.hscale, w.yh, s));
+        CAT_CUDA(launch_centroid_half(centroids, D, K, nullptr, w.a.cnorm, w.a.cmax, w.a.cerr, w.hscale, w.ch, w.a.ctl, s, true, false));
         CAT_CUDA(launch_assign_tc(Yq, N, D, K, centroids, w.a.cnorm, w.a.ynorm2, labels_out, w.a.refine_rows,
                                   w.a.cand_rows, w.a.cand_list, w.a.ctl, nullptr, nullptr, nullptr, s, w.yh, w.ch,
-                                  w.hscale, &fast));
+                                  w.hscale, w.a.cerr, &fast));
         CAT_CUDA(launch_refine_both(Yq, N, D, K, centroids, labels_out, w.a.cand_rows, w.a.cand_list, w.a.refine_rows,
                                     w.a.ctl, nullptr, nullptr, nullptr, s));
         return CAT_OK;
@@ -475,8 +483,10 @@ cat_status_t cat_fit_from(const float *Yq, const float *Yfp, int64_t N, int32_t 
     const bool tc = half || use_tensor_path(N, D, K);
     const void *Yh = half ? w.yh : nullptr;
     if (small) {
-    } else if (half) CAT_CUDA(launch_half_shadow(Yq, N, D, w.a.ynorm2, w.hscale, w.yh, s));
-    else if (tc) CAT_CUDA(launch_row_norms(Yq, N, D, w.a.ynorm2, s));
+    } else if (half) {
+        CAT_CUDA(launch_sample_mean(Yq, N, D, w.a.mean, s));
+        CAT_CUDA(launch_half_shadow(Yq, N, D, w.a.mean, w.a.ynorm2, w.hscale, w.yh, s));
+    } else if (tc) CAT_CUDA(launch_row_norms(Yq, N, D, w.a.ynorm2, s));
 
     // Lloyd rounds.  Two label buffers alternate so that a round sees the previous round's
     // labels and the final assignment lands in `labels`; the running per-cluster sums and
@@ -487,6 +497,7 @@ cat_status_t cat_fit_from(const float *Yq, const float *Yfp, int64_t N, int32_t 
     CAT_CUDA(cudaMemsetAsync(lab[(iters & 1) ^ 1], 0xFF, (size_t)N * sizeof(int32_t), s));
     CAT_CUDA(cudaMemsetAsync(w.sumQ, 0, KD * sizeof(double), s));
     CAT_CUDA(cudaMemsetAsync(w.counts, 0, (size_t)K * sizeof(int64_t), s));
+    CAT_CUDA(cudaMemsetAsync(w.arrivals, 0, (size_t)K * sizeof(uint32_t), s));
     for (int t = 0; t < iters; ++t) {
         int32_t *cur = lab[(iters - t) & 1], *prev = lab[((iters - t) & 1) ^ 1];
         st = run_assign(Yq, N, D, K, C, cur, w.a, nullptr, nullptr, nullptr, s, tc, false, Yh, w.ch, w.hscale,
@@ -556,9 +567,10 @@ cat_status_t cat_fit_shard_begin(const float *Yq, int64_t N, int32_t D, int32_t 
     FitWs w = carve_fit(workspace, N, D, K);
     CAT_CUDA(launch_reset_control(w.a.ctl, s));
     CAT_CUDA(cudaMemsetAsync(w.hscale, 0, 4 * sizeof(float), s));
-    if (use_half_path(N, D, K))
-        CAT_CUDA(launch_half_shadow(Yq, N, D, w.a.ynorm2, w.hscale, w.yh, s, false));
-    else if (use_tensor_path(N, D, K))
+    if (use_half_path(N, D, K)) {
+        CAT_CUDA(launch_sample_mean(Yq, N, D, w.a.mean, s));
+        CAT_CUDA(launch_half_shadow(Yq, N, D, w.a.mean, w.a.ynorm2, w.hscale, w.yh, s, false));
+    } else if (use_tensor_path(N, D, K))
         CAT_CUDA(launch_row_norms(Yq, N, D, w.a.ynorm2, s));
     // (the bit pattern of a non-negative float is the float itself)
     CAT_CUDA(cudaMemcpyAsync(amax_out, w.hscale, sizeof(float), cudaMemcpyDeviceToDevice, s));

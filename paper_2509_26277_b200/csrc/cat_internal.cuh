@@ -95,8 +95,10 @@ struct AssignWs {          // what assign/apply need
     int32_t *cand_rows;    // [N] rows queued with candidates
     uint64_t *cand_list;   // [N] their candidates, 4 x 16 bit
     float *cmax;           // [K] largest magnitude of each centroid
+    float *cerr;           // [K] norms of the rounding errors of the fp16 centroids
+    float *mean;           // [D] what rows and centroids are taken relative to on fp16 operands
     void *ch;              // [K][half_ld(D)] fp16 copy of the centroids (inference on fp16 operands)
-    float *hscale;         // [4] scale of that copy: {s_c, -2 / s_c, 2^-25 / s_c, -}; with yh followed by [N] inverse row scales
+    float *hscale;         // [4] scale of that copy: {s_c, -2 / s_c, 2^-25 / s_c, -}; with yh followed by [N] inverse row scales and [N] rounding errors
     void *prep;            // prepared centroids of the inference kernel that keeps rows in shared memory (or null)
     void *yh;              // [N][half_ld(D)] fp16 copy of the rows (inference with D % 4 != 0), else null
     size_t bytes;
@@ -115,10 +117,12 @@ struct FitWs {
     double *segpart;       // [max_segs][2][D] per-segment partial sums
     void *yh;              // [N][half_ld(D)] fp16 copy of Yq (tensor-core fits)
     void *ch;              // [K][half_ld(D)] fp16 copy of the centroids
-    float *hscale;         // [4 + N] scale of the fp16 centroids, then the inverse row scales
+    float *hscale;         // [4 + 2N] scale of the fp16 centroids, the inverse row scales, the rows' rounding errors
     double *sumQ, *sumF, *var, *cov;   // [K*D] each
     double *meanQ, *meanF;             // [K*D] each
     int64_t *counts;       // [K]
+    void *norm_part;       // parts of the centroid norms (centroid update)
+    uint32_t *arrivals;    // [K] CTAs of a cluster that have left theirs
     double *small_part;    // [SMALL_MAX_GRID][K*D] per-CTA sums of the persistent small-problem kernel (or null)
     int32_t *small_counts; // [SMALL_MAX_GRID][K+1]
     size_t bytes;
@@ -199,29 +203,30 @@ cudaError_t launch_assign_tc(const float *Y, int64_t N, int D, int K, const floa
                              int32_t *cand_rows, uint64_t *cand_list, Control *ctl,
                              const float *gamma, const float *beta, float *out, cudaStream_t s,
                              const void *Yh = nullptr, const void *Ch = nullptr, const float *scale = nullptr,
-                             const FastOut *fast = nullptr);
+                             const float *cerr = nullptr, const FastOut *fast = nullptr);
 
 // One warp waits (at most limit_ms, clamped to 1 .. 1000) on a barrier that is never completed.
 cudaError_t launch_wait_selftest(Control *ctl, int limit_ms, cudaStream_t s);
 
-// fp16 copy of a matrix for repeated assignments, made in one sweep: squared row norms, per-row
-// power-of-two scales, Yh[i] = fp16(Y[i] * scale_i), and scale[4 + N] = {centroid scale s_c from the
-// largest magnitude, -2 / s_c, 2^-25 / s_c, unused, then 1 / scale_i for every row}.  Rows of the copies
-// (of the centroids too) are half_ld(D) elements apart, so that any row length suits the tensor maps.
+// fp16 copy of a matrix for repeated assignments, made in one sweep, of the rows less `mean` (null: as they
+// are): squared row norms, per-row power-of-two scales, Yh[i] = fp16((Y[i] - mean) * scale_i), and
+// scale[4 + 2 N] = {centroid scale s_c from the largest magnitude of Y, -2 / s_c, 2^-25 / s_c, unused, then
+// 1 / scale_i for every row, then the norm of every row's rounding error}.  Rows of the copies (of the centroids
+// too) are half_ld(D) elements apart, so that any row length suits the tensor maps.
 __host__ __device__ constexpr int half_ld(int D) { return (D + 7) & ~7; }
 constexpr int TC_HALF_MIN_D = 8;
 bool tc_half_supported(int64_t N, int D, int K);
 // finish_scale = false leaves the bits of the largest magnitude in scale[0] (launch_half_scale turns them
 // into the three scale words later, e.g. once the maximum over several shards is known).
-cudaError_t launch_half_shadow(const float *Y, int64_t N, int D, float *ynorm2, float *scale, void *Yh,
+cudaError_t launch_half_shadow(const float *Y, int64_t N, int D, const float *mean, float *ynorm2, float *scale, void *Yh,
                                cudaStream_t s, bool finish_scale = true);
-// Ch = fp16(C * scale[0])
-cudaError_t launch_to_half(const float *C, int D, int K, const float *scale, void *Ch, cudaStream_t s);
-// Everything an assignment on fp16 operands needs of the centroids: norms, the scale words from their
-// largest magnitude (cmax: [K] scratch), the fp16 copy; empties the exact-pass queues as
-// launch_centroid_norms does.
-cudaError_t launch_centroid_half(const float *C, int D, int K, float *cnorm, float *cmax, float *scale, void *Ch, Control *ctl,
-                                 cudaStream_t s, bool reset_all);
+// A point among the rows to take them relative to: the column means of the first 128 (any point will do).
+cudaError_t launch_sample_mean(const float *Y, int64_t N, int D, float *mean, cudaStream_t s);
+// Everything an assignment on fp16 operands needs of the centroids less `mean` (null: as they are): norms,
+// the fp16 copy, the norms cerr of its rounding errors, and with own_scale the scale words from their largest
+// magnitude (cmax: [K] scratch); empties the exact-pass queues as launch_centroid_norms does.
+cudaError_t launch_centroid_half(const float *C, int D, int K, const float *mean, float *cnorm, float *cmax, float *cerr, float *scale,
+                                 void *Ch, Control *ctl, cudaStream_t s, bool reset_all, bool own_scale = true);
 
 // Exact fp64 decision among the listed candidates of each queued row; optional affine output.
 cudaError_t launch_refine_both(const float *Y, int64_t N, int D, int K, const float *C, int32_t *labels,
@@ -256,10 +261,14 @@ cudaError_t launch_segment_combine3(const double *part, const int32_t *seg_start
                                     double *out1, double *out2, cudaStream_t s);
 
 // Delta-mode centroid update fused with what the next assignment needs: running sums, centroids,
-// their squared norms, (with Ch) their fp16 copy, and the reset of the exact-pass queues.
+// their squared norms, (with Ch) their fp16 copy with its rounding errors' norms -- norms and copy of the
+// centroids less `mean` if that is given -- and the reset of the exact-pass queues.  norm_part: scratch;
+// arrivals: [K], zero before the first call (left at zero).
 cudaError_t launch_centroid_update(const double *part, const int32_t *seg_start, const int64_t *counts, int D,
                                    int K, double *sums, float *C, float *cnorm, const float *scale, void *Ch,
-                                   Control *ctl, cudaStream_t s);
+                                   const float *mean, float *cerr, void *norm_part, uint32_t *arrivals, Control *ctl,
+                                   cudaStream_t s);
+size_t centroid_update_scratch_bytes(int D, int K);
 
 cudaError_t launch_centroids_from_sums(const double *sums, const int64_t *counts, int D, int K,
                                        float *C, cudaStream_t s);

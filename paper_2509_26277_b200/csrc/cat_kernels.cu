@@ -426,117 +426,213 @@ cudaError_t launch_assign(const float *Y, int64_t N, int D, int K, const float *
 constexpr int R_THREADS = 256;
 constexpr int R_WARPS = R_THREADS / 32;
 
-// One CTA per queued row: warp w evaluates centroids w, w + 8, ... in direct form with fp64
-// accumulation; the CTA then takes the smallest distance, lowest index on equality.
-// The same decision for RG queued rows per CTA at a time (rows of at most RG_MAX_D columns): the
-// rows sit in shared memory as fp64, so a centroid element is fetched and converted once for RG
-// rows and a row element is converted once for all K centroids -- the scan is bound by those
-// conversions and by the fp64 pipe, not by memory.  Warp w takes centroids w, w + 8, ... for all
-// rows of the group; lowest index on equality, as in the single-row form.
-constexpr int RG = 4;
-constexpr int RG_MAX_D = 1024;
+// Relative error of a direct-form fp32 sum of squares whose lanes add D / 32 terms each before a tree adds the
+// lanes, with room for the comparison: two sums further apart than this factor are in the order of the exact
+// ones.  Sums below 1e-30 may have lost squares to underflow: whatever is that small stays a candidate.
+__device__ __forceinline__ float fp32_sum_limit(float best, int D)
+{
+    const float eta = 1.0625f * ((float)D * 0.03125f + 12.f) * 5.9604645e-8f;
+    return fmaxf(best, 1e-30f) * (1.f + 2.25f * eta);
+}
+
+__device__ __forceinline__ double exact_distance(const float *y, const float *__restrict__ c, int D, int lane)
+{
+    double s0 = 0.0, s1 = 0.0;
+    int j = lane;
+#pragma unroll 2
+    for (; j + 32 < D; j += 64) {
+        const double d0 = (double)y[j] - (double)c[j], d1 = (double)y[j + 32] - (double)c[j + 32];
+        s0 = fma(d0, d0, s0);
+        s1 = fma(d1, d1, s1);
+    }
+    if (j < D) {
+        const double d0 = (double)y[j] - (double)c[j];
+        s0 = fma(d0, d0, s0);
+    }
+    return warp_sum(s0 + s1);
+}
+
+// Sums of 16 values over the warp, 16 exchanges in place of 80; lanes 2 i and 2 i + 1 end with the sum of acc[i].
+__device__ __forceinline__ float warp_sum16(float *acc, int lane)
+{
+#pragma unroll
+    for (int h = 8, o = 16; h > 0; h >>= 1, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (i < h) {
+                const float send = up ? acc[i] : acc[i + h];
+                const float keep = up ? acc[i + h] : acc[i];
+                acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+    }
+    return acc[0] + __shfl_xor_sync(0xffffffffu, acc[0], 1);
+}
+
+// Scan of all K centroids for RG queued rows per CTA at a time.  The rows sit in shared memory; a warp forms
+// the fp32 direct-form distances of eight rows to four centroids together (12 operand loads for 32 sums, all of
+// a step's centroid loads in flight), then a warp per row takes the smallest and settles what lies within the
+// sums' error of it in fp64, lowest index on equality.  (All distances in fp64, the earlier form, was bound by
+// the fp32 to fp64 conversions: this pass took 43 us of a Lloyd round on 50 000 x 1000 logits, K = 32, and
+// takes 21 now, with a quarter of the rows left undecided that were before.)
+constexpr int RG = 8;
+constexpr int RG_MAX_D = 1536;
+constexpr size_t RG_MAX_SMEM = (size_t)RG * RG_MAX_D * 4 + (size_t)RG * CAT_MAX_K * 4;
+
+// RT: rows a warp takes at a time; fewer where K alone does not occupy the warps
+template <bool VEC, int RT>
+__device__ __forceinline__ void refine_distances(const float *ys_all, int ld, const float *__restrict__ C, int D, int K, float *dist_all)
+{
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int unit = w; unit < (K + 3) / 4 * (RG / RT); unit += R_WARPS) {
+        const int k0 = unit / (RG / RT) * 4, r0 = unit % (RG / RT) * RT;
+        const float *ys = ys_all + r0 * ld;
+        float *dist = dist_all + r0 * K;
+        float acc[RT * 4];
+#pragma unroll
+        for (int i = 0; i < RT * 4; ++i) acc[i] = 0.f;
+        const float *cp[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) cp[q] = C + (size_t)(k0 + q < K ? k0 + q : k0) * D;
+        if (VEC) {
+#pragma unroll 2
+            for (int j = lane; j < (D >> 2); j += 32) {
+                float4 cv[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) cv[q] = reinterpret_cast<const float4 *>(cp[q])[j];
+#pragma unroll
+                for (int r = 0; r < RT; ++r) {
+                    const float4 y = reinterpret_cast<const float4 *>(ys + r * ld)[j];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        float a = acc[r * 4 + q], d;
+                        d = y.x - cv[q].x; a = fmaf(d, d, a);
+                        d = y.y - cv[q].y; a = fmaf(d, d, a);
+                        d = y.z - cv[q].z; a = fmaf(d, d, a);
+                        d = y.w - cv[q].w; a = fmaf(d, d, a);
+                        acc[r * 4 + q] = a;
+                    }
+                }
+            }
+        } else {
+#pragma unroll 4
+            for (int j = lane; j < D; j += 32) {
+                float cv[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) cv[q] = cp[q][j];
+#pragma unroll
+                for (int r = 0; r < RT; ++r) {
+                    const float y = ys[r * ld + j];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float d = y - cv[q];
+                        acc[r * 4 + q] = fmaf(d, d, acc[r * 4 + q]);
+                    }
+                }
+            }
+        }
+        if constexpr (RT == 8) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float s = warp_sum16(acc + 16 * h, lane);
+                const int r = 4 * h + (lane >> 3), q = (lane >> 1) & 3;
+                if ((lane & 1) == 0 && k0 + q < K) dist[r * K + k0 + q] = s;
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < RT * 4; ++i) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
+                if (lane == 0 && k0 + (i & 3) < K) dist[(i >> 2) * K + k0 + (i & 3)] = acc[i];
+            }
+        }
+    }
+}
+
+template <bool VEC>
+__device__ __forceinline__ void refine_distances(const float *ys, int ld, const float *__restrict__ C, int D, int K, float *dist)
+{
+    if (K > 16) refine_distances<VEC, 8>(ys, ld, C, D, K, dist);
+    else if (K > 4) refine_distances<VEC, 2>(ys, ld, C, D, K, dist);
+    else refine_distances<VEC, 1>(ys, ld, C, D, K, dist);
+}
 
 template <bool AFFINE>
 __device__ __forceinline__ void refine_body_grouped(const float *__restrict__ Y, int64_t N, int D, int K,
                                                     const float *__restrict__ C, int32_t *labels,
                                                     const int32_t *__restrict__ refine_rows, Control *ctl,
-                                                    const float *gamma, const float *beta, float *out,
-                                                    double *ys /* [RG][D] shared */)
+                                                    const float *gamma, const float *beta, float *out, float *ys)
 {
-    __shared__ double g_best[R_WARPS][RG];
-    __shared__ int g_idx[R_WARPS][RG];
-    __shared__ int g_label[RG];
-    __shared__ int64_t g_row[RG];
     int count = ctl->refine_count;
     if ((int64_t)count > N) count = (int)N;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         ctl->refined_total += count;
         ctl->refined_last = count + ctl->cand_count;
     }
-    const int lane = threadIdx.x & 31;
-    const int w = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int ld = (D + 3) & ~3;
+    float *dist = ys + RG * ld;   // [RG][K]
+    const bool vec4 = (D & 3) == 0 && ((reinterpret_cast<uintptr_t>(Y) | reinterpret_cast<uintptr_t>(C)) & 15u) == 0;
+    static_assert(RG == R_WARPS, "a warp per row of the group");
     for (int base = blockIdx.x * RG; base < count; base += gridDim.x * RG) {
-        const int nr = (count - base < RG) ? (count - base) : RG;
-        if (threadIdx.x < RG) {
-            int64_t row = (threadIdx.x < nr) ? (int64_t)refine_rows[base + threadIdx.x] : -1;
-            if (row >= N) row = -1;
-            g_row[threadIdx.x] = row;
+        // this warp's row
+        int64_t row = base + w < count ? (int64_t)refine_rows[base + w] : -1;
+        if (row >= N) row = -1;
+        float *y = ys + w * ld;
+        if (vec4) {
+#pragma unroll 4
+            for (int j = lane; j < (D >> 2); j += 32)
+                reinterpret_cast<float4 *>(y)[j] =
+                    row >= 0 ? __ldg(reinterpret_cast<const float4 *>(Y + (size_t)row * D) + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+        } else {
+#pragma unroll 8
+            for (int j = lane; j < D; j += 32) y[j] = row >= 0 ? __ldg(Y + (size_t)row * D + j) : 0.f;
         }
         __syncthreads();
-        for (int r = 0; r < RG; ++r) {
-            const int64_t row = g_row[r];
-            for (int j = threadIdx.x; j < D; j += R_THREADS)
-                ys[r * D + j] = (row >= 0) ? (double)Y[(size_t)row * D + j] : 0.0;
-        }
+        if (vec4) refine_distances<true>(ys, ld, C, D, K, dist);
+        else refine_distances<false>(ys, ld, C, D, K, dist);
         __syncthreads();
-        double best[RG];
-        int bk[RG];
+        if (row >= 0) {
+            const float *d = dist + w * K;
+            float best = CUDART_INF_F;
+            for (int k = lane; k < K; k += 32) best = fminf(best, d[k]);
 #pragma unroll
-        for (int r = 0; r < RG; ++r) {
-            best[r] = CUDART_INF;
-            bk[r] = K;
-        }
-        for (int k = w; k < K; k += R_WARPS) {
-            const float *c = C + (size_t)k * D;
-            double s[RG];
-#pragma unroll
-            for (int r = 0; r < RG; ++r) s[r] = 0.0;
-            for (int j = lane; j < D; j += 32) {
-                const double cv = (double)c[j];
-#pragma unroll
-                for (int r = 0; r < RG; ++r) {
-                    const double d = ys[r * D + j] - cv;
-                    s[r] = fma(d, d, s[r]);
-                }
+            for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
+            const float lim = fp32_sum_limit(best, D);
+            int n = 0, l = -1;
+            for (int b = 0; b < K; b += 32) {
+                const uint32_t m = __ballot_sync(0xffffffffu, b + lane < K && !(d[b + lane < K ? b + lane : 0] > lim));
+                if (m && l < 0) l = b + __ffs(m) - 1;
+                n += __popc(m);
             }
-#pragma unroll
-            for (int r = 0; r < RG; ++r) {
-                const double v = warp_sum(s[r]);
-                if (v < best[r]) {
-                    best[r] = v;
-                    bk[r] = k;
-                }
+            if (n != 1) {
+                double b64 = CUDART_INF;
+                if (l < 0) l = 0;   // only when every distance is NaN
+                for (int b = 0; b < K; b += 32)
+                    for (uint32_t m = __ballot_sync(0xffffffffu, b + lane < K && !(d[b + lane < K ? b + lane : 0] > lim)); m; m &= m - 1) {
+                        const int k = b + __ffs(m) - 1;
+                        const double v = exact_distance(y, C + (size_t)k * D, D, lane);
+                        if (v < b64) {
+                            b64 = v;
+                            l = k;
+                        }
+                    }
             }
-        }
-        if (lane == 0) {
-#pragma unroll
-            for (int r = 0; r < RG; ++r) {
-                g_best[w][r] = best[r];
-                g_idx[w][r] = bk[r];
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x < RG) {
-            const int r = threadIdx.x;
-            double b = g_best[0][r];
-            int k = g_idx[0][r];
-#pragma unroll
-            for (int q = 1; q < R_WARPS; ++q) {
-                if (g_best[q][r] < b || (g_best[q][r] == b && g_idx[q][r] < k)) {
-                    b = g_best[q][r];
-                    k = g_idx[q][r];
-                }
-            }
-            if (k >= K) k = 0;  // only when every distance is NaN
-            if (g_row[r] >= 0) labels[g_row[r]] = k;
-            g_label[r] = k;
-        }
-        __syncthreads();
-        if (AFFINE) {
-            for (int r = 0; r < RG; ++r) {
-                const int64_t row = g_row[r];
-                if (row < 0) continue;
-                const float *y = Y + (size_t)row * D;
-                const float *g = gamma + (size_t)g_label[r] * D;
-                const float *bb = beta + (size_t)g_label[r] * D;
+            if (lane == 0) labels[row] = l;
+            if (AFFINE) {
+                const float *g = gamma + (size_t)l * D;
+                const float *bb = beta + (size_t)l * D;
                 float *o = out + (size_t)row * D;
-                for (int j = threadIdx.x; j < D; j += R_THREADS) o[j] = fmaf(g[j], y[j], bb[j]);
+#pragma unroll 4
+                for (int j = lane; j < D; j += 32) o[j] = fmaf(g[j], y[j], bb[j]);
             }
         }
         __syncthreads();
     }
 }
 
+// One CTA per queued row (rows too long for the form above): warp w evaluates centroids w, w + 8, ... in
+// direct form with fp64 accumulation; the CTA then takes the smallest distance, lowest index on equality.
 template <bool AFFINE>
 __device__ __forceinline__ void refine_body(const float *__restrict__ Y, int64_t N, int D, int K,
                                             const float *__restrict__ C, int32_t *labels,
@@ -624,24 +720,32 @@ __global__ void __launch_bounds__(R_THREADS) refine_kernel(const float *__restri
                                                            Control *ctl, const float *gamma,
                                                            const float *beta, float *out)
 {
-    extern __shared__ double refine_rows_f64[];
-    if (D <= RG_MAX_D) refine_body_grouped<AFFINE>(Y, N, D, K, C, labels, refine_rows, ctl, gamma, beta, out, refine_rows_f64);
+    extern __shared__ __align__(16) float refine_rows_f32[];
+    if (D <= RG_MAX_D) refine_body_grouped<AFFINE>(Y, N, D, K, C, labels, refine_rows, ctl, gamma, beta, out, refine_rows_f32);
     else refine_body<AFFINE>(Y, N, D, K, C, labels, refine_rows, ctl, gamma, beta, out);
 }
 
-// dynamic shared memory of the full-K exact pass: RG rows as fp64 where the grouped form applies
-static size_t refine_smem_bytes(int D) { return D <= RG_MAX_D ? (size_t)RG * D * sizeof(double) : 0; }
+// dynamic shared memory of the full-K exact pass: RG rows and their distances where the grouped form applies
+static size_t refine_smem_bytes(int D, int K) { return D <= RG_MAX_D ? (size_t)RG * ((D + 3) & ~3) * 4 + (size_t)RG * K * 4 : 0; }
+
+template <typename Kern>
+static cudaError_t refine_config(Kern kern)   // (the same value whatever the shape: several threads may be launching)
+{
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RG_MAX_SMEM);
+}
 
 cudaError_t launch_refine(const float *Y, int64_t N, int D, int K, const float *C,
                           int32_t *labels, const int32_t *refine_rows, Control *ctl,
                           const float *gamma, const float *beta, float *out, cudaStream_t s)
 {
     int blocks = (int)(N < 1184 ? N : 1184);
+    cudaError_t e = out ? refine_config(refine_kernel<true>) : refine_config(refine_kernel<false>);
+    if (e != cudaSuccess) return e;
     if (out)
-        refine_kernel<true><<<blocks, R_THREADS, refine_smem_bytes(D), s>>>(Y, N, D, K, C, labels, refine_rows, ctl,
+        refine_kernel<true><<<blocks, R_THREADS, refine_smem_bytes(D, K), s>>>(Y, N, D, K, C, labels, refine_rows, ctl,
                                                          gamma, beta, out);
     else
-        refine_kernel<false><<<blocks, R_THREADS, refine_smem_bytes(D), s>>>(Y, N, D, K, C, labels, refine_rows, ctl,
+        refine_kernel<false><<<blocks, R_THREADS, refine_smem_bytes(D, K), s>>>(Y, N, D, K, C, labels, refine_rows, ctl,
                                                           gamma, beta, out);
     count_launch();
     return cudaGetLastError();
@@ -691,7 +795,7 @@ __device__ __forceinline__ void refine_candidates_body(
             if (k < K) ncand = q + 1;
         }
         const float *y = Y + (size_t)row * D;
-        double s[4] = {0.0, 0.0, 0.0, 0.0};
+        float s[4] = {0.f, 0.f, 0.f, 0.f};
         if (vec4) {
             // rows and centroids as 128-bit loads (D a multiple of 4, bases 16-byte aligned)
             const float4 *y4 = reinterpret_cast<const float4 *>(y);
@@ -704,15 +808,15 @@ __device__ __forceinline__ void refine_candidates_body(
 #pragma unroll 8
                 for (int j = lane; j < D4; j += 32) {
                     const float4 yv = y4[j], a = c0[j], b = c1[j];
-                    double d;
-                    d = (double)yv.x - (double)a.x; s[0] = fma(d, d, s[0]);
-                    d = (double)yv.y - (double)a.y; s[0] = fma(d, d, s[0]);
-                    d = (double)yv.z - (double)a.z; s[0] = fma(d, d, s[0]);
-                    d = (double)yv.w - (double)a.w; s[0] = fma(d, d, s[0]);
-                    d = (double)yv.x - (double)b.x; s[1] = fma(d, d, s[1]);
-                    d = (double)yv.y - (double)b.y; s[1] = fma(d, d, s[1]);
-                    d = (double)yv.z - (double)b.z; s[1] = fma(d, d, s[1]);
-                    d = (double)yv.w - (double)b.w; s[1] = fma(d, d, s[1]);
+                    float d;
+                    d = yv.x - a.x; s[0] = fmaf(d, d, s[0]);
+                    d = yv.y - a.y; s[0] = fmaf(d, d, s[0]);
+                    d = yv.z - a.z; s[0] = fmaf(d, d, s[0]);
+                    d = yv.w - a.w; s[0] = fmaf(d, d, s[0]);
+                    d = yv.x - b.x; s[1] = fmaf(d, d, s[1]);
+                    d = yv.y - b.y; s[1] = fmaf(d, d, s[1]);
+                    d = yv.z - b.z; s[1] = fmaf(d, d, s[1]);
+                    d = yv.w - b.w; s[1] = fmaf(d, d, s[1]);
                 }
             } else {
 #pragma unroll 4
@@ -721,41 +825,52 @@ __device__ __forceinline__ void refine_candidates_body(
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
                         const float4 c = reinterpret_cast<const float4 *>(cp[q])[j];
-                        double d;
-                        d = (double)yv.x - (double)c.x; s[q] = fma(d, d, s[q]);
-                        d = (double)yv.y - (double)c.y; s[q] = fma(d, d, s[q]);
-                        d = (double)yv.z - (double)c.z; s[q] = fma(d, d, s[q]);
-                        d = (double)yv.w - (double)c.w; s[q] = fma(d, d, s[q]);
+                        float d;
+                        d = yv.x - c.x; s[q] = fmaf(d, d, s[q]);
+                        d = yv.y - c.y; s[q] = fmaf(d, d, s[q]);
+                        d = yv.z - c.z; s[q] = fmaf(d, d, s[q]);
+                        d = yv.w - c.w; s[q] = fmaf(d, d, s[q]);
                     }
                 }
             }
-        } else if (ncand <= 2) {
-            // the common case: only the two nearest are in question
-            for (int j = lane; j < D; j += 32) {
-                const double yv = (double)y[j];
-                const double d0 = yv - (double)cp[0][j];
-                const double d1 = yv - (double)cp[1][j];
-                s[0] = fma(d0, d0, s[0]);
-                s[1] = fma(d1, d1, s[1]);
-            }
         } else {
+#pragma unroll 8
             for (int j = lane; j < D; j += 32) {
-                const double yv = (double)y[j];
+                const float yv = y[j];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    const double d = yv - (double)cp[q][j];
-                    s[q] = fma(d, d, s[q]);
+                    const float d = yv - cp[q][j];
+                    s[q] = fmaf(d, d, s[q]);
                 }
             }
         }
-        double best = CUDART_INF;
-        int bk = K;
+        // fp32 sums first; what lies within their error of the smallest is settled in fp64
+        float fbest = CUDART_INF_F;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const double v = warp_sum(s[q]);
-            if (cand[q] >= 0 && (v < best || (v == best && cand[q] < bk))) {
-                best = v;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
+            if (cand[q] >= 0) fbest = fminf(fbest, s[q]);
+        }
+        const float lim = fp32_sum_limit(fbest, D);
+        int left = 0, bk = K;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (cand[q] >= 0 && !(s[q] > lim)) {
+                ++left;
                 bk = cand[q];
+            }
+        if (left != 1) {
+            double best = CUDART_INF;
+            bk = K;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (cand[q] < 0 || s[q] > lim) continue;
+                const double v = exact_distance(y, cp[q], D, lane);
+                if (v < best || (v == best && cand[q] < bk)) {
+                    best = v;
+                    bk = cand[q];
+                }
             }
         }
         if (bk >= K) bk = (cand[0] >= 0) ? cand[0] : 0;   // only when every distance is NaN
@@ -794,8 +909,8 @@ __global__ void __launch_bounds__(R_THREADS) refine_both_kernel(
     pdl_enter();
     refine_candidates_body<AFFINE>(Y, N, D, K, C, labels, cand_rows, cand_list, ctl, gamma, beta, out, AFFINE);
     __syncthreads();   // (block 0's thread 0 updates the counters in both bodies, in this order)
-    extern __shared__ double refine_rows_f64[];
-    if (D <= RG_MAX_D) refine_body_grouped<AFFINE>(Y, N, D, K, C, labels, refine_rows, ctl, gamma, beta, out, refine_rows_f64);
+    extern __shared__ __align__(16) float refine_rows_f32[];
+    if (D <= RG_MAX_D) refine_body_grouped<AFFINE>(Y, N, D, K, C, labels, refine_rows, ctl, gamma, beta, out, refine_rows_f32);
     else refine_body<AFFINE>(Y, N, D, K, C, labels, refine_rows, ctl, gamma, beta, out);
 }
 
@@ -805,11 +920,13 @@ cudaError_t launch_refine_both(const float *Y, int64_t N, int D, int K, const fl
 {
     int64_t want = (N + (RC_THREADS / 32) - 1) / (RC_THREADS / 32);
     int blocks = (int)(want < 1184 ? want : 1184);
+    cudaError_t e = out ? refine_config(refine_both_kernel<true>) : refine_config(refine_both_kernel<false>);
+    if (e != cudaSuccess) return e;
     if (out)
-        launch_pdl(refine_both_kernel<true>, dim3(blocks), dim3(R_THREADS), refine_smem_bytes(D), s, Y, N, D, K, C, labels,
+        launch_pdl(refine_both_kernel<true>, dim3(blocks), dim3(R_THREADS), refine_smem_bytes(D, K), s, Y, N, D, K, C, labels,
                    cand_rows, cand_list, refine_rows, ctl, gamma, beta, out);
     else
-        launch_pdl(refine_both_kernel<false>, dim3(blocks), dim3(R_THREADS), refine_smem_bytes(D), s, Y, N, D, K, C, labels,
+        launch_pdl(refine_both_kernel<false>, dim3(blocks), dim3(R_THREADS), refine_smem_bytes(D, K), s, Y, N, D, K, C, labels,
                    cand_rows, cand_list, refine_rows, ctl, gamma, beta, out);
     count_launch();
     return cudaGetLastError();

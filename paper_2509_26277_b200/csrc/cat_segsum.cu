@@ -400,71 +400,155 @@ __global__ void segment_combine_kernel(const double *__restrict__ part, const in
     }
 }
 
-// Three-plane partials (MODE 3) added up per cluster.
-__global__ void segment_combine3_kernel(const double *__restrict__ part, const int32_t *__restrict__ seg_start, int D,
-                                        size_t KD, double *__restrict__ out0, double *__restrict__ out1,
-                                        double *__restrict__ out2)
+// The kernels that add up a cluster's segments: a CTA takes `cols` columns of a cluster, 512 / cols threads
+// a column, thread g of them the segments first + g, first + g + 512 / cols, ..., whose sums are then added
+// in that order.  (One thread per column, the earlier form, is a chain of loads as long as the cluster has
+// segments: with K = 2 and 100 000 rows 224 us for the three planes and 19 us a Lloyd round.)
+constexpr int COMB_THREADS = 512;
+
+__device__ __forceinline__ double sum_segments(const double *__restrict__ p, int s0, int s1, int step, size_t stride)
 {
-    const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= KD) return;
-    const int k = (int)(e / D);
-    const int j = (int)(e - (size_t)k * D);
-    double a = 0.0, b = 0.0, c = 0.0;
-    for (int sgm = seg_start[k]; sgm < seg_start[k + 1]; ++sgm) {
-        a += part[((size_t)sgm * 3) * D + j];
-        b += part[((size_t)sgm * 3 + 1) * D + j];
-        c += part[((size_t)sgm * 3 + 2) * D + j];
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    int s = s0;
+    for (; s + 3 * step < s1; s += 4 * step) {
+        double v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = __ldg(p + (size_t)(s + u * step) * stride);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) a[u] += v[u];
     }
-    out0[e] = a;
-    out1[e] = b;
-    out2[e] = c;
+    for (; s < s1; s += step) a[0] += __ldg(p + (size_t)s * stride);
+    return (a[0] + a[1]) + (a[2] + a[3]);
 }
 
-// Delta-mode centroid update, one CTA per cluster: S_k += (partials of key k) - (partials of key
-// K + k); c_k = float(S_k / n_k) where n_k > 0; and for the next assignment the squared norm
-// of c_k (fp64, rounded up), optionally the fp16 copy fp16(c_k * scale[0]), and the reset of the
-// exact-pass queues.
-__global__ void __launch_bounds__(1024) centroid_update_kernel(const double *__restrict__ part,
-                                                              const int32_t *__restrict__ seg_start,
-                                                              const int64_t *__restrict__ counts, int D, int K,
-                                                              double *__restrict__ sums, float *__restrict__ C,
-                                                              float *__restrict__ cnorm, const float *__restrict__ scale,
-                                                              __half *__restrict__ Ch, Control *ctl)
+// every thread of a column gets the sum of its threads' values; red: [COMB_THREADS]
+__device__ __forceinline__ double sum_column(double v, int cols, double *red)
+{
+    if (cols == COMB_THREADS) return v;
+    __syncthreads();
+    red[threadIdx.x] = v;
+    __syncthreads();
+    double t = 0.0;
+    for (int g = threadIdx.x & (cols - 1); g < COMB_THREADS; g += cols) t += red[g];
+    return t;
+}
+
+// columns per CTA: as many CTAs as the device holds a few times over, no more
+int comb_cols(int D, int K)
+{
+    int cols = 32;
+    while (cols < COMB_THREADS && (int64_t)K * ((D + cols - 1) / cols) > 4 * 148) cols *= 2;
+    return cols;
+}
+
+// Three-plane partials (MODE 3) added up per cluster.
+__global__ void __launch_bounds__(COMB_THREADS) segment_combine3_kernel(const double *__restrict__ part,
+                                                                        const int32_t *__restrict__ seg_start, int D, int cols,
+                                                                        double *__restrict__ out0, double *__restrict__ out1,
+                                                                        double *__restrict__ out2)
 {
     pdl_enter();
-    __shared__ double red[32];
-    const int k = blockIdx.x;
-    if (k == 0 && threadIdx.x == 0) {
+    __shared__ double red[COMB_THREADS];
+    const int k = blockIdx.x, g = threadIdx.x / cols, G = COMB_THREADS / cols;
+    const int j = (int)blockIdx.y * cols + (threadIdx.x & (cols - 1));
+    const int s0 = seg_start[k], s1 = seg_start[k + 1];
+    double v[3] = {0.0, 0.0, 0.0};
+    if (j < D)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) v[q] = sum_segments(part + (size_t)q * D + j, s0 + g, s1, G, (size_t)3 * D);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) v[q] = sum_column(v[q], cols, red);
+    if (g == 0 && j < D) {
+        const size_t e = (size_t)k * D + j;
+        out0[e] = v[0];
+        out1[e] = v[1];
+        out2[e] = v[2];
+    }
+}
+
+// Delta-mode centroid update: S_k += (partials of key k) - (partials of key K + k); c_k = float(S_k / n_k) where
+// n_k > 0; and for the next assignment the squared norm of c_k (fp64, rounded up), optionally the fp16 copy
+// fp16(c_k * scale[0]) with the norm of its rounding error -- both of c_k less `mean` if that is given -- and the
+// reset of the exact-pass queues.  The CTAs of a cluster leave their parts of the two norms in `norm_part`; the last
+// one to arrive (`arrivals`, which wraps back to zero) adds them up in column order.
+__global__ void __launch_bounds__(COMB_THREADS) centroid_update_kernel(const double *__restrict__ part,
+                                                              const int32_t *__restrict__ seg_start,
+                                                              const int64_t *__restrict__ counts, int D, int K, int cols,
+                                                              double *__restrict__ sums, float *__restrict__ C,
+                                                              float *__restrict__ cnorm, const float *__restrict__ scale,
+                                                              __half *__restrict__ Ch, const float *__restrict__ mean,
+                                                              float *__restrict__ cerr, double2 *__restrict__ norm_part,
+                                                              unsigned int *__restrict__ arrivals, Control *ctl)
+{
+    pdl_enter();
+    __shared__ double red[COMB_THREADS];
+    __shared__ float red_err[COMB_THREADS / 32];
+    __shared__ int s_last;
+    const int k = blockIdx.x, cb = blockIdx.y, g = threadIdx.x / cols, G = COMB_THREADS / cols;
+    if (k == 0 && cb == 0 && threadIdx.x == 0) {
         ctl->refine_count = 0;
         ctl->cand_count = 0;
     }
-    const int a0 = seg_start[k], a1 = seg_start[k + 1], m0 = seg_start[K + k], m1 = seg_start[K + k + 1];
+    const int j = cb * cols + (threadIdx.x & (cols - 1));
     const int64_t n = counts[k];
     const float sc = Ch ? scale[0] : 1.f;
+    double d = 0.0;
+    if (j < D)
+        d = sum_segments(part + j, seg_start[k] + g, seg_start[k + 1], G, (size_t)2 * D) -
+            sum_segments(part + j, seg_start[K + k] + g, seg_start[K + k + 1], G, (size_t)2 * D);
+    d = sum_column(d, cols, red);
     double nrm = 0.0;
-    for (int j = threadIdx.x; j < D; j += blockDim.x) {
+    float left2 = 0.f;
+    if (g == 0 && j < D) {
         const size_t e = (size_t)k * D + j;
-        double a = 0.0, m = 0.0;
-        for (int sgm = a0; sgm < a1; ++sgm) a += part[((size_t)sgm * 2) * D + j];
-        for (int sgm = m0; sgm < m1; ++sgm) m += part[((size_t)sgm * 2) * D + j];
-        const double sum = sums[e] + (a - m);
+        const double sum = sums[e] + d;
         sums[e] = sum;
         float c = C[e];
         if (n > 0) {
             c = (float)(sum / (double)n);
             C[e] = c;
         }
-        nrm += (double)c * (double)c;
-        if (Ch) Ch[(size_t)k * half_ld(D) + j] = __float2half_rn(c * sc);
+        if (mean) c -= __ldg(mean + j);
+        nrm = (double)c * (double)c;
+        if (Ch) {
+            const __half h = __float2half_rn(c * sc);
+            Ch[(size_t)k * half_ld(D) + j] = h;
+            const float l = c * sc - __half2float(h);
+            left2 = l * l;
+        }
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = nrm;
+    for (int o = 16; o > 0; o >>= 1) {
+        nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
+        left2 += __shfl_xor_sync(0xffffffffu, left2, o);
+    }
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) {
+        red[threadIdx.x >> 5] = nrm;
+        red_err[threadIdx.x >> 5] = left2;
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
+        double t = 0.0, l = 0.0;
+        for (int w = 0; w < cols / 32; ++w) {
+            t += red[w];
+            l += (double)red_err[w];
+        }
+        norm_part[(size_t)k * gridDim.y + cb] = make_double2(t, l);
+        __threadfence();
+        s_last = atomicInc(arrivals + k, gridDim.y - 1) == gridDim.y - 1;
+    }
+    __syncthreads();
+    if (s_last && threadIdx.x == 0) {
+        __threadfence();
+        double t = 0.0, l = 0.0;
+        for (int q = 0; q < (int)gridDim.y; ++q) {
+            const double2 v = __ldcg(norm_part + (size_t)k * gridDim.y + q);
+            t += v.x;
+            l += v.y;
+        }
         cnorm[k] = __double2float_ru(t);
+        if (Ch) cerr[k] = sqrtf((float)l) / sc * 1.001f;
     }
 }
 
@@ -570,24 +654,26 @@ cudaError_t launch_segment_combine(const double *part, const int32_t *seg_start,
 cudaError_t launch_segment_combine3(const double *part, const int32_t *seg_start, int D, int K, double *out0,
                                     double *out1, double *out2, cudaStream_t s)
 {
-    const size_t KD = (size_t)K * D;
-    const int threads = 256;
-    const unsigned blocks = (unsigned)((KD + threads - 1) / threads);
-    segment_combine3_kernel<<<blocks, threads, 0, s>>>(part, seg_start, D, KD, out0, out1, out2);
+    const int cols = comb_cols(D, K);
+    const cudaError_t e = launch_pdl(segment_combine3_kernel, dim3((unsigned)K, (unsigned)((D + cols - 1) / cols)), dim3(COMB_THREADS), 0, s,
+                                     part, seg_start, D, cols, out0, out1, out2);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
+
+size_t centroid_update_scratch_bytes(int D, int K) { return (size_t)K * ((D + 31) / 32) * sizeof(double2); }
 
 cudaError_t launch_centroid_update(const double *part, const int32_t *seg_start, const int64_t *counts, int D,
                                    int K, double *sums, float *C, float *cnorm, const float *scale, void *Ch,
-                                   Control *ctl, cudaStream_t s)
+                                   const float *mean, float *cerr, void *norm_part, uint32_t *arrivals, Control *ctl,
+                                   cudaStream_t s)
 {
-    // one thread per column where the row is short enough: the loads of a column depend on each other
-    const int threads = D >= 1024 ? 1024 : (D >= 512 ? 512 : 256);
-    launch_pdl(centroid_update_kernel, dim3(K), dim3(threads), 0, s, part, seg_start, counts, D, K, sums, C, cnorm, scale,
-               reinterpret_cast<__half *>(Ch), ctl);
+    const int cols = comb_cols(D, K);
+    const cudaError_t e = launch_pdl(centroid_update_kernel, dim3((unsigned)K, (unsigned)((D + cols - 1) / cols)), dim3(COMB_THREADS), 0, s,
+                                     part, seg_start, counts, D, K, cols, sums, C, cnorm, scale, reinterpret_cast<__half *>(Ch), mean, cerr,
+                                     reinterpret_cast<double2 *>(norm_part), arrivals, ctl);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace cat

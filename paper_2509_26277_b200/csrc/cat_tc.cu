@@ -132,7 +132,6 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
     constexpr int BK = HALF ? 64 : 32;   // columns per slab
     const int nslabs = (p.D + BK - 1) / BK;
     const float coef_c = HALF ? p.scale[1] : -2.f;             // score = cn + coef * accumulator
-    const float abs_err_c = HALF ? p.scale[2] : 0.f;
 
     if (tid == 0) {
         for (int s = 0; s < na; ++s) {
@@ -156,15 +155,22 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
     }
     // centroid norms (a huge finite value beyond K) and their maximum
     {
-        float m = 0.f;
+        float m = 0.f, me = 0.f;
         for (int k = tid; k < 256; k += blockDim.x) {
             float v = (k < p.K) ? p.cnorm[k] : TC_KEY_INIT;
             sh.cn[k] = v;
             if (k < p.K) m = fmaxf(m, v);
+            if (HALF && k < p.K) me = fmaxf(me, p.cerr[k]);
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (lane == 0) sh.red[warp] = m;
+        for (int o = 16; o > 0; o >>= 1) {
+            m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+            if (HALF) me = fmaxf(me, __shfl_xor_sync(0xffffffffu, me, o));
+        }
+        if (lane == 0) {
+            sh.red[warp] = m;
+            sh.red_err[warp] = me;
+        }
     }
     if (warp == 1) {
         if (PAIR) {
@@ -179,8 +185,11 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
     __syncthreads();
     if (PAIR) cluster_sync();   // the peer's barriers exist before anything arrives on them
     tc_fence_after();
-    float cmax2 = 0.f;
-    for (int w2 = 0; w2 < (int)(blockDim.x >> 5); ++w2) cmax2 = fmaxf(cmax2, sh.red[w2]);
+    float cmax2 = 0.f, dcmax = 0.f;
+    for (int w2 = 0; w2 < (int)(blockDim.x >> 5); ++w2) {
+        cmax2 = fmaxf(cmax2, sh.red[w2]);
+        dcmax = fmaxf(dcmax, sh.red_err[w2]);
+    }
     const uint32_t tmem_base = sh.tmem_base;
 
     // With the affine epilogue each warpgroup first trades registers: the control and score
@@ -370,7 +379,7 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
             } else {
                 const int64_t row = row0 + r;
                 if (row < p.N) {
-                    const float e = HALF ? tc_error_bound_half(p.D, yn2, cmax2, 2.9802322e-8f * rinv, abs_err_c)
+                    const float e = HALF ? tc_error_bound_measured(p.D, yn2, cmax2, p.scale[4 + p.N + row], dcmax)
                                          : tc_error_bound(p.D, yn2, cmax2);
                     p.labels[row] = key_label(b1, p.K);
                     if (p.fast.best) p.fast.best[row] = b1;
@@ -902,15 +911,40 @@ __global__ void half_scale_kernel(float *scale)
     scale[2] = 2.9802322e-8f / sc;
 }
 
+// entries of `mean` (null: zeros) for column unit c of a row of D
+template <bool VEC4>
+__device__ __forceinline__ void load_mean(const float *__restrict__ mean, int c, int D, float (&mu)[VEC4 ? 4 : 2])
+{
+    constexpr int V = VEC4 ? 4 : 2;
+#pragma unroll
+    for (int q = 0; q < V; ++q) mu[q] = 0.f;
+    if (!mean) return;
+    if (VEC4) {
+        if (4 * c < D) {
+            const float4 t = __ldg(reinterpret_cast<const float4 *>(mean) + c);
+            mu[0] = t.x;
+            mu[1] = t.y;
+            mu[V - 2] = t.z;
+            mu[V - 1] = t.w;
+        }
+    } else {
+        if (2 * c < D) mu[0] = __ldg(mean + 2 * c);
+        if (2 * c + 1 < D) mu[1] = __ldg(mean + 2 * c + 1);
+    }
+}
+
 // One sweep over the rows: squared norm (slightly over-estimated), the row's own power-of-two
 // scale s_i (largest magnitude to [2^13, 2^14)), rinv[i] = 1 / s_i, Yh[i, :] = fp16(Y[i, :] * s_i)
-// rounded to nearest (rows of Yh ld elements apart), and the largest magnitude of the matrix (float
-// bits, one atomicMax per CTA).  A row is handled by G lanes and read twice; the second read comes
+// rounded to nearest (rows of Yh ld elements apart), the norm rerr[i] of what the rounding left, and the
+// largest magnitude of the matrix (float bits, one atomicMax per CTA).  With `mean` everything but that
+// magnitude is of Y[i, :] - mean: nearest centroids do not depend on the origin, and smaller operands make
+// smaller errors.  A row is handled by G lanes and read twice; the second read comes
 // out of L1/L2.  VEC4: 128-bit loads (D % 4 == 0); otherwise a lane takes pairs of columns with
 // scalar loads, whose warp-wide accesses still cover whole lines.
 template <bool VEC4>
 __global__ void __launch_bounds__(256) half_shadow_kernel(const float *__restrict__ Y, int64_t N, int D, int ld, int G,
-                                                          float *__restrict__ ynorm2, float *__restrict__ rinv,
+                                                          const float *__restrict__ mean, float *__restrict__ ynorm2,
+                                                          float *__restrict__ rinv, float *__restrict__ rerr,
                                                           unsigned int *__restrict__ amax_bits, __half *__restrict__ Yh)
 {
     pdl_enter();
@@ -926,7 +960,7 @@ __global__ void __launch_bounds__(256) half_shadow_kernel(const float *__restric
         const int64_t row = base + sub;
         const bool live = row < N;
         const float *y = Y + (size_t)(live ? row : 0) * D;
-        float s = 0.f, m = 0.f;
+        float s = 0.f, m = 0.f, big = 0.f;
         for (int c = c0; c < DV; c += 8 * G) {
             float v[8][V];
 #pragma unroll
@@ -944,12 +978,17 @@ __global__ void __launch_bounds__(256) half_shadow_kernel(const float *__restric
                 }
             }
 #pragma unroll
-            for (int u = 0; u < 8; ++u)
+            for (int u = 0; u < 8; ++u) {
+                float mu[V];
+                load_mean<VEC4>(mean, c + u * G, live ? D : 0, mu);
 #pragma unroll
                 for (int q = 0; q < V; ++q) {
-                    s = fmaf(v[u][q], v[u][q], s);
-                    m = fmaxf(m, fabsf(v[u][q]));
+                    big = fmaxf(big, fabsf(v[u][q]));
+                    const float x = v[u][q] - mu[q];
+                    s = fmaf(x, x, s);
+                    m = fmaxf(m, fabsf(x));
                 }
+            }
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -964,28 +1003,48 @@ __global__ void __launch_bounds__(256) half_shadow_kernel(const float *__restric
         if (sh > 100) sh = 100;
         if (sh < -100) sh = -100;
         const float sc = ldexpf(1.f, sh);
-        if (!live) continue;
-        if (c0 == 0) {
+        if (live && big < CUDART_INF_F) cta_max = fmaxf(cta_max, big);
+        __half *h = Yh + (size_t)row * ld;
+        float left2 = 0.f;
+        if (live) {
+#pragma unroll 4
+            for (int c = c0; c < DV; c += G) {
+                float x[V];
+                if (VEC4) {
+                    const float4 t = __ldg(reinterpret_cast<const float4 *>(y) + c);
+                    x[0] = t.x;
+                    x[1] = t.y;
+                    x[V - 2] = t.z;
+                    x[V - 1] = t.w;
+                } else {
+                    x[0] = __ldg(y + 2 * c);
+                    x[1] = 2 * c + 1 < D ? __ldg(y + 2 * c + 1) : 0.f;
+                }
+                uint32_t w[V / 2];
+                float mu[V];
+                load_mean<VEC4>(mean, c, D, mu);
+#pragma unroll
+                for (int q = 0; q < V; ++q) x[q] = (x[q] - mu[q]) * sc;
+#pragma unroll
+                for (int q = 0; q < V; q += 2) {
+                    const __half2 hh = __floats2half2_rn(x[q], x[q + 1]);
+                    const float2 f = __half22float2(hh);
+                    left2 = fmaf(x[q] - f.x, x[q] - f.x, left2);
+                    left2 = fmaf(x[q + 1] - f.y, x[q + 1] - f.y, left2);
+                    w[q / 2] = *reinterpret_cast<const uint32_t *>(&hh);
+                }
+                // (ld is even and at least D: a pair that starts inside the row fits)
+                if (VEC4) reinterpret_cast<uint2 *>(h)[c] = make_uint2(w[0], w[V / 2 - 1]);
+                else reinterpret_cast<uint32_t *>(h)[c] = w[0];
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            if (o < G) left2 += __shfl_xor_sync(0xffffffffu, left2, o);
+        if (live && c0 == 0) {
             ynorm2[row] = s * 1.0001f;
             rinv[row] = ldexpf(1.f, -sh);
-        }
-        if (m == m && m < CUDART_INF_F) cta_max = fmaxf(cta_max, m);
-        __half *h = Yh + (size_t)row * ld;
-        if (VEC4) {
-            for (int c = c0; c < DV; c += G) {
-                const float4 v = __ldg(reinterpret_cast<const float4 *>(y) + c);
-                const __half2 lo = __floats2half2_rn(v.x * sc, v.y * sc);
-                const __half2 hi = __floats2half2_rn(v.z * sc, v.w * sc);
-                uint2 o2;
-                o2.x = *reinterpret_cast<const unsigned int *>(&lo);
-                o2.y = *reinterpret_cast<const unsigned int *>(&hi);
-                reinterpret_cast<uint2 *>(h)[c] = o2;
-            }
-        } else {
-#pragma unroll 4
-            for (int c = c0; c < DV; c += G)   // (ld is even and at least D: the pair fits)
-                reinterpret_cast<__half2 *>(h)[c] =
-                    __floats2half2_rn(__ldg(y + 2 * c) * sc, 2 * c + 1 < D ? __ldg(y + 2 * c + 1) * sc : 0.f);
+            rerr[row] = sqrtf(left2) * ldexpf(1.f, -sh) * 1.001f;
         }
     }
 #pragma unroll
@@ -999,12 +1058,14 @@ __global__ void __launch_bounds__(256) half_shadow_kernel(const float *__restric
     }
 }
 
-// dst[k, :] = fp16(src[k, :] * scale[0]), round to nearest; one CTA per row, rows of dst ld apart.
+// dst[k, :] = fp16((src[k, :] - mean) * scale[0]), round to nearest; one CTA per row, rows of dst ld apart;
+// cerr[k] = norm of what the rounding left.
 // With cmax (the rows' largest magnitudes) the scale words are made here first (as half_scale_kernel
 // does) and CTA 0 leaves them in `scale`.
 __global__ void __launch_bounds__(256) to_half_kernel(const float *__restrict__ src, int K, int D, int ld,
-                                                      const float *__restrict__ cmax, float *__restrict__ scale,
-                                                      __half *__restrict__ dst)
+                                                      const float *__restrict__ mean, const float *__restrict__ cmax,
+                                                      float *__restrict__ scale, __half *__restrict__ dst,
+                                                      float *__restrict__ cerr)
 {
     pdl_enter();
     __shared__ float wmax[8];
@@ -1028,13 +1089,30 @@ __global__ void __launch_bounds__(256) to_half_kernel(const float *__restrict__ 
         sc = scale[0];
     const float *c = src + (size_t)blockIdx.x * D;
     __half *h = dst + (size_t)blockIdx.x * ld;
+    float left2 = 0.f;
 #pragma unroll 4
-    for (int j = threadIdx.x; j < D; j += 256) h[j] = __float2half_rn(__ldg(c + j) * sc);
+    for (int j = threadIdx.x; j < D; j += 256) {
+        const float x = (mean ? __ldg(c + j) - __ldg(mean + j) : __ldg(c + j)) * sc;
+        const __half v = __float2half_rn(x);
+        h[j] = v;
+        const float d = x - __half2float(v);
+        left2 = fmaf(d, d, left2);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) left2 += __shfl_xor_sync(0xffffffffu, left2, o);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = left2;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) left2 += wmax[w];
+        cerr[blockIdx.x] = sqrtf(left2) / sc * 1.001f;
+    }
 }
 
-// Squared norms (fp64 sum, rounded up) and largest finite magnitudes of the centroids, one CTA each;
+// Squared norms (fp64 sum, rounded up) and largest finite magnitudes of the centroids less `mean`, one CTA each;
 // the exact-pass queues are emptied, with reset_all the status word and counters too.
-__global__ void __launch_bounds__(256) centroid_prep_kernel(const float *__restrict__ C, int D, float *__restrict__ cnorm,
+__global__ void __launch_bounds__(256) centroid_prep_kernel(const float *__restrict__ C, int D,
+                                                            const float *__restrict__ mean, float *__restrict__ cnorm,
                                                             float *__restrict__ cmax, Control *ctl, int reset_all)
 {
     pdl_enter();
@@ -1054,7 +1132,7 @@ __global__ void __launch_bounds__(256) centroid_prep_kernel(const float *__restr
     float m = 0.f;
 #pragma unroll 4
     for (int j = threadIdx.x; j < D; j += 256) {
-        const float v = __ldg(c + j);
+        const float v = mean ? __ldg(c + j) - __ldg(mean + j) : __ldg(c + j);
         s = fma((double)v, (double)v, s);
         if (fabsf(v) < CUDART_INF_F) m = fmaxf(m, fabsf(v));
     }
@@ -1075,6 +1153,24 @@ __global__ void __launch_bounds__(256) centroid_prep_kernel(const float *__restr
         }
         cnorm[blockIdx.x] = __double2float_ru(s);
         cmax[blockIdx.x] = m;
+    }
+}
+
+// Column means of the first `rows` rows: 32 columns per CTA, eight groups of rows.
+__global__ void __launch_bounds__(256) sample_mean_kernel(const float *__restrict__ Y, int rows, int D, float *__restrict__ mean)
+{
+    pdl_enter();
+    __shared__ float part[8][32];
+    const int c = threadIdx.x & 31, g = threadIdx.x >> 5, j = blockIdx.x * 32 + c;
+    float s = 0.f;
+    if (j < D)
+#pragma unroll 16
+        for (int r = g; r < rows; r += 8) s += __ldg(Y + (size_t)r * D + j);
+    part[g][c] = s;
+    __syncthreads();
+    if (g == 0 && j < D) {
+        for (int q = 1; q < 8; ++q) s += part[q][c];
+        mean[j] = s / (float)rows;
     }
 }
 
@@ -1187,10 +1283,10 @@ cudaError_t launch_row_norms(const float *Y, int64_t N, int D, float *out, cudaS
     return cudaGetLastError();
 }
 
-cudaError_t launch_half_shadow(const float *Y, int64_t N, int D, float *ynorm2, float *scale, void *Yh,
+cudaError_t launch_half_shadow(const float *Y, int64_t N, int D, const float *mean, float *ynorm2, float *scale, void *Yh,
                                cudaStream_t s, bool finish_scale)
 {
-    float *rinv = scale + 4;
+    float *rinv = scale + 4, *rerr = scale + 4 + N;
     cudaError_t e = cudaMemsetAsync(scale, 0, 4 * sizeof(float), s);
     if (e != cudaSuccess) return e;
     const int G = lanes_per_row(D);
@@ -1198,33 +1294,27 @@ cudaError_t launch_half_shadow(const float *Y, int64_t N, int D, float *ynorm2, 
     int64_t blocks = (N + rows_per_cta - 1) / rows_per_cta;
     const int64_t cap = (int64_t)sm_count() * 8;
     if (blocks > cap) blocks = cap;
-    unsigned int *amax = reinterpret_cast<unsigned int *>(scale);
-    if (D % 4 == 0)
-        e = launch_pdl(half_shadow_kernel<true>, dim3((unsigned)blocks), dim3(256), 0, s, Y, N, D, half_ld(D), G, ynorm2, rinv,
-                       amax, reinterpret_cast<__half *>(Yh));
-    else
-        e = launch_pdl(half_shadow_kernel<false>, dim3((unsigned)blocks), dim3(256), 0, s, Y, N, D, half_ld(D), G, ynorm2, rinv,
-                       amax, reinterpret_cast<__half *>(Yh));
+    e = launch_pdl(D % 4 == 0 ? half_shadow_kernel<true> : half_shadow_kernel<false>, dim3((unsigned)blocks), dim3(256), 0, s, Y, N, D,
+                   half_ld(D), G, mean, ynorm2, rinv, rerr, reinterpret_cast<unsigned int *>(scale), reinterpret_cast<__half *>(Yh));
     if (e != cudaSuccess) return e;
     count_launch();
     return finish_scale ? launch_half_scale(scale, s) : cudaGetLastError();
 }
 
-cudaError_t launch_to_half(const float *C, int D, int K, const float *scale, void *Ch, cudaStream_t s)
+cudaError_t launch_sample_mean(const float *Y, int64_t N, int D, float *mean, cudaStream_t s)
 {
-    const cudaError_t e = launch_pdl(to_half_kernel, dim3((unsigned)K), dim3(256), 0, s, C, K, D, half_ld(D), nullptr,
-                                     const_cast<float *>(scale), reinterpret_cast<__half *>(Ch));
+    const cudaError_t e = launch_pdl(sample_mean_kernel, dim3((unsigned)((D + 31) / 32)), dim3(256), 0, s, Y, (int)(N < 128 ? N : 128), D, mean);
     count_launch();
     return e;
 }
 
-cudaError_t launch_centroid_half(const float *C, int D, int K, float *cnorm, float *cmax, float *scale, void *Ch, Control *ctl,
-                                 cudaStream_t s, bool reset_all)
+cudaError_t launch_centroid_half(const float *C, int D, int K, const float *mean, float *cnorm, float *cmax, float *cerr, float *scale,
+                                 void *Ch, Control *ctl, cudaStream_t s, bool reset_all, bool own_scale)
 {
-    cudaError_t e = launch_pdl(centroid_prep_kernel, dim3((unsigned)K), dim3(256), 0, s, C, D, cnorm, cmax, ctl, reset_all ? 1 : 0);
+    cudaError_t e = launch_pdl(centroid_prep_kernel, dim3((unsigned)K), dim3(256), 0, s, C, D, mean, cnorm, cmax, ctl, reset_all ? 1 : 0);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(to_half_kernel, dim3((unsigned)K), dim3(256), 0, s, C, K, D, half_ld(D), cmax, scale,
-                   reinterpret_cast<__half *>(Ch));
+    e = launch_pdl(to_half_kernel, dim3((unsigned)K), dim3(256), 0, s, C, K, D, half_ld(D), mean, own_scale ? cmax : nullptr, scale,
+                   reinterpret_cast<__half *>(Ch), cerr);
     count_launch(2);
     return e;
 }
@@ -1361,7 +1451,7 @@ cudaError_t launch_assign_tc(const float *Y, int64_t N, int D, int K, const floa
                              const float *ynorm2, int32_t *labels, int32_t *refine_rows,
                              int32_t *cand_rows, uint64_t *cand_list, Control *ctl,
                              const float *gamma, const float *beta, float *out, cudaStream_t s,
-                             const void *Yh, const void *Ch, const float *scale, const FastOut *fast)
+                             const void *Yh, const void *Ch, const float *scale, const float *cerr, const FastOut *fast)
 {
     TcParams p{};
     if (fast) p.fast = *fast;
@@ -1387,6 +1477,7 @@ cudaError_t launch_assign_tc(const float *Y, int64_t N, int D, int K, const floa
     const bool affine = out != nullptr;
     const bool half = (Yh != nullptr) && !affine;
     p.scale = scale;
+    p.cerr = cerr;
     if (affine) {
         const int cs = choose_column_split(N, D, K);
         if (cs == 2 || cs == 4) return launch_apply_split(cs, p, C, s);

@@ -314,7 +314,8 @@ struct TcParams {
     const float *cnorm;
     const float *ynorm2;   // [N] squared row norms (labels-only mode)
     const float *scale;    // fp16 operands: {centroid scale s_c, -2 / s_c, 2^-25 / s_c, -} followed by
-                           // [N] 1 / (row scale), in device memory
+                           // [N] 1 / (row scale) and [N] norms of the rows' rounding errors, in device memory
+    const float *cerr;     // fp16 operands: [K] norms of the centroids' rounding errors
     int32_t *labels;
     int32_t *refine_rows;
     int32_t *cand_rows;    // rows whose exact decision only needs the listed candidates
@@ -347,6 +348,7 @@ struct TcShared {
     int abort_flag;
     int rows_streamed;            // row slots the streaming warps have finished, all tiles
     float red[32];
+    float red_err[32];
     float cn[256];
     float4 top_key[2][TC_BM];     // four smallest keys of each row, ascending
 };
@@ -396,6 +398,18 @@ __device__ __forceinline__ float tc_error_bound_half(int D, float ysq, float cma
     const float yn = sqrtf(ysq), cn = sqrtf(cmax2);
     return 1.0625f * ((r + 2.f * pk) * yn * cn + 2.f * sqrtf((float)D) * (ac * yn + ay * cn) +
                       2.f * (float)D * ay * ac + (4.f * u + pk) * cmax2);
+}
+
+// The same where the rounding errors of the fp16 operands were measured while the copies were made (norms dy
+// of the row's, dc the largest of the centroids'): |y.c - fp16(y).fp16(c)| <= dy c + (y + dy) dc.  y and c may be
+// taken relative to a common point (rounded to fp32 once: the 2 in 2 D + 4).
+__device__ __forceinline__ float tc_error_bound_measured(int D, float ysq, float cmax2, float dy, float dc)
+{
+    const float u = 5.9604645e-8f;   // 2^-24
+    const float a = (2.f * (float)D + 4.f) * 2.3841858e-7f;   // (2D+4) 2^-22
+    const float pk = 3.0517578e-5f;
+    const float yn = sqrtf(ysq), cn = sqrtf(cmax2);
+    return 1.0625f * ((a + 2.f * pk) * yn * cn + 2.f * (dy * cn + (yn + dy) * dc) + (8.f * u + pk) * cmax2);
 }
 
 // Decision for one row from its four smallest keys.  Returns true when the fast argmin is
