@@ -205,7 +205,7 @@ struct TridiagParams {
 // that update to its own rows and in the same sweep multiplies them with the new reflection; each CTA
 // publishes its products and collects everybody's, word by word, without a barrier.
 //   bound: latency.  A step moves 2 D values between CTAs and does 6 (D - j)^2 / G operations per CTA;
-//   the exchange, three block-wide sums and a square root and two divisions in fp64 make it 3.1 us (D = 1000).
+//   the exchange, three block-wide sums and a square root and two divisions in fp64 make it 3.1 us (D = 1000; 3.7 with 512 threads).
 //   With a grid barrier (a flag per CTA, polled by all) in place of the self-validating words the exchange alone
 //   took 6 of 9 us.
 template <int C, bool REGS>
@@ -403,7 +403,7 @@ __device__ __forceinline__ int count_below(const double *d, const double *e2, in
 //                  different starts, so their vectors span the eigenspace.
 //   back           the reflections in reverse order, then sign, fp32 store
 // Three rounds of solve and orthogonalise, the last one orthogonalised twice.
-//   bound: latency of the serial chains (D = 1000, p = 50: 1.9 ms in all).
+//   bound: latency of the serial chains (D = 1000, p = 50: 1.7 ms in all).
 template <int C>
 __global__ void __launch_bounds__(ET) eigvec_kernel(EigvecParams P)
 {
@@ -464,10 +464,14 @@ __global__ void __launch_bounds__(ET) eigvec_kernel(EigvecParams P)
         for (int q = 0; q < NV; ++q) {
             const int m = me + q * G;
             __syncthreads();
-            for (int k = tid; k < D; k += ET) sd[k] = P.d[k];
-            for (int k = tid; k + 1 < D; k += ET) l[k] = P.e[k];
+            // (a CTA with one vector keeps its factors over the rounds)
+            const bool factor = round == 0 || NV > 1;
+            if (factor) {
+                for (int k = tid; k < D; k += ET) sd[k] = P.d[k];
+                for (int k = tid; k + 1 < D; k += ET) l[k] = P.e[k];
+            }
             __syncthreads();
-            if (tid == 0) {
+            if (factor && tid == 0) {
                 // P L U = T - lambda: u0 (inverted), u1, u2 the rows of U; l overwrites the off-diagonal
                 const double lm = lam[q];
                 double a = sd[0] - lm, b = D > 1 ? l[0] : 0.0;

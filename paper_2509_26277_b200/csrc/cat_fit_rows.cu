@@ -485,7 +485,7 @@ bool fit_rows_supported(int64_t N, int D, int K)
     FitRowsParams p{};
     int grid;
     size_t smem;
-    return fit_rows_plan(N, D, K, &p, &grid, &smem);
+    return fit_rows_plan(N, D, K, &p, &grid, &smem) && grid <= tc_sm_count();   // (all CTAs resident)
 }
 
 cudaError_t launch_fit_rows(const float *Y, int64_t N, int D, int K, float *C, int passes, int32_t *labels, double *sums,

@@ -150,7 +150,8 @@ __global__ void cov_finish_kernel(const double *__restrict__ part, int splits, i
 
 // ---------------------------------------------------------------- projection
 // Z[i, r] = sum_j (Y[i, j] - mean[j]) * comps[r, j], fp64 accumulation: one CTA per 64 rows x 64 components.
-//   bound: fp64 multiply-adds (50 000 x 1000, p = 50: 2.8 GFMA with p rounded up to 56, 0.15 ms at 64 per clock and SM).
+//   bound: the fp64 tensor pipe, 73 % busy (50 000 x 1000, p = 50: 2.8 GFMA with p rounded up to 56, 0.15 ms at 64
+//   per clock and SM; takes 0.27; tiles of 32 rows, for a fuller last wave, 0.30).
 __global__ void __launch_bounds__(P_THREADS) project_kernel(const float *__restrict__ Y, int64_t N, int D, int p,
                                                             const float *__restrict__ mean, const float *__restrict__ comps,
                                                             float *__restrict__ Z)
