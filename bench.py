@@ -363,9 +363,17 @@ def run_cuda(args):
     if ((B.cat_get_small_problem_kernels() & 1) and D in (32, 64, 128) and B.cat_get_tensor_core_min_k() <= K <= 128
             and N_apply >= 128):
         apply_kernel = "small_kernel<inference> (one persistent launch: TF32 scores, in-kernel exact pass, affine from the staged tile)"
+    elif ((B.cat_get_small_problem_kernels() & 1) and form == 0 and 2 <= K <= 128
+            and (K * D <= 32768 or D % 8 or N_apply < 4096 or D > 1024)):
+        apply_kernel = "apply_rows_kernel (groups of eight rows in shared memory, exact decision inside)"
     small_fit = ((B.cat_get_small_problem_kernels() & 2) and D in (32, 64, 128) and K * D <= 4096
                  and B.cat_get_tensor_core_min_k() <= K <= 128 and N_fit >= 128)
-    if small_fit:
+    if (B.cat_get_small_problem_kernels() & 2) and N_fit <= 8192 and N_fit * K * max(D, 256) <= (1 << 27 if N_fit > 6144 else 1 << 28):
+        # (the rounds end at a fixed point, so a round of the difference may be shorter than a full one)
+        roofline_fit = {"bound": "latency", "kernel": "one Lloyd round inside fit_rows_kernel (one cooperative launch for the whole "
+                        "fit, rows in shared memory)", "achieved": lloyd_alg_gbs, "peak": peak, "unit": "GB/s",
+                        "frac": lloyd_alg_gbs / peak, "peak_source": peak_src, "tflops": lloyd_tflops}
+    elif small_fit:
         # all rounds in one persistent launch: a round reads the fp32 rows once (TF32 scores from the staged tile)
         roofline_fit = {"bound": "hbm", "kernel": "one Lloyd round inside small_kernel<fit> (one cooperative launch for the "
                         "whole fit: TF32 scores, in-kernel exact pass, fp64 sums in shared memory, ordered grid-wide combine)",
@@ -396,7 +404,7 @@ def run_cuda(args):
             "fit_s_per_lloyd_iter": lloyd_ms * 1e-3,
             "fit_ms": fit_ms_step, "fit_one_round_ms": fit1_ms, "apply_ms": apply_ms_step,
             "wall_s": t_wall,
-            "roofline": {"bound": "hbm", "kernel": apply_kernel + ("" if apply_kernel.startswith("small_kernel") else " (the one kernel of cat_apply besides the exact pass)"),
+            "roofline": {"bound": "hbm", "kernel": apply_kernel + ("" if apply_kernel.startswith(("small_kernel", "apply_rows")) else " (the one kernel of cat_apply besides the exact pass)"),
                          "achieved": apply_gbs, "peak": peak, "unit": "GB/s", "frac": apply_gbs / peak,
                          "peak_source": peak_src, "traffic": traffic},
             "roofline_fit": roofline_fit,
