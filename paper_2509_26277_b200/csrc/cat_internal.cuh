@@ -79,7 +79,7 @@ struct Control {
 // at launch time.
 struct SegGeom {
     int nblk;       // 1024-entry blocks of the sort
-    int seg_rows;   // largest rows per segment (multiple of 128); a sort may choose shorter segments
+    int seg_rows;   // largest rows per segment (multiple of 16); a sort may choose shorter segments
     int max_segs;   // upper bound on the number of segments: ceil(NE / seg_rows) + KK
 };
 SegGeom seg_geometry(int64_t NE, int D, int KK);
