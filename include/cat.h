@@ -142,9 +142,10 @@ cat_status_t cat_apply_blend(const float *Yq, int64_t N, int32_t D, int32_t K,
  * cat_apply with a bf16 result: Y_out_bf16 [N, D] receives bf16(gamma_l * Yq_i + beta_l), the fp32
  * fused multiply-add of cat_apply rounded to nearest even (Algorithm 2 with alpha = 1; Section 3.1
  * notes that the correction suits low-precision deployment, without fixing a format).  The labels
- * are exact as in cat_apply.  Halves the bytes written.  For shapes the 64-row-tile kernel takes
- * (K >= the tensor-core threshold, K <= 256, D >= 128, D % 8 == 0, N > 64) assignment and correction
- * are fused; other shapes run the assignment, then one pass that reads the rows again.
+ * are exact as in cat_apply.  Halves the bytes written.  Where a fused kernel takes the shape
+ * (rows kept in shared memory, see cat_set_small_problem_kernels; 64-row tiles for K >= the tensor-core threshold,
+ * K <= 256, D >= 128, D % 8 == 0, N > 64) assignment and correction are one pass over the rows; other shapes
+ * run the assignment, then one pass that reads the rows again.
  * Workspace: cat_apply_workspace_bytes(N, D, K).
  */
 cat_status_t cat_apply_bf16(const float *Yq, int64_t N, int32_t D, int32_t K,
