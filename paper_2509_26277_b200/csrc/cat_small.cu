@@ -429,10 +429,12 @@ small_kernel(const __grid_constant__ CUtensorMap mapA, SmallParams p)
                 float lim = 0.f;
                 if (row < p.N) {
                     lab = key_label(b1, p.K);
-                    lim = 2.f * tc_error_bound(p.D, yn2 * 1.0001f, cmax2);
+                    const float e = tc_error_bound(p.D, yn2 * 1.0001f, cmax2);
+                    const bool trusted = tc_trusted(e);
+                    lim = trusted ? 2.f * e : CUDART_INF_F;   // (no trust: every centroid is a candidate)
                     if (p.K > 1 && !((b2 - b1) > lim)) {
                         undecided = true;
-                        wide = !((b4 - b1) > lim) && p.K > 4;
+                        wide = !trusted || (!((b4 - b1) > lim) && p.K > 4);
                         if (!wide) {
                             const float bk[4] = {b1, b2, b3, b4};
 #pragma unroll

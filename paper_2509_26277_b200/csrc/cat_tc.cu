@@ -379,8 +379,9 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
             } else {
                 const int64_t row = row0 + r;
                 if (row < p.N) {
-                    const float e = HALF ? tc_error_bound_measured(p.D, yn2, cmax2, p.scale[4 + p.N + row], dcmax)
-                                         : tc_error_bound(p.D, yn2, cmax2);
+                    float e = HALF ? tc_error_bound_measured(p.D, yn2, cmax2, p.scale[4 + p.N + row], dcmax)
+                                   : tc_error_bound(p.D, yn2, cmax2);
+                    if (HALF && !(fabsf(coef) < CUDART_INF_F)) e = CUDART_INF_F;   // (the scales' product overflowed)
                     p.labels[row] = key_label(b1, p.K);
                     if (p.fast.best) p.fast.best[row] = b1;
                     if (p.fast.second) p.fast.second[row] = b2;

@@ -412,15 +412,22 @@ __device__ __forceinline__ float tc_error_bound_measured(int D, float ysq, float
     return 1.0625f * ((a + 2.f * pk) * yn * cn + 2.f * (dy * cn + (yn + dy) * dc) + (8.f * u + pk) * cmax2);
 }
 
+// True where a bound e on the error of a row's scores also says that its keys mean what they should.  e is at
+// least 2^-14 |y| |c| and 2^-15 |c|^2: below the upper limit every score is below 7e37 in magnitude, so none
+// overflowed (the pattern of an infinity with an index in its low bits is a NaN, which key_insert drops) and
+// none reached TC_KEY_INIT.  Above the lower limit products that vanished below 2^-126 are less than e.
+__device__ __forceinline__ bool tc_trusted(float e) { return e > 1e-33f && e < 1e33f; }
+
 // Decision for one row from its four smallest keys.  Returns true when the fast argmin is
 // certainly exact.  Otherwise the row is queued: with the centroids whose key lies within
 // 2e of the best when those are known to be among the four, else for a scan of all K.
 __device__ __forceinline__ bool tc_decide(const TcParams &p, int64_t row, float4 sc, float e)
 {
     const float lim = 2.f * e;
-    if (p.K == 1 || (sc.y - sc.x) > lim) return true;
-    const bool more = !((sc.w - sc.x) > lim);   // the 4th is a candidate too (or NaN): others may be
-    if (more && p.K > 4) {
+    const bool trusted = tc_trusted(e);
+    if (p.K == 1 || (trusted && (sc.y - sc.x) > lim)) return true;
+    const bool more = p.K > 4 && !((sc.w - sc.x) > lim);   // the 4th is a candidate too (or NaN): others may be
+    if (more || !trusted) {
         int slot = atomicAdd(&p.ctl->refine_count, 1);
         p.refine_rows[slot] = (int32_t)row;
     } else {

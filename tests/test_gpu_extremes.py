@@ -1,0 +1,70 @@
+"""Finite rows whose squared norms leave the range of fp32: fast scores are infinities, NaN or zeros there, and
+every label has to come from the exact pass.  Against the CPU oracle (fp64)."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import cat_oracle as O
+from paper_2509_26277_b200 import binding as B
+from tests.parity import close, labels_match
+
+pytestmark = pytest.mark.gpu
+
+
+def dev(a):
+    return torch.as_tensor(np.ascontiguousarray(a)).cuda()
+
+
+def host(t):
+    return t.detach().cpu().numpy()
+
+
+@pytest.fixture(params=[3, 0], ids=["small kernels", "general path"])
+def small_kernels(request):
+    old = B.cat_get_small_problem_kernels()
+    B.cat_set_small_problem_kernels(request.param)
+    yield request.param
+    B.cat_set_small_problem_kernels(old)
+
+
+def _clusters(n, d, k, mag):
+    """Rows around k points (the first k rows one of each), and the points' magnitudes."""
+    rng = np.random.default_rng(n + 7 * d + k)
+    size = {"huge": np.full(k, 1e19), "one huge": np.where(np.arange(k) == k // 2, 1e19, 1.0),
+            "overflow in the products": np.full(k, 1.2e19 / np.sqrt(d)), "tiny": np.full(k, 1e-24)}[mag]
+    cen = rng.normal(size=(k, d)) * size[:, None]
+    pick = np.concatenate([np.arange(k), rng.integers(0, k, size=n - k)])
+    Yq = cen[pick] + 0.4 * size[pick][:, None] * rng.normal(size=(n, d))
+    return Yq.astype(np.float32), cen.astype(np.float32), size
+
+
+MAGS = ["huge", "one huge", "overflow in the products", "tiny"]
+
+
+@pytest.mark.parametrize("n,d", [(9001, 256), (700, 516), (8500, 513), (300, 64)])
+@pytest.mark.parametrize("k", [2, 3, 4, 5, 9])
+@pytest.mark.parametrize("mag", MAGS)
+def test_fit(n, d, k, mag, small_kernels):
+    Yq, _, size = _clusters(n, d, k, mag)
+    Yfp = (0.9 * Yq).astype(np.float32)
+    ora = O.fit(Yq, Yfp, k, 3)
+    assert int(ora.near.sum()) == 0
+    for diag in (False, True):
+        C, G, Bt, lab = B.cat_fit(dev(Yq), dev(Yfp), k, 3, want_diag=diag)[:4]
+        assert np.array_equal(host(lab), ora.labels), f"{int((host(lab) != ora.labels).sum())} labels differ"
+        scale = np.abs(ora.centroids).max(axis=1, keepdims=True)
+        close(host(C) / scale, ora.centroids / scale, "centroids")
+
+
+@pytest.mark.parametrize("n,d", [(513, 256), (513, 264), (500, 1001), (300, 64), (300, 10)])
+@pytest.mark.parametrize("k", [2, 3, 4, 5, 9])
+@pytest.mark.parametrize("mag", MAGS)
+def test_inference(n, d, k, mag, small_kernels):
+    Yq, C, size = _clusters(n, d, k, mag)
+    g = np.linspace(0.5, 1.5, k * d, dtype=np.float32).reshape(k, d)
+    b = (g * size[:, None]).astype(np.float32)
+    want, lab, best, second = O.apply(Yq, C, g, b)
+    assert np.array_equal(host(B.cat_assign(dev(Yq), dev(C))), lab)
+    out, glab = B.cat_apply(dev(Yq), dev(C), dev(g), dev(b), want_labels=True)
+    assert np.array_equal(host(glab), lab)
+    np.testing.assert_array_equal(host(out), O.affine_with_labels(Yq, lab, g, b))
