@@ -212,7 +212,11 @@ template <int C, bool REGS>
 __global__ void __launch_bounds__(ET) tridiag_kernel(TridiagParams P)
 {
     extern __shared__ double sm[];
-    __shared__ double red[2][EW], red_rows[EW][MAX_ROWS], s_x1;
+    __shared__ double red[2][EW], red_rows[EW][MAX_ROWS];
+    // Each is written before a step's barrier and read behind it, and written again only behind another barrier of
+    // the step: s_x1 around the sum of squares, s_w1 around v'Av.  (One word for both would be written by a warp that
+    // is a step ahead while another has yet to read it.)
+    __shared__ double s_x1, s_w1;
     constexpr int RR = REGS ? 8 : 1;
     const int D = P.D, G = gridDim.x, me = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int R = REGS ? (D - me * 8 < 8 ? D - me * 8 : 8) : (D - me + G - 1) / G;
@@ -351,12 +355,12 @@ __global__ void __launch_bounds__(ET) tridiag_kernel(TridiagParams P)
         for (int c = 0; c < C; ++c) {
             wo[c] *= tau;
             pv = fma(wo[c], vn[c], pv);
-            if (tid + c * ET == j + 1) s_x1 = wo[c];
+            if (tid + c * ET == j + 1) s_w1 = wo[c];
         }
         const double half = 0.5 * tau * block_sum(pv, red[1], ok);
         if (!ok) break;
         v1 = ss > 0.0 ? 1.0 : 0.0;
-        w1 = s_x1 - half * v1;
+        w1 = s_w1 - half * v1;
 #pragma unroll
         for (int c = 0; c < C; ++c) {
             const int k = tid + c * ET;

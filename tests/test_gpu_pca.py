@@ -136,3 +136,18 @@ def test_leading_eigenpairs_of_special_spectra(n, d, p, kind):
             assert P.projector_distance(C[:r], o_comps[:r]) < 1e-5
     again = B.cat_pca_fit(dev(Y), p)
     assert torch.equal(again[1], comps)
+
+
+@pytest.mark.parametrize("n,d,p", [(1200, 1000, 50), (300, 250, 20), (600, 515, 30), (200, 1300, 8)])
+def test_eigenpairs_do_not_vary_from_run_to_run(n, d, p):
+    """Twenty runs give the same bits: the reduction's CTAs exchange values without barriers, and a value read too
+    late or overwritten too early would show in some of them."""
+    rng = np.random.default_rng(n + d)
+    Y = dev((rng.normal(size=(n, d)) * np.linspace(3.0, 1.0, d) + 1.0).astype(np.float32))
+    first = B.cat_pca_fit(Y, p, want_eigenvalues=True)
+    _, o_comps, o_eig = P.pca_fit(host(Y), p)
+    np.testing.assert_allclose(host(first[2]), o_eig, rtol=1e-9)
+    for _ in range(20):
+        again = B.cat_pca_fit(Y, p, want_eigenvalues=True)
+        for x, y in zip(first, again):
+            assert torch.equal(x, y)
