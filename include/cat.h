@@ -46,7 +46,7 @@ enum {
     CAT_ERR_ALIGN = 3,       /* a base pointer is not 16-byte aligned */
     CAT_ERR_WORKSPACE = 4,   /* workspace NULL or smaller than the query says */
     CAT_ERR_CUDA = 5,        /* a CUDA runtime call failed: see cat_last_cuda_error() */
-    CAT_ERR_DEVICE_TIMEOUT = 6, /* a bounded device-side wait gave up (reported by cat_device_status) */
+    CAT_ERR_DEVICE_TIMEOUT = 6, /* a bounded device-side wait gave up (reported by cat_workspace_report) */
     CAT_ERR_UNSUPPORTED = 7  /* K > CAT_MAX_K, D > CAT_MAX_D or N >= 2^31 */
 };
 
@@ -375,12 +375,14 @@ cat_status_t cat_fit_host(const float *Yq_host, const float *Yfp_host, int64_t N
  * `stream`, then copies to the HOST pointers (each may be NULL) the number of rows
  * whose label needed the exact fp64 pass in the latest assignment, the running
  * total since the last cat_fit started on that workspace, and the device status
- * word (CAT_OK or CAT_ERR_DEVICE_TIMEOUT). */
+ * word (CAT_OK or CAT_ERR_DEVICE_TIMEOUT: outputs of that call are undefined).  For the calls that
+ * compose several steps -- cat_pca_fit, cat_fit_pca, cat_apply_pca -- the block speaks for all of them.  (The
+ * host-buffer calls keep theirs behind their staging buffers, out of this call's reach.) */
 cat_status_t cat_workspace_report(const void *workspace, void *stream, int64_t *refined_last_host,
                                   int64_t *refined_total_host, int32_t *device_status_host);
 
-/* Self-test of the failure path of the device-side waits.  The tensor-core kernels wait on
- * barriers with a time limit; a wait that runs out records CAT_ERR_DEVICE_TIMEOUT in the
+/* Self-test of the failure path of the device-side waits.  The tensor-core kernels, the kernels that keep rows in
+ * shared memory and the eigensolver wait on barriers and flags with a time limit; a wait that runs out records CAT_ERR_DEVICE_TIMEOUT in the
  * workspace's control block and the kernel returns instead of hanging.  This call enqueues one
  * warp that waits limit_ms (clamped to 1 .. 1000) on a barrier nothing completes; afterwards
  * cat_workspace_report on the same workspace gives device_status = CAT_ERR_DEVICE_TIMEOUT.

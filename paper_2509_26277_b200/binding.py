@@ -378,20 +378,26 @@ def cat_fit_shard_update(delta_sums, delta_counts, sums, counts, centroids):
                                       _dev(centroids, torch.float32, (K, D)), _stream()), "cat_fit_shard_update")
 
 
-def _scratch(nbytes: int, device, where: str):
+def pca_workspace(kind: str, N: int, D: int, p: int, device, K: int = 0) -> torch.Tensor:
+    """Device scratch for one call of cat_pca_fit ("pca"), cat_fit_pca ("fit_pca") or cat_apply_pca
+    ("apply_pca"); pass it as `ws` to read its status with cat_workspace_report afterwards."""
+    if kind == "pca":
+        nbytes = lib().cat_pca_workspace_bytes(N, D, p)
+    else:
+        nbytes = {"fit_pca": lib().cat_fit_pca_workspace_bytes, "apply_pca": lib().cat_apply_pca_workspace_bytes}[kind](N, D, K, p)
     if nbytes == 0:
-        raise CatError(7, where + " workspace query")
+        raise CatError(7, {"pca": "cat_pca_fit"}.get(kind, "cat_" + kind) + " workspace query")
     return torch.empty(int(nbytes), dtype=torch.uint8, device=device)
 
 
-def cat_pca_fit(Yq, p: int, want_eigenvalues=False):
+def cat_pca_fit(Yq, p: int, want_eigenvalues=False, ws=None):
     """Returns (mean [D], components [p, D][, eigenvalues float64 [p]])."""
     N, D = Yq.shape
     dev = Yq.device
     mean = torch.empty((D,), dtype=torch.float32, device=dev)
     comps = torch.empty((p, D), dtype=torch.float32, device=dev)
     eig = torch.empty((p,), dtype=torch.float64, device=dev) if want_eigenvalues else None
-    ws = _scratch(lib().cat_pca_workspace_bytes(N, D, p), dev, "cat_pca_fit")
+    ws = pca_workspace("pca", N, D, p, dev) if ws is None else ws
     _check(lib().cat_pca_fit(_dev(Yq, torch.float32, None, "Yq"), N, D, p, _dev(mean, torch.float32),
                              _dev(comps, torch.float32), _dev(eig, torch.float64),
                              ctypes.c_void_p(ws.data_ptr()), ws.numel(), _stream()), "cat_pca_fit")
@@ -419,7 +425,7 @@ def cat_affine_with_labels(Yq, labels, gamma, beta, out=None):
     return out
 
 
-def cat_fit_pca(Yq, Yfp, K: int, iters: int, p: int):
+def cat_fit_pca(Yq, Yfp, K: int, iters: int, p: int, ws=None):
     """Returns dict(mean, comps, centroids [K, p], gamma, beta [K, D], labels)."""
     N, D = Yq.shape
     dev = Yq.device
@@ -429,7 +435,7 @@ def cat_fit_pca(Yq, Yfp, K: int, iters: int, p: int):
              gamma=torch.empty((K, D), dtype=torch.float32, device=dev),
              beta=torch.empty((K, D), dtype=torch.float32, device=dev),
              labels=torch.empty((N,), dtype=torch.int32, device=dev))
-    ws = _scratch(lib().cat_fit_pca_workspace_bytes(N, D, K, p), dev, "cat_fit_pca")
+    ws = pca_workspace("fit_pca", N, D, p, dev, K) if ws is None else ws
     _check(lib().cat_fit_pca(_dev(Yq, torch.float32, None, "Yq"), _dev(Yfp, torch.float32, (N, D), "Yfp"), N, D, K, iters, p,
                              _dev(r["mean"], torch.float32), _dev(r["comps"], torch.float32),
                              _dev(r["centroids"], torch.float32), _dev(r["gamma"], torch.float32),
@@ -438,14 +444,14 @@ def cat_fit_pca(Yq, Yfp, K: int, iters: int, p: int):
     return r
 
 
-def cat_apply_pca(Yq, mean, comps, centroids, gamma, beta, out=None, want_labels=False):
+def cat_apply_pca(Yq, mean, comps, centroids, gamma, beta, out=None, want_labels=False, ws=None):
     N, D = Yq.shape
     K, p = centroids.shape
     dev = Yq.device
     if out is None:
         out = torch.empty_like(Yq)
     labels = torch.empty((N,), dtype=torch.int32, device=dev) if want_labels else None
-    ws = _scratch(lib().cat_apply_pca_workspace_bytes(N, D, K, p), dev, "cat_apply_pca")
+    ws = pca_workspace("apply_pca", N, D, p, dev, K) if ws is None else ws
     _check(lib().cat_apply_pca(_dev(Yq, torch.float32, None, "Yq"), N, D, K, p, _dev(mean, torch.float32, (D,)),
                                _dev(comps, torch.float32, (p, D)), _dev(centroids, torch.float32, (K, p)),
                                _dev(gamma, torch.float32, (K, D)), _dev(beta, torch.float32, (K, D)),

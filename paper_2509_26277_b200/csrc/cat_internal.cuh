@@ -291,6 +291,8 @@ cudaError_t launch_fit_diag_round(const float *Y, int64_t N, int D, int K, const
                                   const int32_t *refine_rows, const int32_t *cand_rows, const Control *ctl,
                                   cat_fit_diag_t *diag, int slot, int recorded, cudaStream_t s);
 cudaError_t launch_reset_control(Control *ctl, cudaStream_t s);
+// Adds the counters of a step that ran on a workspace of its own to ctl; its status too, unless ctl has one already.
+cudaError_t launch_absorb_control(Control *ctl, const Control *from, cudaStream_t s);
 
 // Y_out_i = gamma_l * Y_i + beta_l, l = labels[i]; a label outside [0, K) copies the row
 cudaError_t launch_affine_labels(const float *Y, int64_t N, int D, int K, const int32_t *labels, const float *gamma,

@@ -1190,6 +1190,23 @@ __global__ void reset_control_kernel(Control *ctl)
     }
 }
 
+__global__ void absorb_control_kernel(Control *ctl, const Control *from)
+{
+    pdl_enter();
+    if (threadIdx.x == 0 && blockIdx.x == 0) {
+        if (ctl->device_status == CAT_OK) ctl->device_status = from->device_status;
+        ctl->refined_total += from->refined_total;
+        ctl->refined_last = from->refined_last;
+    }
+}
+
+cudaError_t launch_absorb_control(Control *ctl, const Control *from, cudaStream_t s)
+{
+    const cudaError_t e = launch_pdl(absorb_control_kernel, dim3(1), dim3(32), 0, s, ctl, from);
+    count_launch();
+    return e;
+}
+
 cudaError_t launch_reset_control(Control *ctl, cudaStream_t s)
 {
     const cudaError_t e = launch_pdl(reset_control_kernel, dim3(1), dim3(32), 0, s, ctl);

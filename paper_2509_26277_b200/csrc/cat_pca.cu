@@ -491,7 +491,7 @@ cat_status_t cat_affine_with_labels(const float *Yq, int64_t N, int32_t D, int32
 
 namespace {
 struct FitPcaWs {
-    void *pca;  size_t pca_bytes;
+    void *pca;  size_t pca_bytes;   // (first: its control block speaks for the whole call)
     float *Z;                       // [N, p]
     float *gp, *bp;                 // [K, p] closed form of the reduced rows (not used further)
     int32_t *labels;                // [N]
@@ -559,10 +559,11 @@ cat_status_t cat_fit_pca(const float *Yq, const float *Yfp, int64_t N, int32_t D
     if ((st = cat_pca_project(Yq, N, D, p, mean_out, components_out, w.Z, stream)) != CAT_OK) return st;
     if ((st = cat_fit(w.Z, w.Z, N, p, K, iters, centroids_out, w.gp, w.bp, labels, w.fit, w.fit_bytes, stream)) != CAT_OK)
         return st;
+    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    CAT_CUDA(launch_absorb_control(reinterpret_cast<Control *>(w.pca), reinterpret_cast<const Control *>(w.fit), s));
     // the loop over the clusters: moments and the closed form in the original space
     if ((st = cat_cluster_sums(Yq, labels, N, D, K, w.sumQ, w.counts, w.fit, w.fit_bytes, stream)) != CAT_OK) return st;
     if ((st = cat_cluster_sums(Yfp, labels, N, D, K, w.sumF, w.counts, w.fit, w.fit_bytes, stream)) != CAT_OK) return st;
-    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     CAT_CUDA(launch_means_from_sums(w.sumQ, w.counts, D, K, w.meanQ, s));
     CAT_CUDA(launch_means_from_sums(w.sumF, w.counts, D, K, w.meanF, s));
     if ((st = cat_centred_moments(Yq, Yfp, labels, N, D, K, w.meanQ, w.meanF, w.var, w.cov, w.fit, w.fit_bytes, stream)) !=
@@ -576,7 +577,7 @@ size_t cat_apply_pca_workspace_bytes(int64_t N, int32_t D, int32_t K, int32_t p)
     if (N < 1 || D < 1 || p < 1 || p > D || D > CAT_PCA_MAX_D || p > CAT_PCA_MAX_P) return 0;
     const size_t a = cat_apply_workspace_bytes(N, p, K);
     if (a == 0) return 0;
-    return align_up((size_t)N * p * sizeof(float), 256) + align_up((size_t)N * sizeof(int32_t), 256) + a;
+    return align_up(a, 256) + align_up((size_t)N * p * sizeof(float), 256) + align_up((size_t)N * sizeof(int32_t), 256);
 }
 
 cat_status_t cat_apply_pca(const float *Yq, int64_t N, int32_t D, int32_t K, int32_t p, const float *mean,
@@ -588,15 +589,16 @@ cat_status_t cat_apply_pca(const float *Yq, int64_t N, int32_t D, int32_t K, int
     const size_t need = cat_apply_pca_workspace_bytes(N, D, K, p);
     if (need == 0) return (N < 1 || D < 1 || p < 1 || p > D || K < 1) ? CAT_ERR_SHAPE : CAT_ERR_UNSUPPORTED;
     if (!workspace || !al16(workspace) || workspace_bytes < need) return CAT_ERR_WORKSPACE;
+    // (the assignment's part first: its control block is where cat_workspace_report looks)
     unsigned char *b = reinterpret_cast<unsigned char *>(workspace);
-    float *Z = reinterpret_cast<float *>(b);
-    size_t off = align_up((size_t)N * p * sizeof(float), 256);
-    int32_t *labels = labels_out ? labels_out : reinterpret_cast<int32_t *>(b + off);
-    off += align_up((size_t)N * sizeof(int32_t), 256);
+    const size_t assign_bytes = align_up(cat_apply_workspace_bytes(N, p, K), 256);
+    float *Z = reinterpret_cast<float *>(b + assign_bytes);
+    int32_t *labels =
+        labels_out ? labels_out : reinterpret_cast<int32_t *>(b + assign_bytes + align_up((size_t)N * p * sizeof(float), 256));
     cat_status_t st;
     // Algorithm 2 step 1: project; step 2: predict the cluster; steps 4-8: correct in the original space
     if ((st = cat_pca_project(Yq, N, D, p, mean, components, Z, stream)) != CAT_OK) return st;
-    if ((st = cat_assign(Z, N, p, K, centroids, labels, b + off, workspace_bytes - off, stream)) != CAT_OK) return st;
+    if ((st = cat_assign(Z, N, p, K, centroids, labels, b, assign_bytes, stream)) != CAT_OK) return st;
     return cat_affine_with_labels(Yq, N, D, K, labels, gamma, beta, Y_out, stream);
 }
 

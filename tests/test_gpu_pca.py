@@ -151,3 +151,36 @@ def test_eigenpairs_do_not_vary_from_run_to_run(n, d, p):
         again = B.cat_pca_fit(Y, p, want_eigenvalues=True)
         for x, y in zip(first, again):
             assert torch.equal(x, y)
+
+
+def test_one_control_block_speaks_for_the_composed_calls():
+    """cat_workspace_report on the workspace of cat_fit_pca and cat_apply_pca: the counters of their K-Means and
+    assignment steps, and a status that every call starts afresh."""
+    n, d, k, p = 900, 60, 6, 8
+    rng = np.random.default_rng(3)
+    Y = rng.normal(size=(n, d)).astype(np.float32)
+    Y[n // 2:] = Y[:n - n // 2]                              # (each row twice: equal centroids, rows left to the exact pass)
+    Y[1] = Y[0]
+    Y = dev(Y)
+    ws = B.pca_workspace("pca", n, d, p, "cuda")
+    B.cat_selftest_wait_timeout(ws, limit_ms=5)
+    B.cat_pca_fit(Y, p, ws=ws)
+    assert B.cat_workspace_report(ws)["device_status"] == 0
+    ws = B.pca_workspace("fit_pca", n, d, p, "cuda", K=k)
+    B.cat_selftest_wait_timeout(ws, limit_ms=5)
+    assert B.cat_workspace_report(ws)["device_status"] == 6
+    r = B.cat_fit_pca(Y, Y, k, 0, p, ws=ws)
+    rep = B.cat_workspace_report(ws)
+    Z = B.cat_pca_project(Y, r["mean"], r["comps"])
+    wz = B.workspace("fit", n, p, k, "cuda")
+    B.cat_fit(Z, Z, k, 0, ws=wz)
+    assert rep == B.cat_workspace_report(wz)
+    assert rep["device_status"] == 0 and rep["refined_rows_last"] > 0
+    ws = B.pca_workspace("apply_pca", n, d, p, "cuda", K=k)
+    B.cat_selftest_wait_timeout(ws, limit_ms=5)
+    B.cat_apply_pca(Y, r["mean"], r["comps"], r["centroids"], r["gamma"], r["beta"], ws=ws)
+    rep = B.cat_workspace_report(ws)
+    wz = B.workspace("apply", n, p, k, "cuda")
+    B.cat_assign(Z, r["centroids"], ws=wz)
+    assert rep == B.cat_workspace_report(wz)
+    assert rep["device_status"] == 0 and rep["refined_rows_last"] > 0
