@@ -119,6 +119,9 @@ cat_status_t cat_fit_from(const float *Yq, const float *Yfp, int64_t N, int32_t 
  *
  * Yq [N, D] in; centroids, gamma, beta [K, D] in; Y_out [N, D] out (must not
  * overlap Yq); labels_out [N] out, may be NULL.  N >= 1 (N < K is allowed).
+ * The workspace holds tables of a few N and K*D words.  For D % 4 != 0, D >= 8 and K <= 256 it also has room for an
+ * fp16 copy of a slab of rows (about N*D*2 bytes, at most 512 MiB), which
+ * cat_assign uses, and cat_apply and cat_apply_bf16 where the kernel that keeps rows in shared memory does not go.
  */
 size_t cat_apply_workspace_bytes(int64_t N, int32_t D, int32_t K);
 

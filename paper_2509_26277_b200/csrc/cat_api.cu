@@ -27,7 +27,18 @@ struct Carver {
     }
 };
 
-// inference: room for what only inference needs (prepared centroids; an fp16 copy of rows that TMA cannot address)
+// Rows of an inference call's fp16 copy (rows that TMA cannot address): at most 512 MiB of them at a time, so that
+// the scratch of a call does not grow with N * D.  A further slab costs about 17 us (two kernels that fill and drain
+// the device once more: 400 000 x 1001, K = 200 takes 970 us in one piece, 988 in two).  The rows are split evenly.
+static int64_t copy_slab_rows(int64_t N, int D)
+{
+    const int64_t cap = ((int64_t)512 << 20) / (2 * half_ld(D));
+    const int64_t slabs = (N + cap - 1) / cap;
+    const int64_t rows = ((N + slabs - 1) / slabs + 255) & ~(int64_t)255;
+    return rows < N ? rows : N;
+}
+
+// inference: room for what only inference needs (prepared centroids; the fp16 copy of a slab of rows)
 static void carve_assign_into(Carver &c, AssignWs &w, int64_t N, int D, int K, bool inference)
 {
     const bool row_copy = inference && D % 4 != 0 && D >= TC_HALF_MIN_D && K <= 256;
@@ -44,10 +55,11 @@ static void carve_assign_into(Carver &c, AssignWs &w, int64_t N, int D, int K, b
     w.cerr = c.take<float>((size_t)K);
     w.mean = c.take<float>((size_t)D);
     w.ch = c.take<uint16_t>((size_t)K * half_ld(D));
-    w.hscale = c.take<float>(row_copy ? 4 + 2 * (size_t)N : 4);
+    const size_t slab = row_copy ? (size_t)copy_slab_rows(N, D) : 0;
+    w.hscale = c.take<float>(4 + 2 * slab);
     const size_t prep = inference ? apply_rows_prep_bytes(N, D, K) : 0;
     w.prep = prep ? c.take<unsigned char>(prep) : nullptr;
-    w.yh = row_copy ? c.take<uint16_t>((size_t)N * half_ld(D)) : nullptr;
+    w.yh = row_copy ? c.take<uint16_t>(slab * half_ld(D)) : nullptr;
 }
 
 AssignWs carve_assign(void *base, int64_t N, int D, int K)
@@ -214,10 +226,16 @@ static cat_status_t run_assign(const float *Y, int64_t N, int D, int K, const fl
         // tensor cores (49 999 x 1001, K = 50: 233 us against 1546 us on the fp32 pipes, whose loads of
         // such rows are scalar).
         CAT_CUDA(launch_sample_mean(Y, N, D, w.mean, s));
-        CAT_CUDA(launch_half_shadow(Y, N, D, w.mean, w.ynorm2, w.hscale, w.yh, s, false));
-        CAT_CUDA(launch_centroid_half(C, D, K, w.mean, w.cnorm, w.cmax, w.cerr, w.hscale, w.ch, w.ctl, s, top_level));
-        CAT_CUDA(launch_assign_tc(Y, N, D, K, C, w.cnorm, w.ynorm2, labels, w.refine_rows, w.cand_rows, w.cand_list, w.ctl,
-                                  nullptr, nullptr, nullptr, s, w.yh, w.ch, w.hscale, w.cerr));
+        const int64_t slab = copy_slab_rows(N, D);
+        for (int64_t r = 0; r < N; r += slab) {
+            const int64_t n = N - r < slab ? N - r : slab;
+            const float *y = Y + (size_t)r * D;
+            CAT_CUDA(launch_half_shadow(y, n, D, w.mean, w.ynorm2, w.hscale, w.yh, s, false));
+            if (r == 0)
+                CAT_CUDA(launch_centroid_half(C, D, K, w.mean, w.cnorm, w.cmax, w.cerr, w.hscale, w.ch, w.ctl, s, top_level));
+            CAT_CUDA(launch_assign_tc(y, n, D, K, C, w.cnorm, w.ynorm2, labels + r, w.refine_rows, w.cand_rows, w.cand_list, w.ctl,
+                                      nullptr, nullptr, nullptr, s, w.yh, w.ch, w.hscale, w.cerr, nullptr, r));
+        }
         CAT_CUDA(launch_refine_both(Y, N, D, K, C, labels, w.cand_rows, w.cand_list, w.refine_rows, w.ctl, nullptr,
                                     nullptr, nullptr, s));
         if (out) CAT_CUDA(launch_affine_labels(Y, N, D, K, labels, gamma, beta, out, s));
@@ -569,7 +587,7 @@ cat_status_t cat_fit_shard_begin(const float *Yq, int64_t N, int32_t D, int32_t 
     CAT_CUDA(cudaMemsetAsync(w.hscale, 0, 4 * sizeof(float), s));
     if (use_half_path(N, D, K)) {
         CAT_CUDA(launch_sample_mean(Yq, N, D, w.a.mean, s));
-        CAT_CUDA(launch_half_shadow(Yq, N, D, w.a.mean, w.a.ynorm2, w.hscale, w.yh, s, false));
+        CAT_CUDA(launch_half_shadow(Yq, N, D, w.a.mean, w.a.ynorm2, w.hscale, w.yh, s, true, false));
     } else if (use_tensor_path(N, D, K))
         CAT_CUDA(launch_row_norms(Yq, N, D, w.a.ynorm2, s));
     // (the bit pattern of a non-negative float is the float itself)

@@ -98,9 +98,9 @@ struct AssignWs {          // what assign/apply need
     float *cerr;           // [K] norms of the rounding errors of the fp16 centroids
     float *mean;           // [D] what rows and centroids are taken relative to on fp16 operands
     void *ch;              // [K][half_ld(D)] fp16 copy of the centroids (inference on fp16 operands)
-    float *hscale;         // [4] scale of that copy: {s_c, -2 / s_c, 2^-25 / s_c, -}; with yh followed by [N] inverse row scales and [N] rounding errors
+    float *hscale;         // [4] scale of that copy: {s_c, -2 / s_c, 2^-25 / s_c, -}; with yh followed by [slab] inverse row scales and [slab] rounding errors
     void *prep;            // prepared centroids of the inference kernel that keeps rows in shared memory (or null)
-    void *yh;              // [N][half_ld(D)] fp16 copy of the rows (inference with D % 4 != 0), else null
+    void *yh;              // [slab][half_ld(D)] fp16 copy of a slab of rows (inference with D % 4 != 0), else null
     size_t bytes;
 };
 AssignWs carve_assign(void *base, int64_t N, int D, int K);
@@ -203,7 +203,7 @@ cudaError_t launch_assign_tc(const float *Y, int64_t N, int D, int K, const floa
                              int32_t *cand_rows, uint64_t *cand_list, Control *ctl,
                              const float *gamma, const float *beta, float *out, cudaStream_t s,
                              const void *Yh = nullptr, const void *Ch = nullptr, const float *scale = nullptr,
-                             const float *cerr = nullptr, const FastOut *fast = nullptr);
+                             const float *cerr = nullptr, const FastOut *fast = nullptr, int64_t row_base = 0);
 
 // One warp waits (at most limit_ms, clamped to 1 .. 1000) on a barrier that is never completed.
 cudaError_t launch_wait_selftest(Control *ctl, int limit_ms, cudaStream_t s);
@@ -217,9 +217,10 @@ __host__ __device__ constexpr int half_ld(int D) { return (D + 7) & ~7; }
 constexpr int TC_HALF_MIN_D = 8;
 bool tc_half_supported(int64_t N, int D, int K);
 // finish_scale = false leaves the bits of the largest magnitude in scale[0] (launch_half_scale turns them
-// into the three scale words later, e.g. once the maximum over several shards is known).
+// into the three scale words later, e.g. once the maximum over several shards is known); want_amax = false leaves
+// those words alone.
 cudaError_t launch_half_shadow(const float *Y, int64_t N, int D, const float *mean, float *ynorm2, float *scale, void *Yh,
-                               cudaStream_t s, bool finish_scale = true);
+                               cudaStream_t s, bool want_amax = true, bool finish_scale = true);
 // A point among the rows to take them relative to: the column means of the first 128 (any point will do).
 cudaError_t launch_sample_mean(const float *Y, int64_t N, int D, float *mean, cudaStream_t s);
 // Everything an assignment on fp16 operands needs of the centroids less `mean` (null: as they are): norms,

@@ -937,7 +937,7 @@ __device__ __forceinline__ void load_mean(const float *__restrict__ mean, int c,
 // One sweep over the rows: squared norm (slightly over-estimated), the row's own power-of-two
 // scale s_i (largest magnitude to [2^13, 2^14)), rinv[i] = 1 / s_i, Yh[i, :] = fp16(Y[i, :] * s_i)
 // rounded to nearest (rows of Yh ld elements apart), the norm rerr[i] of what the rounding left, and the
-// largest magnitude of the matrix (float bits, one atomicMax per CTA).  With `mean` everything but that
+// largest magnitude of the matrix (float bits, one atomicMax per CTA; amax_bits may be null).  With `mean` everything but that
 // magnitude is of Y[i, :] - mean: nearest centroids do not depend on the origin, and smaller operands make
 // smaller errors.  A row is handled by G lanes and read twice; the second read comes
 // out of L1/L2.  VEC4: 128-bit loads (D % 4 == 0); otherwise a lane takes pairs of columns with
@@ -1055,7 +1055,7 @@ __global__ void __launch_bounds__(256) half_shadow_kernel(const float *__restric
     if (threadIdx.x == 0) {
         float t = 0.f;
         for (int w = 0; w < 8; ++w) t = fmaxf(t, wmax[w]);
-        atomicMax(amax_bits, __float_as_uint(t));
+        if (amax_bits) atomicMax(amax_bits, __float_as_uint(t));
     }
 }
 
@@ -1285,21 +1285,24 @@ cudaError_t launch_row_norms(const float *Y, int64_t N, int D, float *out, cudaS
 }
 
 cudaError_t launch_half_shadow(const float *Y, int64_t N, int D, const float *mean, float *ynorm2, float *scale, void *Yh,
-                               cudaStream_t s, bool finish_scale)
+                               cudaStream_t s, bool want_amax, bool finish_scale)
 {
     float *rinv = scale + 4, *rerr = scale + 4 + N;
-    cudaError_t e = cudaMemsetAsync(scale, 0, 4 * sizeof(float), s);
+    cudaError_t e = want_amax ? cudaMemsetAsync(scale, 0, 4 * sizeof(float), s) : cudaSuccess;
     if (e != cudaSuccess) return e;
     const int G = lanes_per_row(D);
     const int rows_per_cta = 256 / G;
     int64_t blocks = (N + rows_per_cta - 1) / rows_per_cta;
     const int64_t cap = (int64_t)sm_count() * 8;
     if (blocks > cap) blocks = cap;
-    e = launch_pdl(D % 4 == 0 ? half_shadow_kernel<true> : half_shadow_kernel<false>, dim3((unsigned)blocks), dim3(256), 0, s, Y, N, D,
-                   half_ld(D), G, mean, ynorm2, rinv, rerr, reinterpret_cast<unsigned int *>(scale), reinterpret_cast<__half *>(Yh));
-    if (e != cudaSuccess) return e;
+    // (An ordinary launch: a dependent one that starts beside the tail of a kernel with much shared memory keeps that
+    // kernel's split of the L1, and the second read of a row misses -- 100 000 x 1001: K = 200: 335 us a cat_assign against 311.)
+    const auto kern = D % 4 == 0 ? half_shadow_kernel<true> : half_shadow_kernel<false>;
+    kern<<<(unsigned)blocks, 256, 0, s>>>(Y, N, D, half_ld(D), G, mean, ynorm2, rinv, rerr,
+                                          want_amax ? reinterpret_cast<unsigned int *>(scale) : nullptr, reinterpret_cast<__half *>(Yh));
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     count_launch();
-    return finish_scale ? launch_half_scale(scale, s) : cudaGetLastError();
+    return want_amax && finish_scale ? launch_half_scale(scale, s) : cudaGetLastError();
 }
 
 cudaError_t launch_sample_mean(const float *Y, int64_t N, int D, float *mean, cudaStream_t s)
@@ -1452,9 +1455,10 @@ cudaError_t launch_assign_tc(const float *Y, int64_t N, int D, int K, const floa
                              const float *ynorm2, int32_t *labels, int32_t *refine_rows,
                              int32_t *cand_rows, uint64_t *cand_list, Control *ctl,
                              const float *gamma, const float *beta, float *out, cudaStream_t s,
-                             const void *Yh, const void *Ch, const float *scale, const float *cerr, const FastOut *fast)
+                             const void *Yh, const void *Ch, const float *scale, const float *cerr, const FastOut *fast, int64_t row_base)
 {
     TcParams p{};
+    p.row_base = row_base;
     if (fast) p.fast = *fast;
     p.Y = Y;
     p.cnorm = cnorm;

@@ -325,6 +325,7 @@ struct TcParams {
     const float *beta;
     float *out;
     int64_t N;
+    int64_t row_base;   // added to a row's number where it is queued (a slab of a larger matrix)
     int D;
     int K;
     int npad;       // K rounded up to 32 (the score warps read TMEM 32 columns per step)
@@ -429,13 +430,13 @@ __device__ __forceinline__ bool tc_decide(const TcParams &p, int64_t row, float4
     const bool more = p.K > 4 && !((sc.w - sc.x) > lim);   // the 4th is a candidate too (or NaN): others may be
     if (more || !trusted) {
         int slot = atomicAdd(&p.ctl->refine_count, 1);
-        p.refine_rows[slot] = (int32_t)row;
+        p.refine_rows[slot] = (int32_t)(p.row_base + row);
     } else {
         uint64_t c = (uint64_t)(uint16_t)key_index(sc.x) | ((uint64_t)(uint16_t)key_index(sc.y) << 16);
         c |= (uint64_t)(((sc.z - sc.x) > lim || p.K < 3) ? 0xFFFFu : (uint16_t)key_index(sc.z)) << 32;
         c |= (uint64_t)(((sc.w - sc.x) > lim || p.K < 4) ? 0xFFFFu : (uint16_t)key_index(sc.w)) << 48;
         int slot = atomicAdd(&p.ctl->cand_count, 1);
-        p.cand_rows[slot] = (int32_t)row;
+        p.cand_rows[slot] = (int32_t)(p.row_base + row);
         p.cand_list[slot] = c;
     }
     return false;

@@ -591,3 +591,32 @@ def test_rows_of_any_length_on_padded_fp16_copies(n, d, k, scale):
         if ora.near.sum() == 0:
             assert np.array_equal(host(lg), ora.labels)
             close(host(Cg) / scale, ora.centroids / scale, "centroids")
+
+
+@pytest.mark.parametrize("n,d,k", [(600_000, 1001, 130), (1_400_077, 255, 200), (20_000, 16_383, 40)])
+def test_rows_copied_in_slabs(n, d, k):
+    """More rows of a length no tensor map can address than the workspace's fp16 copy holds at a time: labels as the
+    oracle gives them across the seams, undecided rows counted over all slabs, a workspace well below the whole copy."""
+    rng = np.random.default_rng(n)
+    slabs = -(-n // ((512 << 20) // (2 * ((d + 7) // 8 * 8))))
+    slab = (-(-n // slabs) + 255) // 256 * 256
+    assert slab < n
+    ws = B.workspace("apply", n, d, k, "cuda")
+    assert ws.numel() < (520 << 20) + 40 * n + 64 * k * d
+    g = torch.Generator(device="cuda").manual_seed(n)
+    C = torch.randn((k, d), device="cuda", generator=g)
+    pick = torch.randint(0, k, (n,), device="cuda", generator=g)
+    Y = C[pick] + 0.5 * torch.randn((n, d), device="cuda", generator=g)
+    seams = [i for s in range(slab, n, slab) for i in range(s - 3, min(s + 3, n))]
+    Y[seams] = 0.5 * (C[0] + C[1])                           # undecided rows on both sides of every seam
+    labels = B.cat_assign(Y, C, ws=ws)
+    rep = B.cat_workspace_report(ws)
+    at = np.unique(np.concatenate([np.arange(200), slab + np.arange(-200, 200), n - 1 - np.arange(200), seams,
+                                   rng.integers(0, n, size=400)]) % n)
+    want, best, second = O.assign(host(Y[torch.as_tensor(at).cuda()]), host(C))
+    labels_match(host(labels)[at], want, best, second, "labels")
+    assert rep["device_status"] == 0 and len(seams) <= rep["refined_rows_last"] < n
+    pick[seams] = labels[seams].long()
+    assert bool((labels == pick).all())
+    out, lab2 = B.cat_apply(Y, C, torch.ones_like(C), torch.zeros_like(C), want_labels=True, ws=ws)
+    assert torch.equal(lab2, labels) and torch.equal(out, Y)
