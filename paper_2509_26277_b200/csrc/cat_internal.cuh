@@ -221,7 +221,8 @@ bool tc_half_supported(int64_t N, int D, int K);
 // those words alone.
 cudaError_t launch_half_shadow(const float *Y, int64_t N, int D, const float *mean, float *ynorm2, float *scale, void *Yh,
                                cudaStream_t s, bool want_amax = true, bool finish_scale = true);
-// A point among the rows to take them relative to: the column means of the first 128 (any point will do).
+// A point among the rows to take them relative to, from the first 128 (any finite point will do; one that a few stray
+// rows do not move keeps the operands small).
 cudaError_t launch_sample_mean(const float *Y, int64_t N, int D, float *mean, cudaStream_t s);
 // Everything an assignment on fp16 operands needs of the centroids less `mean` (null: as they are): norms,
 // the fp16 copy, the norms cerr of its rounding errors, and with own_scale the scale words from their largest

@@ -1157,22 +1157,35 @@ __global__ void __launch_bounds__(256) centroid_prep_kernel(const float *__restr
     }
 }
 
-// Column means of the first `rows` rows: 32 columns per CTA, eight groups of rows.
+// A point among the first `rows` rows, per column: the median of the means of eight interleaved groups of them
+// (32 columns per CTA).  A row far off all others moves the mean of its own group only, and a group whose sum is not
+// finite does not count, so that up to three such rows leave the point where it is; a plain mean would carry them
+// into the operands of every row.
 __global__ void __launch_bounds__(256) sample_mean_kernel(const float *__restrict__ Y, int rows, int D, float *__restrict__ mean)
 {
     pdl_enter();
-    __shared__ float part[8][32];
+    __shared__ float part[8][32];   // NaN: does not count
     const int c = threadIdx.x & 31, g = threadIdx.x >> 5, j = blockIdx.x * 32 + c;
     float s = 0.f;
     if (j < D)
 #pragma unroll 16
         for (int r = g; r < rows; r += 8) s += __ldg(Y + (size_t)r * D + j);
-    part[g][c] = s;
+    part[g][c] = g < rows && fabsf(s) < CUDART_INF_F ? s / (float)((rows - g + 7) >> 3) : CUDART_NAN_F;
     __syncthreads();
-    if (g == 0 && j < D) {
-        for (int q = 1; q < 8; ++q) s += part[q][c];
-        mean[j] = s / (float)rows;
+    if (j >= D) return;
+    // each group's thread ranks its own mean among the groups that have one; the middle one or two make the median
+    const float v = part[g][c];
+    int rank = 0, valid = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const float o = part[q][c];
+        valid += o == o;
+        rank += o < v || (o == v && q < g);
     }
+    __syncthreads();
+    if (v == v) part[rank][c] = v;
+    __syncthreads();
+    if (g == 0) mean[j] = valid == 0 ? 0.f : 0.5f * part[(valid - 1) / 2][c] + 0.5f * part[valid / 2][c];
 }
 
 // Self-test of the bounded wait: one warp waits on a barrier that nothing ever completes, with

@@ -68,3 +68,21 @@ def test_inference(n, d, k, mag, small_kernels):
     out, glab = B.cat_apply(dev(Yq), dev(C), dev(g), dev(b), want_labels=True)
     assert np.array_equal(host(glab), lab)
     np.testing.assert_array_equal(host(out), O.affine_with_labels(Yq, lab, g, b))
+
+
+@pytest.mark.parametrize("stray", [[], [3], [5, 64, 120]])
+@pytest.mark.parametrize("value", [1e30, -3e38, np.inf, np.nan])
+def test_stray_rows_do_not_reach_the_others(stray, value):
+    """Rows of huge or non-finite entries among the first 128, which the fp16 copies take their common point from: the
+    other rows are still decided by their fast scores (exact labels either way)."""
+    n, d, k = 4000, 1001, 20
+    rng = np.random.default_rng(9)
+    C = rng.normal(size=(k, d)).astype(np.float32)
+    Yq = (C[rng.integers(0, k, size=n)] + 0.4 * rng.normal(size=(n, d))).astype(np.float32)
+    Yq[stray] = value
+    ws = B.workspace("apply", n, d, k, "cuda")
+    labels = host(B.cat_assign(dev(Yq), dev(C), ws=ws))
+    rest = np.setdiff1d(np.arange(n), stray)
+    assert np.array_equal(labels[rest], O.assign(Yq[rest], C)[0])
+    assert ((labels >= 0) & (labels < k)).all()
+    assert len(stray) <= B.cat_workspace_report(ws)["refined_rows_last"] < 100
