@@ -614,7 +614,8 @@ __global__ void __launch_bounds__(RES_MAX_THREADS, 1) apply_rows_kernel(ResParam
 #pragma unroll
             for (int o = LPR / 2; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
             const float e = 1.0625f * 2.f * (sqrt_approx(left2 * slack) * cnorm + sqrt_approx(yn2 * slack) * e_y) + e_abs;
-            const float lim = best + 2.f * e;
+            // (a score that overflowed downwards is no lower than the lowest finite one as far as the bound goes)
+            const float lim = fmaxf(best, -3.4028235e38f) + 2.f * e;
             int cands = 0;
 #pragma unroll
             for (int i = 0; i < KI; ++i) cands += __popc(__ballot_sync(0xffffffffu, l + LPR * i < p.K && !(sc[i] > lim)) & mine);

@@ -86,3 +86,28 @@ def test_stray_rows_do_not_reach_the_others(stray, value):
     assert np.array_equal(labels[rest], O.assign(Yq[rest], C)[0])
     assert ((labels >= 0) & (labels < k)).all()
     assert len(stray) <= B.cat_workspace_report(ws)["refined_rows_last"] < 100
+
+
+@pytest.mark.parametrize("n,d", [(6000, 60), (3000, 1000), (3000, 301)])
+def test_scores_around_the_lowest_finite_one(n, d, small_kernels):
+    """Two near centroids and ten far ones, placed so that the scores ||y - c||^2 - ||y - m||^2 (m: the centroids'
+    mean) of the two near ones pass the lowest finite fp32 number while every norm is finite: one of
+    the two may come out as an infinity, the other not."""
+    k = 12
+    rng = np.random.default_rng(d)
+    u, w = np.linalg.qr(rng.normal(size=(d, 2)))[0].T
+    C = np.concatenate([[1.7e19 * u + 3e16 * w, 1.7e19 * u - 3e16 * w], np.tile(-4.6e18 * u, (k - 2, 1))])
+    C[2:] += 1e17 * rng.normal(size=(k - 2, d)) / np.sqrt(d)
+    C = C.astype(np.float32)
+    m = C.astype(np.float64).mean(0)
+    # along u: score(h) = |h u - c|^2 - |h u - m|^2 = 2 h (m - c).u + |c|^2 - |m|^2
+    c = 1.7e19 * u
+    h = (-3.4028235e38 - c @ c + m @ m) / (2 * (m - c) @ u)
+    Yq = (h * (1 + 1e-5 * rng.normal(size=n)))[:, None] * u + (1e14 * rng.normal(size=n))[:, None] * w
+    Yq = Yq.astype(np.float32)
+    assert np.isfinite((Yq * Yq).sum(1)).all()
+    lab, best, second = O.assign(Yq, C)
+    g, b = rng.normal(size=(k, d)).astype(np.float32), rng.normal(size=(k, d)).astype(np.float32)
+    labels_match(host(B.cat_assign(dev(Yq), dev(C))), lab, best, second, "labels")
+    out, glab = B.cat_apply(dev(Yq), dev(C), dev(g), dev(b), want_labels=True)
+    labels_match(host(glab), lab, best, second, "labels")
