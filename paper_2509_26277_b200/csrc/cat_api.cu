@@ -485,7 +485,7 @@ cat_status_t cat_fit_from(const float *Yq, const float *Yfp, int64_t N, int32_t 
     if (rows) {
         // (scratch: the list of changed rows where the general path sorts, its counts where segments are
         // summed, the padded centroids where the moments come to lie)
-        CAT_CUDA(launch_fit_rows(Yq, N, D, K, C, iters + 1, labels, w.sumQ, w.counts, w.order, reinterpret_cast<int32_t *>(w.segpart),
+        CAT_CUDA(launch_fit_rows(Yq, N, D, K, C, iters + 1, labels, w.sumQ, w.counts, w.order, w.segpart,
                                  reinterpret_cast<float *>(w.var), w.a.ctl, s));
     } else if (small) {
         unsigned int bar_count = 0;   // (the control block was reset above)

@@ -19,6 +19,10 @@
 // A round in which no label changes leaves the centroids as they are, bit for bit, and so do all that would
 // follow: the rounds end there.  The last pass assigns against the final centroids and leaves them alone;
 // its sums and sizes feed the closed form.
+//
+// Sums that follow a list keep what the addition of a row rounded off after that row has left.  That is harmless as long
+// as no row is far larger than the others; where the largest row's exponent is more than F_SPREAD above the rows'
+// average, every round adds up all rows afresh instead (and none ends early).
 //   bound: latency (barriers, staging the centroids, the list's row fetches) for small sets -- 1024 x 1000,
 //   K = 16: 7 us a round --, staging and fp32 issue for the largest that are taken (4096 x 1000, K = 32: 36 us).
 #include "cat_tc.cuh"
@@ -32,6 +36,7 @@ constexpr int FW = FT / 32;
 constexpr int F_LIST = 2048;          // list entries staged at a time
 constexpr int F_QUEUE = 64;           // hits a warp holds before it fetches their rows
 constexpr int F_MAX_GRID = 160;
+constexpr int F_SPREAD = 16;          // (2^16 of the 2^53 that fp64 resolves)
 constexpr size_t F_SMEM = 225 * 1024;
 
 struct FitRowsParams {
@@ -42,7 +47,7 @@ struct FitRowsParams {
     double *sums;            // [K, D] out
     int64_t *counts;         // [K] out
     uint2 *list;             // [G][rpc] {row, new label | old label << 16}
-    int32_t *list_count;     // [G]
+    int4 *list_count;        // [G] {entries; first pass, of the rows' largest magnitudes: sum of exponents, number above zero, largest exponent}
     Control *ctl;
     int64_t N;
     int D, K, passes;
@@ -136,7 +141,8 @@ __device__ __forceinline__ void add_entry(uint32_t w, float v, int k0, int k1, i
 __global__ void __launch_bounds__(FT, 1) fit_rows_kernel(FitRowsParams p)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int s_total, s_fail;
+    __shared__ int s_total, s_fail, s_afresh;
+    __shared__ int3 s_exp[FW];
     __shared__ __align__(8) uint64_t s_bar;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int D = p.D, K = p.K, G = gridDim.x;
@@ -162,9 +168,18 @@ __global__ void __launch_bounds__(FT, 1) fit_rows_kernel(FitRowsParams p)
 
     // rows, zero-padded to whole groups of four rows and columns
     const int n4 = (nrows + 3) & ~3, ld4 = p.ldy >> 2;
-    for (int r = warp; r < n4; r += FW)
-        for (int j = lane; j < p.ldy; j += 32)
-            ys[(size_t)r * p.ldy + j] = r < nrows && j < D ? __ldg(p.Y + (size_t)(row0 + r) * D + j) : 0.f;
+    int3 ex = make_int3(0, 0, 0);
+    for (int r = warp; r < n4; r += FW) {
+        float m = 0.f;
+        for (int j = lane; j < p.ldy; j += 32) {
+            const float v = r < nrows && j < D ? __ldg(p.Y + (size_t)(row0 + r) * D + j) : 0.f;
+            ys[(size_t)r * p.ldy + j] = v;
+            m = fmaxf(m, fabsf(v));
+        }
+        const uint32_t bits = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+        if (bits) ex = make_int3(ex.x + (int)(bits >> 23), ex.y + 1, max(ex.z, (int)(bits >> 23)));
+    }
+    if (lane == 0) s_exp[warp] = ex;
     for (int r = tid; r < p.rpc; r += FT) prev[r] = -1;
     if (tw == 0) {
         for (int e = lane; e < p.span * 8; e += 32) sum[e] = 0.0;
@@ -181,6 +196,7 @@ __global__ void __launch_bounds__(FT, 1) fit_rows_kernel(FitRowsParams p)
     const float eta = 1.0625f * ((float)D * 0.03125f + 12.f) * 5.9604645e-8f;
     int refined = 0, refined_pass = 0;
     uint32_t bar = 0;
+    bool afresh = false;
     for (int pass = 0; pass < p.passes; ++pass) {
         // ---- distances to all centroids, a chunk of them at a time
         for (int c0 = 0; c0 < K; c0 += p.chunk) {
@@ -276,28 +292,40 @@ __global__ void __launch_bounds__(FT, 1) fit_rows_kernel(FitRowsParams p)
         }
         refined += refined_pass;
         __syncthreads();
-        // ---- rows that changed, in row order
+        // ---- rows that changed (or all of them), in row order
         if (warp == 0) {
             int n = 0;
             for (int b = 0; b < nrows; b += 32) {
                 const int r = b + lane;
                 const int l = r < nrows ? lab[r] : 0, o = r < nrows ? prev[r] : 0;
-                const bool moved = r < nrows && l != o;
+                const bool moved = r < nrows && (afresh || l != o);
                 const uint32_t m = __ballot_sync(0xffffffffu, moved);
                 if (moved) {
                     p.list[(size_t)row0 + n + __popc(m & ((1u << lane) - 1u))] =
-                        make_uint2((uint32_t)(row0 + r), (uint32_t)l | ((uint32_t)(o < 0 ? 0xFFFF : o) << 16));
+                        make_uint2((uint32_t)(row0 + r), (uint32_t)l | ((uint32_t)(o < 0 || afresh ? 0xFFFF : o) << 16));
                     prev[r] = l;
                 }
                 n += __popc(m);
             }
-            if (lane == 0) p.list_count[blockIdx.x] = n;
+            if (lane == 0) {
+                int4 w = make_int4(n, 0, 0, 0);
+                for (int q = 0; pass == 0 && q < FW; ++q) {
+                    w.y += s_exp[q].x;
+                    w.z += s_exp[q].y;
+                    w.w = max(w.w, s_exp[q].z);
+                }
+                p.list_count[blockIdx.x] = w;
+            }
         }
         if (!fit_barrier(p.ctl, ++bar)) return;
         if (warp == 0) {
-            int run = 0;
+            int run = 0, esum = 0, rows = 0, emax = 0;
             for (int b = 0; b < G; b += 32) {
-                const int v = b + lane < G ? __ldcg(p.list_count + b + lane) : 0;
+                const int4 w = b + lane < G ? __ldcg(p.list_count + b + lane) : make_int4(0, 0, 0, 0);
+                const int v = w.x;
+                esum += w.y;
+                rows += w.z;
+                emax = max(emax, w.w);
                 int incl = v;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
@@ -311,11 +339,20 @@ __global__ void __launch_bounds__(FT, 1) fit_rows_kernel(FitRowsParams p)
                 pref[G] = run;
                 s_total = run;
             }
+            if (pass == 0) {
+                esum = __reduce_add_sync(0xffffffffu, esum);
+                rows = __reduce_add_sync(0xffffffffu, rows);
+                emax = __reduce_max_sync(0xffffffffu, emax);
+                if (lane == 0) s_afresh = (emax - F_SPREAD) * rows > esum;
+            }
         }
         __syncthreads();
         const int M = s_total;
         const bool last = pass + 1 == p.passes;
         if (M == 0) break;   // nothing moved: nothing would from here on
+        // (the first list has all rows in either case; the same decision in every CTA)
+        const bool carried = !afresh;
+        afresh = s_afresh != 0;
 
         // ---- the sums follow the list
         if (owner) {
@@ -381,7 +418,7 @@ __global__ void __launch_bounds__(FT, 1) fit_rows_kernel(FitRowsParams p)
         __syncthreads();
         if (owner && tw == 0) {
             for (int e = lane; e < (k1 - k0) * 8; e += 32) {
-                double a = sum[e];
+                double a = carried ? sum[e] : 0.0;
                 for (int w = 0; w < p.tu; ++w) {
                     const double *q = part + (size_t)w * p.parts * p.span * 8 + e;
                     const int st = p.span * 8;
@@ -390,7 +427,7 @@ __global__ void __launch_bounds__(FT, 1) fit_rows_kernel(FitRowsParams p)
                 sum[e] = a;
             }
             for (int e = lane; e < k1 - k0; e += 32) {
-                int n = cnt[e];
+                int n = carried ? cnt[e] : 0;
                 for (int w = 0; w < p.tu * p.parts; ++w) n += pcnt[w * p.span + e];
                 cnt[e] = n;
             }
@@ -489,7 +526,7 @@ bool fit_rows_supported(int64_t N, int D, int K)
 }
 
 cudaError_t launch_fit_rows(const float *Y, int64_t N, int D, int K, float *C, int passes, int32_t *labels, double *sums,
-                            int64_t *counts, void *list, int32_t *list_count, float *padded, Control *ctl, cudaStream_t s)
+                            int64_t *counts, void *list, void *list_count, float *padded, Control *ctl, cudaStream_t s)
 {
     FitRowsParams p{};
     int grid;
@@ -502,7 +539,7 @@ cudaError_t launch_fit_rows(const float *Y, int64_t N, int D, int K, float *C, i
     p.sums = sums;
     p.counts = counts;
     p.list = reinterpret_cast<uint2 *>(list);
-    p.list_count = list_count;
+    p.list_count = reinterpret_cast<int4 *>(list_count);
     p.ctl = ctl;
     p.N = N;
     p.D = D;

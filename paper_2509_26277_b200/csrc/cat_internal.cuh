@@ -162,11 +162,11 @@ cudaError_t launch_small_apply(const float *Y, int64_t N, int D, int K, const fl
                                const float *beta, float *out, int32_t *labels, Control *ctl, cudaStream_t s);
 
 // The Lloyd rounds of a fit and its final assignment in one cooperative launch, the rows in shared memory
-// (cat_fit_rows.cu); ctl must have been reset.  passes = rounds + 1.  list: N 8-byte entries, list_count: one
-// int per SM, padded: [K][D rounded up to 4].  Leaves final labels, per-cluster sums and sizes.
+// (cat_fit_rows.cu); ctl must have been reset.  passes = rounds + 1.  list: N 8-byte entries, list_count: 16
+// bytes per CTA (four rows of one at least), padded: [K][D rounded up to 4].  Leaves final labels, per-cluster sums and sizes.
 bool fit_rows_supported(int64_t N, int D, int K);
 cudaError_t launch_fit_rows(const float *Y, int64_t N, int D, int K, float *C, int passes, int32_t *labels, double *sums,
-                            int64_t *counts, void *list, int32_t *list_count, float *padded, Control *ctl, cudaStream_t s);
+                            int64_t *counts, void *list, void *list_count, float *padded, Control *ctl, cudaStream_t s);
 
 // Inference on groups of eight rows held in shared memory, exact decisions included (cat_apply_rows.cu).
 // Resets ctl.  out_bf16: `out` is a [N, D] bf16 matrix; prep: apply_rows_prep_bytes of scratch.

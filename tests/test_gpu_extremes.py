@@ -111,3 +111,31 @@ def test_scores_around_the_lowest_finite_one(n, d, small_kernels):
     labels_match(host(B.cat_assign(dev(Yq), dev(C))), lab, best, second, "labels")
     out, glab = B.cat_apply(dev(Yq), dev(C), dev(g), dev(b), want_labels=True)
     labels_match(host(glab), lab, best, second, "labels")
+
+
+def _visitors(n, d, k):
+    """Ordinary rows, and one huge row for each of the first k centroids.  The huge row of the most populated cluster
+    is drawn to another cluster's centroid in the second round, while all ordinary rows gather in the cluster it leaves."""
+    rng = np.random.default_rng(n + d + k)
+    cen = np.eye(k, d) * 3.0
+    cen[1] = 3.0 * np.array([0.75, np.sqrt(1 - 0.75 ** 2)] + [0.0] * (d - 2))
+    pick = np.where(rng.random(n) < 0.9, 0, rng.integers(0, k, size=n))
+    pick[:k] = np.arange(k)
+    Yq = cen[pick] + 0.05 * rng.normal(size=(n, d))
+    big = np.zeros((k, d))
+    big[:] = 2e14 * cen / 3.0
+    big[1] *= (pick == 1).sum() + 1                          # its cluster's mean is about as long as big[0]
+    Yq = np.concatenate([Yq, big]).astype(np.float32)
+    return Yq
+
+
+@pytest.mark.parametrize("n,d,k", [(1000, 64, 8), (3000, 32, 16), (600, 128, 8)])
+def test_sums_survive_the_visit_of_a_huge_row(n, d, k):
+    Yq = _visitors(n, d, k)
+    ora = O.fit(Yq, Yq, k, 2)
+    assert ora.centroids[0].max() < 10
+    C, G, Bt, lab = B.cat_fit(dev(Yq), dev(Yq), k, 2)
+    assert np.array_equal(host(lab), ora.labels)
+    scale = np.abs(ora.centroids).max(axis=1, keepdims=True)
+    # both are means in fp64, rounded once to fp32
+    close(host(C) / scale, ora.centroids / scale, "centroids", abs_tol=2.0 ** -23, rel_tol=0.0)
