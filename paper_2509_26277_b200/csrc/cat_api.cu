@@ -164,23 +164,35 @@ static bool use_small_apply(int64_t N, int D, int K)
     return (g_small_kernels.load(std::memory_order_relaxed) & 1) && use_tensor_path(N, D, K) && small_apply_supported(N, D, K);
 }
 
-// The kernel that keeps rows in shared memory, where it is the faster one.
-//   K from a quarter of the tensor-core threshold on: the alternative there is the fp32 pipes (50 000 x 1000,
-//   K = 2: 107 us against 270).
-//   Large K * D: its contraction runs on mma.sync with little reuse of the centroids, so on data whose clusters
-//   are far apart the 64-row-tile kernel is ahead (131 072 rows of a mixture: D = 512, K = 64 178 us against 170,
-//   D = 768, K = 48 239 against 212, D = 1000, K = 32 264 against 262).  The other way round where that kernel does
-//   not go (D % 8 != 0), for batches that leave its tiles idle, and for rows above 1024 columns, whose exact pass
-//   outside costs more than anything (60 000 x 2048 logits, K = 24: 415 us against 1219).
+// The kernel that keeps rows in shared memory, where it is the faster one: K from a quarter of the tensor-core
+// threshold on (the alternative there is the fp32 pipes: 50 000 x 1000, K = 2: 107 us against 270).
+//
+// Which one is faster depends on the data more than on the shape.  On logits, whose rows the other kernels' scores often
+// leave undecided, this one gains because it settles them from shared memory; on clusters far apart nothing is left to
+// settle, and its contraction (mma.sync, the centroids read once per eight rows) loses as K * D grows.  The lines
+// lie where the two about balance, so each side of a line loses on one kind of data (us for 131 072 rows, fp32
+// output, here against the other kernel, logits / mixture):
+//   batches below 4096 rows leave the other kernels' tiles idle (4095 x 1004, K = 128: 62 against 95 / 56 against 54)
+//   D % 4 != 0         the alternative is two more passes over a copy (1001, K = 32: 386 against 616 / 280 against 501)
+//   K > 64             eight groups of 16 centroids however many there are.  Rows of 128 to 256: 240, K = 96 181 against
+//                      268 / 139 against 122; shorter: 96, K = 96 106 against 103 / 76 against 68, with bf16 output 105
+//                      against 107 / 73 against 81; longer: 504, K = 65 438 against 497 / 403 against 177, 1004, K = 128 886 against
+//                      1351 / 802 against 293
+//   K * D > 32768      with D % 8 == 0 the 64-row tiles: 512, K = 64 204 against 408 / 178 against 169, 1000, K = 32 330 against 536 / 263
+//                      against 260; beyond, 60 000 x 1504, K = 64: 412 against 485 / 335 against 209
+//   rows above 1536 columns, whose exact pass outside takes one row at a time (60 000 x 2048, K = 64: 514 against 2869 / 435
+//                      against 264; K = 128 878 against 5186 / 760 against 270)
 //   Short rows with many centroids: a group of eight rows is too little work (128 406 x 48, K = 106: 83 against 75).
-static bool use_apply_rows(int64_t N, int D, int K)
+static bool use_apply_rows(int64_t N, int D, int K, bool bf16)
 {
     const int min_k = g_tc_min_k.load(std::memory_order_relaxed);
     if (!(g_small_kernels.load(std::memory_order_relaxed) & 1) || get_apply_column_split() != 0 ||
         K < min_k / 4 + (min_k % 4 != 0) || !apply_rows_supported(N, D, K))
         return false;
     if (D < 64) return K <= 64;
-    return (int64_t)K * D <= 32768 || D % 8 != 0 || N < 4096 || D > 1024;
+    if (N < 4096 || D % 4 != 0 || D > 1536) return true;
+    if (K > 64) return D <= 256 && (bf16 ? D % 8 == 0 || D <= 128 : D >= 128);
+    return (int64_t)K * D <= 32768 || D % 8 != 0;
 }
 
 // norms -> fast assignment (tensor cores for large K, fp32 pipes otherwise) -> exact pass for
@@ -198,7 +210,7 @@ static cat_status_t run_assign(const float *Y, int64_t N, int D, int K, const fl
         CAT_CUDA(launch_small_apply(Y, N, D, K, C, gamma, beta, out, labels, w.ctl, s));
         return CAT_OK;
     }
-    if (out && labels && top_level && !fast && use_apply_rows(N, D, K)) {
+    if (out && labels && top_level && !fast && use_apply_rows(N, D, K, false)) {
         // rows kept in shared memory from the first read to the corrected store (behind the kernel above
         // where both apply: 200 704 x 64, K = 64 takes 69 us here and 43 there)
         CAT_CUDA(launch_apply_rows(Y, N, D, K, C, gamma, beta, out, false, labels, w.ctl, w.prep, s));
@@ -374,7 +386,7 @@ cat_status_t cat_apply_bf16(const float *Yq, int64_t N, int32_t D, int32_t K, co
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     AssignWs w = carve_assign(workspace, N, D, K);
     int32_t *labels = labels_out ? labels_out : w.labels;
-    if (use_apply_rows(N, D, K)) {
+    if (use_apply_rows(N, D, K, true)) {
         CAT_CUDA(launch_apply_rows(Yq, N, D, K, centroids, gamma, beta, Y_out_bf16, true, labels, w.ctl, w.prep, s));
         return CAT_OK;
     }
