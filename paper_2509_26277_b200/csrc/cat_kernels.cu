@@ -712,7 +712,9 @@ __device__ __forceinline__ void refine_body(const float *__restrict__ Y, int64_t
     }
 }
 
-template <bool AFFINE>
+// GROUPED: rows of at most RG_MAX_D columns.  (A kernel of its own for longer ones: the grouped form's 128 registers
+// a thread would leave two CTAs per SM where the other fits five, and its scan lives on loads in flight.)
+template <bool AFFINE, bool GROUPED>
 __global__ void __launch_bounds__(R_THREADS) refine_kernel(const float *__restrict__ Y, int64_t N,
                                                            int D, int K, const float *__restrict__ C,
                                                            int32_t *labels,
@@ -721,7 +723,7 @@ __global__ void __launch_bounds__(R_THREADS) refine_kernel(const float *__restri
                                                            const float *beta, float *out)
 {
     extern __shared__ __align__(16) float refine_rows_f32[];
-    if (D <= RG_MAX_D) refine_body_grouped<AFFINE>(Y, N, D, K, C, labels, refine_rows, ctl, gamma, beta, out, refine_rows_f32);
+    if constexpr (GROUPED) refine_body_grouped<AFFINE>(Y, N, D, K, C, labels, refine_rows, ctl, gamma, beta, out, refine_rows_f32);
     else refine_body<AFFINE>(Y, N, D, K, C, labels, refine_rows, ctl, gamma, beta, out);
 }
 
@@ -729,8 +731,9 @@ __global__ void __launch_bounds__(R_THREADS) refine_kernel(const float *__restri
 static size_t refine_smem_bytes(int D, int K) { return D <= RG_MAX_D ? (size_t)RG * ((D + 3) & ~3) * 4 + (size_t)RG * K * 4 : 0; }
 
 template <typename Kern>
-static cudaError_t refine_config(Kern kern)   // (the same value whatever the shape: several threads may be launching)
+static cudaError_t refine_config(Kern kern, size_t smem)   // (the same value whatever the shape: several threads may be launching)
 {
+    if (smem <= 48 * 1024) return cudaSuccess;   // (what any kernel may have; the call costs the host a microsecond)
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RG_MAX_SMEM);
 }
 
@@ -738,15 +741,14 @@ cudaError_t launch_refine(const float *Y, int64_t N, int D, int K, const float *
                           int32_t *labels, const int32_t *refine_rows, Control *ctl,
                           const float *gamma, const float *beta, float *out, cudaStream_t s)
 {
-    int blocks = (int)(N < 1184 ? N : 1184);
-    cudaError_t e = out ? refine_config(refine_kernel<true>) : refine_config(refine_kernel<false>);
+    const bool grouped = D <= RG_MAX_D;
+    const int blocks = (int)(N < 1184 ? N : 1184);
+    const auto kern = out ? (grouped ? refine_kernel<true, true> : refine_kernel<true, false>)
+                          : (grouped ? refine_kernel<false, true> : refine_kernel<false, false>);
+    const size_t smem = refine_smem_bytes(D, K);
+    const cudaError_t e = refine_config(kern, smem);
     if (e != cudaSuccess) return e;
-    if (out)
-        refine_kernel<true><<<blocks, R_THREADS, refine_smem_bytes(D, K), s>>>(Y, N, D, K, C, labels, refine_rows, ctl,
-                                                         gamma, beta, out);
-    else
-        refine_kernel<false><<<blocks, R_THREADS, refine_smem_bytes(D, K), s>>>(Y, N, D, K, C, labels, refine_rows, ctl,
-                                                          gamma, beta, out);
+    kern<<<blocks, R_THREADS, smem, s>>>(Y, N, D, K, C, labels, refine_rows, ctl, gamma, beta, out);
     count_launch();
     return cudaGetLastError();
 }
@@ -900,7 +902,7 @@ __device__ __forceinline__ void refine_candidates_body(
 // Both exact passes in one launch: the rows queued with their candidates (a warp each), then the
 // rows queued for a scan of all K (a CTA each).  A row is in one queue only.
 static_assert(RC_THREADS == R_THREADS, "the fused exact pass runs both bodies with one block size");
-template <bool AFFINE>
+template <bool AFFINE, bool GROUPED>
 __global__ void __launch_bounds__(R_THREADS) refine_both_kernel(
     const float *__restrict__ Y, int64_t N, int D, int K, const float *__restrict__ C, int32_t *labels,
     const int32_t *__restrict__ cand_rows, const uint64_t *__restrict__ cand_list,
@@ -910,7 +912,7 @@ __global__ void __launch_bounds__(R_THREADS) refine_both_kernel(
     refine_candidates_body<AFFINE>(Y, N, D, K, C, labels, cand_rows, cand_list, ctl, gamma, beta, out, AFFINE);
     __syncthreads();   // (block 0's thread 0 updates the counters in both bodies, in this order)
     extern __shared__ __align__(16) float refine_rows_f32[];
-    if (D <= RG_MAX_D) refine_body_grouped<AFFINE>(Y, N, D, K, C, labels, refine_rows, ctl, gamma, beta, out, refine_rows_f32);
+    if constexpr (GROUPED) refine_body_grouped<AFFINE>(Y, N, D, K, C, labels, refine_rows, ctl, gamma, beta, out, refine_rows_f32);
     else refine_body<AFFINE>(Y, N, D, K, C, labels, refine_rows, ctl, gamma, beta, out);
 }
 
@@ -919,15 +921,16 @@ cudaError_t launch_refine_both(const float *Y, int64_t N, int D, int K, const fl
                                Control *ctl, const float *gamma, const float *beta, float *out, cudaStream_t s)
 {
     int64_t want = (N + (RC_THREADS / 32) - 1) / (RC_THREADS / 32);
-    int blocks = (int)(want < 1184 ? want : 1184);
-    cudaError_t e = out ? refine_config(refine_both_kernel<true>) : refine_config(refine_both_kernel<false>);
+    const bool grouped = D <= RG_MAX_D;
+    const int blocks = (int)(want < 1184 ? want : 1184);
+    const auto kern = out ? (grouped ? refine_both_kernel<true, true> : refine_both_kernel<true, false>)
+                          : (grouped ? refine_both_kernel<false, true> : refine_both_kernel<false, false>);
+    const size_t smem = refine_smem_bytes(D, K);
+    cudaError_t e = refine_config(kern, smem);
     if (e != cudaSuccess) return e;
-    if (out)
-        launch_pdl(refine_both_kernel<true>, dim3(blocks), dim3(R_THREADS), refine_smem_bytes(D, K), s, Y, N, D, K, C, labels,
-                   cand_rows, cand_list, refine_rows, ctl, gamma, beta, out);
-    else
-        launch_pdl(refine_both_kernel<false>, dim3(blocks), dim3(R_THREADS), refine_smem_bytes(D, K), s, Y, N, D, K, C, labels,
-                   cand_rows, cand_list, refine_rows, ctl, gamma, beta, out);
+    e = launch_pdl(kern, dim3(blocks), dim3(R_THREADS), smem, s, Y, N, D, K, C, labels, cand_rows, cand_list, refine_rows, ctl, gamma, beta,
+                   out);
+    if (e != cudaSuccess) return e;
     count_launch();
     return cudaGetLastError();
 }
