@@ -303,7 +303,7 @@ static cat_status_t run_delta_update(const float *Yq, const int32_t *labels, con
                                w.seg_start, w.order, s));
     CAT_CUDA(launch_segment_sums(0, Yq, nullptr, w.order, w.cluster_start, w.seg_start, nullptr, nullptr, D,
                                  2 * K, g, w.segpart, s));
-    CAT_CUDA(launch_centroid_update(w.segpart, w.seg_start, w.counts, D, K, w.sumQ, C, w.a.cnorm, w.hscale,
+    CAT_CUDA(launch_centroid_update(w.segpart, w.seg_start, w.counts, D, K, g.max_segs, w.sumQ, C, w.a.cnorm, w.hscale,
                                     half ? w.ch : nullptr, half ? w.a.mean : nullptr, w.a.cerr, w.norm_part, w.arrivals, w.a.ctl, s));
     return CAT_OK;
 }
@@ -566,7 +566,7 @@ cat_status_t cat_fit_from(const float *Yq, const float *Yfp, int64_t N, int32_t 
         SegGeom g = seg_geometry(N, D, K);
         CAT_CUDA(launch_segment_sums(3, Yq, Yfp, w.order, w.cluster_start, w.seg_start, meanQ, nullptr, D, K, g,
                                      w.segpart, s));
-        CAT_CUDA(launch_segment_combine3(w.segpart, w.seg_start, D, K, w.var, w.cov, w.sumF, s));
+        CAT_CUDA(launch_segment_combine3(w.segpart, w.seg_start, D, K, g.max_segs, w.var, w.cov, w.sumF, s));
     }
     CAT_CUDA(launch_solve(w.sumQ, w.sumF, w.var, w.cov, w.counts, D, K, gamma_out, beta_out, s));
     if (diag) CAT_CUDA(launch_fit_diag(w.a.ctl, w.counts, K, diag, s));

@@ -259,7 +259,7 @@ cudaError_t launch_segment_combine(const double *part, const int32_t *seg_start,
                                    int K, bool delta, double *out0, double *out1, float *C, cudaStream_t s);
 
 // Sums of the three planes of mode 3 per cluster: out0 = sum (q-muQ)^2, out1 = sum (q-muQ)(f-muQ), out2 = sum f.
-cudaError_t launch_segment_combine3(const double *part, const int32_t *seg_start, int D, int K, double *out0,
+cudaError_t launch_segment_combine3(const double *part, const int32_t *seg_start, int D, int K, int max_segs, double *out0,
                                     double *out1, double *out2, cudaStream_t s);
 
 // Delta-mode centroid update fused with what the next assignment needs: running sums, centroids,
@@ -267,7 +267,7 @@ cudaError_t launch_segment_combine3(const double *part, const int32_t *seg_start
 // centroids less `mean` if that is given -- and the reset of the exact-pass queues.  norm_part: scratch;
 // arrivals: [K], zero before the first call (left at zero).
 cudaError_t launch_centroid_update(const double *part, const int32_t *seg_start, const int64_t *counts, int D,
-                                   int K, double *sums, float *C, float *cnorm, const float *scale, void *Ch,
+                                   int K, int max_segs, double *sums, float *C, float *cnorm, const float *scale, void *Ch,
                                    const float *mean, float *cerr, void *norm_part, uint32_t *arrivals, Control *ctl,
                                    cudaStream_t s);
 size_t centroid_update_scratch_bytes(int D, int K);

@@ -400,45 +400,70 @@ __global__ void segment_combine_kernel(const double *__restrict__ part, const in
     }
 }
 
-// The kernels that add up a cluster's segments: a CTA takes `cols` columns of a cluster, 512 / cols threads
-// a column, thread g of them the segments first + g, first + g + 512 / cols, ..., whose sums are then added
-// in that order.  (One thread per column, the earlier form, is a chain of loads as long as the cluster has
-// segments: with K = 2 and 100 000 rows 224 us for the three planes and 19 us a Lloyd round.)
+// The kernels that add up a cluster's segments: a CTA takes `cols` columns of a cluster, G = threads / cols threads
+// a column, thread g of them the segments first + g, first + g + G, ..., whose sums are then added
+// in that order.  (One thread per column is a chain of loads as long as the cluster has segments: with K = 2 and
+// 100 000 rows 224 us for the three planes and 19 us a Lloyd round.  More threads than segments are a longer
+// exchange for nothing: 8192 x 64, K = 200 takes 8.6 us a round with 16 of them, 6.3 with two and whole rows.)
 constexpr int COMB_THREADS = 512;
 
-__device__ __forceinline__ double sum_segments(const double *__restrict__ p, int s0, int s1, int step, size_t stride)
+// P planes of a segment lie `plane` apart; four segments' loads are in flight together
+template <int P>
+__device__ __forceinline__ void sum_segments(const double *__restrict__ p, int s0, int s1, int step, size_t stride, size_t plane,
+                                             double (&out)[P])
 {
-    double a[4] = {0.0, 0.0, 0.0, 0.0};
-    int s = s0;
-    for (; s + 3 * step < s1; s += 4 * step) {
-        double v[4];
+    double a[P][4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = __ldg(p + (size_t)(s + u * step) * stride);
+    for (int q = 0; q < P; ++q)
 #pragma unroll
-        for (int u = 0; u < 4; ++u) a[u] += v[u];
+        for (int u = 0; u < 4; ++u) a[q][u] = 0.0;
+    for (int s = s0; s < s1; s += 4 * step) {
+        double v[P][4];
+#pragma unroll
+        for (int q = 0; q < P; ++q)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[q][u] = s + u * step < s1 ? __ldg(p + (size_t)(s + u * step) * stride + q * plane) : 0.0;
+#pragma unroll
+        for (int q = 0; q < P; ++q)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) a[q][u] += v[q][u];
     }
-    for (; s < s1; s += step) a[0] += __ldg(p + (size_t)s * stride);
-    return (a[0] + a[1]) + (a[2] + a[3]);
+#pragma unroll
+    for (int q = 0; q < P; ++q) out[q] = (a[q][0] + a[q][1]) + (a[q][2] + a[q][3]);
 }
 
 // every thread of a column gets the sum of its threads' values; red: [COMB_THREADS]
 __device__ __forceinline__ double sum_column(double v, int cols, double *red)
 {
-    if (cols == COMB_THREADS) return v;
+    if (cols == (int)blockDim.x) return v;
     __syncthreads();
     red[threadIdx.x] = v;
     __syncthreads();
     double t = 0.0;
-    for (int g = threadIdx.x & (cols - 1); g < COMB_THREADS; g += cols) t += red[g];
+    for (int g = threadIdx.x & (cols - 1); g < (int)blockDim.x; g += cols) t += red[g];
     return t;
 }
 
-// columns per CTA: as many CTAs as the device holds a few times over, no more
-int comb_cols(int D, int K)
+// Columns and threads of a CTA: as many CTAs as the device holds a few times over, no more; as many threads a column as
+// a cluster has segments on average; whole rows where they fit then.
+struct CombGeom {
+    int cols, threads;
+};
+CombGeom comb_geometry(int D, int K, int max_segs)
 {
-    int cols = 32;
+    int cols = 32, G = 1;
     while (cols < COMB_THREADS && (int64_t)K * ((D + cols - 1) / cols) > 4 * 148) cols *= 2;
-    return cols;
+    while (cols * G < COMB_THREADS && 2 * G * (int64_t)K <= max_segs) G *= 2;
+    int whole = 32;
+    while (whole < D && whole < COMB_THREADS) whole *= 2;
+    if (whole >= D && whole > cols) {
+        const int Gw = G < COMB_THREADS / whole ? G : COMB_THREADS / whole;
+        if (max_segs <= (int64_t)K * Gw * 8) {   // (two batches of loads a thread at most)
+            cols = whole;
+            G = Gw;
+        }
+    }
+    return {cols, cols * G};
 }
 
 // Three-plane partials (MODE 3) added up per cluster.
@@ -449,13 +474,11 @@ __global__ void __launch_bounds__(COMB_THREADS) segment_combine3_kernel(const do
 {
     pdl_enter();
     __shared__ double red[COMB_THREADS];
-    const int k = blockIdx.x, g = threadIdx.x / cols, G = COMB_THREADS / cols;
+    const int k = blockIdx.x, g = threadIdx.x / cols, G = (int)blockDim.x / cols;
     const int j = (int)blockIdx.y * cols + (threadIdx.x & (cols - 1));
     const int s0 = seg_start[k], s1 = seg_start[k + 1];
     double v[3] = {0.0, 0.0, 0.0};
-    if (j < D)
-#pragma unroll
-        for (int q = 0; q < 3; ++q) v[q] = sum_segments(part + (size_t)q * D + j, s0 + g, s1, G, (size_t)3 * D);
+    if (j < D) sum_segments<3>(part + j, s0 + g, s1, G, (size_t)3 * D, (size_t)D, v);
 #pragma unroll
     for (int q = 0; q < 3; ++q) v[q] = sum_column(v[q], cols, red);
     if (g == 0 && j < D) {
@@ -470,8 +493,9 @@ __global__ void __launch_bounds__(COMB_THREADS) segment_combine3_kernel(const do
 // n_k > 0; and for the next assignment the squared norm of c_k (fp64, rounded up), optionally the fp16 copy
 // fp16(c_k * scale[0]) with the norm of its rounding error -- both of c_k less `mean` if that is given -- and the
 // reset of the exact-pass queues.  The CTAs of a cluster leave their parts of the two norms in `norm_part`; the last
-// one to arrive (`arrivals`, which wraps back to zero) adds them up in column order.
-__global__ void __launch_bounds__(COMB_THREADS) centroid_update_kernel(const double *__restrict__ part,
+// one to arrive (`arrivals`, which wraps back to zero) adds them up, in an order that does not depend on who came when.
+// (32 registers a thread: four CTAs per SM, so that the 592 CTAs of the geometry above are one wave)
+__global__ void __launch_bounds__(COMB_THREADS, 4) centroid_update_kernel(const double *__restrict__ part,
                                                               const int32_t *__restrict__ seg_start,
                                                               const int64_t *__restrict__ counts, int D, int K, int cols,
                                                               double *__restrict__ sums, float *__restrict__ C,
@@ -484,7 +508,7 @@ __global__ void __launch_bounds__(COMB_THREADS) centroid_update_kernel(const dou
     __shared__ double red[COMB_THREADS];
     __shared__ float red_err[COMB_THREADS / 32];
     __shared__ int s_last;
-    const int k = blockIdx.x, cb = blockIdx.y, g = threadIdx.x / cols, G = COMB_THREADS / cols;
+    const int k = blockIdx.x, cb = blockIdx.y, g = threadIdx.x / cols, G = (int)blockDim.x / cols;
     if (k == 0 && cb == 0 && threadIdx.x == 0) {
         ctl->refine_count = 0;
         ctl->cand_count = 0;
@@ -492,10 +516,12 @@ __global__ void __launch_bounds__(COMB_THREADS) centroid_update_kernel(const dou
     const int j = cb * cols + (threadIdx.x & (cols - 1));
     const int64_t n = counts[k];
     const float sc = Ch ? scale[0] : 1.f;
-    double d = 0.0;
-    if (j < D)
-        d = sum_segments(part + j, seg_start[k] + g, seg_start[k + 1], G, (size_t)2 * D) -
-            sum_segments(part + j, seg_start[K + k] + g, seg_start[K + k + 1], G, (size_t)2 * D);
+    double in[1] = {0.0}, gone[1] = {0.0};
+    if (j < D) {
+        sum_segments<1>(part + j, seg_start[k] + g, seg_start[k + 1], G, (size_t)2 * D, 0, in);
+        sum_segments<1>(part + j, seg_start[K + k] + g, seg_start[K + k + 1], G, (size_t)2 * D, 0, gone);
+    }
+    double d = in[0] - gone[0];
     d = sum_column(d, cols, red);
     double nrm = 0.0;
     float left2 = 0.f;
@@ -534,19 +560,31 @@ __global__ void __launch_bounds__(COMB_THREADS) centroid_update_kernel(const dou
             t += red[w];
             l += (double)red_err[w];
         }
-        norm_part[(size_t)k * gridDim.y + cb] = make_double2(t, l);
-        __threadfence();
-        s_last = atomicInc(arrivals + k, gridDim.y - 1) == gridDim.y - 1;
+        if (gridDim.y == 1) {
+            cnorm[k] = __double2float_ru(t);
+            if (Ch) cerr[k] = sqrtf((float)l) / sc * 1.001f;
+        } else {
+            norm_part[(size_t)k * gridDim.y + cb] = make_double2(t, l);
+            __threadfence();
+            s_last = atomicInc(arrivals + k, gridDim.y - 1) == gridDim.y - 1;
+        }
     }
+    if (gridDim.y == 1) return;
     __syncthreads();
-    if (s_last && threadIdx.x == 0) {
+    if (s_last && threadIdx.x < 32) {
         __threadfence();
         double t = 0.0, l = 0.0;
-        for (int q = 0; q < (int)gridDim.y; ++q) {
+        for (int q = threadIdx.x; q < (int)gridDim.y; q += 32) {
             const double2 v = __ldcg(norm_part + (size_t)k * gridDim.y + q);
             t += v.x;
             l += v.y;
         }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            t += __shfl_xor_sync(0xffffffffu, t, o);
+            l += __shfl_xor_sync(0xffffffffu, l, o);
+        }
+        if (threadIdx.x != 0) return;
         cnorm[k] = __double2float_ru(t);
         if (Ch) cerr[k] = sqrtf((float)l) / sc * 1.001f;
     }
@@ -653,11 +691,12 @@ cudaError_t launch_segment_combine(const double *part, const int32_t *seg_start,
     return cudaGetLastError();
 }
 
-cudaError_t launch_segment_combine3(const double *part, const int32_t *seg_start, int D, int K, double *out0,
+cudaError_t launch_segment_combine3(const double *part, const int32_t *seg_start, int D, int K, int max_segs, double *out0,
                                     double *out1, double *out2, cudaStream_t s)
 {
-    const int cols = comb_cols(D, K);
-    const cudaError_t e = launch_pdl(segment_combine3_kernel, dim3((unsigned)K, (unsigned)((D + cols - 1) / cols)), dim3(COMB_THREADS), 0, s,
+    const CombGeom cg = comb_geometry(D, K, max_segs);
+    const int cols = cg.cols;
+    const cudaError_t e = launch_pdl(segment_combine3_kernel, dim3((unsigned)K, (unsigned)((D + cols - 1) / cols)), dim3((unsigned)cg.threads), 0, s,
                                      part, seg_start, D, cols, out0, out1, out2);
     count_launch();
     return e;
@@ -666,12 +705,13 @@ cudaError_t launch_segment_combine3(const double *part, const int32_t *seg_start
 size_t centroid_update_scratch_bytes(int D, int K) { return (size_t)K * ((D + 31) / 32) * sizeof(double2); }
 
 cudaError_t launch_centroid_update(const double *part, const int32_t *seg_start, const int64_t *counts, int D,
-                                   int K, double *sums, float *C, float *cnorm, const float *scale, void *Ch,
+                                   int K, int max_segs, double *sums, float *C, float *cnorm, const float *scale, void *Ch,
                                    const float *mean, float *cerr, void *norm_part, uint32_t *arrivals, Control *ctl,
                                    cudaStream_t s)
 {
-    const int cols = comb_cols(D, K);
-    const cudaError_t e = launch_pdl(centroid_update_kernel, dim3((unsigned)K, (unsigned)((D + cols - 1) / cols)), dim3(COMB_THREADS), 0, s,
+    const CombGeom cg = comb_geometry(D, K, max_segs);
+    const int cols = cg.cols;
+    const cudaError_t e = launch_pdl(centroid_update_kernel, dim3((unsigned)K, (unsigned)((D + cols - 1) / cols)), dim3((unsigned)cg.threads), 0, s,
                                      part, seg_start, counts, D, K, cols, sums, C, cnorm, scale, reinterpret_cast<__half *>(Ch), mean, cerr,
                                      reinterpret_cast<double2 *>(norm_part), arrivals, ctl);
     count_launch();
