@@ -468,8 +468,13 @@ bool fit_rows_plan(int64_t N, int D, int K, FitRowsParams *p, int *grid, size_t 
     // update a latency per changed row.  25 rounds against the general rounds: 1024 x 1000, K = 16 0.24 ms and 0.96,
     // 4096 x 1000, K = 64 1.15 and 1.76, 8192 x 50, K = 32 0.57 and 0.82, 3000 x 300, K = 256 0.57 and 2.0; past the lines
     // drawn here 7000 x 400, K = 90 1.47 and 1.40, 8000 x 16, K = 256 1.50 and 0.88, 20 000 x 50, K = 64 1.25 and 1.19.
+    // From 256 columns on the line comes down with the rows a CTA holds (logits, whose labels change in every round; well
+    // separated clusters reach their fixed point early and gain throughout): up to 32 rows 4500 x 768, K = 48 1.01 and 1.08;
+    // up to 48 6144 x 256, K = 96 0.86 and 0.88, past it K = 128 1.09 and 0.89; above 8192 x 256, K = 32 0.80 and 0.86, past it
+    // K = 64 1.08 and 0.93.
     if (D < 4 || K < 2 || K > CAT_MAX_K || N < K || N > 8192) return false;
-    if (N * (int64_t)K * (D < 256 ? 256 : D) > (N > 6144 ? (int64_t)1 << 27 : (int64_t)1 << 28)) return false;
+    const int shift = D < 256 ? N > 6144 : (N > 148 * 48 ? 2 : N > 148 * 32);
+    if (N * (int64_t)K * (D < 256 ? 256 : D) > ((int64_t)1 << 28) >> shift) return false;
     const int sms = 148;
     int64_t rpc = (N + sms - 1) / sms;
     if (rpc < 4) rpc = 4;
