@@ -440,6 +440,15 @@ int32_t cat_tensor_path_available(void);
 void cat_set_apply_column_split(int32_t cs);
 int32_t cat_get_apply_column_split(void);
 
+/* Name of the kernel that decides the labels in a call of this shape under the current settings -- in a fit of
+ * all rounds, with the default start and without diag -- for reports and tests; "" where the shape is out of range or
+ * there is nothing to decide (K = 1). */
+#define CAT_CALL_APPLY 0
+#define CAT_CALL_APPLY_BF16 1
+#define CAT_CALL_ASSIGN 2
+#define CAT_CALL_FIT 3
+const char *cat_kernel_for(int32_t call, int64_t N, int32_t D, int32_t K);
+
 const char *cat_status_string(cat_status_t status);
 int cat_last_cuda_error(void);           /* cudaError_t of the last failing runtime call on this thread */
 const char *cat_version(void);

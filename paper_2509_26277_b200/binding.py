@@ -44,7 +44,7 @@ EXPORTS = [
     "cat_selftest_wait_timeout",
     "cat_set_tensor_core_min_k", "cat_get_tensor_core_min_k", "cat_tensor_path_available",
     "cat_set_small_problem_kernels", "cat_get_small_problem_kernels",
-    "cat_set_apply_column_split", "cat_get_apply_column_split", "cat_status_string",
+    "cat_set_apply_column_split", "cat_get_apply_column_split", "cat_kernel_for", "cat_status_string",
     "cat_last_cuda_error", "cat_version", "cat_kernel_launches",
 ]
 
@@ -141,6 +141,8 @@ def lib():
     L.cat_set_apply_column_split.argtypes = [i32]
     L.cat_set_apply_column_split.restype = None
     L.cat_get_apply_column_split.restype = i32
+    L.cat_kernel_for.argtypes = [i32, i64, i32, i32]
+    L.cat_kernel_for.restype = ctypes.c_char_p
     L.cat_status_string.argtypes = [ctypes.c_int]
     L.cat_status_string.restype = ctypes.c_char_p
     L.cat_last_cuda_error.restype = ctypes.c_int
@@ -584,6 +586,11 @@ def cat_set_apply_column_split(cs: int) -> None:
 
 def cat_get_apply_column_split() -> int:
     return int(lib().cat_get_apply_column_split())
+
+
+def cat_kernel_for(call: str, N: int, D: int, K: int) -> str:
+    """Name of the kernel that decides the labels: call is "apply", "apply_bf16", "assign" or "fit" (see cat.h)."""
+    return lib().cat_kernel_for(["apply", "apply_bf16", "assign", "fit"].index(call), N, D, K).decode()
 
 
 def cat_version() -> str:

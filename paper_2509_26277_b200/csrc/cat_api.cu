@@ -763,6 +763,35 @@ int32_t cat_get_small_problem_kernels(void) { return g_small_kernels.load(std::m
 
 int32_t cat_tensor_path_available(void) { return tc_supported(1, 4, 1) ? 1 : 0; }
 
+// (the order of run_assign, cat_apply_bf16 and cat_fit_from)
+const char *cat_kernel_for(int32_t call, int64_t N, int32_t D, int32_t K)
+{
+    if (check_shape(N, D, K, call == CAT_CALL_FIT) != CAT_OK) return "";
+    const bool tc = use_tensor_path(N, D, K);
+    switch (call) {
+    case CAT_CALL_APPLY:
+        if (use_small_apply(N, D, K)) return "small_kernel";
+        if (use_apply_rows(N, D, K, false)) return "apply_rows_kernel";
+        break;
+    case CAT_CALL_APPLY_BF16:
+        if (use_apply_rows(N, D, K, true)) return "apply_rows_kernel";
+        break;
+    case CAT_CALL_FIT:
+        if (use_fit_rows(N, D, K)) return "fit_rows_kernel";
+        if (use_small_fit(N, D, K)) return "small_kernel";
+        break;
+    case CAT_CALL_ASSIGN: break;
+    default: return "";
+    }
+    if (K == 1) return "";
+    if (call == CAT_CALL_FIT) return use_half_path(N, D, K) ? "assign_tc_kernel, fp16 copies" : tc ? "assign_tc_kernel" : "assign_kernel";
+    if (call == CAT_CALL_APPLY_BF16 ? tc && apply_h64_supported(N, D, K) : call == CAT_CALL_APPLY && tc && choose_apply_form(N, D, K) == 64)
+        return "apply_h64_kernel";
+    if (D % 4 != 0 && use_half_path(N, D, K)) return "assign_tc_kernel, fp16 copies";
+    if (!tc) return "assign_kernel";
+    return call == CAT_CALL_APPLY && choose_apply_form(N, D, K) > 1 ? "apply_split_kernel" : "assign_tc_kernel";
+}
+
 void cat_set_apply_column_split(int32_t cs) { set_apply_column_split((int)cs); }
 
 int32_t cat_get_apply_column_split(void) { return (int32_t)get_apply_column_split(); }

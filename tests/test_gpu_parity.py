@@ -34,6 +34,16 @@ def contraction_path(request):
     B.cat_set_tensor_core_min_k(old)
 
 
+@pytest.fixture(params=[3, 0], ids=["small kernels", "general path"])
+def small_kernels(request):
+    """With the kernels that take small sets and keep rows in shared memory, and without: the shapes of a test are small
+    enough for the oracle, so only the second form reaches the kernels that large inputs take."""
+    old = B.cat_get_small_problem_kernels()
+    B.cat_set_small_problem_kernels(request.param)
+    yield request.param
+    B.cat_set_small_problem_kernels(old)
+
+
 def dev(a):
     return torch.as_tensor(np.ascontiguousarray(a)).cuda()
 
@@ -161,7 +171,7 @@ def _rand(seed, n, d):
                                    (2000, 20, 1), (900, 1024, 256), (700, 12, 512), (600, 1540, 48), (300, 1100, 6),
                                    # N not a multiple of the rows a warp shares when a row takes fewer than 32 lanes
                                    (1001, 64, 65), (67, 8, 64), (515, 32, 40), (333, 120, 33)])
-def test_ragged_shapes_apply_and_fit(n, d, k):
+def test_ragged_shapes_apply_and_fit(n, d, k, small_kernels):
     Yq = _rand(n * 7 + d, n, d)
     Yfp = (Yq * 1.1 + 0.1 * _rand(n + d + 1, n, d)).astype(np.float32)
     C = _rand(k, k, d)
@@ -187,13 +197,15 @@ def test_ragged_shapes_apply_and_fit(n, d, k):
 @pytest.mark.parametrize("n,d,k,scale", [(600, 2048, 40, 1.0),      # rows longer than one streaming step
                                          (300, 120, 33, 1.0),       # short rows, 30 float4 (not a power of two)
                                          (700, 1032, 64, 1.0),      # last fp16 slab partly outside the matrix
-                                         (520, 1028, 48, 1.0),      # D % 8 != 0: the fit stays on TF32 operands
+                                         (520, 1028, 48, 1.0),      # D % 8 != 0: padded rows of the fp16 copy
                                          (3000, 256, 128, 1.0),
                                          (1500, 512, 256, 3.0e4),   # magnitudes far above the fp16 range
                                          (1500, 512, 256, 2.0e-7)])  # ... and far below it
-def test_tensor_paths_shapes_and_scales(n, d, k, scale):
+def test_tensor_paths_shapes_and_scales(n, d, k, scale, small_kernels, contraction_path):
     """Shapes and magnitudes that steer the tensor-core kernels through their variants (fp16 copy of
     the rows with its power-of-two scale, TF32, short and long rows).  Tolerances scale with the data."""
+    if small_kernels == 0 and contraction_path == "tensor":
+        assert B.cat_kernel_for("fit", n, d, k) == "assign_tc_kernel, fp16 copies"
     Yq = (_rand(n + d, n, d) * scale).astype(np.float32)
     Yfp = (Yq * 0.9 + 0.05 * scale * _rand(n + d + 1, n, d)).astype(np.float32)
     Cg, Gg, Bg, lg = B.cat_fit(dev(Yq), dev(Yfp), k, 4)
@@ -339,13 +351,15 @@ def test_apply_column_split_falls_back_where_the_shape_does_not_allow_it():
     assert torch.equal(out, ref)
 
 
-@pytest.mark.parametrize("d,k", [(256, 32), (1024, 64), (64, 40), (120, 33), (68, 40)])
-def test_rows_between_two_centroids_are_decided_like_the_oracle(d, k):
+@pytest.mark.parametrize("offset", [0.0, 300.0])
+@pytest.mark.parametrize("d,k", [(256, 32), (1024, 64), (64, 40), (120, 33), (68, 40), (257, 33), (1001, 20)])
+def test_rows_between_two_centroids_are_decided_like_the_oracle(d, k, offset, small_kernels):
     """Rows placed next to the bisector of two centroids, with relative distance gaps from 1e-6 to
     1e-4: all of them are undecidable for the tensor-core scores, and they straddle the margin
-    below which the exact pass leaves its fp32 pre-decision for fp64."""
+    below which the exact pass leaves its fp32 pre-decision for fp64.  With an offset that all rows and centroids
+    have in common, which the fp16 copies take off first: their error bound has to cover that too."""
     rng = np.random.default_rng(d + k)
-    C = rng.normal(size=(k, d)).astype(np.float32)
+    C = (offset + rng.normal(size=(k, d))).astype(np.float32)
     n = 6000
     a = rng.integers(0, k, size=n)
     b = (a + 1 + rng.integers(0, k - 1, size=n)) % k
@@ -367,13 +381,20 @@ def test_rows_between_two_centroids_are_decided_like_the_oracle(d, k):
     assert torch.equal(glab2, glab)
 
 
-def test_fit_fp16_and_tf32_operands_agree():
+def test_fit_fp16_and_tf32_operands_agree(contraction_path):
     """The default start lets cat_fit assign from an fp16 copy of the rows; an explicit start (here the
     same first K rows) keeps TF32 operands.  Labels are decided exactly either way."""
     w, _ = workload("cfg4s")
     Yq, Yfp = dev(w.Yq_fit.numpy()), dev(w.Yfp_fit.numpy())
-    a = B.cat_fit(Yq, Yfp, w.K, 6)
-    b = B.cat_fit(Yq, Yfp, w.K, 6, init_centroids=Yq[:w.K].clone())
+    old = B.cat_get_small_problem_kernels()
+    B.cat_set_small_problem_kernels(0)
+    try:
+        if contraction_path == "tensor":
+            assert B.cat_kernel_for("fit", *Yq.shape, w.K) == "assign_tc_kernel, fp16 copies"
+        a = B.cat_fit(Yq, Yfp, w.K, 6)
+        b = B.cat_fit(Yq, Yfp, w.K, 6, init_centroids=Yq[:w.K].clone())
+    finally:
+        B.cat_set_small_problem_kernels(old)
     assert torch.equal(a[3], b[3])
     for x, y in zip(a[:3], b[:3]):
         close(host(x), host(y), "fp16 vs tf32 fit")
@@ -561,9 +582,14 @@ def test_bounded_device_wait_reports_a_timeout_and_leaves_the_context_usable():
 @pytest.mark.parametrize("n,d,k,scale", [(65, 9, 8, 1.0), (300, 10, 64, 1.0), (513, 33, 8, 1.0), (129, 63, 40, 1.0),
                                          (257, 65, 129, 1.0), (1000, 1001, 50, 1.0), (700, 2047, 256, 1.0),
                                          (90, 1003, 9, 3.0e4), (600, 510, 100, 2.0e-7)])
-def test_rows_of_any_length_on_padded_fp16_copies(n, d, k, scale):
-    """Row lengths that no tensor map can address (D % 4 != 0) through inference (fp32 and bf16 output,
-    blended too), labels alone and fitting: the scores come from padded fp16 copies there."""
+def test_rows_of_any_length_on_padded_fp16_copies(n, d, k, scale, small_kernels, contraction_path):
+    """Row lengths that no tensor map can address (mostly D % 4 != 0) through inference (fp32 and bf16 output,
+    blended too), labels alone and fitting.  Without the kernels that keep rows in shared memory the scores come
+    from padded fp16 copies, as they do in larger calls; the threshold of the fp32 pipes moves short rows with few
+    centroids off them (K * D < 1024)."""
+    if small_kernels == 0 and contraction_path == "tensor" and k * d >= 1024:
+        assert B.cat_kernel_for("fit", n, d, k) == "assign_tc_kernel, fp16 copies"
+        assert d % 4 == 0 or B.cat_kernel_for("apply", n, d, k) == "assign_tc_kernel, fp16 copies"
     Yq = (_rand(n + d, n, d) * scale).astype(np.float32)
     Yfp = (Yq * 0.9 + 0.05 * scale * _rand(n + d + 1, n, d)).astype(np.float32)
     C = (_rand(k, k, d) * scale).astype(np.float32)
@@ -620,3 +646,24 @@ def test_rows_copied_in_slabs(n, d, k):
     assert bool((labels == pick).all())
     out, lab2 = B.cat_apply(Y, C, torch.ones_like(C), torch.zeros_like(C), want_labels=True, ws=ws)
     assert torch.equal(lab2, labels) and torch.equal(out, Y)
+
+
+@pytest.mark.parametrize("n,d,k", [(3000, 259, 5), (2000, 510, 40), (1500, 1001, 130)])
+@pytest.mark.parametrize("offset", [50.0, 3000.0])
+def test_fit_of_rows_with_a_common_offset(n, d, k, offset, small_kernels):
+    """Rows whose distance from the origin is far larger than their spread: the fp16 copies hold them relative to a
+    point among them, through several rounds of moving centroids."""
+    rng = np.random.default_rng(n + d)
+    Yq = (offset + rng.normal(size=(n, d))).astype(np.float32)
+    Yfp = (0.9 * Yq + 0.1 * rng.normal(size=(n, d))).astype(np.float32)
+    C, G, Bt, lab = B.cat_fit(dev(Yq), dev(Yfp), k, 6)
+    ora = O.fit(Yq, Yfp, k, 6, near_rel=NEAR_REL)
+    want, best, second = O.assign(Yq, host(C))
+    labels_match(host(lab), want, best, second, "labels")
+    g_want, b_want = O.solve_gamma_beta(Yq, Yfp, host(lab), k)
+    close(host(G), g_want, "gamma")
+    # beta = muF - gamma muQ, means of the size of the offset: a rounding of gamma (2^-24) moves it by that much of it
+    close(host(Bt), b_want, "beta", abs_tol=1e-6 + 2.0 ** -23 * offset)
+    if int(ora.near.sum()) == 0:
+        assert np.array_equal(host(lab), ora.labels)
+        close(host(C), ora.centroids, "centroids")

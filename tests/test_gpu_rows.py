@@ -100,3 +100,55 @@ def test_fit_with_rows_in_shared_memory(n, d, k, kind):
         close(host(G), g, "gamma")
         close(host(Bt), b, "beta")
     assert B.cat_workspace_report(B.workspace("fit", n, d, k, "cuda"))["device_status"] == 0
+
+
+# Several groups of rows for every team of every CTA (148 CTAs of T teams take 8 rows each at a time), and a last group
+# that is not full: slots that are loaded again, barriers' phases, the prefetch into the other slot.  Teams of 1, 2, 4
+# and 8 warps, aligned and ragged rows, fragments in shared memory and in L2.
+MANY = [(75_001, 10, 16), (75_003, 60, 12), (36_001, 200, 9), (36_003, 201, 33), (24_001, 528, 9), (24_003, 1000, 16),
+        (20_003, 1001, 50), (20_001, 1004, 60), (20_005, 131, 100), (9_003, 1600, 20), (9_001, 2047, 64)]
+
+
+@pytest.mark.parametrize("n,d,k", MANY)
+def test_teams_that_take_many_groups(n, d, k):
+    rng = np.random.default_rng(n + d)
+    C = rng.normal(size=(k, d)).astype(np.float32)
+    Yq = (C[rng.integers(0, k, size=n)] + rng.normal(size=(n, d), scale=0.7)).astype(np.float32)
+    Yq[::97] = 0.5 * (C[0] + C[1])                           # undecided rows all over the matrix
+    g, b = rng.normal(size=(k, d)).astype(np.float32), rng.normal(size=(k, d)).astype(np.float32)
+    assert B.cat_kernel_for("apply", n, d, k) == B.cat_kernel_for("apply_bf16", n, d, k) == "apply_rows_kernel"
+    _check(Yq, C, g, b)
+    first = B.cat_apply(dev(Yq), dev(C), dev(g), dev(b))
+    for _ in range(3):
+        assert torch.equal(B.cat_apply(dev(Yq), dev(C), dev(g), dev(b)), first)
+
+
+@pytest.mark.parametrize("call,n,d,k,kernel", [
+    ("apply", 4095, 1004, 128, "apply_rows_kernel"), ("apply", 4096, 1004, 128, "assign_tc_kernel"),
+    ("apply", 4096, 256, 128, "apply_rows_kernel"), ("apply", 4096, 264, 65, "assign_tc_kernel"),
+    ("apply", 4096, 120, 65, "assign_tc_kernel"), ("apply_bf16", 4096, 120, 65, "apply_rows_kernel"),
+    ("apply_bf16", 4096, 132, 65, "assign_tc_kernel"), ("apply", 4096, 132, 65, "apply_rows_kernel"),
+    ("apply", 4096, 512, 64, "apply_rows_kernel"), ("apply", 4096, 1000, 33, "apply_h64_kernel"),
+    ("apply", 4096, 1000, 32, "apply_rows_kernel"), ("apply", 4096, 1504, 64, "apply_h64_kernel"),
+    ("apply", 4096, 1544, 64, "apply_rows_kernel"), ("apply", 4096, 1001, 128, "apply_rows_kernel"),
+    ("apply", 4096, 48, 65, "assign_tc_kernel"), ("apply", 4096, 64, 64, "small_kernel"),
+    ("fit", 4096, 1000, 32, "fit_rows_kernel"), ("fit", 8192, 256, 32, "fit_rows_kernel"),
+    ("fit", 8192, 256, 64, "assign_tc_kernel, fp16 copies"), ("fit", 6144, 256, 128, "assign_tc_kernel, fp16 copies"),
+    ("fit", 8192, 50, 64, "fit_rows_kernel"), ("fit", 5000, 64, 64, "small_kernel"), ("fit", 4096, 64, 64, "fit_rows_kernel"),
+])
+def test_lines_of_the_dispatch(call, n, d, k, kernel):
+    """One shape on each side of the lines; results of either side against the oracle."""
+    assert B.cat_kernel_for(call, n, d, k) == kernel
+    rng = np.random.default_rng(n + d + k)
+    cen = rng.normal(size=(k, d)).astype(np.float32)
+    Yq = (cen[rng.integers(0, k, size=n)] + rng.normal(size=(n, d))).astype(np.float32)
+    if call == "fit":
+        C, G, Bt, lab = B.cat_fit(dev(Yq), dev(Yq), k, 3)
+        want, best, second = O.assign(Yq, host(C))
+        labels_match(host(lab), want, best, second, "labels")
+        ora = O.fit(Yq, Yq, k, 3)
+        if int(ora.near.sum()) == 0:
+            close(host(C), ora.centroids, "centroids")
+    else:
+        g, b = rng.normal(size=(k, d)).astype(np.float32), rng.normal(size=(k, d)).astype(np.float32)
+        _check(Yq, cen, g, b)

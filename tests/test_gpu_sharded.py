@@ -41,7 +41,9 @@ def test_one_shard_equals_cat_fit(config, scale):
     assert torch.equal(out, B.cat_apply(w.Yq_apply[:4096].contiguous(), C, G, Bt))
 
 
-@pytest.mark.parametrize("shape", [(3001, 1000, 16), (5000, 64, 64), (2500, 256, 40), (130, 12, 7)])
+@pytest.mark.parametrize("shape", [(3001, 1000, 16), (5000, 64, 64), (2500, 256, 40), (130, 12, 7),
+                                   # rows of the fp16 copy that need padding; few centroids on it
+                                   (2501, 1001, 12), (3003, 258, 33), (2000, 512, 4)])
 def test_two_shards_on_one_device_equal_the_oracle(shape):
     """Ranks emulated in one process: each shard has its own backend (workspace, label history);
     the sums of the deltas stand in for the all-reduce."""

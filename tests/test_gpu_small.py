@@ -59,7 +59,8 @@ def test_inference_matches_the_oracle(n, d, k, small_mask):
     assert B.cat_workspace_report(ws)["device_status"] == 0
 
 
-@pytest.mark.parametrize("n,d,k", SHAPES)
+# (a fit of up to 4096 rows takes the kernel that keeps them in shared memory)
+@pytest.mark.parametrize("n,d,k", SHAPES + [(4097, 64, 33), (4224, 64, 64), (5001, 32, 128), (4200, 128, 8)])
 def test_fit_matches_the_oracle_and_repeats(n, d, k, small_mask):
     Yq, Yfp = _data(2 * n + d + k, n, d)
     iters = 4
@@ -173,10 +174,13 @@ def test_fit_without_rounds_is_the_assignment_to_the_first_rows(small_mask):
     close(host(Bt), b_want, "beta")
 
 
-def test_shapes_outside_the_small_kernels_take_the_general_path(small_mask):
-    """K * D above 4096 (fitting) or a D that is not 32, 64 or 128: same results, other kernels."""
-    B.cat_set_small_problem_kernels(3)
+@pytest.mark.parametrize("mask", [3, 0])
+def test_shapes_outside_the_small_kernels_take_other_kernels(mask, small_mask):
+    """K * D above 4096 (fitting) or a D that is not 32, 64 or 128: the kernels that keep rows in shared memory, and with
+    those off the general path; same results."""
+    B.cat_set_small_problem_kernels(mask)
     for n, d, k in [(2000, 128, 64), (1500, 96, 40)]:
+        assert B.cat_kernel_for("fit", n, d, k) == ("fit_rows_kernel" if mask else "assign_tc_kernel, fp16 copies")
         Yq, Yfp = _data(n + d, n, d)
         C, G, Bt, labels = B.cat_fit(dev(Yq), dev(Yfp), k, 3)
         lab, best, second = O.assign(Yq, host(C))
