@@ -244,9 +244,7 @@ __device__ __noinline__ int settle(const float *y, const float *C, int D, uint4 
             if (first < 0) first = ka;
         }
     }
-    const float eta = 1.0625f * ((float)D * 0.03125f + 12.f) * 5.9604645e-8f;
-    // (below 1e-30 squares may have lost bits to underflow: whatever is that small stays a candidate)
-    const float lim = fmaxf(best, 1e-30f) * (1.f + 2.25f * eta);
+    const float lim = fp32_sum_limit(best, D);
     int left = 0;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {

@@ -60,40 +60,6 @@ struct FitRowsParams {
     uint32_t o_c, o_dist, o_sum, o_cnt, o_part, o_pcnt, o_list, o_queue, o_lab, o_pref;   // shared memory (rows first)
 };
 
-__device__ __forceinline__ uint32_t load_acquire(const uint32_t *p)
-{
-    uint32_t v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-// n-th grid barrier; false once the time limit is over anywhere
-__device__ __forceinline__ bool fit_barrier(Control *ctl, uint32_t n)
-{
-    __syncthreads();
-    bool ok = true;
-    if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(&ctl->grid_bar, 1u);
-        uint64_t t0 = 0;
-        for (uint32_t it = 0; (int32_t)(load_acquire(&ctl->grid_bar) - n * gridDim.x) < 0; ++it) {
-            if ((it & 63u) != 63u) continue;
-            if (*(volatile int *)&ctl->device_status != (int)CAT_OK) {
-                ok = false;
-                break;
-            }
-            const uint64_t now = global_timer();
-            if (t0 == 0) t0 = now;
-            else if (now - t0 > TC_TIMEOUT_NS) {
-                atomicExch(&ctl->device_status, (int)CAT_ERR_DEVICE_TIMEOUT);
-                ok = false;
-                break;
-            }
-        }
-    }
-    return __syncthreads_and(ok);
-}
-
 __device__ __forceinline__ double exact_distance(const float *y, const float *c, int D, int lane)
 {
     double s = 0.0;
@@ -105,23 +71,6 @@ __device__ __forceinline__ double exact_distance(const float *y, const float *c,
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     return s;
-}
-
-// Sums of 16 values over the warp; lanes 2 i and 2 i + 1 end with the sum of acc[i].
-__device__ __forceinline__ float warp_sum16(float (&acc)[16], int lane)
-{
-#pragma unroll
-    for (int h = 8, o = 16; h > 0; h >>= 1, o >>= 1) {
-        const bool up = lane & o;
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-            if (i < h) {
-                const float send = up ? acc[i] : acc[i + h];
-                const float keep = up ? acc[i + h] : acc[i];
-                acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-            }
-    }
-    return acc[0] + __shfl_xor_sync(0xffffffffu, acc[0], 1);
 }
 
 // one list entry's value into the sums of the clusters [k0, k1) that its row entered and left
@@ -193,7 +142,6 @@ __global__ void __launch_bounds__(FT, 1) fit_rows_kernel(FitRowsParams p)
     }
     uint32_t copies = 0;
 
-    const float eta = 1.0625f * ((float)D * 0.03125f + 12.f) * 5.9604645e-8f;
     int refined = 0, refined_pass = 0;
     uint32_t bar = 0;
     bool afresh = false;
@@ -266,8 +214,7 @@ __global__ void __launch_bounds__(FT, 1) fit_rows_kernel(FitRowsParams p)
             for (int k = lane; k < K; k += 32) best = fminf(best, d[k]);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
-            // (below 1e-30 squares may have lost bits to underflow: whatever is that small is a candidate)
-            const float lim = fmaxf(best, 1e-30f) * (1.f + 2.25f * eta);
+            const float lim = fp32_sum_limit(best, D);
             int n = 0, l = -1;
             for (int b = 0; b < K; b += 32) {
                 const uint32_t m = __ballot_sync(0xffffffffu, b + lane < K && !(d[b + lane < K ? b + lane : 0] > lim));
@@ -317,7 +264,7 @@ __global__ void __launch_bounds__(FT, 1) fit_rows_kernel(FitRowsParams p)
                 p.list_count[blockIdx.x] = w;
             }
         }
-        if (!fit_barrier(p.ctl, ++bar)) return;
+        if (!grid_barrier(&p.ctl->grid_bar, ++bar, p.ctl)) return;
         if (warp == 0) {
             int run = 0, esum = 0, rows = 0, emax = 0;
             for (int b = 0; b < G; b += 32) {
@@ -448,7 +395,7 @@ __global__ void __launch_bounds__(FT, 1) fit_rows_kernel(FitRowsParams p)
             }
             asm volatile("fence.proxy.async;" ::: "memory");
         }
-        if (!fit_barrier(p.ctl, ++bar)) return;
+        if (!grid_barrier(&p.ctl->grid_bar, ++bar, p.ctl)) return;
     }
     for (int r = tid; r < nrows; r += FT) p.labels[row0 + r] = lab[r];
     if (owner && tw == 0)

@@ -52,6 +52,33 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
+
+// Direct-form fp32 sums of squares whose lanes add D / 32 terms each before a tree adds the lanes have a relative error of
+// at most eta = (D / 32 + 12) 2^-24.  Sums above this limit are in the order of the exact ones against `best`; what lies
+// within it is settled in fp64.  Sums below 1e-30 may have lost squares to underflow: whatever is that small stays a
+// candidate.  (Every exact decision of the library goes by this line.)
+__device__ __forceinline__ float fp32_sum_limit(float best, int D)
+{
+    const float eta = 1.0625f * ((float)D * 0.03125f + 12.f) * 5.9604645e-8f;
+    return fmaxf(best, 1e-30f) * (1.f + 2.25f * eta);
+}
+
+// Sums of 16 values over the warp, 16 exchanges in place of 80; lanes 2 i and 2 i + 1 end with the sum of acc[i].
+__device__ __forceinline__ float warp_sum16(float *acc, int lane)
+{
+#pragma unroll
+    for (int h = 8, o = 16; h > 0; h >>= 1, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (i < h) {
+                const float send = up ? acc[i] : acc[i + h];
+                const float keep = up ? acc[i + h] : acc[i];
+                acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+    }
+    return acc[0] + __shfl_xor_sync(0xffffffffu, acc[0], 1);
+}
 #endif
 
 // ---------------------------------------------------------------- workspace layouts

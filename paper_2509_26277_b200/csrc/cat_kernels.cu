@@ -426,15 +426,6 @@ cudaError_t launch_assign(const float *Y, int64_t N, int D, int K, const float *
 constexpr int R_THREADS = 256;
 constexpr int R_WARPS = R_THREADS / 32;
 
-// Relative error of a direct-form fp32 sum of squares whose lanes add D / 32 terms each before a tree adds the
-// lanes, with room for the comparison: two sums further apart than this factor are in the order of the exact
-// ones.  Sums below 1e-30 may have lost squares to underflow: whatever is that small stays a candidate.
-__device__ __forceinline__ float fp32_sum_limit(float best, int D)
-{
-    const float eta = 1.0625f * ((float)D * 0.03125f + 12.f) * 5.9604645e-8f;
-    return fmaxf(best, 1e-30f) * (1.f + 2.25f * eta);
-}
-
 __device__ __forceinline__ double exact_distance(const float *y, const float *__restrict__ c, int D, int lane)
 {
     double s0 = 0.0, s1 = 0.0;
@@ -450,23 +441,6 @@ __device__ __forceinline__ double exact_distance(const float *y, const float *__
         s0 = fma(d0, d0, s0);
     }
     return warp_sum(s0 + s1);
-}
-
-// Sums of 16 values over the warp, 16 exchanges in place of 80; lanes 2 i and 2 i + 1 end with the sum of acc[i].
-__device__ __forceinline__ float warp_sum16(float *acc, int lane)
-{
-#pragma unroll
-    for (int h = 8, o = 16; h > 0; h >>= 1, o >>= 1) {
-        const bool up = lane & o;
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-            if (i < h) {
-                const float send = up ? acc[i] : acc[i + h];
-                const float keep = up ? acc[i + h] : acc[i];
-                acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-            }
-    }
-    return acc[0] + __shfl_xor_sync(0xffffffffu, acc[0], 1);
 }
 
 // Scan of all K centroids for RG queued rows per CTA at a time.  The rows sit in shared memory; a warp forms

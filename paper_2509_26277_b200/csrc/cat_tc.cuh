@@ -88,6 +88,45 @@ __device__ __forceinline__ uint64_t global_timer()
     return t;
 }
 
+__device__ __forceinline__ uint32_t load_flag(const uint32_t *p)
+{
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// waits until *flag >= value; false when the time limit is over or another CTA has given up
+__device__ __forceinline__ bool wait_flag(const uint32_t *flag, uint32_t value, Control *ctl)
+{
+    uint64_t t0 = 0;
+    for (uint32_t it = 0;; ++it) {
+        if ((int32_t)(load_flag(flag) - value) >= 0) return true;
+        if ((it & 255u) == 255u) {
+            if (*(volatile int *)&ctl->device_status != (int)CAT_OK) return false;
+            const uint64_t now = global_timer();
+            if (t0 == 0) t0 = now;
+            else if (now - t0 > TC_TIMEOUT_NS) {
+                atomicExch(&ctl->device_status, (int)CAT_ERR_DEVICE_TIMEOUT);
+                return false;
+            }
+        }
+    }
+}
+
+// Grid barrier: a counter that only grows, polled by one thread per CTA; the n-th barrier is over at
+// n * gridDim.x arrivals.  The whole CTA calls it; false once the time limit is over anywhere.
+__device__ __forceinline__ bool grid_barrier(uint32_t *counter, uint32_t n, Control *ctl)
+{
+    __syncthreads();
+    bool ok = true;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(counter, 1u);
+        ok = wait_flag(counter, n * gridDim.x, ctl);
+    }
+    return __syncthreads_and(ok);
+}
+
 // Bounded wait.  Returns false after a timeout or once another role has given up.
 // (Inlined on purpose: a called function inside the re-divided register budgets of the
 // affine kernel sends ptxas into a very long compile.)
