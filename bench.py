@@ -329,7 +329,7 @@ def run_cuda(args):
     # What a round moves and computes.  With K at or above the tensor threshold and D % 8 == 0 the assignment reads the fp16 copy of
     # the rows (N D 2 bytes, plus labels) and is paced by the tensor cores (2 N K D flop); otherwise it
     # reads the fp32 rows.  The algorithmic figure (one fp32 read of Yq per round) is reported beside it.
-    fp16_rounds = (K >= B.cat_get_tensor_core_min_k() and D % 8 == 0 and K <= 256 and B.cat_tensor_path_available())
+    fp16_rounds = B.cat_kernel_for("fit", N_fit, D, K).endswith("fp16 copies")
     lloyd_alg_gbs = 1.0 * N_fit * D * 4 / (lloyd_ms * 1e-3) / 1e9
     lloyd_moved_gbs = (N_fit * D * (2.0 if fp16_rounds else 4.0) + 8.0 * N_fit) / (lloyd_ms * 1e-3) / 1e9
     lloyd_tflops = 2.0 * N_fit * K * D / (lloyd_ms * 1e-3) / 1e12
@@ -356,24 +356,18 @@ def run_cuda(args):
                                         "objective_first": d["objective"][0], "objective_last": d["objective"][-1],
                                         "objective_never_rises": bool(all(b <= a * (1 + 1e-12) for a, b in
                                                                           zip(d["objective"], d["objective"][1:])))}
-    form = B.lib().cat_get_apply_column_split()
-    apply_kernel = ("apply_h64_kernel (64-row tiles, fp16 operands made in the kernel)"
-                    if (form in (0, 64) and K >= B.cat_get_tensor_core_min_k() and K <= 256 and 640 <= D <= 2048
-                        and D % 8 == 0 and N_apply >= 4096) else "assign_tc_kernel<affine> / assign_kernel<affine>")
-    if ((B.cat_get_small_problem_kernels() & 1) and D in (32, 64, 128) and B.cat_get_tensor_core_min_k() <= K <= 128
-            and N_apply >= 128):
-        apply_kernel = "small_kernel<inference> (one persistent launch: TF32 scores, in-kernel exact pass, affine from the staged tile)"
-    elif ((B.cat_get_small_problem_kernels() & 1) and form == 0 and 2 <= K <= 128
-            and (K * D <= 32768 or D % 8 or N_apply < 4096 or D > 1024)):
-        apply_kernel = "apply_rows_kernel (groups of eight rows in shared memory, exact decision inside)"
-    small_fit = ((B.cat_get_small_problem_kernels() & 2) and D in (32, 64, 128) and K * D <= 4096
-                 and B.cat_get_tensor_core_min_k() <= K <= 128 and N_fit >= 128)
-    if (B.cat_get_small_problem_kernels() & 2) and N_fit <= 8192 and N_fit * K * max(D, 256) <= (1 << 27 if N_fit > 6144 else 1 << 28):
+    apply_kernel = {"small_kernel": "small_kernel<inference> (one persistent launch: TF32 scores, in-kernel exact pass, affine from the staged tile)",
+                    "apply_rows_kernel": "apply_rows_kernel (groups of eight rows in shared memory, exact decision inside)",
+                    "apply_h64_kernel": "apply_h64_kernel (64-row tiles, fp16 operands made in the kernel)"}
+    apply_name = B.cat_kernel_for("apply", N_apply, D, K)
+    apply_kernel = apply_kernel.get(apply_name, apply_name)
+    fit_name = B.cat_kernel_for("fit", N_fit, D, K)
+    if fit_name == "fit_rows_kernel":
         # (the rounds end at a fixed point, so a round of the difference may be shorter than a full one)
         roofline_fit = {"bound": "latency", "kernel": "one Lloyd round inside fit_rows_kernel (one cooperative launch for the whole "
                         "fit, rows in shared memory)", "achieved": lloyd_alg_gbs, "peak": peak, "unit": "GB/s",
                         "frac": lloyd_alg_gbs / peak, "peak_source": peak_src, "tflops": lloyd_tflops}
-    elif small_fit:
+    elif fit_name == "small_kernel":
         # all rounds in one persistent launch: a round reads the fp32 rows once (TF32 scores from the staged tile)
         roofline_fit = {"bound": "hbm", "kernel": "one Lloyd round inside small_kernel<fit> (one cooperative launch for the "
                         "whole fit: TF32 scores, in-kernel exact pass, fp64 sums in shared memory, ordered grid-wide combine)",
