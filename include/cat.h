@@ -61,7 +61,7 @@ enum {
  * always recorded, at index min(iters, CAT_DIAG_MAX_ROUNDS - 1). */
 #define CAT_DIAG_MAX_ROUNDS 64
 typedef struct cat_fit_diag {
-    int64_t refined_rows_total;   /* rows whose label needed the exact fp64 pass, summed over all assignments */
+    int64_t refined_rows_total;   /* rows whose label needed the exact pass, summed over all assignments */
     int64_t refined_rows_final;   /* same, final assignment only */
     int64_t empty_clusters_final; /* clusters with no rows in the final assignment */
     int64_t device_status;        /* CAT_OK or CAT_ERR_DEVICE_TIMEOUT */
@@ -93,10 +93,14 @@ typedef struct cat_fit_diag {
  * labels_out    [N] out, may be NULL.
  * init_centroids [K, D] in, may be NULL; must not alias centroids_out.
  * diag          device pointer to one cat_fit_diag_t, may be NULL.
- * Labels are decided in fp64 whenever the fast scores cannot separate the two
- * nearest centroids; sums and moments are accumulated in fp64.  In the Lloyd
+ * Labels are those of exact arithmetic wherever fp64 distances separate the two nearest centroids: the fast scores
+ * (fp32, TF32 or fp16 operands) carry a bound on their error -- for fp16 operands from the rounding errors that were
+ * measured when the copies were made -- and rows they cannot decide go to the exact pass: direct-form distances, in fp32
+ * as far as their own error bound decides, the rest in fp64, lowest index on equality.  Rows whose squared norms leave
+ * the range of fp32 always go there.  Sums and moments are accumulated in fp64.  In the Lloyd
  * rounds the per-cluster sums are carried from round to round and updated with
- * the rows whose label changed (the same sums up to fp64 rounding).
+ * the rows whose label changed (the same sums up to fp64 rounding; a row far larger than the others leaves its rounding
+ * behind when it moves on -- one-launch fits notice that spread and add up afresh).
  * The workspace holds, besides tables of a few N and K*D words, an fp16 copy
  * of Yq (N*D*2 bytes) that the tensor-core assignment reads in every round.
  */
@@ -169,7 +173,7 @@ cat_status_t cat_assign(const float *Yq, int64_t N, int32_t D, int32_t K,
  * cat_assign that also hands out what its fast pass saw, so that the label decision can be
  * audited from outside (Alg. 2 step 2; the decision rule is the library's own: a row's label is
  * taken from fast scores t_k = ||c_k||^2 - 2 y.c_k when the two smallest are more than 2e apart,
- * e being a bound on the error of a fast score, and from fp64 direct-form distances otherwise).
+ * e being a bound on the error of a fast score, and by the exact pass otherwise).
  * Every array of `scores` has N entries and may be NULL:
  *   best, second  the two smallest fast scores of the row.  On the tensor-core path a score
  *                 carries the index of its centroid in the low 8 bits of its fp32 pattern.
@@ -304,7 +308,8 @@ cat_status_t cat_solve_gamma_beta(const double *sumQ, const double *sumF,
  * (1 / (N - 1)); its largest eigenpairs in fp64 on the device (tridiagonal reduction, bisection, inverse iteration);
  * the p directions of largest variance -> components_out [p, D] (rows, unit length, decreasing variance;
  * the sign of a row is fixed so that its entry of largest magnitude is positive); their variances
- * -> eigenvalues_out [p] double, may be NULL.  Deterministic.  N >= 2, 1 <= p <= D,
+ * -> eigenvalues_out [p] double, may be NULL: each within a few D ulp (2^-53) of the LARGEST one, so variances that
+ * are smaller than that are known to that absolute error only.  Deterministic.  N >= 2, 1 <= p <= D,
  * D <= CAT_PCA_MAX_D, p <= CAT_PCA_MAX_P.  Directions whose variances coincide are determined
  * only up to a rotation among themselves.
  * cat_pca_project: Z_out [N, p] = (Y - mean) components^T, fp64 accumulation, fp32 result.
@@ -376,7 +381,7 @@ cat_status_t cat_fit_host(const float *Yq_host, const float *Yfp_host, int64_t N
 
 /* Reads back counters kept in a workspace by the calls that used it last: waits for
  * `stream`, then copies to the HOST pointers (each may be NULL) the number of rows
- * whose label needed the exact fp64 pass in the latest assignment, the running
+ * whose label needed the exact pass in the latest assignment, the running
  * total since the last cat_fit started on that workspace, and the device status
  * word (CAT_OK or CAT_ERR_DEVICE_TIMEOUT: outputs of that call are undefined).  For the calls that
  * compose several steps -- cat_pca_fit, cat_fit_pca, cat_apply_pca -- the block speaks for all of them.  (The
@@ -395,8 +400,8 @@ cat_status_t cat_selftest_wait_timeout(void *workspace, size_t workspace_bytes, 
 /* Kernel selection for the distance contraction.  With K >= min_k (and D % 4 == 0,
  * K <= 256) the scores are formed on the tensor cores (tcgen05, TF32 or fp16 operands, fp32
  * accumulation); below it on the fp32 pipes.  Fits (and inference on rows with D % 4 != 0) use a padded
- * fp16 copy of the rows from K >= min_k / 4 and K * D >= 1024 on, short rows excepted.  Either way undecided rows are settled in
- * fp64, so the labels are the same.  Default 8: measured at K = 8, 16 and 32 (rows of 1000
+ * fp16 copy of the rows from K >= min_k / 4 and K * D >= 1024 on, short rows excepted.  Either way undecided rows are settled
+ * exactly, so the labels are the same.  Default 8: measured at K = 8, 16 and 32 (rows of 1000
  * columns) a Lloyd round takes half the time on the tensor path and so does inference, except
  * where low-precision scores leave most rows undecided (unimodal data, K = 32: there the fp32
  * pipes are a quarter faster for inference).
@@ -408,13 +413,15 @@ int32_t cat_get_tensor_core_min_k(void);
 
 /* Small problems (D one of 32, 64, 128; K <= 128, and K * D <= 4096 for fitting; at least 128
  * rows; K >= the tensor-core threshold above) have persistent single-launch kernels: scores on the
- * tensor cores, undecided rows settled in fp64 inside the kernel, and for fitting the per-cluster
+ * tensor cores, undecided rows settled inside the kernel, and for fitting the per-cluster
  * sums kept on chip and combined across the grid in a fixed order, all rounds in one launch.
  * mask bit 0: the whole of cat_apply (Algorithm 2) runs that way; so it does for other shapes with
- * K <= 128 (K >= a quarter of the threshold, rows up to about 3300 columns), in two launches that keep
- * each row in shared memory.  mask bit 1: so do the K-Means
+ * K <= 128 (K >= a quarter of the threshold; rows up to about 3300 columns for K <= 32, 3000 for K <= 64, 2500 above), in
+ * two launches that keep each row in shared memory -- except, for 4096 rows and more with D % 4 == 0 and D <= 1536, where
+ * K * D > 32768 (D % 8 == 0) or K > 64 (rows of 128 to 256 columns excepted), and short rows with many centroids: those
+ * stay on the tile kernels (cat_kernel_for tells).  mask bit 1: so do the K-Means
  * rounds and the final assignment of cat_fit / cat_fit_from (Algorithm 1, step 2; calls without
- * per-round diagnostics), and of other sets of up to 8192 rows with moderate N * K * D.  Default 3:
+ * per-round diagnostics), and of other sets of up to 8192 rows with moderate N * K * D (of those shapes too up to 4096 rows).  Default 3:
  * both are the faster form where they apply.  Clearing a bit sends these shapes down the general multi-launch path instead: same labels (rows on a bisector
  * apart, when a centroid differs in its last bit); sums that agree to fp64 rounding.  A PROCESS-WIDE
  * tuning and test hook like the one above. */

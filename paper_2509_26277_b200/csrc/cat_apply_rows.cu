@@ -16,7 +16,7 @@
 // What bounds it: latency and instruction issue -- a group's way through its phases takes about 7 us, and
 // shared memory holds five groups of rows of 1000 columns per SM.  Measured against the kernels that read
 // a row twice (64-row tiles with a separate exact pass; padded copies where D % 4 != 0): 1024 x 1000, K = 8
-// 26 us against 63; 50 000 x 1000, K = 16 113 against 158, K = 32 142 against 262; 50 000 x 1001, K = 50 250
+// 18 us against 62; 50 000 x 1000, K = 16 113 against 158, K = 32 142 against 262; 50 000 x 1001, K = 50 250
 // against 342; 1 000 000 x 768, K = 32 1.47 ms against 2.39.
 //
 // Scores.  t_k = ||c_k||^2 - ||m||^2 - 2 y.(c_k - m) with m the mean of the centroids: m changes all

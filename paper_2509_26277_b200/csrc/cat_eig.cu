@@ -474,7 +474,7 @@ __global__ void __launch_bounds__(ET) eigvec_kernel(EigvecParams P)
             for (int k = tid; k < D; k += ET) {
                 double v = 0.0;
                 if (round == 0) {
-                    uint32_t h = (uint32_t)m * 0x9E3779B9u + (uint32_t)k * 0x85EBCA6Bu + 1u;   // a different start for each vector
+                    uint32_t h = (uint32_t)m * 0x9E3779B9u + (uint32_t)k * 0x85EBCA6Bu + 1u;   // a different start for each vector (Wellons' lowbias32 mixer)
                     h ^= h >> 16;
                     h *= 0x7FEB352Du;
                     h ^= h >> 15;
