@@ -86,8 +86,7 @@ FitWs carve_fit(void *base, int64_t N, int D, int K)
     w.labels_prev = c.take<int32_t>((size_t)N);
     {
         // two planes per segment in delta mode, three in the single-sweep final pass (full mode)
-        const SegGeom gf = seg_geometry(N, D, K);
-        const size_t a = (size_t)g.max_segs * 2, b = (size_t)gf.max_segs * 3;
+        const size_t a = (size_t)seg_capacity(2 * N, 2 * K) * 2, b = (size_t)seg_capacity(N, K) * 3;
         w.segpart = c.take<double>((a > b ? a : b) * D);
     }
     w.yh = c.take<uint16_t>((size_t)N * half_ld(D));

@@ -110,6 +110,7 @@ struct SegGeom {
     int max_segs;   // upper bound on the number of segments: ceil(NE / seg_rows) + KK
 };
 SegGeom seg_geometry(int64_t NE, int D, int KK);
+int seg_capacity(int64_t NE, int KK);
 
 struct AssignWs {          // what assign/apply need
     Control *ctl;

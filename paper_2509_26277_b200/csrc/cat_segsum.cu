@@ -615,6 +615,18 @@ SegGeom seg_geometry(int64_t NE, int D, int KK)
     return g;
 }
 
+// Room for the segments of any list of up to NE entries (never less for a longer list: a workspace for more rows
+// serves fewer).
+int seg_capacity(int64_t NE, int KK)
+{
+    int64_t n = (NE + 15) / 16;
+    if (NE > 8192) {
+        n = (NE + 127) / 128;
+        n = n < 512 ? 512 : (n < 2048 ? n : 2048);
+    }
+    return (int)n + KK;
+}
+
 cudaError_t launch_label_sort(const int32_t *labels, const int32_t *prev, int64_t N, int K, const SegGeom &g,
                               uint32_t *blk_hist, uint32_t *key_total, int64_t *counts, int32_t *cluster_start,
                               int32_t *seg_start, int32_t *order, cudaStream_t s)

@@ -122,3 +122,14 @@ def test_binding_refuses_cpu_tensors():
     x = torch.zeros((8, 4))
     with pytest.raises(TypeError):
         binding.cat_assign(x, x[:2].contiguous(), ws=torch.zeros(1024, dtype=torch.uint8))
+
+
+ROWS = [1, 2, 64, 127, 128, 129, 1000, 2048, 4095, 4096, 4097, 4737, 5000, 8191, 8192, 8193, 9000, 16384, 16385, 65536, 131072,
+        131073, 262144, 262145, 267520, 267521, 300000, 535040, 535041, 600000, 1048576, 1048577, 2000000, 4194304]
+
+
+@pytest.mark.parametrize("d,k", [(1001, 4), (1001, 200), (1000, 16), (64, 64), (10, 500), (4099, 30), (1024, 256)])
+def test_a_fit_workspace_for_more_rows_serves_fewer(d, k):
+    """A caller may size one workspace for its largest call (shards, the last chunk of a stream of rows)."""
+    size = [binding.lib().cat_fit_workspace_bytes(n, d, k) for n in ROWS]
+    assert size[0] > 0 and size == sorted(size)
