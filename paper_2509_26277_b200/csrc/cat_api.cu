@@ -29,10 +29,16 @@ struct Carver {
 
 // Rows of an inference call's fp16 copy (rows that TMA cannot address): at most 512 MiB of them at a time, so that
 // the scratch of a call does not grow with N * D.  A further slab costs about 17 us (two kernels that fill and drain
-// the device once more: 400 000 x 1001, K = 200 takes 970 us in one piece, 988 in two).  The rows are split evenly.
+// the device once more: 400 000 x 1001, K = 200 takes 970 us in one piece, 988 in two).  The rows are split evenly; the
+// room is what the longest slab of any smaller call needs.
+static int64_t copy_room_rows(int64_t N, int D)
+{
+    const int64_t cap = (((int64_t)512 << 20) / (2 * half_ld(D))) & ~(int64_t)255;
+    return N < cap ? N : cap;
+}
 static int64_t copy_slab_rows(int64_t N, int D)
 {
-    const int64_t cap = ((int64_t)512 << 20) / (2 * half_ld(D));
+    const int64_t cap = (((int64_t)512 << 20) / (2 * half_ld(D))) & ~(int64_t)255;
     const int64_t slabs = (N + cap - 1) / cap;
     const int64_t rows = ((N + slabs - 1) / slabs + 255) & ~(int64_t)255;
     return rows < N ? rows : N;
@@ -55,7 +61,7 @@ static void carve_assign_into(Carver &c, AssignWs &w, int64_t N, int D, int K, b
     w.cerr = c.take<float>((size_t)K);
     w.mean = c.take<float>((size_t)D);
     w.ch = c.take<uint16_t>((size_t)K * half_ld(D));
-    const size_t slab = row_copy ? (size_t)copy_slab_rows(N, D) : 0;
+    const size_t slab = row_copy ? (size_t)copy_room_rows(N, D) : 0;
     w.hscale = c.take<float>(4 + 2 * slab);
     const size_t prep = inference ? apply_rows_prep_bytes(N, D, K) : 0;
     w.prep = prep ? c.take<unsigned char>(prep) : nullptr;

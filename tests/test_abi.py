@@ -129,7 +129,9 @@ ROWS = [1, 2, 64, 127, 128, 129, 1000, 2048, 4095, 4096, 4097, 4737, 5000, 8191,
 
 
 @pytest.mark.parametrize("d,k", [(1001, 4), (1001, 200), (1000, 16), (64, 64), (10, 500), (4099, 30), (1024, 256)])
-def test_a_fit_workspace_for_more_rows_serves_fewer(d, k):
+@pytest.mark.parametrize("call", ["fit", "apply"])
+def test_a_workspace_for_more_rows_serves_fewer(call, d, k):
     """A caller may size one workspace for its largest call (shards, the last chunk of a stream of rows)."""
-    size = [binding.lib().cat_fit_workspace_bytes(n, d, k) for n in ROWS]
+    query = getattr(binding.lib(), f"cat_{call}_workspace_bytes")
+    size = [query(n, d, k) for n in ROWS]
     assert size[0] > 0 and size == sorted(size)

@@ -624,7 +624,7 @@ def test_rows_copied_in_slabs(n, d, k):
     """More rows of a length no tensor map can address than the workspace's fp16 copy holds at a time: labels as the
     oracle gives them across the seams, undecided rows counted over all slabs, a workspace well below the whole copy."""
     rng = np.random.default_rng(n)
-    slabs = -(-n // ((512 << 20) // (2 * ((d + 7) // 8 * 8))))
+    slabs = -(-n // ((512 << 20) // (2 * ((d + 7) // 8 * 8)) // 256 * 256))
     slab = (-(-n // slabs) + 255) // 256 * 256
     assert slab < n
     ws = B.workspace("apply", n, d, k, "cuda")
