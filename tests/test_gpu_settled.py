@@ -1,0 +1,45 @@
+"""Fits on the multi-launch path whose labels come to rest before the last round: the rounds behind that one do no
+work, and the result is that of running them."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import cat_oracle as O
+from paper_2509_26277_b200 import binding as B
+
+pytestmark = pytest.mark.gpu
+
+
+def _clusters(seed, n, d, k, spread):
+    rng = np.random.default_rng(seed)
+    cen = rng.normal(size=(k, d)) * spread
+    Yq = (cen[np.arange(n) % k] + rng.normal(size=(n, d))).astype(np.float32)
+    return Yq, (0.9 * Yq + 0.05 * rng.normal(size=(n, d))).astype(np.float32)
+
+
+@pytest.mark.parametrize("n,d,k,spread", [(9001, 64, 16, 20.0), (9001, 63, 20, 20.0), (20_000, 256, 40, 1.0), (9000, 40, 3, 20.0),
+                                          (9000, 16, 300, 20.0), (9000, 64, 1, 20.0)])
+def test_rounds_after_a_fixed_point_change_nothing(n, d, k, spread):
+    Yq, Yfp = _clusters(3, n, d, k, spread)
+    q, f = torch.from_numpy(Yq).cuda(), torch.from_numpy(Yfp).cuda()
+    old = B.cat_get_small_problem_kernels()
+    B.cat_set_small_problem_kernels(0)
+    try:
+        ws = torch.empty(B.lib().cat_fit_workspace_bytes(n, d, k), dtype=torch.uint8, device="cuda")
+        want = O.fit(Yq, Yfp, k, 60, near_rel=1e-6)
+        got = {}
+        for iters in (60, 59, 12, 0, 60):   # both parities of the label buffers; a fit that settles, then others on its workspace
+            C, G, Bt, lab = B.cat_fit(q, f, k, iters, ws=ws)
+            got.setdefault(iters, []).append([t.cpu() for t in (C, G, Bt, lab)])
+        sums, counts = B.cat_cluster_sums(q, got[60][0][3].cuda(), k, ws=ws)
+    finally:
+        B.cat_set_small_problem_kernels(old)
+    assert all(torch.equal(a, b) for a, b in zip(got[60][0], got[60][1]))
+    if np.array_equal(want.labels, O.fit(Yq, Yfp, k, 59).labels):
+        assert all(torch.equal(a, b) for a, b in zip(got[60][0], got[59][0]))
+    if want.near.sum() == 0:
+        assert np.array_equal(got[60][0][3].numpy(), want.labels)
+        np.testing.assert_allclose(got[60][0][0].numpy(), want.centroids, rtol=1e-5, atol=1e-6)
+    first = O.fit(Yq, Yfp, k, 0)
+    assert (got[0][0][3].numpy() != first.labels).mean() < 1e-3
+    np.testing.assert_array_equal(counts.cpu().numpy(), np.bincount(got[60][0][3].numpy(), minlength=k))
