@@ -207,7 +207,7 @@ static cat_status_t run_assign(const float *Y, int64_t N, int D, int K, const fl
                                const float *beta, float *out, cudaStream_t s,
                                bool row_norms_ready = false, bool top_level = true,
                                const void *Yh = nullptr, void *Ch = nullptr, float *hscale = nullptr,
-                               bool centroids_ready = false, const FastOut *fast = nullptr)
+                               bool centroids_ready = false, const FastOut *fast = nullptr, const int32_t *settled = nullptr)
 {
     if (out && labels && top_level && !fast && use_small_apply(N, D, K)) {
         // small problems: everything in one persistent launch (exact decisions included)
@@ -266,11 +266,11 @@ static cat_status_t run_assign(const float *Y, int64_t N, int D, int K, const fl
         if (Yh && !centroids_ready)
             CAT_CUDA(launch_centroid_half(C, D, K, w.mean, w.cnorm, w.cmax, w.cerr, hscale, Ch, w.ctl, s, top_level, false));
         CAT_CUDA(launch_assign_tc(Y, N, D, K, C, w.cnorm, w.ynorm2, labels, w.refine_rows, w.cand_rows,
-                                  w.cand_list, w.ctl, gamma, beta, out, s, Yh, Ch, hscale, w.cerr, fast));
+                                  w.cand_list, w.ctl, gamma, beta, out, s, Yh, Ch, hscale, w.cerr, fast, 0, settled));
         CAT_CUDA(launch_refine_both(Y, N, D, K, C, labels, w.cand_rows, w.cand_list, w.refine_rows, w.ctl, gamma,
                                     beta, out, s));
     } else {
-        CAT_CUDA(launch_assign(Y, N, D, K, C, w.cnorm, labels, w.refine_rows, w.ctl, gamma, beta, out, s, fast));
+        CAT_CUDA(launch_assign(Y, N, D, K, C, w.cnorm, labels, w.refine_rows, w.ctl, gamma, beta, out, s, fast, settled));
         if (K > 1) CAT_CUDA(launch_refine(Y, N, D, K, C, labels, w.refine_rows, w.ctl, gamma, beta, out, s));
     }
     return CAT_OK;
@@ -301,15 +301,15 @@ static cat_status_t run_sums(const float *M, int64_t N, int D, int K, const FitW
 // and sizes in the workspace (sumQ, counts) move by what entered and left each cluster, then
 // c_k = sumQ_k / n_k.  `prev` = all -1 makes every row an entry (the first round).
 static cat_status_t run_delta_update(const float *Yq, const int32_t *labels, const int32_t *prev, int64_t N, int D,
-                                     int K, const FitWs &w, float *C, bool half, cudaStream_t s)
+                                     int K, const FitWs &w, float *C, bool half, cudaStream_t s, int32_t *settled)
 {
     SegGeom g = seg_geometry(2 * N, D, 2 * K);
     CAT_CUDA(launch_label_sort(labels, prev, N, K, g, w.blk_hist, w.key_total, w.counts, w.cluster_start,
-                               w.seg_start, w.order, s));
+                               w.seg_start, w.order, s, settled));
     CAT_CUDA(launch_segment_sums(0, Yq, nullptr, w.order, w.cluster_start, w.seg_start, nullptr, nullptr, D,
-                                 2 * K, g, w.segpart, s));
+                                 2 * K, g, w.segpart, s, settled));
     CAT_CUDA(launch_centroid_update(w.segpart, w.seg_start, w.counts, D, K, g.max_segs, w.sumQ, C, w.a.cnorm, w.hscale,
-                                    half ? w.ch : nullptr, half ? w.a.mean : nullptr, w.a.cerr, w.norm_part, w.arrivals, w.a.ctl, s));
+                                    half ? w.ch : nullptr, half ? w.a.mean : nullptr, w.a.cerr, w.norm_part, w.arrivals, w.a.ctl, s, settled));
     return CAT_OK;
 }
 
@@ -528,6 +528,9 @@ cat_status_t cat_fit_from(const float *Yq, const float *Yfp, int64_t N, int32_t 
     // sizes start at zero with "no previous label" (-1) for every row.
     const int diag_recorded = iters + 1 < CAT_DIAG_MAX_ROUNDS ? iters + 1 : CAT_DIAG_MAX_ROUNDS;
     int32_t *lab[2] = {labels, w.labels_prev};
+    // (a round that moves no row ends the work of those behind it -- both label buffers hold the same labels then --,
+    // except where every assignment is to be recorded)
+    int32_t *settled = diag ? nullptr : &w.a.ctl->settled;
     if (!small) {
     CAT_CUDA(cudaMemsetAsync(lab[(iters & 1) ^ 1], 0xFF, (size_t)N * sizeof(int32_t), s));
     CAT_CUDA(cudaMemsetAsync(w.sumQ, 0, KD * sizeof(double), s));
@@ -536,18 +539,18 @@ cat_status_t cat_fit_from(const float *Yq, const float *Yfp, int64_t N, int32_t 
     for (int t = 0; t < iters; ++t) {
         int32_t *cur = lab[(iters - t) & 1], *prev = lab[((iters - t) & 1) ^ 1];
         st = run_assign(Yq, N, D, K, C, cur, w.a, nullptr, nullptr, nullptr, s, tc, false, Yh, w.ch, w.hscale,
-                        t > 0);
+                        t > 0, nullptr, settled);
         if (st != CAT_OK) return st;
         if (diag && t < CAT_DIAG_MAX_ROUNDS - 1)
             CAT_CUDA(launch_fit_diag_round(Yq, N, D, K, C, cur, w.a.refine_rows, w.a.cand_rows, w.a.ctl, diag, t,
                                            diag_recorded, s));
-        st = run_delta_update(Yq, cur, prev, N, D, K, w, C, half, s);
+        st = run_delta_update(Yq, cur, prev, N, D, K, w, C, half, s, settled);
         if (st != CAT_OK) return st;
     }
 
     // final assignment, then the closed form
     st = run_assign(Yq, N, D, K, C, labels, w.a, nullptr, nullptr, nullptr, s, tc, false, Yh, w.ch, w.hscale,
-                    iters > 0);
+                    iters > 0, nullptr, settled);
     if (st != CAT_OK) return st;
     if (diag)
         CAT_CUDA(launch_fit_diag_round(Yq, N, D, K, C, labels, w.a.refine_rows, w.a.cand_rows, w.a.ctl, diag,

@@ -98,7 +98,9 @@ struct Control {
     int64_t refined_last;        // rows of the latest finished assignment that took an exact pass
     int32_t cand_count;          // rows queued with a short candidate list by the current assignment
     uint32_t grid_bar;           // arrival counter of the grid-wide barrier of the persistent small-problem kernel
-    int64_t pad[4];
+    int32_t settled;             // a Lloyd round of cat_fit moved no row: the rounds behind it have nothing to do
+    int32_t pad32;
+    int64_t pad[3];
 };
 
 // Geometry of the sort-based segmented sums for NE entries over KK keys (full mode: N rows,
@@ -169,7 +171,7 @@ cudaError_t launch_centroid_norms(const float *C, int D, int K, float *cnorm, Co
 cudaError_t launch_assign(const float *Y, int64_t N, int D, int K, const float *C,
                           const float *cnorm, int32_t *labels, int32_t *refine_rows, Control *ctl,
                           const float *gamma, const float *beta, float *out, cudaStream_t s,
-                          const FastOut *fast = nullptr);
+                          const FastOut *fast = nullptr, const int32_t *settled = nullptr);
 
 // Exact fp64 direct-form labels for the queued rows; optional affine output.
 cudaError_t launch_refine(const float *Y, int64_t N, int D, int K, const float *C,
@@ -231,7 +233,8 @@ cudaError_t launch_assign_tc(const float *Y, int64_t N, int D, int K, const floa
                              int32_t *cand_rows, uint64_t *cand_list, Control *ctl,
                              const float *gamma, const float *beta, float *out, cudaStream_t s,
                              const void *Yh = nullptr, const void *Ch = nullptr, const float *scale = nullptr,
-                             const float *cerr = nullptr, const FastOut *fast = nullptr, int64_t row_base = 0);
+                             const float *cerr = nullptr, const FastOut *fast = nullptr, int64_t row_base = 0,
+                             const int32_t *settled = nullptr);
 
 // One warp waits (at most limit_ms, clamped to 1 .. 1000) on a barrier that is never completed.
 cudaError_t launch_wait_selftest(Control *ctl, int limit_ms, cudaStream_t s);
@@ -267,9 +270,13 @@ cudaError_t launch_refine_both(const float *Y, int64_t N, int D, int K, const fl
 // cluster k.  prev != NULL (delta mode): entries only for rows with labels[i] != prev[i], under keys
 // labels[i] and K + prev[i]; counts[k] += (rows that entered k) - (rows that left k).  Tables have one
 // entry per key (+1).  Labels outside [0, K) are left out.
+// settled (delta mode, here and in the launchers below and of the assignments; may be null): the sort of a round in
+// which no label changed sets it, and once it is set the kernels return at once.  Such a round leaves sums, centroids
+// and labels as they are, bit for bit, and so do all that would follow.  262 144 x 1024 rows in 256 far-apart clusters
+// stand still after about seventeen of 25 rounds.
 cudaError_t launch_label_sort(const int32_t *labels, const int32_t *prev, int64_t N, int K, const SegGeom &g,
                               uint32_t *blk_hist, uint32_t *key_total, int64_t *counts, int32_t *cluster_start,
-                              int32_t *seg_start, int32_t *order, cudaStream_t s);
+                              int32_t *seg_start, int32_t *order, cudaStream_t s, int32_t *settled = nullptr);
 
 // Per-segment partial sums over KK keys.  mode 0: column sums of Yq (plane 0); mode 1: of Yq and Yf
 // (planes 0, 1); mode 2 (full mode only): centred moments sum (q-muQ)^2 (plane 0) and
@@ -278,7 +285,7 @@ cudaError_t launch_label_sort(const int32_t *labels, const int32_t *prev, int64_
 cudaError_t launch_segment_sums(int mode, const float *Yq, const float *Yf, const int32_t *order,
                                 const int32_t *cluster_start, const int32_t *seg_start, const double *meanQ,
                                 const double *meanF, int D, int KK, const SegGeom &g, double *part,
-                                cudaStream_t s);
+                                cudaStream_t s, const int32_t *settled = nullptr);
 
 // Adds each cluster's segment partials in order into out0 (and out1 if not NULL); in delta mode
 // out0[k] += (partials of key k) - (partials of key K + k).  With C also writes the centroid
@@ -297,7 +304,7 @@ cudaError_t launch_segment_combine3(const double *part, const int32_t *seg_start
 cudaError_t launch_centroid_update(const double *part, const int32_t *seg_start, const int64_t *counts, int D,
                                    int K, int max_segs, double *sums, float *C, float *cnorm, const float *scale, void *Ch,
                                    const float *mean, float *cerr, void *norm_part, uint32_t *arrivals, Control *ctl,
-                                   cudaStream_t s);
+                                   cudaStream_t s, const int32_t *settled = nullptr);
 size_t centroid_update_scratch_bytes(int D, int K);
 
 cudaError_t launch_centroids_from_sums(const double *sums, const int64_t *counts, int D, int K,

@@ -112,6 +112,7 @@ struct AssignParams {
     int D;
     int K;
     FastOut fast;
+    const int32_t *settled;   // nothing to do once this is set (or null)
 };
 
 template <int BN>
@@ -171,6 +172,7 @@ __device__ __forceinline__ void assign_load_tile(AssignSmem<BN> &sm, int stage, 
 template <int BN, bool VEC4, bool AFFINE>
 __global__ void __launch_bounds__(A_THREADS) assign_kernel(AssignParams p)
 {
+    if (p.settled && *p.settled) return;
     constexpr int TX = BN / 8;
     constexpr int TY = A_THREADS / TX;
     constexpr int TM = A_BM / TY;
@@ -410,9 +412,9 @@ static cudaError_t launch_assign_bn(const AssignParams &p, cudaStream_t s)
 cudaError_t launch_assign(const float *Y, int64_t N, int D, int K, const float *C,
                           const float *cnorm, int32_t *labels, int32_t *refine_rows, Control *ctl,
                           const float *gamma, const float *beta, float *out, cudaStream_t s,
-                          const FastOut *fast)
+                          const FastOut *fast, const int32_t *settled)
 {
-    AssignParams p{Y, C, cnorm, labels, refine_rows, ctl, gamma, beta, out, N, D, K, fast ? *fast : FastOut{}};
+    AssignParams p{Y, C, cnorm, labels, refine_rows, ctl, gamma, beta, out, N, D, K, fast ? *fast : FastOut{}, settled};
     const bool vec = (D % 4 == 0);
     const bool affine = (out != nullptr);
     if (vec) return affine ? launch_assign_bn<true, true>(p, s) : launch_assign_bn<true, false>(p, s);
@@ -1164,6 +1166,7 @@ __global__ void reset_control_kernel(Control *ctl)
         ctl->refined_total = 0;
         ctl->refined_last = 0;
         ctl->grid_bar = 0;
+        ctl->settled = 0;
     }
 }
 

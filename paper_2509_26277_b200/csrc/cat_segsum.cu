@@ -54,9 +54,11 @@ __device__ __forceinline__ int entry_key(const int32_t *__restrict__ cur, const 
 
 __global__ void __launch_bounds__(SORT_BLOCK) label_hist_kernel(const int32_t *__restrict__ cur,
                                                                  const int32_t *__restrict__ prev, int64_t N, int K,
-                                                                 int KK, uint32_t *__restrict__ blk_hist)
+                                                                 int KK, uint32_t *__restrict__ blk_hist,
+                                                                 const int32_t *settled)
 {
     pdl_enter();
+    if (settled && *settled) return;
     extern __shared__ uint32_t hist[];   // [KK]
     for (int k = threadIdx.x; k < KK; k += SORT_BLOCK) hist[k] = 0;
     __syncthreads();
@@ -70,9 +72,10 @@ __global__ void __launch_bounds__(SORT_BLOCK) label_hist_kernel(const int32_t *_
 // One warp per key: blk_hist[k][b] becomes the number of entries of key k in blocks before
 // b, key_total[k] their total.
 __global__ void __launch_bounds__(256) label_scan_blocks_kernel(uint32_t *__restrict__ blk_hist, int nblk, int KK,
-                                                                 uint32_t *__restrict__ key_total)
+                                                                 uint32_t *__restrict__ key_total, const int32_t *settled)
 {
     pdl_enter();
+    if (settled && *settled) return;
     const int k = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     if (k >= KK) return;
@@ -136,7 +139,7 @@ __device__ __forceinline__ uint32_t cta_exclusive_scan(uint32_t v, uint32_t *wsu
 __device__ __forceinline__ uint32_t scan_keys(const uint32_t *__restrict__ key_total, int K, int KK, int seg_rows_max,
                                               int64_t NE, int delta, bool publish, int64_t *__restrict__ counts,
                                               int32_t *__restrict__ cluster_start, int32_t *__restrict__ seg_start,
-                                              uint32_t *wsum /*[33] shared*/)
+                                              int32_t *settled, uint32_t *wsum /*[33] shared*/)
 {
     const int k = threadIdx.x;
     const uint32_t tot = (k < KK) ? key_total[k] : 0u;
@@ -158,6 +161,7 @@ __device__ __forceinline__ uint32_t scan_keys(const uint32_t *__restrict__ key_t
         cluster_start[KK] = (int32_t)M;
         seg_start[KK] = (int32_t)nseg;
         seg_start[KK + 1] = (int32_t)sr;
+        if (settled && M == 0) *settled = 1;   // (read by later launches; a CTA of this one that sees it has no entry to place)
     }
     if (k < K) {
         if (delta) counts[k] += (int64_t)tot - (int64_t)key_total[K + k];
@@ -176,9 +180,11 @@ __global__ void __launch_bounds__(SORT_BLOCK) label_scatter_kernel(const int32_t
                                                                     int64_t *__restrict__ counts,
                                                                     int32_t *__restrict__ cluster_start,
                                                                     int32_t *__restrict__ seg_start,
-                                                                    int32_t *__restrict__ order)
+                                                                    int32_t *__restrict__ order, int32_t *settled)
 {
     pdl_enter();
+    // (one read per CTA: CTA 0 may set the word while others of this launch are here)
+    if (settled && __syncthreads_or(threadIdx.x == 0 && *(volatile int32_t *)settled)) return;
     extern __shared__ uint32_t scatter_smem[];   // [KK] key offsets, then [32][KK] 16-bit warp histograms
     __shared__ uint32_t wsum[33];
     uint32_t *key_off = scatter_smem;
@@ -187,7 +193,7 @@ __global__ void __launch_bounds__(SORT_BLOCK) label_scatter_kernel(const int32_t
     for (int e = tid; e < 32 * KK; e += SORT_BLOCK) warp_hist[e] = 0;
     {
         const uint32_t ea = scan_keys(key_total, K, KK, seg_rows_max, NE, delta, blockIdx.x == 0, counts, cluster_start,
-                                      seg_start, wsum);
+                                      seg_start, settled, wsum);
         if (tid < KK) key_off[tid] = ea;
     }
     __syncthreads();
@@ -226,6 +232,7 @@ struct SegParams {
     int K;
     int seg_rows;
     int tpr;                    // threads per row (power of two <= 256)
+    const int32_t *settled;
 };
 
 __device__ __forceinline__ void add4(double (&a)[4], const float4 v)
@@ -271,6 +278,7 @@ template <int MODE, int VEC>
 __global__ void __launch_bounds__(SEG_THREADS) segment_sums_kernel(SegParams p)
 {
     pdl_enter();
+    if (p.settled && *p.settled) return;
     __shared__ int32_t rows_s[128];
     __shared__ double red_s[SEG_THREADS * VEC];
     const int nseg_total = p.seg_start[p.K];
@@ -502,7 +510,8 @@ __global__ void __launch_bounds__(COMB_THREADS, 4) centroid_update_kernel(const 
                                                               float *__restrict__ cnorm, const float *__restrict__ scale,
                                                               __half *__restrict__ Ch, const float *__restrict__ mean,
                                                               float *__restrict__ cerr, double2 *__restrict__ norm_part,
-                                                              unsigned int *__restrict__ arrivals, Control *ctl)
+                                                              unsigned int *__restrict__ arrivals, Control *ctl,
+                                                              const int32_t *settled)
 {
     pdl_enter();
     __shared__ double red[COMB_THREADS];
@@ -513,6 +522,7 @@ __global__ void __launch_bounds__(COMB_THREADS, 4) centroid_update_kernel(const 
         ctl->refine_count = 0;
         ctl->cand_count = 0;
     }
+    if (settled && *settled) return;
     const int j = cb * cols + (threadIdx.x & (cols - 1));
     const int64_t n = counts[k];
     const float sc = Ch ? scale[0] : 1.f;
@@ -629,11 +639,13 @@ int seg_capacity(int64_t NE, int KK)
 
 cudaError_t launch_label_sort(const int32_t *labels, const int32_t *prev, int64_t N, int K, const SegGeom &g,
                               uint32_t *blk_hist, uint32_t *key_total, int64_t *counts, int32_t *cluster_start,
-                              int32_t *seg_start, int32_t *order, cudaStream_t s)
+                              int32_t *seg_start, int32_t *order, cudaStream_t s, int32_t *settled)
 {
     const int KK = prev ? 2 * K : K;
-    launch_pdl(label_hist_kernel, dim3(g.nblk), dim3(SORT_BLOCK), (size_t)KK * sizeof(uint32_t), s, labels, prev, N, K, KK, blk_hist);
-    launch_pdl(label_scan_blocks_kernel, dim3((KK * 32 + 255) / 256), dim3(256), 0, s, blk_hist, g.nblk, KK, key_total);
+    launch_pdl(label_hist_kernel, dim3(g.nblk), dim3(SORT_BLOCK), (size_t)KK * sizeof(uint32_t), s, labels, prev, N, K, KK, blk_hist,
+               settled);
+    launch_pdl(label_scan_blocks_kernel, dim3((KK * 32 + 255) / 256), dim3(256), 0, s, blk_hist, g.nblk, KK, key_total,
+               settled);
     // (the scan over the keys -- key offsets, segment table, cluster sizes -- runs inside the scatter
     // kernel: every CTA needs the offsets, CTA 0 publishes the tables)
     const size_t sc_smem = (size_t)KK * sizeof(uint32_t) + (size_t)32 * KK * sizeof(uint16_t);
@@ -643,7 +655,7 @@ cudaError_t launch_label_sort(const int32_t *labels, const int32_t *prev, int64_
         if (e != cudaSuccess) return e;
     }
     launch_pdl(label_scatter_kernel, dim3(g.nblk), dim3(SORT_BLOCK), sc_smem, s, labels, prev, N, K, KK, blk_hist, key_total,
-               g.seg_rows, prev ? 2 * N : N, prev ? 1 : 0, counts, cluster_start, seg_start, order);
+               g.seg_rows, prev ? 2 * N : N, prev ? 1 : 0, counts, cluster_start, seg_start, order, settled);
     count_launch(3);
     return cudaGetLastError();
 }
@@ -668,7 +680,7 @@ static cudaError_t launch_segment_sums_mode(const SegParams &p, const SegGeom &g
 cudaError_t launch_segment_sums(int mode, const float *Yq, const float *Yf, const int32_t *order,
                                 const int32_t *cluster_start, const int32_t *seg_start, const double *meanQ,
                                 const double *meanF, int D, int K, const SegGeom &g, double *part,
-                                cudaStream_t s)
+                                cudaStream_t s, const int32_t *settled)
 {
     SegParams p{};
     p.Yq = Yq;
@@ -682,6 +694,7 @@ cudaError_t launch_segment_sums(int mode, const float *Yq, const float *Yf, cons
     p.D = D;
     p.K = K;
     p.seg_rows = g.seg_rows;
+    p.settled = settled;
     const int units = (D % 4 == 0) ? D / 4 : D;
     p.tpr = tpr_for(units);
     switch (mode) {
@@ -719,13 +732,13 @@ size_t centroid_update_scratch_bytes(int D, int K) { return (size_t)K * ((D + 31
 cudaError_t launch_centroid_update(const double *part, const int32_t *seg_start, const int64_t *counts, int D,
                                    int K, int max_segs, double *sums, float *C, float *cnorm, const float *scale, void *Ch,
                                    const float *mean, float *cerr, void *norm_part, uint32_t *arrivals, Control *ctl,
-                                   cudaStream_t s)
+                                   cudaStream_t s, const int32_t *settled)
 {
     const CombGeom cg = comb_geometry(D, K, max_segs);
     const int cols = cg.cols;
     const cudaError_t e = launch_pdl(centroid_update_kernel, dim3((unsigned)K, (unsigned)((D + cols - 1) / cols)), dim3((unsigned)cg.threads), 0, s,
                                      part, seg_start, counts, D, K, cols, sums, C, cnorm, scale, reinterpret_cast<__half *>(Ch), mean, cerr,
-                                     reinterpret_cast<double2 *>(norm_part), arrivals, ctl);
+                                     reinterpret_cast<double2 *>(norm_part), arrivals, ctl, settled);
     count_launch();
     return e;
 }

@@ -111,6 +111,7 @@ __global__ void __launch_bounds__(AFFINE ? TC_THREADS_AFFINE : TC_THREADS_LABELS
 assign_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, TcParams p)
 {
     pdl_enter();
+    if (!AFFINE && p.settled && *p.settled) return;   // (the same word for every CTA: no earlier kernel of the stream runs any more)
     extern __shared__ unsigned char smem_raw[];
     // operand tiles need 1024-byte alignment for the 128-byte swizzle
     const uint32_t raw = smem_u32(smem_raw);
@@ -1468,10 +1469,12 @@ cudaError_t launch_assign_tc(const float *Y, int64_t N, int D, int K, const floa
                              const float *ynorm2, int32_t *labels, int32_t *refine_rows,
                              int32_t *cand_rows, uint64_t *cand_list, Control *ctl,
                              const float *gamma, const float *beta, float *out, cudaStream_t s,
-                             const void *Yh, const void *Ch, const float *scale, const float *cerr, const FastOut *fast, int64_t row_base)
+                             const void *Yh, const void *Ch, const float *scale, const float *cerr, const FastOut *fast, int64_t row_base,
+                             const int32_t *settled)
 {
     TcParams p{};
     p.row_base = row_base;
+    p.settled = settled;
     if (fast) p.fast = *fast;
     p.Y = Y;
     p.cnorm = cnorm;

@@ -372,6 +372,7 @@ struct TcParams {
     int a_stages;   // ring depths (<= TC_MAX_A_STAGES, TC_MAX_B_STAGES)
     int b_stages;
     FastOut fast;   // optional record of the fast pass (labels-only kernels)
+    const int32_t *settled;   // nothing to do once this is set (labels-only kernels; or null)
 };
 
 struct TcShared {
