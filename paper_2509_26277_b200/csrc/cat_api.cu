@@ -107,10 +107,11 @@ FitWs carve_fit(void *base, int64_t N, int D, int K)
     w.counts = c.take<int64_t>((size_t)K);
     w.norm_part = c.take<unsigned char>(centroid_update_scratch_bytes(D, K));
     w.arrivals = c.take<uint32_t>((size_t)K);
-    if (small_fit_supported(N, D, K)) {
-        // per-CTA partial sums and sizes of the persistent small-problem kernel
-        w.small_part = c.take<double>(small_part_doubles(D, K));
-        w.small_counts = c.take<int32_t>(small_part_counts(K));
+    const size_t tiles = fit_tiles_part_doubles(D, K);   // (by D and K alone: a workspace for more rows serves fewer)
+    if (tiles || small_fit_supported(N, D, K)) {
+        const size_t a = small_fit_supported(N, D, K) ? small_part_doubles(D, K) : 0, b = small_part_counts(K), t = fit_tiles_counts(K);
+        w.small_part = c.take<double>(a > tiles ? a : tiles);
+        w.small_counts = c.take<int32_t>(b > t ? b : t);
     }
     w.bytes = align_up(c.off, 256);
     return w;
@@ -163,6 +164,10 @@ static bool use_fit_rows(int64_t N, int D, int K)
 {
     return (g_small_kernels.load(std::memory_order_relaxed) & 2) && fit_rows_supported(N, D, K) &&
            (N <= 4096 || !use_small_fit(N, D, K));
+}
+static bool use_fit_tiles(int64_t N, int D, int K)
+{
+    return (g_small_kernels.load(std::memory_order_relaxed) & 2) && N > 8192 && fit_tiles_supported(N, D, K);
 }
 static bool use_small_apply(int64_t N, int D, int K)
 {
@@ -497,9 +502,13 @@ cat_status_t cat_fit_from(const float *Yq, const float *Yfp, int64_t N, int32_t 
 
     // Small problems without per-round diagnostics: every round, the final assignment and the
     // per-cluster sums and sizes that follow its labels come from one persistent launch.
-    const bool rows = !diag && use_fit_rows(N, D, K);
-    const bool small = rows || (!diag && use_small_fit(N, D, K));
-    if (rows) {
+    const bool tiles = !diag && use_fit_tiles(N, D, K);
+    const bool rows = !diag && !tiles && use_fit_rows(N, D, K);
+    const bool small = tiles || rows || (!diag && use_small_fit(N, D, K));
+    if (tiles) {
+        CAT_CUDA(launch_sample_mean(Yq, N, D, w.a.mean, s));
+        CAT_CUDA(launch_fit_tiles(Yq, N, D, K, C, w.a.mean, iters + 1, labels, w.small_part, w.small_counts, w.sumQ, w.counts, w.a.ctl, s));
+    } else if (rows) {
         // (scratch: the list of changed rows where the general path sorts, its counts where segments are
         // summed, the padded centroids where the moments come to lie)
         CAT_CUDA(launch_fit_rows(Yq, N, D, K, C, iters + 1, labels, w.sumQ, w.counts, w.order, w.segpart,
@@ -785,6 +794,7 @@ const char *cat_kernel_for(int32_t call, int64_t N, int32_t D, int32_t K)
         if (use_apply_rows(N, D, K, true)) return "apply_rows_kernel";
         break;
     case CAT_CALL_FIT:
+        if (use_fit_tiles(N, D, K)) return "fit_tiles_kernel";
         if (use_fit_rows(N, D, K)) return "fit_rows_kernel";
         if (use_small_fit(N, D, K)) return "small_kernel";
         break;

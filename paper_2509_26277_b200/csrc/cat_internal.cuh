@@ -153,8 +153,8 @@ struct FitWs {
     int64_t *counts;       // [K]
     void *norm_part;       // parts of the centroid norms (centroid update)
     uint32_t *arrivals;    // [K] CTAs of a cluster that have left theirs
-    double *small_part;    // [SMALL_MAX_GRID][K*D] per-CTA sums of the persistent small-problem kernel (or null)
-    int32_t *small_counts; // [SMALL_MAX_GRID][K+1]
+    double *small_part;    // per-CTA sums of the single-launch fits that keep them in planes (or null)
+    int32_t *small_counts; // ... and their counters
     size_t bytes;
 };
 FitWs carve_fit(void *base, int64_t N, int D, int K);
@@ -197,6 +197,14 @@ cudaError_t launch_small_apply(const float *Y, int64_t N, int D, int K, const fl
 bool fit_rows_supported(int64_t N, int D, int K);
 cudaError_t launch_fit_rows(const float *Y, int64_t N, int D, int K, float *C, int passes, int32_t *labels, double *sums,
                             int64_t *counts, void *list, void *list_count, float *padded, Control *ctl, cudaStream_t s);
+
+// The same for many rows of few columns, held as fp16 operand fragments (cat_fit_tiles.cu); ctl must have been reset, mean
+// is a point among the rows (launch_sample_mean).  part: fit_tiles_part_doubles, part_counts: fit_tiles_counts.
+bool fit_tiles_supported(int64_t N, int D, int K);
+size_t fit_tiles_part_doubles(int D, int K);   // (0: no such shape whatever N is)
+size_t fit_tiles_counts(int K);
+cudaError_t launch_fit_tiles(const float *Y, int64_t N, int D, int K, float *C, const float *mean, int passes, int32_t *labels, double *part,
+                             int32_t *part_counts, double *sums, int64_t *counts, Control *ctl, cudaStream_t s);
 
 // Inference on groups of eight rows held in shared memory, exact decisions included (cat_apply_rows.cu).
 // Resets ctl.  out_bf16: `out` is a [N, D] bf16 matrix; prep: apply_rows_prep_bytes of scratch.
