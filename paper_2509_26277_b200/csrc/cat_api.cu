@@ -107,6 +107,7 @@ FitWs carve_fit(void *base, int64_t N, int D, int K)
     w.counts = c.take<int64_t>((size_t)K);
     w.norm_part = c.take<unsigned char>(centroid_update_scratch_bytes(D, K));
     w.arrivals = c.take<uint32_t>((size_t)K);
+    w.moved_flags = c.take<uint64_t>(moved_flag_words());
     const size_t tiles = fit_tiles_part_doubles(D, K);   // (by D and K alone: a workspace for more rows serves fewer)
     if (tiles || small_fit_supported(N, D, K)) {
         const size_t a = small_fit_supported(N, D, K) ? small_part_doubles(D, K) : 0, b = small_part_counts(K), t = fit_tiles_counts(K);
@@ -316,6 +317,12 @@ static cat_status_t run_delta_update(const float *Yq, const int32_t *labels, con
     CAT_CUDA(launch_centroid_update(w.segpart, w.seg_start, w.counts, D, K, g.max_segs, w.sumQ, C, w.a.cnorm, w.hscale,
                                     half ? w.ch : nullptr, half ? w.a.mean : nullptr, w.a.cerr, w.norm_part, w.arrivals, w.a.ctl, s, settled));
     return CAT_OK;
+}
+
+// Rounds whose moved rows are listed instead of sorted: from the fourth on, where a tenth of the rows or fewer moves.
+static bool use_moved_list(int round, int64_t N, int D, int K, bool may_settle)
+{
+    return may_settle && round >= 3 && K >= 8;
 }
 
 static cat_status_t run_centred(const float *Yq, const float *Yfp, int64_t N, int D, int K, const FitWs &w,
@@ -544,7 +551,8 @@ cat_status_t cat_fit_from(const float *Yq, const float *Yfp, int64_t N, int32_t 
     CAT_CUDA(cudaMemsetAsync(lab[(iters & 1) ^ 1], 0xFF, (size_t)N * sizeof(int32_t), s));
     CAT_CUDA(cudaMemsetAsync(w.sumQ, 0, KD * sizeof(double), s));
     CAT_CUDA(cudaMemsetAsync(w.counts, 0, (size_t)K * sizeof(int64_t), s));
-    CAT_CUDA(cudaMemsetAsync(w.arrivals, 0, (size_t)K * sizeof(uint32_t), s));
+    // (arrivals, and behind them the flags)
+    CAT_CUDA(cudaMemsetAsync(w.arrivals, 0, (size_t)((char *)(w.moved_flags + moved_flag_words()) - (char *)w.arrivals), s));
     for (int t = 0; t < iters; ++t) {
         int32_t *cur = lab[(iters - t) & 1], *prev = lab[((iters - t) & 1) ^ 1];
         st = run_assign(Yq, N, D, K, C, cur, w.a, nullptr, nullptr, nullptr, s, tc, false, Yh, w.ch, w.hscale,
@@ -553,8 +561,13 @@ cat_status_t cat_fit_from(const float *Yq, const float *Yfp, int64_t N, int32_t 
         if (diag && t < CAT_DIAG_MAX_ROUNDS - 1)
             CAT_CUDA(launch_fit_diag_round(Yq, N, D, K, C, cur, w.a.refine_rows, w.a.cand_rows, w.a.ctl, diag, t,
                                            diag_recorded, s));
-        st = run_delta_update(Yq, cur, prev, N, D, K, w, C, half, s, settled);
-        if (st != CAT_OK) return st;
+        if (use_moved_list(t, N, D, K, settled != nullptr)) {
+            CAT_CUDA(launch_moved_update(Yq, cur, prev, N, D, K, (uint32_t)t, w.order, w.moved_flags, w.counts, w.sumQ, C, w.a.cnorm, w.hscale,
+                                         half ? w.ch : nullptr, half ? w.a.mean : nullptr, w.a.cerr, w.norm_part, w.arrivals, w.a.ctl, settled, s));
+        } else {
+            st = run_delta_update(Yq, cur, prev, N, D, K, w, C, half, s, settled);
+            if (st != CAT_OK) return st;
+        }
     }
 
     // final assignment, then the closed form

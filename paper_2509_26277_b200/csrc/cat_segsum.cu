@@ -32,6 +32,7 @@ namespace {
 
 constexpr int SORT_BLOCK = 1024;     // rows per histogram / scatter block
 constexpr int SEG_THREADS = 256;
+constexpr int COMB_THREADS = 512;
 
 // Key of virtual entry e: entries [0, N) are the rows under their current label; in delta
 // mode (prev != NULL) a row whose label did not change has no entry, and entries [N, 2N)
@@ -413,8 +414,6 @@ __global__ void segment_combine_kernel(const double *__restrict__ part, const in
 // in that order.  (One thread per column is a chain of loads as long as the cluster has segments: with K = 2 and
 // 100 000 rows 224 us for the three planes and 19 us a Lloyd round.  More threads than segments are a longer
 // exchange for nothing: 8192 x 64, K = 200 takes 8.6 us a round with 16 of them, 6.3 with two and whole rows.)
-constexpr int COMB_THREADS = 512;
-
 // P planes of a segment lie `plane` apart; four segments' loads are in flight together
 template <int P>
 __device__ __forceinline__ void sum_segments(const double *__restrict__ p, int s0, int s1, int step, size_t stride, size_t plane,
@@ -497,58 +496,47 @@ __global__ void __launch_bounds__(COMB_THREADS) segment_combine3_kernel(const do
     }
 }
 
-// Delta-mode centroid update: S_k += (partials of key k) - (partials of key K + k); c_k = float(S_k / n_k) where
+// What a Lloyd round does with a cluster once the change d of its sums is known: S_k += d; c_k = float(S_k / n_k) where
 // n_k > 0; and for the next assignment the squared norm of c_k (fp64, rounded up), optionally the fp16 copy
-// fp16(c_k * scale[0]) with the norm of its rounding error -- both of c_k less `mean` if that is given -- and the
-// reset of the exact-pass queues.  The CTAs of a cluster leave their parts of the two norms in `norm_part`; the last
-// one to arrive (`arrivals`, which wraps back to zero) adds them up, in an order that does not depend on who came when.
-// (32 registers a thread: four CTAs per SM, so that the 592 CTAs of the geometry above are one wave)
-__global__ void __launch_bounds__(COMB_THREADS, 4) centroid_update_kernel(const double *__restrict__ part,
-                                                              const int32_t *__restrict__ seg_start,
-                                                              const int64_t *__restrict__ counts, int D, int K, int cols,
-                                                              double *__restrict__ sums, float *__restrict__ C,
-                                                              float *__restrict__ cnorm, const float *__restrict__ scale,
-                                                              __half *__restrict__ Ch, const float *__restrict__ mean,
-                                                              float *__restrict__ cerr, double2 *__restrict__ norm_part,
-                                                              unsigned int *__restrict__ arrivals, Control *ctl,
-                                                              const int32_t *settled)
+// fp16(c_k * scale[0]) with the norm of its rounding error -- both of c_k less `mean` if that is given.  The CTAs
+// (k, 0 ... gridDim.y - 1) of a cluster have `cols` columns each, thread j of the first `cols` the j-th; they leave their
+// parts of the two norms in `norm_part`, and the last one to arrive (`arrivals`, which wraps back to zero) adds them up, in an
+// order that does not depend on who came when.
+struct FinishParams {
+    double *sums;
+    float *C;
+    float *cnorm;
+    const float *scale;
+    __half *Ch;
+    const float *mean;
+    float *cerr;
+    double2 *norm_part;
+    unsigned int *arrivals;
+    int64_t *counts_out;   // the cluster's size is left here by whoever finishes last (or null)
+    int D, cols;
+};
+
+__device__ __forceinline__ void finish_centroid(const FinishParams &f, double d, int64_t n, double *red, float *red_err, int *s_last)
 {
-    pdl_enter();
-    __shared__ double red[COMB_THREADS];
-    __shared__ float red_err[COMB_THREADS / 32];
-    __shared__ int s_last;
-    const int k = blockIdx.x, cb = blockIdx.y, g = threadIdx.x / cols, G = (int)blockDim.x / cols;
-    if (k == 0 && cb == 0 && threadIdx.x == 0) {
-        ctl->refine_count = 0;
-        ctl->cand_count = 0;
-    }
-    if (settled && *settled) return;
-    const int j = cb * cols + (threadIdx.x & (cols - 1));
-    const int64_t n = counts[k];
-    const float sc = Ch ? scale[0] : 1.f;
-    double in[1] = {0.0}, gone[1] = {0.0};
-    if (j < D) {
-        sum_segments<1>(part + j, seg_start[k] + g, seg_start[k + 1], G, (size_t)2 * D, 0, in);
-        sum_segments<1>(part + j, seg_start[K + k] + g, seg_start[K + k + 1], G, (size_t)2 * D, 0, gone);
-    }
-    double d = in[0] - gone[0];
-    d = sum_column(d, cols, red);
+    const int D = f.D, cols = f.cols;
+    const int k = blockIdx.x, cb = blockIdx.y, j = cb * cols + (int)threadIdx.x;
+    const float sc = f.Ch ? f.scale[0] : 1.f;
     double nrm = 0.0;
     float left2 = 0.f;
-    if (g == 0 && j < D) {
+    if ((int)threadIdx.x < cols && j < D) {
         const size_t e = (size_t)k * D + j;
-        const double sum = sums[e] + d;
-        sums[e] = sum;
-        float c = C[e];
+        const double sum = f.sums[e] + d;
+        f.sums[e] = sum;
+        float c = f.C[e];
         if (n > 0) {
             c = (float)(sum / (double)n);
-            C[e] = c;
+            f.C[e] = c;
         }
-        if (mean) c -= __ldg(mean + j);
+        if (f.mean) c -= __ldg(f.mean + j);
         nrm = (double)c * (double)c;
-        if (Ch) {
+        if (f.Ch) {
             const __half h = __float2half_rn(c * sc);
-            Ch[(size_t)k * half_ld(D) + j] = h;
+            f.Ch[(size_t)k * half_ld(D) + j] = h;
             const float l = c * sc - __half2float(h);
             left2 = l * l;
         }
@@ -571,21 +559,22 @@ __global__ void __launch_bounds__(COMB_THREADS, 4) centroid_update_kernel(const 
             l += (double)red_err[w];
         }
         if (gridDim.y == 1) {
-            cnorm[k] = __double2float_ru(t);
-            if (Ch) cerr[k] = sqrtf((float)l) / sc * 1.001f;
+            f.cnorm[k] = __double2float_ru(t);
+            if (f.Ch) f.cerr[k] = sqrtf((float)l) / sc * 1.001f;
+            if (f.counts_out) f.counts_out[k] = n;
         } else {
-            norm_part[(size_t)k * gridDim.y + cb] = make_double2(t, l);
+            f.norm_part[(size_t)k * gridDim.y + cb] = make_double2(t, l);
             __threadfence();
-            s_last = atomicInc(arrivals + k, gridDim.y - 1) == gridDim.y - 1;
+            *s_last = atomicInc(f.arrivals + k, gridDim.y - 1) == gridDim.y - 1;
         }
     }
     if (gridDim.y == 1) return;
     __syncthreads();
-    if (s_last && threadIdx.x < 32) {
+    if (*s_last && threadIdx.x < 32) {
         __threadfence();
         double t = 0.0, l = 0.0;
         for (int q = threadIdx.x; q < (int)gridDim.y; q += 32) {
-            const double2 v = __ldcg(norm_part + (size_t)k * gridDim.y + q);
+            const double2 v = __ldcg(f.norm_part + (size_t)k * gridDim.y + q);
             t += v.x;
             l += v.y;
         }
@@ -595,9 +584,231 @@ __global__ void __launch_bounds__(COMB_THREADS, 4) centroid_update_kernel(const 
             l += __shfl_xor_sync(0xffffffffu, l, o);
         }
         if (threadIdx.x != 0) return;
-        cnorm[k] = __double2float_ru(t);
-        if (Ch) cerr[k] = sqrtf((float)l) / sc * 1.001f;
+        f.cnorm[k] = __double2float_ru(t);
+        if (f.Ch) f.cerr[k] = sqrtf((float)l) / sc * 1.001f;
+        if (f.counts_out) f.counts_out[k] = n;
     }
+}
+
+// Delta-mode centroid update from the segments' partial sums: the change of a cluster's sums is (partials of key k) -
+// (partials of key K + k).  Also resets the exact-pass queues.
+// (32 registers a thread: four CTAs per SM, so that the 592 CTAs of the geometry above are one wave)
+__global__ void __launch_bounds__(COMB_THREADS, 4) centroid_update_kernel(const double *__restrict__ part,
+                                                              const int32_t *__restrict__ seg_start,
+                                                              const int64_t *__restrict__ counts, int K, FinishParams f,
+                                                              Control *ctl, const int32_t *settled)
+{
+    pdl_enter();
+    __shared__ double red[COMB_THREADS];
+    __shared__ float red_err[COMB_THREADS / 32];
+    __shared__ int s_last;
+    const int D = f.D, cols = f.cols;
+    const int k = blockIdx.x, cb = blockIdx.y, g = threadIdx.x / cols, G = (int)blockDim.x / cols;
+    if (k == 0 && cb == 0 && threadIdx.x == 0) {
+        ctl->refine_count = 0;
+        ctl->cand_count = 0;
+    }
+    if (settled && *settled) return;
+    const int j = cb * cols + (threadIdx.x & (cols - 1));
+    const int64_t n = counts[k];
+    double in[1] = {0.0}, gone[1] = {0.0};
+    if (j < D) {
+        sum_segments<1>(part + j, seg_start[k] + g, seg_start[k + 1], G, (size_t)2 * D, 0, in);
+        sum_segments<1>(part + j, seg_start[K + k] + g, seg_start[K + k + 1], G, (size_t)2 * D, 0, gone);
+    }
+    finish_centroid(f, sum_column(in[0] - gone[0], cols, red), n, red, red_err, &s_last);
+}
+
+// ---- rounds in which few rows move: two launches in place of five
+//
+// The sort, its tables and the segments cost 25 to 45 us a round whatever moves (histograms of 2 K keys for every 1024
+// rows of two label buffers; five launches).  Once the clustering has found its shape a hundredth of the rows moves: those are
+// listed, in row order, and a cluster's CTAs pick theirs out of the list.
+
+constexpr int MOVE_THREADS = 512;
+constexpr int MOVE_GRID = 148;
+constexpr int MOVE_CHUNK = 2048;
+
+// list[] = {row, new label | old label << 16} of the rows whose label changed, in row order; *total their number, and
+// *settled set if there is none.  A CTA has `per` consecutive rows, a thread `per` / 512 of them; the CTAs' counts
+// pass through flag[] (count | tag << 32; tags differ between the launches that share the words), waits are bounded.
+__global__ void __launch_bounds__(MOVE_THREADS) moved_list_kernel(const int32_t *__restrict__ cur, const int32_t *__restrict__ prev, int64_t N,
+                                                                  int per, uint32_t tag, uint2 *__restrict__ list,
+                                                                  unsigned long long *flag, int32_t *total, int32_t *settled,
+                                                                  Control *ctl)
+{
+    pdl_enter();
+    if (*settled) return;   // (set by the last CTA of an earlier launch: this one's sets it behind its wait for all others)
+    __shared__ int s_warp[MOVE_THREADS / 32], s_before;
+    __shared__ int s_ok;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, R = per / MOVE_THREADS;
+    const int64_t r0 = (int64_t)blockIdx.x * per + (int64_t)tid * R;
+    if (tid == 0) {
+        s_before = 0;
+        s_ok = 1;
+    }
+    // (R is a multiple of 4; the label buffers are 16-byte aligned)
+    int n = 0;
+    for (int q = 0; q < R; q += 4) {
+        const int64_t r = r0 + q;
+        if (r + 4 <= N) {
+            const int4 a = __ldg(reinterpret_cast<const int4 *>(cur + r)), b = __ldg(reinterpret_cast<const int4 *>(prev + r));
+            n += (a.x != b.x) + (a.y != b.y) + (a.z != b.z) + (a.w != b.w);
+        } else
+            for (int64_t i = r; i < N && i < r + 4; ++i) n += cur[i] != prev[i];
+    }
+    int incl = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    int at = incl - n, all = 0;
+#pragma unroll
+    for (int w = 0; w < MOVE_THREADS / 32; ++w) {
+        const int c = s_warp[w];
+        if (w < warp) at += c;
+        all += c;
+    }
+    if (tid == 0) atomicExch(flag + blockIdx.x, (unsigned long long)tag << 32 | (unsigned)all);
+    if (tid < (int)blockIdx.x) {
+        uint64_t t0 = 0;
+        for (uint32_t it = 0;; ++it) {
+            const unsigned long long v = *(volatile unsigned long long *)(flag + tid);
+            if ((uint32_t)(v >> 32) == tag) {
+                if ((uint32_t)v) atomicAdd(&s_before, (int)(uint32_t)v);
+                break;
+            }
+            if ((it & 255u) == 255u) {
+                uint64_t now;
+                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+                if (t0 == 0) t0 = now;
+                if (*(volatile int *)&ctl->device_status != (int)CAT_OK || now - t0 > 2000000000ull) {
+                    atomicExch(&ctl->device_status, (int)CAT_ERR_DEVICE_TIMEOUT);
+                    s_ok = 0;
+                    break;
+                }
+            }
+        }
+    }
+    __syncthreads();
+    at += s_before;
+    if (blockIdx.x == gridDim.x - 1 && tid == 0) {
+        const int m = s_ok ? s_before + all : 0;
+        *total = m;
+        if (m == 0 && s_ok) *settled = 1;
+    }
+    if (!s_ok || n == 0) return;
+    for (int q = 0; q < R; ++q) {
+        const int64_t r = r0 + q;
+        if (r >= N) break;
+        const int c = cur[r], p = prev[r];
+        if (c != p) list[at++] = make_uint2((uint32_t)r, ((uint32_t)c & 0xFFFFu) | (uint32_t)p << 16);
+    }
+}
+
+// A CTA per `cols` columns of a cluster: its rows of the list, in order, entering and leaving, then as above.  tpr threads
+// (of VEC columns) have a row, 256 / tpr rows at a time, each group of threads into sums of its own.
+template <int VEC>
+__global__ void __launch_bounds__(SEG_THREADS) cluster_move_kernel(const float *__restrict__ Y, int64_t N, const uint2 *__restrict__ list,
+                                                                   const int32_t *__restrict__ total, const int64_t *__restrict__ counts,
+                                                                   int tpr, FinishParams f, Control *ctl, const int32_t *settled)
+{
+    pdl_enter();
+    __shared__ double red[SEG_THREADS * VEC];
+    __shared__ float red_err[SEG_THREADS / 32];
+    __shared__ uint32_t sel[MOVE_CHUNK];   // row, bit 31: it leaves
+    __shared__ int s_cnt[MOVE_CHUNK / 32], s_last;
+    const int k = blockIdx.x, cb = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (k == 0 && cb == 0 && tid == 0) {
+        ctl->refine_count = 0;
+        ctl->cand_count = 0;
+    }
+    if (*settled) return;
+    const int D = f.D, M = *total, g = tid / tpr, G = SEG_THREADS / tpr, col = cb * f.cols + (tid & (tpr - 1)) * VEC;
+    int64_t n = counts[k];
+    double acc[VEC];
+#pragma unroll
+    for (int q = 0; q < VEC; ++q) acc[q] = 0.0;
+    constexpr int PER = MOVE_CHUNK / SEG_THREADS;   // entries a thread looks at: e0 + 256 u + tid
+    for (int e0 = 0; e0 < M; e0 += MOVE_CHUNK) {
+        uint2 w[PER];
+        uint32_t m[PER];
+#pragma unroll
+        for (int u = 0; u < PER; ++u) w[u] = e0 + u * SEG_THREADS + tid < M ? __ldg(list + e0 + u * SEG_THREADS + tid) : make_uint2(0xFFFFFFFFu, 0u);
+        __syncthreads();   // (the rows of the chunk before are through)
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            const bool hit = (int64_t)w[u].x < N && ((int)(w[u].y & 0xFFFFu) == k || (int)(w[u].y >> 16) == k);
+            m[u] = __ballot_sync(0xffffffffu, hit);
+            if (lane == 0) s_cnt[u * (SEG_THREADS / 32) + warp] = __popc(m[u]);
+        }
+        __syncthreads();
+        if (warp == 0) {
+            // exclusive scan of the 64 counts, in the entries' order
+            const int a = s_cnt[2 * lane], b = s_cnt[2 * lane + 1];
+            int incl = a + b;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += t;
+            }
+            s_cnt[2 * lane] = incl - a - b;
+            s_cnt[2 * lane + 1] = incl - b;
+            if (lane == 31) s_last = incl;
+        }
+        __syncthreads();
+        const int hits = s_last;
+#pragma unroll
+        for (int u = 0; u < PER; ++u)
+            if (m[u] >> lane & 1u)
+                sel[s_cnt[u * (SEG_THREADS / 32) + warp] + __popc(m[u] & ((1u << lane) - 1u))] =
+                    w[u].x | ((int)(w[u].y & 0xFFFFu) == k ? 0u : 0x80000000u);
+        __syncthreads();
+        for (int e = g; e < hits; e += 4 * G) {
+            float4 y[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int i = e + u * G;
+                y[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (i < hits && col < D) {
+                    const float *src = Y + (size_t)(sel[i] & 0x7FFFFFFFu) * D + col;
+                    if (VEC == 4) y[u] = __ldg(reinterpret_cast<const float4 *>(src));
+                    else y[u].x = __ldg(src);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int i = e + u * G;
+                if (i >= hits) break;
+                const float v[4] = {y[u].x, y[u].y, y[u].z, y[u].w};
+                const bool leaves = sel[i] >> 31;
+#pragma unroll
+                for (int q = 0; q < VEC; ++q) acc[q] += leaves ? -(double)v[q] : (double)v[q];
+            }
+        }
+        int dn = 0;
+        for (int e = tid; e < hits; e += SEG_THREADS) dn += sel[e] >> 31 ? -1 : 1;
+        // the change of the cluster's size (integers: any order will do)
+        __syncthreads();
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) dn += __shfl_xor_sync(0xffffffffu, dn, o);
+        if (lane == 0) s_cnt[warp] = dn;
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < SEG_THREADS / 32; ++q) n += s_cnt[q];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < VEC; ++q) red[tid * VEC + q] = acc[q];
+    __syncthreads();
+    double d = 0.0;
+    if (tid < f.cols)
+        for (int q = 0; q < G; ++q) d += red[q * f.cols + tid];   // (thread tid of a group's tpr has columns VEC tid ... )
+    __syncthreads();
+    finish_centroid(f, d, n, red, red_err, &s_last);
 }
 
 int tpr_for(int units)
@@ -736,10 +947,40 @@ cudaError_t launch_centroid_update(const double *part, const int32_t *seg_start,
 {
     const CombGeom cg = comb_geometry(D, K, max_segs);
     const int cols = cg.cols;
+    const FinishParams f{sums, C, cnorm, scale, reinterpret_cast<__half *>(Ch), mean, cerr, reinterpret_cast<double2 *>(norm_part), arrivals,
+                         nullptr, D, cols};
     const cudaError_t e = launch_pdl(centroid_update_kernel, dim3((unsigned)K, (unsigned)((D + cols - 1) / cols)), dim3((unsigned)cg.threads), 0, s,
-                                     part, seg_start, counts, D, K, cols, sums, C, cnorm, scale, reinterpret_cast<__half *>(Ch), mean, cerr,
-                                     reinterpret_cast<double2 *>(norm_part), arrivals, ctl, settled);
+                                     part, seg_start, counts, K, f, ctl, settled);
     count_launch();
+    return e;
+}
+
+size_t moved_flag_words() { return MOVE_GRID + 1; }
+
+// One centroid update from the rows whose label changed, for rounds in which few do.
+cudaError_t launch_moved_update(const float *Y, const int32_t *cur, const int32_t *prev, int64_t N, int D, int K, uint32_t tag, void *list,
+                                void *flags, int64_t *counts, double *sums, float *C, float *cnorm, const float *scale, void *Ch,
+                                const float *mean, float *cerr, void *norm_part, uint32_t *arrivals, Control *ctl, int32_t *settled,
+                                cudaStream_t s)
+{
+    int64_t per = ((N + MOVE_GRID - 1) / MOVE_GRID + 4 * MOVE_THREADS - 1) / (4 * MOVE_THREADS) * (4 * MOVE_THREADS);
+    const unsigned grid = (unsigned)((N + per - 1) / per);
+    unsigned long long *flag = reinterpret_cast<unsigned long long *>(flags);
+    int32_t *total = reinterpret_cast<int32_t *>(flag + MOVE_GRID);
+    cudaError_t e = launch_pdl(moved_list_kernel, dim3(grid), dim3(MOVE_THREADS), 0, s, cur, prev, N, (int)per, tag,
+                               reinterpret_cast<uint2 *>(list), flag, total, settled, ctl);
+    if (e != cudaSuccess) return e;
+    // columns per CTA: as many CTAs as there are SMs, no fewer columns than a warp has
+    const int vec = D % 4 == 0 ? 4 : 1;
+    int cols = 256;
+    while (cols > 32 && (int64_t)K * ((D + cols - 1) / cols) < 2 * 148) cols >>= 1;
+    while (cols > 32 && cols / 2 >= D) cols >>= 1;
+    const FinishParams f{sums, C, cnorm, scale, reinterpret_cast<__half *>(Ch), mean, cerr, reinterpret_cast<double2 *>(norm_part), arrivals,
+                         counts, D, cols};
+    const dim3 blocks((unsigned)K, (unsigned)((D + cols - 1) / cols));
+    e = launch_pdl(vec == 4 ? cluster_move_kernel<4> : cluster_move_kernel<1>, blocks, dim3(SEG_THREADS), 0, s, Y, N,
+                   reinterpret_cast<const uint2 *>(list), total, counts, cols / vec, f, ctl, settled);
+    count_launch(2);
     return e;
 }
 
