@@ -166,9 +166,9 @@ static bool use_fit_rows(int64_t N, int D, int K)
     return (g_small_kernels.load(std::memory_order_relaxed) & 2) && fit_rows_supported(N, D, K) &&
            (N <= 4096 || !use_small_fit(N, D, K));
 }
-static bool use_fit_tiles(int64_t N, int D, int K)
+static bool use_fit_tiles(int64_t N, int D, int K, bool clusters_only)
 {
-    return (g_small_kernels.load(std::memory_order_relaxed) & 2) && N > 8192 && fit_tiles_supported(N, D, K);
+    return (g_small_kernels.load(std::memory_order_relaxed) & 2) && (N > 8192 || (clusters_only && N >= 2048)) && fit_tiles_supported(N, D, K);
 }
 static bool use_small_apply(int64_t N, int D, int K)
 {
@@ -336,6 +336,42 @@ static cat_status_t run_centred(const float *Yq, const float *Yfp, int64_t N, in
     return CAT_OK;
 }
 
+// gamma and beta for given labels.  have_sums: the workspace has the clusters' sums of Yq and sizes already.
+static cat_status_t run_closed_form(const float *Yq, const float *Yfp, int64_t N, int D, int K, const int32_t *labels, const FitWs &w,
+                                    bool have_sums, float *gamma_out, float *beta_out, cudaStream_t s)
+{
+    if (have_sums) CAT_CUDA(launch_means_from_sums(w.sumQ, w.counts, D, K, w.meanQ, s));
+    cat_status_t st = run_sort(labels, N, D, K, w, w.counts, s);
+    if (st != CAT_OK) return st;
+    if (!have_sums) {
+        if ((st = run_sums(Yq, N, D, K, w, w.counts, w.sumQ, nullptr, s)) != CAT_OK) return st;
+        CAT_CUDA(launch_means_from_sums(w.sumQ, w.counts, D, K, w.meanQ, s));
+    }
+    // one sweep over Yq and Yfp forms the centred moments and the sums of Yfp
+    const SegGeom g = seg_geometry(N, D, K);
+    CAT_CUDA(launch_segment_sums(3, Yq, Yfp, w.order, w.cluster_start, w.seg_start, w.meanQ, nullptr, D, K, g, w.segpart, s));
+    CAT_CUDA(launch_segment_combine3(w.segpart, w.seg_start, D, K, g.max_segs, w.var, w.cov, w.sumF, s));
+    CAT_CUDA(launch_solve(w.sumQ, w.sumF, w.var, w.cov, w.counts, D, K, gamma_out, beta_out, s));
+    return CAT_OK;
+}
+
+cat_status_t fit_closed_form(const float *Yq, const float *Yfp, int64_t N, int D, int K, const int32_t *labels, float *gamma_out,
+                             float *beta_out, void *workspace, cudaStream_t s)
+{
+    return run_closed_form(Yq, Yfp, N, D, K, labels, carve_fit(workspace, N, D, K), false, gamma_out, beta_out, s);
+}
+
+// cat_fit_from; without Yfp the clusters alone.
+static cat_status_t fit_from(const float *Yq, const float *Yfp, int64_t N, int32_t D, int32_t K, int32_t iters,
+                             const float *init_centroids, float *centroids_out, float *gamma_out, float *beta_out,
+                             int32_t *labels_out, cat_fit_diag_t *diag, void *workspace, size_t workspace_bytes, void *stream);
+
+cat_status_t fit_clusters(const float *Y, int64_t N, int D, int K, int iters, float *centroids_out, int32_t *labels_out, void *workspace,
+                          size_t workspace_bytes, cudaStream_t s)
+{
+    return fit_from(Y, nullptr, N, D, K, iters, nullptr, centroids_out, nullptr, nullptr, labels_out, nullptr, workspace, workspace_bytes, s);
+}
+
 }  // namespace cat
 
 using namespace cat;
@@ -484,12 +520,22 @@ cat_status_t cat_fit_from(const float *Yq, const float *Yfp, int64_t N, int32_t 
                           void *stream)
 {
     if (!Yq || !Yfp || !centroids_out || !gamma_out || !beta_out) return CAT_ERR_NULL;
+    return fit_from(Yq, Yfp, N, D, K, iters, init_centroids, centroids_out, gamma_out, beta_out, labels_out, diag, workspace,
+                    workspace_bytes, stream);
+}
+
+}  // extern "C"
+
+static cat_status_t cat::fit_from(const float *Yq, const float *Yfp, int64_t N, int32_t D, int32_t K, int32_t iters,
+                                  const float *init_centroids, float *centroids_out, float *gamma_out, float *beta_out,
+                                  int32_t *labels_out, cat_fit_diag_t *diag, void *workspace, size_t workspace_bytes, void *stream)
+{
     cat_status_t st = check_shape(N, D, K, true);
     if (st != CAT_OK) return st;
     if (iters < 0) return CAT_ERR_SHAPE;
     if (N >= ((int64_t)1 << 30)) return CAT_ERR_UNSUPPORTED;   // a round may sort 2N entries with 32-bit positions
     if (!aligned16(Yq) || !aligned16(Yfp) || !aligned16(centroids_out) || !aligned16(gamma_out) ||
-        !aligned16(beta_out) || (labels_out && !aligned16(labels_out)) ||
+        !aligned16(beta_out) || (labels_out && !aligned16(labels_out)) ||   // (a null pointer is aligned)
         (init_centroids && !aligned16(init_centroids)) || (diag && !aligned16(diag)))
         return CAT_ERR_ALIGN;
     if (init_centroids == centroids_out) return CAT_ERR_SHAPE;
@@ -499,9 +545,9 @@ cat_status_t cat_fit_from(const float *Yq, const float *Yfp, int64_t N, int32_t 
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     FitWs w = carve_fit(workspace, N, D, K);
     const size_t KD = (size_t)K * D;
-    double *meanQ = w.meanQ;
     int32_t *labels = labels_out ? labels_out : w.a.labels;
     float *C = centroids_out;
+    const bool clusters_only = Yfp == nullptr;
 
     CAT_CUDA(launch_reset_control(w.a.ctl, s));
     CAT_CUDA(cudaMemcpyAsync(C, init_centroids ? init_centroids : Yq, KD * sizeof(float),
@@ -509,7 +555,7 @@ cat_status_t cat_fit_from(const float *Yq, const float *Yfp, int64_t N, int32_t 
 
     // Small problems without per-round diagnostics: every round, the final assignment and the
     // per-cluster sums and sizes that follow its labels come from one persistent launch.
-    const bool tiles = !diag && use_fit_tiles(N, D, K);
+    const bool tiles = !diag && use_fit_tiles(N, D, K, clusters_only);
     const bool rows = !diag && !tiles && use_fit_rows(N, D, K);
     const bool small = tiles || rows || (!diag && use_small_fit(N, D, K));
     if (tiles) {
@@ -577,6 +623,7 @@ cat_status_t cat_fit_from(const float *Yq, const float *Yfp, int64_t N, int32_t 
     if (diag)
         CAT_CUDA(launch_fit_diag_round(Yq, N, D, K, C, labels, w.a.refine_rows, w.a.cand_rows, w.a.ctl, diag,
                                        diag_recorded - 1, diag_recorded, s));
+    if (clusters_only) return CAT_OK;
     // The running sums follow the final labels too (without touching the centroids), which gives
     // the cluster means of Yq before the one sweep over Yq and Yfp that forms the centred moments
     // and the sums of Yfp.
@@ -589,19 +636,13 @@ cat_status_t cat_fit_from(const float *Yq, const float *Yfp, int64_t N, int32_t 
         CAT_CUDA(launch_segment_combine(w.segpart, w.seg_start, w.counts, D, K, true, w.sumQ, nullptr, nullptr, s));
     }
     }   // !small
-    CAT_CUDA(launch_means_from_sums(w.sumQ, w.counts, D, K, meanQ, s));
-    st = run_sort(labels, N, D, K, w, w.counts, s);
-    if (st != CAT_OK) return st;
-    {
-        SegGeom g = seg_geometry(N, D, K);
-        CAT_CUDA(launch_segment_sums(3, Yq, Yfp, w.order, w.cluster_start, w.seg_start, meanQ, nullptr, D, K, g,
-                                     w.segpart, s));
-        CAT_CUDA(launch_segment_combine3(w.segpart, w.seg_start, D, K, g.max_segs, w.var, w.cov, w.sumF, s));
-    }
-    CAT_CUDA(launch_solve(w.sumQ, w.sumF, w.var, w.cov, w.counts, D, K, gamma_out, beta_out, s));
+    if (clusters_only) return CAT_OK;
+    if ((st = run_closed_form(Yq, Yfp, N, D, K, labels, w, true, gamma_out, beta_out, s)) != CAT_OK) return st;
     if (diag) CAT_CUDA(launch_fit_diag(w.a.ctl, w.counts, K, diag, s));
     return CAT_OK;
 }
+
+extern "C" {
 
 cat_status_t cat_fit(const float *Yq, const float *Yfp, int64_t N, int32_t D, int32_t K,
                      int32_t iters, float *centroids_out, float *gamma_out, float *beta_out,
@@ -807,7 +848,7 @@ const char *cat_kernel_for(int32_t call, int64_t N, int32_t D, int32_t K)
         if (use_apply_rows(N, D, K, true)) return "apply_rows_kernel";
         break;
     case CAT_CALL_FIT:
-        if (use_fit_tiles(N, D, K)) return "fit_tiles_kernel";
+        if (use_fit_tiles(N, D, K, false)) return "fit_tiles_kernel";
         if (use_fit_rows(N, D, K)) return "fit_rows_kernel";
         if (use_small_fit(N, D, K)) return "small_kernel";
         break;

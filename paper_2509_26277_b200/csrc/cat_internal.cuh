@@ -160,6 +160,13 @@ struct FitWs {
 };
 FitWs carve_fit(void *base, int64_t N, int D, int K);
 
+// K-Means as cat_fit runs it, without the closed form (workspace of cat_fit); and the closed form for given labels (a
+// workspace of cat_fit for this shape).
+cat_status_t fit_clusters(const float *Y, int64_t N, int D, int K, int iters, float *centroids_out, int32_t *labels_out, void *workspace,
+                          size_t workspace_bytes, cudaStream_t s);
+cat_status_t fit_closed_form(const float *Yq, const float *Yfp, int64_t N, int D, int K, const int32_t *labels, float *gamma_out,
+                             float *beta_out, void *workspace, cudaStream_t s);
+
 // ---------------------------------------------------------------- kernel launchers (cat_kernels.cu)
 // All return a cudaError_t from the launch; none synchronises.
 

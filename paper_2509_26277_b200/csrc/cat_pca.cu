@@ -493,10 +493,7 @@ namespace {
 struct FitPcaWs {
     void *pca;  size_t pca_bytes;   // (first: its control block speaks for the whole call)
     float *Z;                       // [N, p]
-    float *gp, *bp;                 // [K, p] closed form of the reduced rows (not used further)
     int32_t *labels;                // [N]
-    double *sumQ, *sumF, *var, *cov, *meanQ, *meanF;   // [K, D]
-    int64_t *counts;                // [K]
     void *fit;  size_t fit_bytes;   // cat_fit workspace for (N, p, K), then for (N, D, K)
     size_t bytes;
 };
@@ -511,20 +508,10 @@ FitPcaWs carve_fit_pca(void *base, int64_t N, int D, int K, int p)
         return q;
     };
     FitPcaWs w{};
-    const size_t KD = (size_t)K * D;
     w.pca_bytes = cat_pca_workspace_bytes(N, D, p);
     w.pca = take(w.pca_bytes);
     w.Z = (float *)take((size_t)N * p * sizeof(float));
-    w.gp = (float *)take((size_t)K * p * sizeof(float));
-    w.bp = (float *)take((size_t)K * p * sizeof(float));
     w.labels = (int32_t *)take((size_t)N * sizeof(int32_t));
-    w.sumQ = (double *)take(KD * sizeof(double));
-    w.sumF = (double *)take(KD * sizeof(double));
-    w.var = (double *)take(KD * sizeof(double));
-    w.cov = (double *)take(KD * sizeof(double));
-    w.meanQ = (double *)take(KD * sizeof(double));
-    w.meanF = (double *)take(KD * sizeof(double));
-    w.counts = (int64_t *)take((size_t)K * sizeof(int64_t));
     const size_t a = cat_fit_workspace_bytes(N, p, K), c = cat_fit_workspace_bytes(N, D, K);
     w.fit_bytes = a > c ? a : c;
     w.fit = take(w.fit_bytes);
@@ -557,19 +544,12 @@ cat_status_t cat_fit_pca(const float *Yq, const float *Yfp, int64_t N, int32_t D
     // Algorithm 1 step 1: the projection; step 2: K-Means on the reduced rows
     if ((st = cat_pca_fit(Yq, N, D, p, mean_out, components_out, nullptr, w.pca, w.pca_bytes, stream)) != CAT_OK) return st;
     if ((st = cat_pca_project(Yq, N, D, p, mean_out, components_out, w.Z, stream)) != CAT_OK) return st;
-    if ((st = cat_fit(w.Z, w.Z, N, p, K, iters, centroids_out, w.gp, w.bp, labels, w.fit, w.fit_bytes, stream)) != CAT_OK)
-        return st;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    if ((st = fit_clusters(w.Z, N, p, K, iters, centroids_out, labels, w.fit, w.fit_bytes, s)) != CAT_OK) return st;
     CAT_CUDA(launch_absorb_control(reinterpret_cast<Control *>(w.pca), reinterpret_cast<const Control *>(w.fit), s));
     // the loop over the clusters: moments and the closed form in the original space
-    if ((st = cat_cluster_sums(Yq, labels, N, D, K, w.sumQ, w.counts, w.fit, w.fit_bytes, stream)) != CAT_OK) return st;
-    if ((st = cat_cluster_sums(Yfp, labels, N, D, K, w.sumF, w.counts, w.fit, w.fit_bytes, stream)) != CAT_OK) return st;
-    CAT_CUDA(launch_means_from_sums(w.sumQ, w.counts, D, K, w.meanQ, s));
-    CAT_CUDA(launch_means_from_sums(w.sumF, w.counts, D, K, w.meanF, s));
-    if ((st = cat_centred_moments(Yq, Yfp, labels, N, D, K, w.meanQ, w.meanF, w.var, w.cov, w.fit, w.fit_bytes, stream)) !=
-        CAT_OK)
-        return st;
-    return cat_solve_gamma_beta(w.sumQ, w.sumF, w.var, w.cov, w.counts, D, K, gamma_out, beta_out, stream);
+    if (!al16(Yfp) || !al16(gamma_out) || !al16(beta_out)) return CAT_ERR_ALIGN;
+    return fit_closed_form(Yq, Yfp, N, D, K, labels, gamma_out, beta_out, w.fit, s);
 }
 
 size_t cat_apply_pca_workspace_bytes(int64_t N, int32_t D, int32_t K, int32_t p)
