@@ -940,10 +940,10 @@ __device__ __forceinline__ void load_mean(const float *__restrict__ mean, int c,
 // rounded to nearest (rows of Yh ld elements apart), the norm rerr[i] of what the rounding left, and the
 // largest magnitude of the matrix (float bits, one atomicMax per CTA; amax_bits may be null).  With `mean` everything but that
 // magnitude is of Y[i, :] - mean: nearest centroids do not depend on the origin, and smaller operands make
-// smaller errors.  A row is handled by G lanes and read twice; the second read comes
-// out of L1/L2.  VEC4: 128-bit loads (D % 4 == 0); otherwise a lane takes pairs of columns with
-// scalar loads, whose warp-wide accesses still cover whole lines.
-template <bool VEC4>
+// smaller errors.  A row is handled by G lanes.  VEC4: 128-bit loads (D % 4 == 0); otherwise a lane takes pairs of columns
+// with scalar loads, whose warp-wide accesses still cover whole lines.  ONCE: a lane's part of a row (8 units at most) stays in
+// registers; longer rows are read twice, the second time out of L1/L2.
+template <bool VEC4, bool ONCE>
 __global__ void __launch_bounds__(256) half_shadow_kernel(const float *__restrict__ Y, int64_t N, int D, int ld, int G,
                                                           const float *__restrict__ mean, float *__restrict__ ynorm2,
                                                           float *__restrict__ rinv, float *__restrict__ rerr,
@@ -963,8 +963,8 @@ __global__ void __launch_bounds__(256) half_shadow_kernel(const float *__restric
         const bool live = row < N;
         const float *y = Y + (size_t)(live ? row : 0) * D;
         float s = 0.f, m = 0.f, big = 0.f;
+        float v[8][V];   // (ONCE: what follows the scale has them less the mean)
         for (int c = c0; c < DV; c += 8 * G) {
-            float v[8][V];
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const int cc = c + u * G;
@@ -987,6 +987,7 @@ __global__ void __launch_bounds__(256) half_shadow_kernel(const float *__restric
                 for (int q = 0; q < V; ++q) {
                     big = fmaxf(big, fabsf(v[u][q]));
                     const float x = v[u][q] - mu[q];
+                    if (ONCE) v[u][q] = x;
                     s = fmaf(x, x, s);
                     m = fmaxf(m, fabsf(x));
                 }
@@ -1009,24 +1010,10 @@ __global__ void __launch_bounds__(256) half_shadow_kernel(const float *__restric
         __half *h = Yh + (size_t)row * ld;
         float left2 = 0.f;
         if (live) {
-#pragma unroll 4
-            for (int c = c0; c < DV; c += G) {
-                float x[V];
-                if (VEC4) {
-                    const float4 t = __ldg(reinterpret_cast<const float4 *>(y) + c);
-                    x[0] = t.x;
-                    x[1] = t.y;
-                    x[V - 2] = t.z;
-                    x[V - 1] = t.w;
-                } else {
-                    x[0] = __ldg(y + 2 * c);
-                    x[1] = 2 * c + 1 < D ? __ldg(y + 2 * c + 1) : 0.f;
-                }
+            auto put = [&](int c, float (&x)[V]) {
                 uint32_t w[V / 2];
-                float mu[V];
-                load_mean<VEC4>(mean, c, D, mu);
 #pragma unroll
-                for (int q = 0; q < V; ++q) x[q] = (x[q] - mu[q]) * sc;
+                for (int q = 0; q < V; ++q) x[q] *= sc;
 #pragma unroll
                 for (int q = 0; q < V; q += 2) {
                     const __half2 hh = __floats2half2_rn(x[q], x[q + 1]);
@@ -1038,6 +1025,30 @@ __global__ void __launch_bounds__(256) half_shadow_kernel(const float *__restric
                 // (ld is even and at least D: a pair that starts inside the row fits)
                 if (VEC4) reinterpret_cast<uint2 *>(h)[c] = make_uint2(w[0], w[V / 2 - 1]);
                 else reinterpret_cast<uint32_t *>(h)[c] = w[0];
+            };
+            if (ONCE) {
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (c0 + u * G < DV) put(c0 + u * G, v[u]);
+            } else {
+#pragma unroll 4
+                for (int c = c0; c < DV; c += G) {
+                    float x[V], mu[V];
+                    if (VEC4) {
+                        const float4 t = __ldg(reinterpret_cast<const float4 *>(y) + c);
+                        x[0] = t.x;
+                        x[1] = t.y;
+                        x[V - 2] = t.z;
+                        x[V - 1] = t.w;
+                    } else {
+                        x[0] = __ldg(y + 2 * c);
+                        x[1] = 2 * c + 1 < D ? __ldg(y + 2 * c + 1) : 0.f;
+                    }
+                    load_mean<VEC4>(mean, c, D, mu);
+#pragma unroll
+                    for (int q = 0; q < V; ++q) x[q] -= mu[q];
+                    put(c, x);
+                }
             }
         }
 #pragma unroll
@@ -1304,14 +1315,19 @@ cudaError_t launch_half_shadow(const float *Y, int64_t N, int D, const float *me
     float *rinv = scale + 4, *rerr = scale + 4 + N;
     cudaError_t e = want_amax ? cudaMemsetAsync(scale, 0, 4 * sizeof(float), s) : cudaSuccess;
     if (e != cudaSuccess) return e;
-    const int G = lanes_per_row(D);
+    int G = lanes_per_row(D);
+    const int units = D % 4 == 0 ? D / 4 : (D + 1) / 2;
+    const bool once = units <= 8 * G;
+    // (as many loads in flight per lane as its registers hold, from whole lines)
+    while (once && G > 8 && units <= 4 * G) G >>= 1;
     const int rows_per_cta = 256 / G;
     int64_t blocks = (N + rows_per_cta - 1) / rows_per_cta;
     const int64_t cap = (int64_t)sm_count() * 8;
     if (blocks > cap) blocks = cap;
     // (An ordinary launch: a dependent one that starts beside the tail of a kernel with much shared memory keeps that
     // kernel's split of the L1, and the second read of a row misses -- 100 000 x 1001: K = 200: 335 us a cat_assign against 311.)
-    const auto kern = D % 4 == 0 ? half_shadow_kernel<true> : half_shadow_kernel<false>;
+    const auto kern = D % 4 == 0 ? (once ? half_shadow_kernel<true, true> : half_shadow_kernel<true, false>)
+                                 : (once ? half_shadow_kernel<false, true> : half_shadow_kernel<false, false>);
     kern<<<(unsigned)blocks, 256, 0, s>>>(Y, N, D, half_ld(D), G, mean, ynorm2, rinv, rerr,
                                           want_amax ? reinterpret_cast<unsigned int *>(scale) : nullptr, reinterpret_cast<__half *>(Yh));
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
