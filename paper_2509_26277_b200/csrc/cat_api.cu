@@ -175,6 +175,14 @@ static bool use_small_apply(int64_t N, int D, int K)
     return (g_small_kernels.load(std::memory_order_relaxed) & 1) && use_tensor_path(N, D, K) && small_apply_supported(N, D, K);
 }
 
+// Short rows in registers: from 8192 rows on (two groups of sixteen rows for every three warps of the device).
+static bool use_apply_short(int64_t N, int D, int K)
+{
+    const int min_k = g_tc_min_k.load(std::memory_order_relaxed);
+    return (g_small_kernels.load(std::memory_order_relaxed) & 1) && get_apply_column_split() == 0 && N >= 8192 && K >= min_k &&
+           apply_short_supported(N, D, K);
+}
+
 // The kernel that keeps rows in shared memory, where it is the faster one: K from a quarter of the tensor-core
 // threshold on (the alternative there is the fp32 pipes: 50 000 x 1000, K = 2: 107 us against 270).
 //
@@ -215,6 +223,11 @@ static cat_status_t run_assign(const float *Y, int64_t N, int D, int K, const fl
                                const void *Yh = nullptr, void *Ch = nullptr, float *hscale = nullptr,
                                bool centroids_ready = false, const FastOut *fast = nullptr, const int32_t *settled = nullptr)
 {
+    if (out && labels && top_level && !fast && use_apply_short(N, D, K)) {
+        CAT_CUDA(launch_reset_control(w.ctl, s));
+        CAT_CUDA(launch_apply_short(Y, N, D, K, C, gamma, beta, out, false, labels, w.ctl, s));
+        return CAT_OK;
+    }
     if (out && labels && top_level && !fast && use_small_apply(N, D, K)) {
         // small problems: everything in one persistent launch (exact decisions included)
         CAT_CUDA(launch_reset_control(w.ctl, s));
@@ -439,6 +452,11 @@ cat_status_t cat_apply_bf16(const float *Yq, int64_t N, int32_t D, int32_t K, co
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     AssignWs w = carve_assign(workspace, N, D, K);
     int32_t *labels = labels_out ? labels_out : w.labels;
+    if (use_apply_short(N, D, K)) {
+        CAT_CUDA(launch_reset_control(w.ctl, s));
+        CAT_CUDA(launch_apply_short(Yq, N, D, K, centroids, gamma, beta, Y_out_bf16, true, labels, w.ctl, s));
+        return CAT_OK;
+    }
     if (use_apply_rows(N, D, K, true)) {
         CAT_CUDA(launch_apply_rows(Yq, N, D, K, centroids, gamma, beta, Y_out_bf16, true, labels, w.ctl, w.prep, s));
         return CAT_OK;
@@ -841,10 +859,12 @@ const char *cat_kernel_for(int32_t call, int64_t N, int32_t D, int32_t K)
     const bool tc = use_tensor_path(N, D, K);
     switch (call) {
     case CAT_CALL_APPLY:
+        if (use_apply_short(N, D, K)) return "apply_short_kernel";
         if (use_small_apply(N, D, K)) return "small_kernel";
         if (use_apply_rows(N, D, K, false)) return "apply_rows_kernel";
         break;
     case CAT_CALL_APPLY_BF16:
+        if (use_apply_short(N, D, K)) return "apply_short_kernel";
         if (use_apply_rows(N, D, K, true)) return "apply_rows_kernel";
         break;
     case CAT_CALL_FIT:

@@ -214,6 +214,12 @@ size_t fit_tiles_counts(int K);
 cudaError_t launch_fit_tiles(const float *Y, int64_t N, int D, int K, float *C, const float *mean, int passes, int32_t *labels, double *part,
                              int32_t *part_counts, double *sums, int64_t *counts, Control *ctl, cudaStream_t s);
 
+// Inference on rows of 32 to 128 columns that stay in a warp's registers, exact decisions included
+// (cat_apply_short.cu); ctl must have been reset.  out_bf16: `out` is a [N, D] bf16 matrix.
+bool apply_short_supported(int64_t N, int D, int K);
+cudaError_t launch_apply_short(const float *Y, int64_t N, int D, int K, const float *C, const float *gamma, const float *beta, void *out,
+                               bool out_bf16, int32_t *labels, Control *ctl, cudaStream_t s);
+
 // Inference on groups of eight rows held in shared memory, exact decisions included (cat_apply_rows.cu).
 // Resets ctl.  out_bf16: `out` is a [N, D] bf16 matrix; prep: apply_rows_prep_bytes of scratch.
 bool apply_rows_supported(int64_t N, int D, int K);
