@@ -353,6 +353,10 @@ static cat_status_t run_centred(const float *Yq, const float *Yfp, int64_t N, in
 static cat_status_t run_closed_form(const float *Yq, const float *Yfp, int64_t N, int D, int K, const int32_t *labels, const FitWs &w,
                                     bool have_sums, float *gamma_out, float *beta_out, cudaStream_t s)
 {
+    if (closed_form_supported(N, D, K)) {
+        CAT_CUDA(launch_closed_form(Yq, Yfp, labels, N, D, K, have_sums ? w.sumQ : nullptr, gamma_out, beta_out, s));
+        return CAT_OK;
+    }
     if (have_sums) CAT_CUDA(launch_means_from_sums(w.sumQ, w.counts, D, K, w.meanQ, s));
     cat_status_t st = run_sort(labels, N, D, K, w, w.counts, s);
     if (st != CAT_OK) return st;

@@ -309,6 +309,11 @@ cudaError_t launch_segment_sums(int mode, const float *Yq, const float *Yf, cons
                                 const double *meanF, int D, int KK, const SegGeom &g, double *part,
                                 cudaStream_t s, const int32_t *settled = nullptr);
 
+// gamma and beta of a small set for given labels (sumQ: the clusters' sums of Yq, or null).
+bool closed_form_supported(int64_t N, int D, int K);
+cudaError_t launch_closed_form(const float *Yq, const float *Yf, const int32_t *labels, int64_t N, int D, int K, const double *sumQ,
+                               float *gamma, float *beta, cudaStream_t s);
+
 // Adds each cluster's segment partials in order into out0 (and out1 if not NULL); in delta mode
 // out0[k] += (partials of key k) - (partials of key K + k).  With C also writes the centroid
 // float(out0 / n_k) for clusters with n_k > 0.
