@@ -30,6 +30,14 @@
 // candidates; one candidate is the label.  Several: direct-form fp32 sums of squares, a lane's D / 32 terms
 // first, then a tree (relative error at most (D / 32 + 12) 2^-24), and among what these leave within that
 // error direct-form fp64, lowest index on equality.
+//
+// Algorithm 2 with PCA (label_i = argmin_k ||z_i - c_k||^2, z_i = fp32 of V (y_i - mean)) is the same kernel: with
+// w_k = V'(c_k - m) in place of c_k - m and y - mean in place of y, t_k = ||c_k||^2 - ||m||^2 - 2 (y - mean).w_k.  The
+// projection is never formed for a row that its scores decide; its rounding to fp32 and that of y - mean enter the bound,
+//   e += 2^-24 ||y - mean|| (||w|| + ||V||_F max ||c_k - m||).
+// Several candidates: the same dot products in fp32 from w_k in fp32; for the rows that these leave (one in a thousand) a kernel
+// behind this one forms the projection in fp64 and the distances in the reduced space.  50 000 x 1000, 50 components, K = 64: the projection in fp64, the assignment of
+// the reduced rows and the correction took 377 us.
 #include "cat_tc.cuh"
 
 #include <cuda_bf16.h>
@@ -47,11 +55,11 @@ constexpr size_t RES_SMEM = 227 * 1024;
 
 // byte offsets in dynamic shared memory
 struct ResLayout {
-    uint32_t bs, ak, coef, part, stat, slots, bars, total;
+    uint32_t bs, ak, coef, mean, part, stat, slots, bars, total;
     uint32_t part_team, slot_bytes;
 };
 
-ResLayout res_layout(int MT, int ldy, int nk, int TW, int T, int S, bool bg)
+ResLayout res_layout(int MT, int ldy, int nk, int TW, int T, int S, bool bg, bool pca)
 {
     ResLayout L{};
     size_t o = 0;
@@ -67,6 +75,8 @@ ResLayout res_layout(int MT, int ldy, int nk, int TW, int T, int S, bool bg)
     o += (size_t)MT * 16 * 4;
     L.coef = (uint32_t)o;
     o += (size_t)MT * 16 * 4;
+    L.mean = (uint32_t)o;
+    o += pca ? (size_t)nk * 64 : 0;
     L.part = (uint32_t)o;
     o += (size_t)T * part_team;
     L.stat = (uint32_t)o;
@@ -80,7 +90,11 @@ ResLayout res_layout(int MT, int ldy, int nk, int TW, int T, int S, bool bg)
 
 // What the preparation leaves for the main kernel: fragments [nk][MT][32] x 16 bytes, then per centroid
 // (MT * 16 of them) ||c||^2 - ||m||^2, -2 / scale, ||c - m||^2 and the norm of its rounding error.
+// With PCA also the norm of each c - m in the reduced space, the squared Frobenius norm of the components, and
+// behind these the w_k in fp32.
+__host__ __device__ constexpr size_t lift_offset(int MT, int nk) { return (size_t)nk * MT * 512 + ((size_t)MT * 16 * 5 + 4) * sizeof(float); }
 size_t prep_bytes(int MT, int nk) { return (size_t)nk * MT * 512 + (size_t)MT * 16 * 4 * sizeof(float); }
+size_t prep_bytes_pca(int MT, int nk, int D, int K) { return lift_offset(MT, nk) + (size_t)K * D * sizeof(float); }
 
 struct ResParams {
     const float *Y, *C, *gamma, *beta;
@@ -94,6 +108,9 @@ struct ResParams {
     int nk;        // 16-column steps of a row, a multiple of KS
     int T, S;      // teams, row slots per team
     int out_bf16;
+    const float *mean;   // PCA: [D]
+    uint4 *open_rows;    // PCA: [N] {row, candidates} that fp32 has not decided
+    int p;
     ResLayout L;
 };
 
@@ -268,6 +285,73 @@ __device__ __noinline__ int settle(const float *y, const float *C, int D, uint4 
     return l;
 }
 
+// (y - mean) . w for two of the w_k, fp32, in every lane; y and mean in shared memory
+template <bool VEC>
+__device__ __forceinline__ void dots2(const float *y, const float *mean, const float *w0, const float *w1, int D, int lane, float &s0,
+                                      float &s1)
+{
+    s0 = s1 = 0.f;
+    if (VEC) {
+#pragma unroll 4
+        for (int j = lane; j < (D >> 2); j += 32) {
+            const float4 a = reinterpret_cast<const float4 *>(w0)[j], b = reinterpret_cast<const float4 *>(w1)[j];
+            const float4 v = reinterpret_cast<const float4 *>(y)[j], m = reinterpret_cast<const float4 *>(mean)[j];
+            const float4 d = make_float4(v.x - m.x, v.y - m.y, v.z - m.z, v.w - m.w);
+            s0 = fmaf(d.x, a.x, fmaf(d.y, a.y, fmaf(d.z, a.z, fmaf(d.w, a.w, s0))));
+            s1 = fmaf(d.x, b.x, fmaf(d.y, b.y, fmaf(d.z, b.z, fmaf(d.w, b.w, s1))));
+        }
+    } else {
+#pragma unroll 8
+        for (int j = lane; j < D; j += 32) {
+            const float d = y[j] - mean[j];
+            s0 = fmaf(d, w0[j], s0);
+            s1 = fmaf(d, w1[j], s1);
+        }
+    }
+    s0 = warp_sum_f(s0);
+    s1 = warp_sum_f(s1);
+}
+
+// Label among the candidates (K <= 64) by the same dot products in fp32; those left are returned where that does not decide.
+// noise: bound on the error of a fp32 score here, the rounding of the projected row included.
+template <bool VEC>
+__device__ __noinline__ int settle_pca(const float *y, const float *mean, const float *lift, const float *ak, int D, uint2 mask2, float noise,
+                                       int lane, uint2 *rest)
+{
+    uint32_t mask[2] = {mask2.x, mask2.y};
+    float sc[2];   // of candidate lane + 32 i
+    float best = CUDART_INF_F;
+    int held = -1;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        sc[i] = CUDART_INF_F;
+        uint32_t m = mask[i];
+        while (m) {
+            const int ka = 32 * i + __ffs(m) - 1;
+            m &= m - 1;
+            const int kb = m ? 32 * i + __ffs(m) - 1 : ka;
+            m &= m ? m - 1 : 0u;
+            float s0, s1;
+            dots2<VEC>(y, mean, lift + (size_t)ka * D, lift + (size_t)kb * D, D, lane, s0, s1);
+            s0 = fmaf(-2.f, s0, ak[ka]);
+            s1 = fmaf(-2.f, s1, ak[kb]);
+            if (lane == (ka & 31)) sc[i] = s0;
+            if (lane == (kb & 31)) sc[i] = s1;
+            best = fminf(best, fminf(s0, s1));
+        }
+    }
+    const float lim = fmaxf(best, -3.4028235e38f) + 2.f * noise;
+    int left = 0;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        mask[i] &= __ballot_sync(0xffffffffu, !(sc[i] > lim));
+        left += __popc(mask[i]);
+        if (mask[i] && held < 0) held = 32 * i + __ffs(mask[i]) - 1;
+    }
+    *rest = left == 1 ? make_uint2(0u, 0u) : make_uint2(mask[0], mask[1]);
+    return held < 0 ? 0 : held;
+}
+
 template <int TW>
 __device__ __forceinline__ void team_sync(int team)
 {
@@ -329,8 +413,11 @@ __device__ __forceinline__ void correct(const ResParams &p, size_t e, const floa
 // One CTA per centroid (MT * 16 of them): the mean of all centroids, c - m, its norm, scale, fp16 fragments
 // and what rounding left.  Also resets the control block.  A launch of its own because the columns' sums
 // over all centroids are latency that every CTA of the main kernel would pay (9 us there, 4 here).
+// With PCA (p > 0) the centroids are [K][p] and what becomes fragments is V'(c - m), formed in fp64.
+template <bool PCA>
 __global__ void __launch_bounds__(PREP_THREADS) centroid_fragments_kernel(const float *__restrict__ C, int D, int K, int MT, int nk,
-                                                                          unsigned char *__restrict__ prep, Control *ctl)
+                                                                          unsigned char *__restrict__ prep, Control *ctl,
+                                                                          const float *__restrict__ V, int p)
 {
     pdl_enter();
     extern __shared__ float4 diff4[];   // [16 nk] c - m, zero beyond D
@@ -349,9 +436,37 @@ __global__ void __launch_bounds__(PREP_THREADS) centroid_fragments_kernel(const 
     const bool live = k < K;
     float mx = 0.f, n2 = 0.f;
     double a = 0.0;
+    double *cred = reinterpret_cast<double *>(diff + 16 * nk);   // PCA: [p] c - m
+    float nred = 0.f, vf2 = 0.f;
+    if constexpr (PCA) {
+        for (int r = tid; r < p; r += PREP_THREADS) {
+            double s = 0.0;
+#pragma unroll 16
+            for (int q = 0; q < K; ++q) s += (double)__ldg(C + (size_t)q * p + r);
+            const double m = s / (double)K, c = live ? (double)__ldg(C + (size_t)k * p + r) : m;
+            cred[r] = c - m;
+            nred = fmaf((float)(c - m), (float)(c - m), nred);
+            a = fma(c - m, c + m, a);
+        }
+        __syncthreads();
+    }
     for (int j = tid; j < 16 * nk; j += PREP_THREADS) {
         float d = 0.f;
-        if (live && j < D) {
+        if (PCA) {
+            if (live && j < D) {
+                double s = 0.0;
+#pragma unroll 8
+                for (int r = 0; r < p; ++r) {
+                    const float v = __ldg(V + (size_t)r * D + j);
+                    s = fma(cred[r], (double)v, s);
+                    if (k == 0) vf2 = fmaf(v, v, vf2);
+                }
+                d = (float)s;
+                mx = fmaxf(mx, fabsf(d));
+                n2 = fmaf(d, d, n2);
+                reinterpret_cast<float *>(prep + lift_offset(MT, nk))[(size_t)k * D + j] = d;
+            }
+        } else if (live && j < D) {
             float s = 0.f;
 #pragma unroll 16
             for (int q = 0; q < K; ++q) s += __ldg(C + (size_t)q * D + j);
@@ -368,11 +483,17 @@ __global__ void __launch_bounds__(PREP_THREADS) centroid_fragments_kernel(const 
         mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         n2 += __shfl_xor_sync(0xffffffffu, n2, o);
         a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (PCA) {
+            nred += __shfl_xor_sync(0xffffffffu, nred, o);
+            vf2 += __shfl_xor_sync(0xffffffffu, vf2, o);
+        }
     }
+    __shared__ float2 rp[PREP_THREADS / 32];
     if (lane == 0) {
         rmax[warp] = mx;
         rn2[warp] = n2;
         ra[warp] = a;
+        if (PCA) rp[warp] = make_float2(nred, vf2);
     }
     __syncthreads();
     mx = 0.f;
@@ -403,11 +524,21 @@ __global__ void __launch_bounds__(PREP_THREADS) centroid_fragments_kernel(const 
         cw[MT * 16 + k] = -2.f * inv;
         cw[2 * MT * 16 + k] = n2;
         cw[3 * MT * 16 + k] = sqrtf(left2) * inv;
+        if (PCA) {
+            nred = vf2 = 0.f;
+            for (int w = 0; w < PREP_THREADS / 32; ++w) {
+                nred += rp[w].x;
+                vf2 += rp[w].y;
+            }
+            cw[4 * MT * 16 + k] = sqrtf(nred);
+            if (k == 0) cw[5 * MT * 16] = vf2;
+        }
     }
 }
 
 // MT: groups of 16 centroids; VEC: D % 4 == 0; TW: warps per team; BG: the fragments stay in global memory (L2).
-template <int MT, bool VEC, int TW, bool BG>
+// PCA: the scores are those of the projected rows.
+template <int MT, bool VEC, int TW, bool BG, bool PCA>
 __global__ void __launch_bounds__(RES_MAX_THREADS, 1) apply_rows_kernel(ResParams p)
 {
     pdl_enter();
@@ -453,18 +584,23 @@ __global__ void __launch_bounds__(RES_MAX_THREADS, 1) apply_rows_kernel(ResParam
         ak[k] = __ldg(cw + k);
         coef[k] = __ldg(cw + MT * 16 + k);
     }
-    float cmax2 = 0.f, amax = 0.f, dc = 0.f;
+    float *mean = reinterpret_cast<float *>(smem + L.mean);   // PCA: zero beyond D
+    if (PCA)
+        for (int j = tid; j < 16 * p.nk; j += blockDim.x) mean[j] = j < p.D ? __ldg(p.mean + j) : 0.f;
+    float cmax2 = 0.f, amax = 0.f, dc = 0.f, cred = 0.f;
     for (int k = lane; k < p.K; k += 32) {
         // (a centroid that is not finite has scores that decide nothing, whatever the bound)
         amax = fmaxf(amax, fabsf(__ldg(cw + k)));
         cmax2 = fmaxf(cmax2, __ldg(cw + 2 * MT * 16 + k));
         dc = fmaxf(dc, __ldg(cw + 3 * MT * 16 + k));
+        if (PCA) cred = fmaxf(cred, __ldg(cw + 4 * MT * 16 + k));
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
         cmax2 = fmaxf(cmax2, __shfl_xor_sync(0xffffffffu, cmax2, o));
         dc = fmaxf(dc, __shfl_xor_sync(0xffffffffu, dc, o));
+        if (PCA) cred = fmaxf(cred, __shfl_xor_sync(0xffffffffu, cred, o));
     }
     __syncthreads();
     if (!BG && !mbar_wait_warp(smem_u32(prep_bar), 0, &fail[team][0], p.ctl)) fail[team][0] = 1;
@@ -473,8 +609,10 @@ __global__ void __launch_bounds__(RES_MAX_THREADS, 1) apply_rows_kernel(ResParam
     const float slack = 1.0001f + (float)p.D * 6.0e-8f;   // covers the rounding of the running sums of squares
     const float cnorm = sqrtf(cmax2 * slack);
     // (c_k - m is rounded to fp32 before it is scaled: 2^-24 of c beside dc)
+    // PCA: y - mean, and the projected row, are rounded to fp32
+    const float e_z = PCA ? 5.9604645e-8f * (1.001f * cnorm + sqrtf(__ldg(cw + 5 * MT * 16) * (slack + (float)p.p * 6.0e-8f)) * cred * 1.01f) : 0.f;
     const float e_y = 1.001f * (dc * slack + 5.9604645e-8f * cnorm) +
-                      (float)(16 * KS * ((nb + TW - 1) / TW) + TW + 2) * 2.3841858e-7f * cnorm;
+                      (float)(16 * KS * ((nb + TW - 1) / TW) + TW + 2) * 2.3841858e-7f * cnorm + e_z;
     const float e_abs = 8.f * 5.9604645e-8f * amax + 1e-30f;   // (squares below that may have underflowed)
 
     int undecided = 0;
@@ -521,6 +659,14 @@ __global__ void __launch_bounds__(RES_MAX_THREADS, 1) apply_rows_kernel(ResParam
                     for (int u = 0; u < KS; ++u) {
                         v[u][0] = pack2(u * 16 < rem ? yb[u * 16] : 0.f, u * 16 + 1 < rem ? yb[u * 16 + 1] : 0.f);
                         v[u][1] = pack2(u * 16 + 2 < rem ? yb[u * 16 + 2] : 0.f, u * 16 + 3 < rem ? yb[u * 16 + 3] : 0.f);
+                    }
+                }
+                if (PCA) {
+#pragma unroll
+                    for (int u = 0; u < KS; ++u) {
+                        const ulonglong2 m = *reinterpret_cast<const ulonglong2 *>(mean + kb * (16 * KS) + u * 16 + 4 * t);
+                        v[u][0] = fma2(m.x, pack2(-1.f, -1.f), v[u][0]);
+                        v[u][1] = fma2(m.y, pack2(-1.f, -1.f), v[u][1]);
                     }
                 }
                 float mx = 0.f;
@@ -632,7 +778,18 @@ __global__ void __launch_bounds__(RES_MAX_THREADS, 1) apply_rows_kernel(ResParam
                     const uint32_t bl = __ballot_sync(0xffffffffu, l + LPR * i < p.K && !(sc[i] > lm));
                     mask[i * LPR / 32] |= (bl >> src & (LPR == 32 ? 0xffffffffu : (1u << (LPR & 31)) - 1u)) << (i * LPR % 32);
                 }
-                const int exact = settle<VEC>(rows + ro * p.ldy, p.C, p.D, make_uint4(mask[0], mask[1], mask[2], mask[3]), lane);
+                int exact;
+                if constexpr (PCA) {
+                    // (fp32 sums of D / 32 terms a lane, then a tree; w_k rounded to fp32)
+                    const float yn = __shfl_sync(0xffffffffu, sqrt_approx(yn2 * slack), src);
+                    const float noise = 1.0625f * 2.f * yn * (((float)p.D * 0.03125f + 13.f) * 5.9604645e-8f * cnorm + e_z) + e_abs;
+                    uint2 rest;
+                    exact = settle_pca<VEC>(rows + ro * p.ldy, mean, reinterpret_cast<const float *>(p.prep + lift_offset(MT, p.nk)), ak, p.D,
+                                            make_uint2(mask[0], mask[1]), noise, lane, &rest);
+                    if ((rest.x | rest.y) != 0u && lane == 0)
+                        p.open_rows[atomicAdd(&p.ctl->refine_count, 1)] = make_uint4((uint32_t)(row0 + ro), rest.x, rest.y, 0u);
+                } else
+                    exact = settle<VEC>(rows + ro * p.ldy, p.C, p.D, make_uint4(mask[0], mask[1], mask[2], mask[3]), lane);
                 if (lane / LPR == src / LPR) label = exact;
             }
             if (l == 0 && live) p.labels[row0 + r] = label;
@@ -644,7 +801,9 @@ __global__ void __launch_bounds__(RES_MAX_THREADS, 1) apply_rows_kernel(ResParam
         constexpr int V = Unit<VEC>::N;
         const int DV = p.D / V;
         if (TW >= 4) {
-            constexpr int U = VEC ? (TW == 8 ? 4 : 2) : (TW == 8 ? 8 : 4);   // column steps at a time, for each of the warp's rows
+            // column steps at a time, for each of the warp's rows (scalar loads: eight, 225 us against 245 with four for
+            // 49 999 x 1001, K = 50)
+            constexpr int U = VEC ? (TW == 8 ? 4 : 2) : 8;
             int lq[RPW];
 #pragma unroll
             for (int q = 0; q < RPW; ++q) lq[q] = __shfl_sync(0xffffffffu, label, q * LPR);
@@ -713,6 +872,81 @@ __global__ void __launch_bounds__(RES_MAX_THREADS, 1) apply_rows_kernel(ResParam
     }
 }
 
+// The rows that fp32 has not decided, a CTA each: the projection in fp64, rounded to fp32, and the candidates' distances to it
+// in fp64, lowest index on equality; then the correction once more.  A launch of its own: a warp of the kernel above
+// would be at one such row for as long as it takes its team to go through three groups of rows.
+constexpr int OPEN_THREADS = 256;
+__global__ void __launch_bounds__(OPEN_THREADS) open_rows_kernel(const float *__restrict__ Y, const float *__restrict__ C, int D, int K, int p,
+                                                                 const float *__restrict__ mean, const float *__restrict__ comps,
+                                                                 const float *__restrict__ gamma, const float *__restrict__ beta,
+                                                                 float *__restrict__ out, int32_t *__restrict__ labels,
+                                                                 const uint4 *__restrict__ open_rows, const Control *ctl)
+{
+    pdl_enter();
+    extern __shared__ double xs[];   // [D] y - mean, then [p] the projected row
+    __shared__ double s_dist[64];
+    __shared__ int s_label;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    float *z = reinterpret_cast<float *>(xs + D);
+    const int n = ctl->refine_count;
+    for (int i = blockIdx.x; i < n; i += gridDim.x) {
+        const uint4 e = open_rows[i];
+        const float *y = Y + (size_t)e.x * D;
+        for (int j = tid; j < D; j += OPEN_THREADS) xs[j] = (double)__ldg(y + j) - (double)__ldg(mean + j);
+        __syncthreads();
+        // (eight components of a warp side by side, 32 loads in flight per lane)
+        for (int r0 = warp * 8; r0 < p; r0 += OPEN_THREADS / 32 * 8) {
+            double s[8];
+            const float *v[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                s[q] = 0.0;
+                v[q] = comps + (size_t)(r0 + q < p ? r0 + q : r0) * D;
+            }
+#pragma unroll 4
+            for (int j = lane; j < D; j += 32) {
+                const double x = xs[j];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) s[q] = fma(x, (double)__ldg(v[q] + j), s[q]);
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
+                if (lane == 0 && r0 + q < p) z[r0 + q] = (float)s[q];
+            }
+        }
+        __syncthreads();
+        for (int k = warp; k < K; k += OPEN_THREADS / 32) {
+            if (!((k < 32 ? e.y >> k : e.z >> (k - 32)) & 1u)) continue;
+            double s = 0.0;
+            for (int r = lane; r < p; r += 32) {
+                const double d = (double)z[r] - (double)__ldg(C + (size_t)k * p + r);
+                s = fma(d, d, s);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) s_dist[k] = s;
+        }
+        __syncthreads();
+        if (tid == 0) {
+            double best = CUDART_INF;
+            int l = e.y ? __ffs(e.y) - 1 : 31 + __ffs(e.z);   // (when every distance is infinite or NaN)
+            for (int k = 0; k < K; ++k)
+                if (((k < 32 ? e.y >> k : e.z >> (k - 32)) & 1u) && s_dist[k] < best) {
+                    best = s_dist[k];
+                    l = k;
+                }
+            s_label = l;
+            labels[e.x] = l;
+        }
+        __syncthreads();
+        const size_t o = (size_t)s_label * D;
+        for (int j = tid; j < D; j += OPEN_THREADS) out[(size_t)e.x * D + j] = fmaf(__ldg(gamma + o + j), __ldg(y + j), __ldg(beta + o + j));
+        __syncthreads();
+    }
+}
+
 struct ResPlan {
     int MT, ldy, nk, TW, T, S;
     bool bg;
@@ -726,7 +960,7 @@ struct ResPlan {
 //   fragments        in shared memory as long as that leaves sixteen warps, else in L2: 50 000 x 600, K = 64
 //                    takes 112 us from shared memory (5 teams) and 135 from L2; 50 000 x 1000, K = 60 270 us (2 teams)
 //                    and 205 (5 teams), 20 000 x 2047, K = 64 237 us from L2 where shared memory has no room
-bool res_plan(int64_t N, int D, int K, ResPlan *pl)
+bool res_plan(int64_t N, int D, int K, ResPlan *pl, bool pca = false)
 {
     if (N < 1 || D < 1 || K < 2 || K > 128) return false;
     const int m16 = (K + 15) / 16;
@@ -738,7 +972,7 @@ bool res_plan(int64_t N, int D, int K, ResPlan *pl)
     for (int bg = 0; bg < 2; ++bg)
         for (int T = RES_MAX_THREADS / 32 / pl->TW; T >= 2 && (bg || T * pl->TW >= 16); --T)
             for (int S = 2; S >= 1; --S) {
-                pl->L = res_layout(pl->MT, pl->ldy, pl->nk, pl->TW, T, S, bg != 0);
+                pl->L = res_layout(pl->MT, pl->ldy, pl->nk, pl->TW, T, S, bg != 0, pca);
                 if (pl->L.total + 1024 <= RES_SMEM) {
                     pl->T = T;
                     pl->S = S;
@@ -749,10 +983,10 @@ bool res_plan(int64_t N, int D, int K, ResPlan *pl)
     return false;
 }
 
-template <int MT, bool VEC, int TW, bool BG>
+template <int MT, bool VEC, int TW, bool BG, bool PCA = false>
 cudaError_t launch_rows(const ResPlan &pl, const ResParams &p, cudaStream_t s)
 {
-    auto kern = apply_rows_kernel<MT, VEC, TW, BG>;
+    auto kern = apply_rows_kernel<MT, VEC, TW, BG, PCA>;
     // (the same value whatever the shape: several threads may be launching)
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(RES_SMEM - 1024));
     if (e != cudaSuccess) return e;
@@ -814,13 +1048,71 @@ cudaError_t launch_apply_rows(const float *Y, int64_t N, int D, int K, const flo
 {
     ResPlan pl;
     if (!res_plan(N, D, K, &pl)) return cudaErrorInvalidValue;
-    cudaError_t e = launch_pdl(centroid_fragments_kernel, dim3((unsigned)pl.MT * 16), dim3(PREP_THREADS), (size_t)pl.nk * 64, s, C, D, K,
-                               pl.MT, pl.nk, reinterpret_cast<unsigned char *>(prep), ctl);
+    cudaError_t e = launch_pdl(centroid_fragments_kernel<false>, dim3((unsigned)pl.MT * 16), dim3(PREP_THREADS), (size_t)pl.nk * 64, s, C, D, K,
+                               pl.MT, pl.nk, reinterpret_cast<unsigned char *>(prep), ctl, nullptr, 0);
     if (e != cudaSuccess) return e;
     count_launch();
     ResParams p{Y, C, gamma, beta, reinterpret_cast<const unsigned char *>(prep), out, labels, ctl, N, D, K, pl.ldy, pl.nk, pl.T, pl.S,
-                out_bf16 ? 1 : 0, pl.L};
+                out_bf16 ? 1 : 0, nullptr, nullptr, 0, pl.L};
     return D % 4 == 0 ? launch_rows_tw<true>(pl, p, s) : launch_rows_tw<false>(pl, p, s);
+}
+
+bool apply_rows_pca_supported(int64_t N, int D, int K)
+{
+    ResPlan pl;
+    return D <= 1024 && K <= 64 && res_plan(N, D, K, &pl, true);
+}
+
+size_t apply_rows_pca_prep_bytes(int64_t N, int D, int K)
+{
+    ResPlan pl;
+    return apply_rows_pca_supported(N, D, K) && res_plan(N, D, K, &pl, true) ? prep_bytes_pca(pl.MT, pl.nk, D, K) : 0;
+}
+
+template <bool VEC, int TW>
+static cudaError_t launch_rows_pca(const ResPlan &pl, const ResParams &p, cudaStream_t s)
+{
+    if constexpr (TW >= 4)
+        if (pl.bg) switch (pl.MT) {
+            case 1: return launch_rows<1, VEC, TW, true, true>(pl, p, s);
+            case 2: return launch_rows<2, VEC, TW, true, true>(pl, p, s);
+            case 3: return launch_rows<3, VEC, TW, true, true>(pl, p, s);
+            default: return launch_rows<4, VEC, TW, true, true>(pl, p, s);
+            }
+    if (pl.bg) return cudaErrorInvalidValue;
+    switch (pl.MT) {
+    case 1: return launch_rows<1, VEC, TW, false, true>(pl, p, s);
+    case 2: return launch_rows<2, VEC, TW, false, true>(pl, p, s);
+    case 3: return launch_rows<3, VEC, TW, false, true>(pl, p, s);
+    default: return launch_rows<4, VEC, TW, false, true>(pl, p, s);
+    }
+}
+
+cudaError_t launch_apply_rows_pca(const float *Y, int64_t N, int D, int K, int p, const float *mean, const float *comps, const float *C,
+                                  const float *gamma, const float *beta, float *out, int32_t *labels, Control *ctl, void *prep,
+                                  void *open_rows, cudaStream_t s)
+{
+    ResPlan pl;
+    if (!apply_rows_pca_supported(N, D, K) || !res_plan(N, D, K, &pl, true)) return cudaErrorInvalidValue;
+    cudaError_t e = launch_pdl(centroid_fragments_kernel<true>, dim3((unsigned)pl.MT * 16), dim3(PREP_THREADS),
+                               (size_t)pl.nk * 64 + (size_t)p * sizeof(double), s, C, D, K, pl.MT, pl.nk,
+                               reinterpret_cast<unsigned char *>(prep), ctl, comps, p);
+    if (e != cudaSuccess) return e;
+    count_launch();
+    ResParams q{Y, C, gamma, beta, reinterpret_cast<const unsigned char *>(prep), out, labels, ctl, N, D, K, pl.ldy, pl.nk, pl.T, pl.S, 0,
+                mean, reinterpret_cast<uint4 *>(open_rows), p, pl.L};
+    const bool vec = D % 4 == 0;
+    switch (pl.TW) {
+    case 1: e = vec ? launch_rows_pca<true, 1>(pl, q, s) : launch_rows_pca<false, 1>(pl, q, s); break;
+    case 2: e = vec ? launch_rows_pca<true, 2>(pl, q, s) : launch_rows_pca<false, 2>(pl, q, s); break;
+    case 4: e = vec ? launch_rows_pca<true, 4>(pl, q, s) : launch_rows_pca<false, 4>(pl, q, s); break;
+    default: return cudaErrorInvalidValue;
+    }
+    if (e != cudaSuccess) return e;
+    e = launch_pdl(open_rows_kernel, dim3((unsigned)tc_sm_count() * 4), dim3(OPEN_THREADS), (size_t)D * sizeof(double) + (size_t)p * sizeof(float), s, Y, C,
+                   D, K, p, mean, comps, gamma, beta, out, labels, reinterpret_cast<const uint4 *>(open_rows), ctl);
+    count_launch();
+    return e;
 }
 
 }  // namespace cat

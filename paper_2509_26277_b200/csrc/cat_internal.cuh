@@ -227,6 +227,14 @@ size_t apply_rows_prep_bytes(int64_t N, int D, int K);
 cudaError_t launch_apply_rows(const float *Y, int64_t N, int D, int K, const float *C, const float *gamma, const float *beta,
                               void *out, bool out_bf16, int32_t *labels, Control *ctl, void *prep, cudaStream_t s);
 
+// The same for clusters in a reduced space: C [K][p], labels by z = fp32 of comps (y - mean) (D <= 1024, K <= 64).  open_rows: N
+// 16-byte entries of scratch.
+bool apply_rows_pca_supported(int64_t N, int D, int K);
+size_t apply_rows_pca_prep_bytes(int64_t N, int D, int K);
+cudaError_t launch_apply_rows_pca(const float *Y, int64_t N, int D, int K, int p, const float *mean, const float *comps, const float *C,
+                                  const float *gamma, const float *beta, float *out, int32_t *labels, Control *ctl, void *prep,
+                                  void *open_rows, cudaStream_t s);
+
 // Tensor-core (tcgen05, TF32) variant of launch_assign; ynorm2 is needed when out == nullptr.
 bool tc_supported(int64_t N, int D, int K);
 // Form of the fused inference kernel on the tensor path: 0 = chosen by shape, 1 = TF32 row tiles

@@ -557,7 +557,17 @@ size_t cat_apply_pca_workspace_bytes(int64_t N, int32_t D, int32_t K, int32_t p)
     if (N < 1 || D < 1 || p < 1 || p > D || D > CAT_PCA_MAX_D || p > CAT_PCA_MAX_P) return 0;
     const size_t a = cat_apply_workspace_bytes(N, p, K);
     if (a == 0) return 0;
-    return align_up(a, 256) + align_up((size_t)N * p * sizeof(float), 256) + align_up((size_t)N * sizeof(int32_t), 256);
+    const size_t three = align_up(a, 256) + align_up((size_t)N * p * sizeof(float), 256) + align_up((size_t)N * sizeof(int32_t), 256);
+    const size_t rows = 256 + align_up(apply_rows_pca_prep_bytes(N, D, K), 256) + align_up((size_t)N * 16, 256) + align_up((size_t)N * sizeof(int32_t), 256);
+    return three > rows ? three : rows;
+}
+
+// One kernel that keeps rows in shared memory, where it takes the shape (the selector of cat_apply's kernel of that kind
+// holds here too): against the three steps, 8000 x 777, K = 16, 8 components 30 us and 123, 50 000 x 1000, K = 64, 50
+// components 240 and 372, 50 000 x 100, K = 40 42 and 81.  (Less than a few hundred rows leave either idle.)
+static bool use_apply_rows_pca(int64_t N, int D, int K)
+{
+    return N * D >= 65536 && (cat_get_small_problem_kernels() & 1) && get_apply_column_split() == 0 && apply_rows_pca_supported(N, D, K);
 }
 
 cat_status_t cat_apply_pca(const float *Yq, int64_t N, int32_t D, int32_t K, int32_t p, const float *mean,
@@ -571,6 +581,16 @@ cat_status_t cat_apply_pca(const float *Yq, int64_t N, int32_t D, int32_t K, int
     if (!workspace || !al16(workspace) || workspace_bytes < need) return CAT_ERR_WORKSPACE;
     // (the assignment's part first: its control block is where cat_workspace_report looks)
     unsigned char *b = reinterpret_cast<unsigned char *>(workspace);
+    if (use_apply_rows_pca(N, D, K)) {
+        if (!al16(Yq) || !al16(mean) || !al16(components) || !al16(centroids) || !al16(gamma) || !al16(beta) || !al16(Y_out) ||
+            (labels_out && !al16(labels_out)))
+            return CAT_ERR_ALIGN;
+        unsigned char *open_rows = b + 256 + align_up(apply_rows_pca_prep_bytes(N, D, K), 256);
+        int32_t *labels = labels_out ? labels_out : reinterpret_cast<int32_t *>(open_rows + align_up((size_t)N * 16, 256));
+        CAT_CUDA(launch_apply_rows_pca(Yq, N, D, K, p, mean, components, centroids, gamma, beta, Y_out, labels,
+                                       reinterpret_cast<Control *>(b), b + 256, open_rows, reinterpret_cast<cudaStream_t>(stream)));
+        return CAT_OK;
+    }
     const size_t assign_bytes = align_up(cat_apply_workspace_bytes(N, p, K), 256);
     float *Z = reinterpret_cast<float *>(b + assign_bytes);
     int32_t *labels =

@@ -1,0 +1,98 @@
+"""cat_apply_pca in the kernel that keeps rows in shared memory (scores of the projected rows without the projection)
+against the oracle, and against the three-step path it takes the place of."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import cat_oracle as O
+from oracle import cat_pca_oracle as P
+from paper_2509_26277_b200 import binding as B
+from tests.parity import labels_match
+
+pytestmark = pytest.mark.gpu
+
+
+def host(t):
+    return t.detach().cpu().numpy()
+
+
+def dev(a):
+    return torch.as_tensor(np.ascontiguousarray(a)).cuda()
+
+
+def _case(seed, n, d, p, k, offset, scale):
+    rng = np.random.default_rng(seed)
+    Y = (rng.normal(size=(n, d)) * scale + offset).astype(np.float32)
+    V = np.linalg.qr(rng.normal(size=(d, p)))[0].T.astype(np.float32)
+    mean = (np.full(d, offset) + 0.1 * scale * rng.normal(size=d)).astype(np.float32)
+    C = (scale * rng.normal(size=(k, p))).astype(np.float32)
+    g, b = rng.normal(size=(k, d)).astype(np.float32), rng.normal(size=(k, d)).astype(np.float32)
+    return Y, mean, V, C, g, b
+
+
+def _check(Y, mean, V, C, g, b):
+    out, lab = B.cat_apply_pca(dev(Y), dev(mean), dev(V), dev(C), dev(g), dev(b), want_labels=True)
+    want, olab, best, second = P.apply_pca(Y, mean, V, C, g, b)
+    labels_match(host(lab), olab, best, second, "labels of the projected rows")
+    np.testing.assert_array_equal(host(out), O.affine_with_labels(Y, host(lab), g, b))
+    return host(lab)
+
+
+@pytest.mark.parametrize("n,d,p,k,offset,scale", [
+    (1, 8, 3, 2, 0.0, 1.0), (7, 1, 1, 2, 0.0, 1.0), (9, 5, 5, 3, 0.0, 1.0), (1000, 64, 8, 16, 0.0, 1.0),
+    (1001, 128, 33, 17, 3.0, 1.0), (997, 129, 50, 32, 0.0, 1e-3), (2003, 256, 50, 33, 100.0, 1.0), (2003, 257, 4, 48, 0.0, 1e3),
+    (3001, 1000, 50, 64, 1.0, 1.0), (3001, 1001, 50, 64, 0.0, 1.0), (513, 1024, 300, 5, 0.0, 1.0), (515, 1023, 64, 49, 50.0, 1.0),
+])
+def test_labels_and_outputs_match_the_oracle(n, d, p, k, offset, scale):
+    case = _case(n + d + p + k, n, d, p, k, offset, scale)
+    lab = _check(*case)
+    old = B.cat_get_small_problem_kernels()
+    B.cat_set_small_problem_kernels(0)
+    try:
+        assert (lab != _check(*case)).mean() <= 2e-3   # (a row within fp32 rounding of a bisector)
+    finally:
+        B.cat_set_small_problem_kernels(old)
+
+
+def test_equal_centroids_and_rows_between_two():
+    """Rows on the bisector of two centroids, and centroids that coincide: lowest index, as the exact distances have it."""
+    rng = np.random.default_rng(5)
+    d, p, k, n = 300, 12, 20, 4000
+    V = np.eye(p, d, dtype=np.float32)   # the projection is exact: the first p columns
+    C = rng.integers(-8, 8, size=(k, p)).astype(np.float32)
+    C[7] = C[3]
+    C[19] = C[3]
+    i, j = rng.integers(0, k, size=n), rng.integers(0, k, size=n)
+    Y = rng.normal(size=(n, d)).astype(np.float32)
+    Y[:, :p] = (C[i] + C[j]) / 2
+    Y[::2, :p] = C[i[::2]]
+    g, b = rng.normal(size=(k, d)).astype(np.float32), rng.normal(size=(k, d)).astype(np.float32)
+    mean = np.zeros(d, np.float32)
+    _, lab = B.cat_apply_pca(dev(Y), dev(mean), dev(V), dev(C), dev(g), dev(b), want_labels=True)
+    olab, _, _ = O.assign(np.ascontiguousarray(Y[:, :p]), C)
+    np.testing.assert_array_equal(host(lab), olab)
+
+
+def test_components_that_are_not_unit_vectors_and_rows_out_of_range():
+    rng = np.random.default_rng(6)
+    Y, mean, V, C, g, b = _case(6, 1200, 200, 10, 24, 0.0, 1.0)
+    V = (V * np.logspace(-3, 3, 10)[:, None]).astype(np.float32)
+    C = (C * np.logspace(-3, 3, 10)[None]).astype(np.float32)
+    Y[3] *= 1e18
+    Y[4] *= 1e-25
+    Y[5] = 0.0
+    _check(Y, mean, V, C, g, b)
+    Y[6, 11] = np.nan
+    Y[7, 12] = np.inf
+    old = B.cat_get_small_problem_kernels()
+    got = []
+    try:
+        for mask in (old, 0):
+            B.cat_set_small_problem_kernels(mask)
+            got.append([host(t) for t in B.cat_apply_pca(dev(Y), dev(mean), dev(V), dev(C), dev(g), dev(b), want_labels=True)])
+    finally:
+        B.cat_set_small_problem_kernels(old)
+    rest = np.setdiff1d(np.arange(1200), [6, 7])
+    np.testing.assert_array_equal(got[0][1][rest], got[1][1][rest])
+    np.testing.assert_array_equal(got[0][0][rest], got[1][0][rest])
+    assert all(0 <= l < 24 for l in got[0][1][[6, 7]])
