@@ -302,28 +302,32 @@ __global__ void __launch_bounds__(ET) tridiag_regs_kernel(TridiagParams P)
             if (lead && k > j && k < D) P.refl[(size_t)j * D + k] = un[c];
         }
         // update j - 1 of the own rows and their products with the new reflection
-        double acc[8];
+        // (rows that are done with go along: a branch per row would leave one row's chain of dependent operations after the
+        // other, 1750 cycles of a step's 5900 where the eight together take a third of that)
+        double acc[8], ui[8], wi[8];
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
             acc[r] = 0.0;
-            const int i = i0 + r;
-            if (i > j && i < D) {
-                const double ui = u_old[i], wi = -fma(-h, ui, tau * s_prod[r]);
+            ui[r] = -u_old[i0 + r];
+            wi[r] = -fma(h, ui[r], tau * s_prod[r]);
+        }
 #pragma unroll
-                for (int c = 0; c < C; ++c)
-                    if (warp * 32 + 31 + c * ET > j) {   // (columns up to j are done with)
-                        ar[r][c] = fma(wi, uo[c], fma(-ui, wo[c], ar[r][c]));
-                        acc[r] = fma(ar[r][c], un[c], acc[r]);
-                    }
-                if (i == j + 1) {
+        for (int c = 0; c < C; ++c)
+            if (warp * 32 + 31 + c * ET > j) {   // (columns up to j are done with)
 #pragma unroll
-                    for (int c = 0; c < C; ++c) {
-                        const int k = tid + c * ET;
-                        if (k > j && k < D) publish(P.next + (size_t)(j + 1) * D + k, ar[r][c]);
-                    }
+                for (int r = 0; r < 8; ++r) ar[r][c] = fma(wi[r], uo[c], fma(ui[r], wo[c], ar[r][c]));
+#pragma unroll
+                for (int r = 0; r < 8; ++r) acc[r] = fma(ar[r][c], un[c], acc[r]);
+            }
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+            if (i0 + r == j + 1) {
+#pragma unroll
+                for (int c = 0; c < C; ++c) {
+                    const int k = tid + c * ET;
+                    if (k > j && k < D) publish(P.next + (size_t)(j + 1) * D + k, ar[r][c]);
                 }
             }
-        }
         const double s = warp_sum8(acc, lane);
         if ((lane & 3) == 0) red_rows[warp][lane >> 2] = s;
         tau = reflect ? 1.0 / fma(fabs(x1), nrm, tt) : 0.0;
@@ -526,8 +530,8 @@ struct EigvecParams {
 // Eigenvalues of the tridiagonal matrix below each of two points: sign changes of the leading minors p_i = (d_i - x) p_{i-1} -
 // e_{i-1}^2 p_{i-2} (Givens' form of the Sturm sequence; the products' rounding amounts to relative changes of d - x and
 // e^2 by a few units, as in the form with quotients, and a step is one dependent operation where a division was some
-// twenty).  Every four steps the pair is scaled by a power of two: entries are below 2^14 and above 2^-65 of the norm, so that
-// four steps stay within fp64's range.  de[i] = {d_i, e_{i-1}^2}; two points keep the fp64 pipe and its latency in balance.
+// twenty).  Every eight steps the pair is scaled by a power of two: entries are below 2^14 and above 2^-65 of the norm, so that
+// eight steps stay within fp64's range.  de[i] = {d_i, e_{i-1}^2}; two points keep the fp64 pipe and its latency in balance.
 __device__ __forceinline__ void count_below(const double2 *de, int D, const double (&x)[2], int (&n)[2])
 {
     double p0[2], p1[2];
@@ -548,12 +552,12 @@ __device__ __forceinline__ void count_below(const double2 *de, int D, const doub
         }
     };
     int i = 1;
-    for (; i + 4 <= D; i += 4) {
-        double2 v[4];
+    for (; i + 8 <= D; i += 8) {
+        double2 v[8];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = de[i + u];
+        for (int u = 0; u < 8; ++u) v[u] = de[i + u];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) step(v[u]);
+        for (int u = 0; u < 8; ++u) step(v[u]);
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             const int ea = __double2hiint(p0[q]) & 0x7FF00000, eb = __double2hiint(p1[q]) & 0x7FF00000;
@@ -904,15 +908,22 @@ __global__ void __launch_bounds__(ET) eigvec_kernel(EigvecParams P)
                 if (lane == 0) s_blk[warp] = t;
             }
             __syncthreads();
+            // (in pairs, then a tree: dependent additions are what a block's time is made of)
 #pragma unroll
-            for (int i = 0; i < RB; ++i) {
-                const double s = -s_blk[i];
+            for (int c = 0; c < C; ++c) {
+                double part[RB / 2];
 #pragma unroll
-                for (int c = 0; c < C; ++c) {
-                    z[c] = fma(s, u[i][c], z[c]);
-                    u[i][c] = un[i][c];
-                }
+                for (int i = 0; i < RB / 2; ++i) part[i] = fma(s_blk[2 * i], u[2 * i][c], s_blk[2 * i + 1] * u[2 * i + 1][c]);
+#pragma unroll
+                for (int o = RB / 4; o > 0; o >>= 1)
+#pragma unroll
+                    for (int i = 0; i < o; ++i) part[i] += part[i + o];
+                z[c] -= part[0];
             }
+#pragma unroll
+            for (int i = 0; i < RB; ++i)
+#pragma unroll
+                for (int c = 0; c < C; ++c) u[i][c] = un[i][c];
             mm = mn;
         }
         // the entry of largest magnitude (lowest index among equals) is made positive
