@@ -9,7 +9,9 @@
 // The kernel this takes such calls from (csrc/cat_small.cu) passes a tile of 128 rows through five warp roles, whose
 // hand-overs bounded it.  tcgen05 would bring them back: its accumulators are read by other warps than those that
 // wait for its operands; the contraction is small here (K <= 128, D <= 128).
-//   bound: instruction issue and the latency of a group's loads, sixteen warps per SM.
+// The next group's rows are on their way into shared memory (cp.async, every lane what it will read itself) while this one's
+// are worked on.
+//   bound: instruction issue, about 700 instructions a group.
 //
 // Scores and error bound as in csrc/cat_apply_rows.cu: t_k = ||c_k||^2 - ||m||^2 - 2 y.(c_k - m), m the centroids' mean; the
 // rounding errors of the fp16 operands are measured.  Rows with several centroids within the bound are settled by the
@@ -38,10 +40,11 @@ struct ShortParams {
 __host__ __device__ constexpr int short_threads(int nks) { return nks <= 4 ? 512 : (nks <= 6 ? 384 : 320); }
 // row stride of what is read by label: 64 bytes off a multiple of 128, so that two rows in a phase collide half as often
 __host__ __device__ constexpr int short_ld(int D) { return D % 32 == 0 ? D + 16 : D; }
-size_t short_smem(int D, int K)
+size_t short_smem(int D, int K, bool ahead)
 {
     const size_t nt = K > 64 ? 8 : (K + 15) / 16;
-    return (size_t)3 * K * short_ld(D) * 4 + nt * 16 * D * 2 + nt * 16 * 2 * 4 + (size_t)D * 4;
+    const size_t rows = ahead ? (size_t)short_threads(D / 16) / 32 * 16 * D * 4 : 0;
+    return rows + (size_t)3 * K * short_ld(D) * 4 + nt * 16 * D * 2 + nt * 16 * 2 * 4 + (size_t)D * 4;
 }
 
 __device__ __forceinline__ void mma_16816(float (&c)[4], const uint4 a, uint32_t b0, uint32_t b1)
@@ -50,6 +53,33 @@ __device__ __forceinline__ void mma_16816(float (&c)[4], const uint4 a, uint32_t
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                  : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
 }
+// pairs of fp32 values in one 64-bit register: one instruction does both
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
 // exponent shift that brings m > 0 to [2^13, 2^14), clamped to +-100; 0 for zero or non-finite m
 __device__ __forceinline__ int half_shift(float m)
 {
@@ -167,8 +197,13 @@ __device__ __forceinline__ void put4(void *out, size_t at, float4 y, float4 g, f
         __stcs(reinterpret_cast<float4 *>(reinterpret_cast<float *>(out) + at), v);
 }
 
-// NKS: steps of sixteen columns; NC: chunks of 64 centroids.
-template <int NKS, int NC, bool BF16>
+__device__ __forceinline__ void copy_async16(float4 *dst, const float4 *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+
+// NKS: steps of sixteen columns; NC: chunks of 64 centroids; AHEAD: rows come through shared memory (where it has room).
+template <int NKS, int NC, bool BF16, bool AHEAD>
 __global__ void __launch_bounds__(short_threads(NKS), 1) apply_short_kernel(ShortParams p)
 {
     pdl_enter();
@@ -177,9 +212,24 @@ __global__ void __launch_bounds__(short_threads(NKS), 1) apply_short_kernel(Shor
     __shared__ float s_max[3][NW];
     const int K = p.K, nt = p.nt;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
-    float *cs = reinterpret_cast<float *>(smem), *gs = cs + K * LD, *bs = gs + K * LD;
+    float4 *ahead = reinterpret_cast<float4 *>(smem) + (size_t)warp * NKS * 64 + lane;   // [2 NKS][32] of this warp
+    float *cs = reinterpret_cast<float *>(smem + (AHEAD ? (size_t)NW * NKS * 1024 : 0)), *gs = cs + K * LD, *bs = gs + K * LD;
     uint4 *bfrag = reinterpret_cast<uint4 *>(bs + K * LD);
     float *ak = reinterpret_cast<float *>(bfrag + (size_t)NKS * nt * 32), *coef = ak + nt * 16, *mean = coef + nt * 16;
+
+    const int64_t groups = (p.N + 15) / 16;
+    // (neighbouring groups on different SMs: a small call spreads over the device)
+    const int64_t first = (int64_t)warp * gridDim.x + blockIdx.x, step = (int64_t)gridDim.x * NW;
+    auto row_of = [&](int64_t row) { return reinterpret_cast<const float4 *>(p.Y + (size_t)(row < p.N ? row : 0) * D) + t; };
+    auto request = [&](int64_t grp) {
+        const float4 *pa = row_of(grp * 16 + g), *pb = row_of(grp * 16 + g + 8);
+#pragma unroll
+        for (int ks = 0; ks < NKS; ++ks) {
+            copy_async16(ahead + (2 * ks) * 32, pa + 4 * ks);
+            copy_async16(ahead + (2 * ks + 1) * 32, pb + 4 * ks);
+        }
+    };
+    if (AHEAD && first < groups) request(first);
 
     // ---- centroids: copy, mean, fragments of c - m
     for (int e = tid; e < K * (D / 4); e += TH) {
@@ -225,7 +275,7 @@ __global__ void __launch_bounds__(short_threads(NKS), 1) apply_short_kernel(Shor
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) left2 += __shfl_xor_sync(0xffffffffu, left2, o);
             if (lane == 0) {
-                ak[k] = k < K ? (float)a : CUDART_INF_F;
+                ak[k] = k < K ? (float)a : TC_KEY_INIT;
                 coef[k] = -2.f * pow2i(-sh);
             }
             if (k < K) {   // (NaN stays out: a centroid that is not finite has scores that decide nothing)
@@ -249,21 +299,30 @@ __global__ void __launch_bounds__(short_threads(NKS), 1) apply_short_kernel(Shor
     }
     const float cnorm = sqrtf(cmax2 * slack);
     // e = 1.0625 * 2 (|dy| c + |y| e_y) + e_abs (c - m is rounded to fp32 before it is scaled: 2^-24 of c beside dc)
-    const float e_y = 1.001f * (dc + 5.9604645e-8f * cnorm) + (float)(D + 2) * 2.3841858e-7f * cnorm;
-    const float e_abs = 8.f * 5.9604645e-8f * amax + 1e-30f;   // (squares below that may have underflowed)
+    // and 2^-16 of a score for the index in its low seven bits
+    const float e_y = 1.001f * (dc + 5.9604645e-8f * cnorm) + ((float)(D + 2) * 2.3841858e-7f + 1.5258789e-5f) * cnorm;
+    const float e_abs = (8.f * 5.9604645e-8f + 1.5258789e-5f) * amax + 1e-30f;   // (squares below that may have underflowed)
 
-    const int64_t groups = (p.N + 15) / 16;
     int undecided = 0;
-    // (neighbouring groups on different SMs: a small call spreads over the device)
-    for (int64_t grp = (int64_t)warp * gridDim.x + blockIdx.x; grp < groups; grp += (int64_t)gridDim.x * NW) {
+    for (int64_t grp = first; grp < groups; grp += step) {
         const int64_t ra = grp * 16 + g, rb = ra + 8;
         const bool ina = ra < p.N, inb = rb < p.N;
-        const float4 *pa = reinterpret_cast<const float4 *>(p.Y + (size_t)(ina ? ra : 0) * D) + t, *pb = reinterpret_cast<const float4 *>(p.Y + (size_t)(inb ? rb : 0) * D) + t;
         float4 ya[NKS], yb[NKS];
+        if constexpr (AHEAD) {
+            asm volatile("cp.async.wait_all;" ::: "memory");
 #pragma unroll
-        for (int ks = 0; ks < NKS; ++ks) {
-            ya[ks] = __ldcs(pa + 4 * ks);
-            yb[ks] = __ldcs(pb + 4 * ks);
+            for (int ks = 0; ks < NKS; ++ks) {
+                ya[ks] = ahead[(2 * ks) * 32];
+                yb[ks] = ahead[(2 * ks + 1) * 32];
+            }
+            if (grp + step < groups) request(grp + step);   // (this lane's pieces are in its registers)
+        } else {
+            const float4 *pa = row_of(ra), *pb = row_of(rb);
+#pragma unroll
+            for (int ks = 0; ks < NKS; ++ks) {
+                ya[ks] = __ldcs(pa + 4 * ks);
+                yb[ks] = __ldcs(pb + 4 * ks);
+            }
         }
         float ma = 0.f, mb = 0.f, na = 0.f, nb = 0.f, la = 0.f, lb = 0.f;
 #pragma unroll
@@ -300,8 +359,7 @@ __global__ void __launch_bounds__(short_threads(NKS), 1) apply_short_kernel(Shor
         const float wb = 2.f * (1.0625f * 2.f * (sqrt_approx(lb * slack) * ib * cnorm + sqrt_approx(nb * slack) * e_y) + e_abs);
 
         float acc[8][4];
-        float a1 = CUDART_INF_F, a2 = CUDART_INF_F, c1 = CUDART_INF_F, c2 = CUDART_INF_F;   // smallest two scores of rows ra and rb
-        int ka = 0, kb = 0;
+        float a1 = TC_KEY_INIT, a2 = TC_KEY_INIT, c1 = TC_KEY_INIT, c2 = TC_KEY_INIT;   // smallest two keys of rows ra and rb
         auto contract = [&](int ch) {
 #pragma unroll
             for (int i = 0; i < 8; ++i)
@@ -318,11 +376,14 @@ __global__ void __launch_bounds__(short_threads(NKS), 1) apply_short_kernel(Shor
                 }
             }
         };
-        auto better = [](float s, int k, float &b1, float &b2, int &l) {
-            b2 = fminf(b2, fmaxf(b1, s));
-            l = s < b1 ? k : l;
-            b1 = fminf(b1, s);
+        // keys: scores with the centroid's index in the low seven bits.  (Those of an infinite or NaN score may get lost, but a
+        // row that has one also has a bound that decides nothing.)
+        auto better = [](float s, int k, float &b1, float &b2) {
+            const float key = __uint_as_float((__float_as_uint(s) & 0xFFFFFF80u) | (uint32_t)k);
+            b2 = fminf(b2, fmaxf(b1, key));
+            b1 = fminf(b1, key);
         };
+        const f32x2 ia2 = pack2(ia, ia), ib2 = pack2(ib, ib);
 #pragma unroll 1
         for (int ch = 0; ch < NC; ++ch) {
             contract(ch);
@@ -330,27 +391,28 @@ __global__ void __launch_bounds__(short_threads(NKS), 1) apply_short_kernel(Shor
             for (int i = 0; i < 8; ++i) {
                 if (ch * 4 + (i >> 1) >= nt) break;
                 const int k = ch * 64 + i * 8 + 2 * t;
-                const float2 n = *reinterpret_cast<const float2 *>(ak + k), f = *reinterpret_cast<const float2 *>(coef + k);
-                better(fmaf(f.x, acc[i][0] * ia, n.x), k, a1, a2, ka);
-                better(fmaf(f.y, acc[i][1] * ia, n.y), k + 1, a1, a2, ka);
-                better(fmaf(f.x, acc[i][2] * ib, n.x), k, c1, c2, kb);
-                better(fmaf(f.y, acc[i][3] * ib, n.y), k + 1, c1, c2, kb);
+                const f32x2 n = *reinterpret_cast<const f32x2 *>(ak + k), f = *reinterpret_cast<const f32x2 *>(coef + k);
+                const float2 ua = unpack2(fma2(f, mul2(pack2(acc[i][0], acc[i][1]), ia2), n));
+                const float2 ub = unpack2(fma2(f, mul2(pack2(acc[i][2], acc[i][3]), ib2), n));
+                better(ua.x, k, a1, a2);
+                better(ua.y, k + 1, a1, a2);
+                better(ub.x, k, c1, c2);
+                better(ub.y, k + 1, c1, c2);
             }
         }
 #pragma unroll
         for (int o = 1; o < 4; o <<= 1) {
             float q1 = __shfl_xor_sync(0xffffffffu, a1, o), q2 = __shfl_xor_sync(0xffffffffu, a2, o);
-            int qk = __shfl_xor_sync(0xffffffffu, ka, o);
             a2 = fminf(fminf(a2, q2), fmaxf(a1, q1));
-            ka = q1 < a1 || (q1 == a1 && qk < ka) ? qk : ka;
             a1 = fminf(a1, q1);
             q1 = __shfl_xor_sync(0xffffffffu, c1, o);
             q2 = __shfl_xor_sync(0xffffffffu, c2, o);
-            qk = __shfl_xor_sync(0xffffffffu, kb, o);
             c2 = fminf(fminf(c2, q2), fmaxf(c1, q1));
-            kb = q1 < c1 || (q1 == c1 && qk < kb) ? qk : kb;
             c1 = fminf(c1, q1);
         }
+        int ka = (int)(__float_as_uint(a1) & 0x7Fu), kb = (int)(__float_as_uint(c1) & 0x7Fu);
+        if (ka >= K) ka = 0;
+        if (kb >= K) kb = 0;
         // (scores of a bound below 1e33 have not overflowed)
         const bool ua = ina && !(a2 - a1 > wa && wa < 2e33f), ub = inb && !(c2 - c1 > wb && wb < 2e33f);
         if (__any_sync(0xffffffffu, ua || ub)) {
@@ -409,31 +471,43 @@ __global__ void __launch_bounds__(short_threads(NKS), 1) apply_short_kernel(Shor
     }
 }
 
-template <int NKS, int NC, bool BF16>
-cudaError_t launch_short(const ShortParams &p, size_t smem, cudaStream_t s)
+template <int NKS, int NC, bool BF16, bool AHEAD>
+cudaError_t launch_short(const ShortParams &p, cudaStream_t s)
 {
-    auto kern = apply_short_kernel<NKS, NC, BF16>;
+    auto kern = apply_short_kernel<NKS, NC, BF16, AHEAD>;
     // (the same value whatever the shape: several threads may be launching)
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH_SMEM);
     if (e != cudaSuccess) return e;
     const int64_t groups = (p.N + 15) / 16;
     const int64_t grid = groups < tc_sm_count() ? groups : tc_sm_count();
-    e = launch_pdl(kern, dim3((unsigned)grid), dim3(short_threads(NKS)), smem, s, p);
+    e = launch_pdl(kern, dim3((unsigned)grid), dim3(short_threads(NKS)), short_smem(16 * NKS, p.K, AHEAD), s, p);
     count_launch();
     return e;
 }
-template <int NKS>
-cudaError_t launch_short_nks(const ShortParams &p, bool bf16, size_t smem, cudaStream_t s)
+template <int NKS, bool BF16>
+cudaError_t launch_short_nks(const ShortParams &p, cudaStream_t s)
 {
-    if (p.nt > 4) return bf16 ? launch_short<NKS, 2, true>(p, smem, s) : launch_short<NKS, 2, false>(p, smem, s);
-    return bf16 ? launch_short<NKS, 1, true>(p, smem, s) : launch_short<NKS, 1, false>(p, smem, s);
+    const bool ahead = short_smem(16 * NKS, p.K, true) <= SH_SMEM;
+    if (p.nt > 4) return ahead ? launch_short<NKS, 2, BF16, true>(p, s) : launch_short<NKS, 2, BF16, false>(p, s);
+    return ahead ? launch_short<NKS, 1, BF16, true>(p, s) : launch_short<NKS, 1, BF16, false>(p, s);
+}
+template <bool BF16>
+cudaError_t launch_short_d(int D, const ShortParams &p, cudaStream_t s)
+{
+    switch (D / 16) {
+    case 2: return launch_short_nks<2, BF16>(p, s);
+    case 3: return launch_short_nks<3, BF16>(p, s);
+    case 4: return launch_short_nks<4, BF16>(p, s);
+    case 6: return launch_short_nks<6, BF16>(p, s);
+    default: return launch_short_nks<8, BF16>(p, s);
+    }
 }
 
 }  // namespace
 
 bool apply_short_supported(int64_t N, int D, int K)
 {
-    return N >= 1 && K >= 2 && K <= 128 && (D == 32 || D == 48 || D == 64 || D == 96 || D == 128) && short_smem(D, K) <= SH_SMEM;
+    return N >= 1 && K >= 2 && K <= 128 && (D == 32 || D == 48 || D == 64 || D == 96 || D == 128) && short_smem(D, K, false) <= SH_SMEM;
 }
 
 cudaError_t launch_apply_short(const float *Y, int64_t N, int D, int K, const float *C, const float *gamma, const float *beta, void *out,
@@ -442,14 +516,7 @@ cudaError_t launch_apply_short(const float *Y, int64_t N, int D, int K, const fl
     if (!apply_short_supported(N, D, K)) return cudaErrorInvalidValue;
     const int nt = K > 64 ? 8 : (K + 15) / 16;
     const ShortParams p{Y, C, gamma, beta, out, labels, ctl, N, K, nt};
-    const size_t smem = short_smem(D, K);
-    switch (D / 16) {
-    case 2: return launch_short_nks<2>(p, out_bf16, smem, s);
-    case 3: return launch_short_nks<3>(p, out_bf16, smem, s);
-    case 4: return launch_short_nks<4>(p, out_bf16, smem, s);
-    case 6: return launch_short_nks<6>(p, out_bf16, smem, s);
-    default: return launch_short_nks<8>(p, out_bf16, smem, s);
-    }
+    return out_bf16 ? launch_short_d<true>(D, p, s) : launch_short_d<false>(D, p, s);
 }
 
 }  // namespace cat
