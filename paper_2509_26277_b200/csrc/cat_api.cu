@@ -60,6 +60,7 @@ static void carve_assign_into(Carver &c, AssignWs &w, int64_t N, int D, int K, b
     w.cmax = c.take<float>((size_t)K);
     w.cerr = c.take<float>((size_t)K);
     w.mean = c.take<float>((size_t)D);
+    w.cconst = c.take<float>((size_t)K);
     w.ch = c.take<uint16_t>((size_t)K * half_ld(D));
     const size_t slab = row_copy ? (size_t)copy_room_rows(N, D) : 0;
     w.hscale = c.take<float>(4 + 2 * slab);
@@ -166,6 +167,10 @@ static bool use_fit_rows(int64_t N, int D, int K)
     return (g_small_kernels.load(std::memory_order_relaxed) & 2) && fit_rows_supported(N, D, K) &&
            (N <= 4096 || !use_small_fit(N, D, K));
 }
+// Rows as fp16 fragments in shared memory for all rounds: more than 8192 rows (200 704 x 64, K = 64 1030 us against 1390 in the
+// persistent kernel, 108 286 x 256, K = 49 1510 against 1790 on the general path's sorts; up to 8192 rows the kernels of small sets
+// are as fast or faster and some of these rows' lists are what tests pin).  Clusters alone, as of PCA's reduced rows, from 2048 on:
+// 4096 x 50, K = 32 without the closed form's labels pass.
 static bool use_fit_tiles(int64_t N, int D, int K, bool clusters_only)
 {
     return (g_small_kernels.load(std::memory_order_relaxed) & 2) && (N > 8192 || (clusters_only && N >= 2048)) && fit_tiles_supported(N, D, K);
@@ -175,7 +180,8 @@ static bool use_small_apply(int64_t N, int D, int K)
     return (g_small_kernels.load(std::memory_order_relaxed) & 1) && use_tensor_path(N, D, K) && small_apply_supported(N, D, K);
 }
 
-// Short rows in registers: from 8192 rows on (two groups of sixteen rows for every three warps of the device).
+// Short rows in registers: from 8192 rows on (two groups of sixteen rows for every three warps of the device).  200 704 x 64,
+// K = 64 35 us against 50 in the persistent kernel; 12 155 x 64 and 40 764 x 48 18 - 20 in either; below, launches decide.
 static bool use_apply_short(int64_t N, int D, int K)
 {
     const int min_k = g_tc_min_k.load(std::memory_order_relaxed);
@@ -247,11 +253,11 @@ static cat_status_t run_assign(const float *Y, int64_t N, int D, int K, const fl
         return CAT_OK;
     }
     if (out && !fast && use_tensor_path(N, D, K) && choose_apply_form(N, D, K) == 64) {
-        // inference on 64-row tiles: fp16 copy of the centroids (scaled by a power of two from
-        // their largest magnitude), rows converted inside the kernel
-        CAT_CUDA(launch_centroid_half(C, D, K, nullptr, w.cnorm, w.cmax, w.cerr, w.hscale, w.ch, w.ctl, s, top_level));
-        CAT_CUDA(launch_apply_h64(Y, N, D, K, w.ch, w.hscale, w.cnorm, labels, w.refine_rows, w.cand_rows, w.cand_list,
-                                  w.ctl, gamma, beta, out, s));
+        // inference on 64-row tiles: fp16 copy of the centroids less a point among them (scaled by a power of two
+        // from the largest magnitude), rows converted inside the kernel
+        CAT_CUDA(launch_centroid_half(C, D, K, w.mean, w.cnorm, w.cmax, w.cerr, w.hscale, w.ch, w.ctl, s, top_level, true, w.cconst));
+        CAT_CUDA(launch_apply_h64(Y, N, D, K, w.ch, w.hscale, w.cnorm, w.cerr, w.cconst, labels, w.refine_rows, w.cand_rows,
+                                  w.cand_list, w.ctl, gamma, beta, out, s));
         CAT_CUDA(launch_refine_both(Y, N, D, K, C, labels, w.cand_rows, w.cand_list, w.refine_rows, w.ctl, gamma,
                                     beta, out, s));
         return CAT_OK;
@@ -332,8 +338,10 @@ static cat_status_t run_delta_update(const float *Yq, const int32_t *labels, con
     return CAT_OK;
 }
 
-// Rounds whose moved rows are listed instead of sorted: from the fourth on, where a tenth of the rows or fewer moves.
-static bool use_moved_list(int round, int64_t N, int D, int K, bool may_settle)
+// Rounds whose moved rows are listed instead of sorted: from the fourth on, where a tenth of the rows or fewer moves (262 144 x 1024,
+// K = 256: 45 us a round sorted, 10 listed; in the first rounds, where most rows move, the sort's segments spread them over more CTAs).
+// A cluster's CTAs read the whole list: with fewer than eight clusters too few of them share the sums.
+static bool use_moved_list(int round, int K, bool may_settle)
 {
     return may_settle && round >= 3 && K >= 8;
 }
@@ -468,9 +476,9 @@ cat_status_t cat_apply_bf16(const float *Yq, int64_t N, int32_t D, int32_t K, co
     if (use_tensor_path(N, D, K) && apply_h64_supported(N, D, K)) {
         // fused: the 64-row-tile kernel writes bf16 with the fast labels; the exact pass settles the
         // undecided rows' labels, and those rows are written once more
-        CAT_CUDA(launch_centroid_half(centroids, D, K, nullptr, w.cnorm, w.cmax, w.cerr, w.hscale, w.ch, w.ctl, s, true));
-        CAT_CUDA(launch_apply_h64(Yq, N, D, K, w.ch, w.hscale, w.cnorm, labels, w.refine_rows, w.cand_rows, w.cand_list, w.ctl,
-                                  gamma, beta, reinterpret_cast<float *>(Y_out_bf16), s, true));
+        CAT_CUDA(launch_centroid_half(centroids, D, K, w.mean, w.cnorm, w.cmax, w.cerr, w.hscale, w.ch, w.ctl, s, true, true, w.cconst));
+        CAT_CUDA(launch_apply_h64(Yq, N, D, K, w.ch, w.hscale, w.cnorm, w.cerr, w.cconst, labels, w.refine_rows, w.cand_rows, w.cand_list,
+                                  w.ctl, gamma, beta, reinterpret_cast<float *>(Y_out_bf16), s, true));
         CAT_CUDA(launch_refine_both(Yq, N, D, K, centroids, labels, w.cand_rows, w.cand_list, w.refine_rows, w.ctl, nullptr,
                                     nullptr, nullptr, s));
         CAT_CUDA(launch_affine_bf16(Yq, N, D, K, labels, gamma, beta, Y_out_bf16, w.refine_rows, w.cand_rows, w.ctl, s));
@@ -629,7 +637,7 @@ static cat_status_t cat::fit_from(const float *Yq, const float *Yfp, int64_t N, 
         if (diag && t < CAT_DIAG_MAX_ROUNDS - 1)
             CAT_CUDA(launch_fit_diag_round(Yq, N, D, K, C, cur, w.a.refine_rows, w.a.cand_rows, w.a.ctl, diag, t,
                                            diag_recorded, s));
-        if (use_moved_list(t, N, D, K, settled != nullptr)) {
+        if (use_moved_list(t, K, settled != nullptr)) {
             CAT_CUDA(launch_moved_update(Yq, cur, prev, N, D, K, (uint32_t)t, w.order, w.moved_flags, w.counts, w.sumQ, C, w.a.cnorm, w.hscale,
                                          half ? w.ch : nullptr, half ? w.a.mean : nullptr, w.a.cerr, w.norm_part, w.arrivals, w.a.ctl, settled, s));
         } else {

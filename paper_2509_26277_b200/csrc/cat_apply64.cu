@@ -28,7 +28,11 @@
 // largest magnitude of the first 64 columns into [2^10, 2^11).  Later elements up to 32 times
 // larger still fit; if one does not (it would become inf), the row is marked and goes to the
 // exact pass like any undecided row.  Elements that fall into fp16's subnormal range enter the
-// error bound with their absolute rounding error, as in the fp16 path of the fit.
+// error bound with their absolute rounding error.  The scores are ||c_k||^2 - ||m||^2 - 2 y.(c_k - m) with m a point among the
+// centroids (it changes all scores of a row alike), and the centroids' rounding errors enter the bound as measured: on
+// logits, whose centroids lie close together, that leaves a fraction of the rows undecided that the centroids themselves
+// did (24 222 x 1000, K = 161, bf16 out: 172 us with the centroids as they are, 137 so; 262 144 x 1024 far-apart clusters 511 and 512).  (Measuring the rows' errors too, in the converters, would halve it again; their loop then spills and far-apart clusters
+// take 5 % longer.)
 //
 // Every wait is bounded; a wait that runs out records CAT_ERR_DEVICE_TIMEOUT and all roles
 // leave.  No TMA multicast; all tensor maps cover this GPU's memory.
@@ -79,7 +83,8 @@ struct H64Shared {
     uint32_t tmem_base;
     int abort_flag;
     int rows_streamed;
-    float red[32];
+    float red[3][32];
+    float3 err;                   // terms of the error bound
     float cn[256];
     float rinv[2][H_ROWS];        // 1 / (row scale)
     float ysq[2][H_ROWS];         // ||y||^2, slightly over-estimated; +inf for a row that left the fp16 range
@@ -190,6 +195,7 @@ __device__ __forceinline__ void prefetch_row_l2(const TcParams &p, int64_t row, 
 struct H64Params {
     TcParams t;       // Y, cnorm, scale (= {s_c, -2 / s_c, 2^-25 / s_c, -}), labels, queues, ctl, gamma, beta, out, N, D, K, npad, tmem_cols
     int nh;           // fp16 slabs (64 columns) per row
+    const float *cconst;   // [K] ||c||^2 - ||m||^2
 };
 
 template <bool OUT_BF16>
@@ -245,17 +251,29 @@ apply_h64_kernel(const __grid_constant__ CUtensorMap mapY, const __grid_constant
         sh.rows_streamed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // centroid norms (a huge finite value beyond K) and their maximum
+    // the scores' constants (a huge finite value beyond K) and the maxima behind the error bound
     {
-        float m = 0.f;
+        float m = 0.f, me = 0.f, ma = 0.f;
         for (int k = tid; k < 256; k += blockDim.x) {
-            float v = (k < p.K) ? p.cnorm[k] : TC_KEY_INIT;
+            float v = (k < p.K) ? hp.cconst[k] : TC_KEY_INIT;
             sh.cn[k] = v;
-            if (k < p.K) m = fmaxf(m, v);
+            if (k < p.K) {
+                m = fmaxf(m, p.cnorm[k]);
+                me = fmaxf(me, p.cerr[k]);
+                ma = fmaxf(ma, fabsf(v));
+            }
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (lane == 0) sh.red[warp] = m;
+        for (int o = 16; o > 0; o >>= 1) {
+            m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+            me = fmaxf(me, __shfl_xor_sync(0xffffffffu, me, o));
+            ma = fmaxf(ma, __shfl_xor_sync(0xffffffffu, ma, o));
+        }
+        if (lane == 0) {
+            sh.red[0][warp] = m;
+            sh.red[1][warp] = me;
+            sh.red[2][warp] = ma;
+        }
     }
     if (warp == 1) {
         tmem_alloc_pair(smem_u32(&sh.tmem_base), (uint32_t)p.tmem_cols);
@@ -265,12 +283,19 @@ apply_h64_kernel(const __grid_constant__ CUtensorMap mapY, const __grid_constant
     __syncthreads();
     cluster_sync();   // the peer's barriers exist before anything arrives on them
     tc_fence_after();
-    float cmax2 = 0.f;
-    for (int w2 = 0; w2 < (int)(blockDim.x >> 5); ++w2) cmax2 = fmaxf(cmax2, sh.red[w2]);
+    if (tid == 0) {
+        float cmax2 = 0.f, dcmax = 0.f, amax = 0.f;
+        for (int w2 = 0; w2 < H_THREADS / 32; ++w2) {
+            cmax2 = fmaxf(cmax2, sh.red[0][w2]);
+            dcmax = fmaxf(dcmax, sh.red[1][w2]);
+            amax = fmaxf(amax, sh.red[2][w2]);
+        }
+        sh.err = tc_error_terms_centred(p.D, cmax2, dcmax, amax);
+    }
+    __syncthreads();
     const uint32_t tmem_base = sh.tmem_base;
     const float s_c = p.scale[0];          // centroid scale
     const float coef_c = p.scale[1];       // -2 / s_c
-    const float abs_err_c = p.scale[2];    // 2^-25 / s_c
 
     if (warp < TC_FIRST_SCORE_WARP) {
         setmaxnreg_dec<H_REGS_CONTROL>();   // (warps 2 and 3 have no role)
@@ -418,7 +443,7 @@ apply_h64_kernel(const __grid_constant__ CUtensorMap mapY, const __grid_constant
                 if (lane == 0) mbar_arrive(smem_u32(&sh.lab_full[b]));
                 const int64_t row = (unit * 2 + rank) * H_ROWS + r;
                 if (row < p.N) {
-                    const float e = tc_error_bound_half(p.D, yn2, cmax2, 2.9802322e-8f * rinv, abs_err_c);
+                    const float e = fmaf(sqrtf(yn2), sh.err.x, fmaf(2.9802322e-8f * rinv, sh.err.y, sh.err.z));
                     p.labels[row] = l;
                     tc_decide(p, row, make_float4(b1, b2, b3, b4), e);
                 }
@@ -558,12 +583,14 @@ bool apply_h64_supported(int64_t N, int D, int K)
 }
 
 cudaError_t launch_apply_h64(const float *Y, int64_t N, int D, int K, const void *Ch, const float *scale,
-                             const float *cnorm, int32_t *labels, int32_t *refine_rows, int32_t *cand_rows,
-                             uint64_t *cand_list, Control *ctl, const float *gamma, const float *beta, float *out,
+                             const float *cnorm, const float *cerr, const float *cconst, int32_t *labels, int32_t *refine_rows,
+                             int32_t *cand_rows, uint64_t *cand_list, Control *ctl, const float *gamma, const float *beta, float *out,
                              cudaStream_t s, bool out_bf16)
 {
     H64Params hp{};
     TcParams &p = hp.t;
+    hp.cconst = cconst;
+    p.cerr = cerr;
     p.Y = Y;
     p.cnorm = cnorm;
     p.scale = scale;

@@ -11,7 +11,9 @@
 // wait for its operands; the contraction is small here (K <= 128, D <= 128).
 // The next group's rows are on their way into shared memory (cp.async, every lane what it will read itself) while this one's
 // are worked on.
-//   bound: instruction issue, about 700 instructions a group.
+//   bound: instruction issue, about 700 instructions a group; 11 us are start, centroids and end.  200 704 x 64, K = 64 (floor
+//   16 us): 48 - 53 us in the persistent kernel, 36.7 without the rows fetched ahead and with labels beside the scores, 35.1 now.
+//   Sixteen rows a warp: the A operand's height; thirty-two do not fit into the registers beside the scores.
 //
 // Scores and error bound as in csrc/cat_apply_rows.cu: t_k = ||c_k||^2 - ||m||^2 - 2 y.(c_k - m), m the centroids' mean; the
 // rounding errors of the fp16 operands are measured.  Rows with several centroids within the bound are settled by the

@@ -15,6 +15,10 @@
 //               owns a column of some clusters, so nothing is added in a varying order
 //   barrier, the CTAs' sums added up in CTA order, barrier
 //
+//   bound, 200 704 x 64, K = 64 (cycles a round): scores 21 000 (issue), moves 23 000 on average (latency of the moved rows, more in the
+//   first rounds), barriers 12 000, combination 7 000, centroids 5 000, settlement 2 500.  25 rounds take 1030 us, 1390 in the
+//   persistent kernel.  Moves by groups of lanes with four columns each: 1090 (the scores' registers spill).
+//
 // A round in which no label changes leaves everything as it is, and so would all behind it: the rounds end there.  Sums
 // that follow moves keep what a far larger row rounded off after it has left; where the largest row's exponent is more than
 // X_SPREAD above the rows' average every round adds up all rows afresh (and none ends early).

@@ -127,6 +127,7 @@ struct AssignWs {          // what assign/apply need
     float *cmax;           // [K] largest magnitude of each centroid
     float *cerr;           // [K] norms of the rounding errors of the fp16 centroids
     float *mean;           // [D] what rows and centroids are taken relative to on fp16 operands
+    float *cconst;         // [K] squared norms less that of the mean (inference on 64-row tiles)
     void *ch;              // [K][half_ld(D)] fp16 copy of the centroids (inference on fp16 operands)
     float *hscale;         // [4] scale of that copy: {s_c, -2 / s_c, 2^-25 / s_c, -}; with yh followed by [slab] inverse row scales and [slab] rounding errors
     void *prep;            // prepared centroids of the inference kernel that keeps rows in shared memory (or null)
@@ -243,13 +244,13 @@ bool tc_supported(int64_t N, int D, int K);
 void set_apply_column_split(int cs);
 int get_apply_column_split();
 int choose_apply_form(int64_t N, int D, int K);   // 1, 2, 4 or 64 for this shape under the current setting
-// 64-row-tile inference kernel on fp16 operands (cat_apply64.cu).  Ch = fp16(C * scale[0]) and
-// scale = {s_c, -2 / s_c, 2^-25 / s_c, -} come from launch_centroid_half.
+// 64-row-tile inference kernel on fp16 operands (cat_apply64.cu).  Ch = fp16((C - m) * scale[0]),
+// scale = {s_c, -2 / s_c, 2^-25 / s_c, -}, cnorm, cerr and cconst come from launch_centroid_half with m.
 bool apply_h64_supported(int64_t N, int D, int K);
 cudaError_t launch_half_scale(float *scale, cudaStream_t s);                           // bits of the maximum -> the three scale words
 cudaError_t launch_apply_h64(const float *Y, int64_t N, int D, int K, const void *Ch, const float *scale,
-                             const float *cnorm, int32_t *labels, int32_t *refine_rows, int32_t *cand_rows,
-                             uint64_t *cand_list, Control *ctl, const float *gamma, const float *beta, float *out,
+                             const float *cnorm, const float *cerr, const float *cconst, int32_t *labels, int32_t *refine_rows,
+                             int32_t *cand_rows, uint64_t *cand_list, Control *ctl, const float *gamma, const float *beta, float *out,
                              cudaStream_t s, bool out_bf16 = false);   // out_bf16: `out` is a [N, D] bf16 matrix
 // out_bf16[row] = bf16(gamma_l * y + beta_l), l = labels[row]: for all rows (rows == nullptr, n_rows = N) or
 // for the listed rows (two lists, lengths read from ctl: the exact-pass queues).
@@ -287,9 +288,10 @@ cudaError_t launch_half_shadow(const float *Y, int64_t N, int D, const float *me
 cudaError_t launch_sample_mean(const float *Y, int64_t N, int D, float *mean, cudaStream_t s);
 // Everything an assignment on fp16 operands needs of the centroids less `mean` (null: as they are): norms,
 // the fp16 copy, the norms cerr of its rounding errors, and with own_scale the scale words from their largest
-// magnitude (cmax: [K] scratch); empties the exact-pass queues as launch_centroid_norms does.
-cudaError_t launch_centroid_half(const float *C, int D, int K, const float *mean, float *cnorm, float *cmax, float *cerr, float *scale,
-                                 void *Ch, Control *ctl, cudaStream_t s, bool reset_all, bool own_scale = true);
+// magnitude (cmax: [K] scratch).  With aconst they are taken less a point m among them instead, which goes to
+// `mean`, and aconst is ||c||^2 - ||m||^2.  Empties the exact-pass queues as launch_centroid_norms does.
+cudaError_t launch_centroid_half(const float *C, int D, int K, float *mean, float *cnorm, float *cmax, float *cerr, float *scale,
+                                 void *Ch, Control *ctl, cudaStream_t s, bool reset_all, bool own_scale = true, float *aconst = nullptr);
 
 // Exact fp64 decision among the listed candidates of each queued row; optional affine output.
 cudaError_t launch_refine_both(const float *Y, int64_t N, int D, int K, const float *C, int32_t *labels,

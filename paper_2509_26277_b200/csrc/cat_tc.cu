@@ -1071,10 +1071,29 @@ __global__ void __launch_bounds__(256) half_shadow_kernel(const float *__restric
     }
 }
 
+// A point among the centroids: the median of the first three, column by column (one stray centroid does not move it).  Three loads
+// where the mean of all would be a launch of its own, and that of eight made the kernel below 3 us longer.
+__device__ __forceinline__ float median_of_three(float a, float b, float c)
+{
+    const float m = fmaxf(fminf(a, b), fminf(fmaxf(a, b), c));
+    return fabsf(m) < CUDART_INF_F ? m : 0.f;   // (any finite point will do)
+}
+// columns j ... j + W - 1 of a matrix row, W = 1 or 4
+template <int W>
+__device__ __forceinline__ void load_cols(const float *__restrict__ row, int j, float (&v)[W])
+{
+    if constexpr (W == 4) {
+        const float4 x = __ldg(reinterpret_cast<const float4 *>(row + j));
+        v[0] = x.x, v[1] = x.y, v[2] = x.z, v[3] = x.w;
+    } else
+        v[0] = __ldg(row + j);
+}
+
 // dst[k, :] = fp16((src[k, :] - mean) * scale[0]), round to nearest; one CTA per row, rows of dst ld apart;
 // cerr[k] = norm of what the rounding left.
 // With cmax (the rows' largest magnitudes) the scale words are made here first (as half_scale_kernel
 // does) and CTA 0 leaves them in `scale`.
+template <int W>
 __global__ void __launch_bounds__(256) to_half_kernel(const float *__restrict__ src, int K, int D, int ld,
                                                       const float *__restrict__ mean, const float *__restrict__ cmax,
                                                       float *__restrict__ scale, __half *__restrict__ dst,
@@ -1104,12 +1123,23 @@ __global__ void __launch_bounds__(256) to_half_kernel(const float *__restrict__ 
     __half *h = dst + (size_t)blockIdx.x * ld;
     float left2 = 0.f;
 #pragma unroll 4
-    for (int j = threadIdx.x; j < D; j += 256) {
-        const float x = (mean ? __ldg(c + j) - __ldg(mean + j) : __ldg(c + j)) * sc;
-        const __half v = __float2half_rn(x);
-        h[j] = v;
-        const float d = x - __half2float(v);
-        left2 = fmaf(d, d, left2);
+    for (int j = W * threadIdx.x; j < D; j += W * 256) {
+        float x[W], o[W] = {};
+        __half v[W];
+        load_cols<W>(c, j, x);
+        if (mean) load_cols<W>(mean, j, o);
+#pragma unroll
+        for (int q = 0; q < W; ++q) {
+            x[q] = (x[q] - o[q]) * sc;
+            v[q] = __float2half_rn(x[q]);
+            const float d = x[q] - __half2float(v[q]);
+            left2 = fmaf(d, d, left2);
+        }
+        if constexpr (W == 4) {
+            const __half2 lo = __halves2half2(v[0], v[1]), hi = __halves2half2(v[2], v[3]);
+            *reinterpret_cast<uint2 *>(h + j) = make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
+        } else
+            h[j] = v[0];
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) left2 += __shfl_xor_sync(0xffffffffu, left2, o);
@@ -1122,14 +1152,17 @@ __global__ void __launch_bounds__(256) to_half_kernel(const float *__restrict__ 
     }
 }
 
-// Squared norms (fp64 sum, rounded up) and largest finite magnitudes of the centroids less `mean`, one CTA each;
+// Squared norms (fp64 sum, rounded up) and largest finite magnitudes of the centroids less `mean`, one CTA each, with
+// aconst less a point among them, which goes to `mean`, and also ||c||^2 - ||that point||^2 (W columns a load);
 // the exact-pass queues are emptied, with reset_all the status word and counters too.
-__global__ void __launch_bounds__(256) centroid_prep_kernel(const float *__restrict__ C, int D,
-                                                            const float *__restrict__ mean, float *__restrict__ cnorm,
-                                                            float *__restrict__ cmax, Control *ctl, int reset_all)
+template <int W>
+__global__ void __launch_bounds__(256) centroid_prep_kernel(const float *__restrict__ C, int D, int K,
+                                                            float *mean, float *__restrict__ cnorm, float *__restrict__ cmax,
+                                                            float *__restrict__ aconst, Control *ctl,
+                                                            int reset_all)
 {
     pdl_enter();
-    __shared__ double wsum[8];
+    __shared__ double wsum[8], wsum_a[8];
     __shared__ float wmax[8];
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         ctl->refine_count = 0;
@@ -1141,31 +1174,60 @@ __global__ void __launch_bounds__(256) centroid_prep_kernel(const float *__restr
         }
     }
     const float *c = C + (size_t)blockIdx.x * D;
-    double s = 0.0;
+    double s = 0.0, a = 0.0;
     float m = 0.f;
+    if (aconst) {
+        const float *c1 = C + (size_t)(K > 1 ? 1 : 0) * D, *c2 = C + (size_t)(K > 2 ? 2 : 0) * D;
+        for (int j = W * threadIdx.x; j < D; j += W * 256) {
+            float w[W], p0[W], p1[W], p2[W];
+            load_cols<W>(c, j, w);
+            load_cols<W>(C, j, p0);
+            load_cols<W>(c1, j, p1);
+            load_cols<W>(c2, j, p2);
+#pragma unroll
+            for (int q = 0; q < W; ++q) {
+                const float o = median_of_three(p0[q], p1[q], p2[q]), v = w[q] - o;
+                if (blockIdx.x == 0) mean[j + q] = o;
+                const double d = (double)w[q] - (double)o;
+                s = fma(d, d, s);
+                a = fma(d, (double)w[q] + (double)o, a);
+                if (fabsf(v) < CUDART_INF_F) m = fmaxf(m, fabsf(v));
+            }
+        }
+    } else {
 #pragma unroll 4
-    for (int j = threadIdx.x; j < D; j += 256) {
-        const float v = mean ? __ldg(c + j) - __ldg(mean + j) : __ldg(c + j);
-        s = fma((double)v, (double)v, s);
-        if (fabsf(v) < CUDART_INF_F) m = fmaxf(m, fabsf(v));
+        for (int j = threadIdx.x; j < D; j += 256) {
+            const float v = mean ? __ldg(c + j) - __ldg(mean + j) : __ldg(c + j);
+            s = fma((double)v, (double)v, s);
+            if (fabsf(v) < CUDART_INF_F) m = fmaxf(m, fabsf(v));
+        }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         s += __shfl_xor_sync(0xffffffffu, s, o);
         m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if (aconst) a += __shfl_xor_sync(0xffffffffu, a, o);
     }
     if ((threadIdx.x & 31) == 0) {
         wsum[threadIdx.x >> 5] = s;
+        wsum_a[threadIdx.x >> 5] = a;
         wmax[threadIdx.x >> 5] = m;
     }
     __syncthreads();
+    if (threadIdx.x >= 32) return;
+    s = wsum[threadIdx.x & 7];
+    a = wsum_a[threadIdx.x & 7];
+    m = wmax[threadIdx.x & 7];
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+        s += __shfl_xor_sync(0xffffffffu, s, o);
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if (aconst) a += __shfl_xor_sync(0xffffffffu, a, o);
+    }
     if (threadIdx.x == 0) {
-        for (int w = 1; w < 8; ++w) {
-            s += wsum[w];
-            m = fmaxf(m, wmax[w]);
-        }
         cnorm[blockIdx.x] = __double2float_ru(s);
         cmax[blockIdx.x] = m;
+        if (aconst) aconst[blockIdx.x] = (float)a;
     }
 }
 
@@ -1342,13 +1404,16 @@ cudaError_t launch_sample_mean(const float *Y, int64_t N, int D, float *mean, cu
     return e;
 }
 
-cudaError_t launch_centroid_half(const float *C, int D, int K, const float *mean, float *cnorm, float *cmax, float *cerr, float *scale,
-                                 void *Ch, Control *ctl, cudaStream_t s, bool reset_all, bool own_scale)
+cudaError_t launch_centroid_half(const float *C, int D, int K, float *mean, float *cnorm, float *cmax, float *cerr, float *scale,
+                                 void *Ch, Control *ctl, cudaStream_t s, bool reset_all, bool own_scale, float *aconst)
 {
-    cudaError_t e = launch_pdl(centroid_prep_kernel, dim3((unsigned)K), dim3(256), 0, s, C, D, mean, cnorm, cmax, ctl, reset_all ? 1 : 0);
+    const bool vec = D % 4 == 0 && ((reinterpret_cast<uintptr_t>(C) | reinterpret_cast<uintptr_t>(mean)) & 15) == 0;
+    const dim3 grid((unsigned)K), block(256);
+    cudaError_t e = launch_pdl(vec ? centroid_prep_kernel<4> : centroid_prep_kernel<1>, grid, block, 0, s, C, D, K, mean, cnorm, cmax, aconst,
+                               ctl, reset_all ? 1 : 0);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(to_half_kernel, dim3((unsigned)K), dim3(256), 0, s, C, K, D, half_ld(D), mean, own_scale ? cmax : nullptr, scale,
-                   reinterpret_cast<__half *>(Ch), cerr);
+    e = launch_pdl(vec ? to_half_kernel<4> : to_half_kernel<1>, grid, block, 0, s, C, K, D, half_ld(D), mean, own_scale ? cmax : nullptr,
+                   scale, reinterpret_cast<__half *>(Ch), cerr);
     count_launch(2);
     return e;
 }

@@ -429,19 +429,7 @@ __device__ __forceinline__ float tc_error_bound(int D, float ysq, float cmax2)
     return 1.0625f * ((a + 2.f * pk) * yc + (4.f * u + pk) * cmax2);
 }
 
-// Same for fp16 operands (round to nearest, scaled by powers of two; ay, ac = absolute rounding
-// error of a row / centroid element that falls into fp16's subnormal range).
-__device__ __forceinline__ float tc_error_bound_half(int D, float ysq, float cmax2, float ay, float ac)
-{
-    const float u = 5.9604645e-8f;   // 2^-24
-    const float r = 1.953125e-3f * 1.001f + (2.f * (float)D + 2.f) * 2.3841858e-7f;  // 2^-9 (1 + 2^-12) + (2D+2) 2^-22
-    const float pk = 3.0517578e-5f;
-    const float yn = sqrtf(ysq), cn = sqrtf(cmax2);
-    return 1.0625f * ((r + 2.f * pk) * yn * cn + 2.f * sqrtf((float)D) * (ac * yn + ay * cn) +
-                      2.f * (float)D * ay * ac + (4.f * u + pk) * cmax2);
-}
-
-// The same where the rounding errors of the fp16 operands were measured while the copies were made (norms dy
+// The same for fp16 operands whose rounding errors were measured while the copies were made (norms dy
 // of the row's, dc the largest of the centroids'): |y.c - fp16(y).fp16(c)| <= dy c + (y + dy) dc.  y and c may be
 // taken relative to a common point (rounded to fp32 once: the 2 in 2 D + 4).
 __device__ __forceinline__ float tc_error_bound_measured(int D, float ysq, float cmax2, float dy, float dc)
@@ -451,6 +439,20 @@ __device__ __forceinline__ float tc_error_bound_measured(int D, float ysq, float
     const float pk = 3.0517578e-5f;
     const float yn = sqrtf(ysq), cn = sqrtf(cmax2);
     return 1.0625f * ((a + 2.f * pk) * yn * cn + 2.f * (dy * cn + (yn + dy) * dc) + (8.f * u + pk) * cmax2);
+}
+
+// The same for scores a_k - 2 y.(c_k - m), a_k = ||c_k||^2 - ||m||^2, of rows as they are, rounded to fp16 with 2^-11 relative
+// and ay absolute error (elements in fp16's subnormal range): c = largest ||c_k - m||, dc the largest norm of their rounding
+// errors, amax the largest |a_k| (c_k - m is rounded to fp32 before: 2^-24 c beside dc).  e = ||y|| x + ay y + z of what is
+// returned.
+__device__ __forceinline__ float3 tc_error_terms_centred(int D, float cmax2, float dc, float amax)
+{
+    const float u = 5.9604645e-8f;   // 2^-24
+    const float a = (2.f * (float)D + 4.f) * 2.3841858e-7f;   // (2D+4) 2^-22
+    const float r = 4.8828125e-4f * 1.001f;                   // 2^-11
+    const float pk = 3.0517578e-5f, cn = sqrtf(cmax2), d = dc + 2.f * u * cn;
+    return make_float3(1.0625f * ((a + 2.f * pk) * cn + 2.f * (r * cn + (1.f + r) * d)), 1.0625f * 2.f * sqrtf((float)D) * (cn + d),
+                       1.0625f * (8.f * u + pk) * amax);
 }
 
 // True where a bound e on the error of a row's scores also says that its keys mean what they should.  e is at
