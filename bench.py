@@ -357,14 +357,15 @@ def run_cuda(args):
                                         "objective_never_rises": bool(all(b <= a * (1 + 1e-12) for a, b in
                                                                           zip(d["objective"], d["objective"][1:])))}
     apply_kernel = {"small_kernel": "small_kernel<inference> (one persistent launch: TF32 scores, in-kernel exact pass, affine from the staged tile)",
+                    "apply_short_kernel": "apply_short_kernel (sixteen rows in a warp's registers, exact decision inside)",
                     "apply_rows_kernel": "apply_rows_kernel (groups of eight rows in shared memory, exact decision inside)",
                     "apply_h64_kernel": "apply_h64_kernel (64-row tiles, fp16 operands made in the kernel)"}
     apply_name = B.cat_kernel_for("apply", N_apply, D, K)
     apply_kernel = apply_kernel.get(apply_name, apply_name)
     fit_name = B.cat_kernel_for("fit", N_fit, D, K)
-    if fit_name == "fit_rows_kernel":
+    if fit_name in ("fit_rows_kernel", "fit_tiles_kernel"):
         # (the rounds end at a fixed point, so a round of the difference may be shorter than a full one)
-        roofline_fit = {"bound": "latency", "kernel": "one Lloyd round inside fit_rows_kernel (one cooperative launch for the whole "
+        roofline_fit = {"bound": "latency", "kernel": f"one Lloyd round inside {fit_name} (one cooperative launch for the whole "
                         "fit, rows in shared memory)", "achieved": lloyd_alg_gbs, "peak": peak, "unit": "GB/s",
                         "frac": lloyd_alg_gbs / peak, "peak_source": peak_src, "tflops": lloyd_tflops}
     elif fit_name == "small_kernel":
@@ -398,7 +399,7 @@ def run_cuda(args):
             "fit_s_per_lloyd_iter": lloyd_ms * 1e-3,
             "fit_ms": fit_ms_step, "fit_one_round_ms": fit1_ms, "apply_ms": apply_ms_step,
             "wall_s": t_wall,
-            "roofline": {"bound": "hbm", "kernel": apply_kernel + ("" if apply_kernel.startswith(("small_kernel", "apply_rows")) else " (the one kernel of cat_apply besides the exact pass)"),
+            "roofline": {"bound": "hbm", "kernel": apply_kernel + ("" if apply_kernel.startswith(("small_kernel", "apply_rows", "apply_short")) else " (the one kernel of cat_apply besides the exact pass)"),
                          "achieved": apply_gbs, "peak": peak, "unit": "GB/s", "frac": apply_gbs / peak,
                          "peak_source": peak_src, "traffic": traffic},
             "roofline_fit": roofline_fit,

@@ -419,9 +419,12 @@ int32_t cat_get_tensor_core_min_k(void);
  * K <= 128 (K >= a quarter of the threshold; rows up to about 3300 columns for K <= 32, 3000 for K <= 64, 2500 above), in
  * two launches that keep each row in shared memory -- except, for 4096 rows and more with D % 4 == 0 and D <= 1536, where
  * K * D > 32768 (D % 8 == 0) or K > 64 (rows of 128 to 256 columns excepted), and short rows with many centroids: those
- * stay on the tile kernels (cat_kernel_for tells).  mask bit 1: so do the K-Means
+ * stay on the tile kernels (cat_kernel_for tells); 8192 and more rows of 32, 48, 64, 96 or 128 columns with K * D small enough for
+ * shared memory stay in registers in one launch.  mask bit 1: so do the K-Means
  * rounds and the final assignment of cat_fit / cat_fit_from (Algorithm 1, step 2; calls without
- * per-round diagnostics), and of other sets of up to 8192 rows with moderate N * K * D (of those shapes too up to 4096 rows).  Default 3:
+ * per-round diagnostics), and of other sets of up to 8192 rows with moderate N * K * D (of those shapes too up to 4096 rows), and
+ * of more than 8192 rows of 4 to 256 columns with K * D <= 8192 as far as their fp16 form fits into the device's shared
+ * memory.  Default 3:
  * both are the faster form where they apply.  Clearing a bit sends these shapes down the general multi-launch path instead: same labels (rows on a bisector
  * apart, when a centroid differs in its last bit); sums that agree to fp64 rounding.  A PROCESS-WIDE
  * tuning and test hook like the one above. */

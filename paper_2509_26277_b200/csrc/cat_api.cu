@@ -168,12 +168,11 @@ static bool use_fit_rows(int64_t N, int D, int K)
            (N <= 4096 || !use_small_fit(N, D, K));
 }
 // Rows as fp16 fragments in shared memory for all rounds: more than 8192 rows (200 704 x 64, K = 64 1030 us against 1390 in the
-// persistent kernel, 108 286 x 256, K = 49 1510 against 1790 on the general path's sorts; up to 8192 rows the kernels of small sets
-// are as fast or faster and some of these rows' lists are what tests pin).  Clusters alone, as of PCA's reduced rows, from 2048 on:
-// 4096 x 50, K = 32 without the closed form's labels pass.
-static bool use_fit_tiles(int64_t N, int D, int K, bool clusters_only)
+// persistent kernel, 108 286 x 256, K = 49 1510 against 1790 on the general path).  Up to there the kernels of small sets have the
+// shorter rounds (PCA fits with reduced sets of 2048 x 20, K = 10 1314 us against 1358 here, 4096 x 50, K = 32 the same).
+static bool use_fit_tiles(int64_t N, int D, int K)
 {
-    return (g_small_kernels.load(std::memory_order_relaxed) & 2) && (N > 8192 || (clusters_only && N >= 2048)) && fit_tiles_supported(N, D, K);
+    return (g_small_kernels.load(std::memory_order_relaxed) & 2) && N > 8192 && fit_tiles_supported(N, D, K);
 }
 static bool use_small_apply(int64_t N, int D, int K)
 {
@@ -585,7 +584,7 @@ static cat_status_t cat::fit_from(const float *Yq, const float *Yfp, int64_t N, 
 
     // Small problems without per-round diagnostics: every round, the final assignment and the
     // per-cluster sums and sizes that follow its labels come from one persistent launch.
-    const bool tiles = !diag && use_fit_tiles(N, D, K, clusters_only);
+    const bool tiles = !diag && use_fit_tiles(N, D, K);
     const bool rows = !diag && !tiles && use_fit_rows(N, D, K);
     const bool small = tiles || rows || (!diag && use_small_fit(N, D, K));
     if (tiles) {
@@ -880,7 +879,7 @@ const char *cat_kernel_for(int32_t call, int64_t N, int32_t D, int32_t K)
         if (use_apply_rows(N, D, K, true)) return "apply_rows_kernel";
         break;
     case CAT_CALL_FIT:
-        if (use_fit_tiles(N, D, K, false)) return "fit_tiles_kernel";
+        if (use_fit_tiles(N, D, K)) return "fit_tiles_kernel";
         if (use_fit_rows(N, D, K)) return "fit_rows_kernel";
         if (use_small_fit(N, D, K)) return "small_kernel";
         break;
