@@ -240,8 +240,8 @@ static cat_status_t run_assign(const float *Y, int64_t N, int D, int K, const fl
         return CAT_OK;
     }
     if (out && labels && top_level && !fast && use_apply_rows(N, D, K, false)) {
-        // rows kept in shared memory from the first read to the corrected store (behind the kernel above
-        // where both apply: 200 704 x 64, K = 64 takes 69 us here and 43 there)
+        // rows kept in shared memory from the first read to the corrected store (behind the kernels above
+        // where both apply: 200 704 x 64, K = 64 takes 69 us here, 35 and 50 there)
         CAT_CUDA(launch_apply_rows(Y, N, D, K, C, gamma, beta, out, false, labels, w.ctl, w.prep, s));
         return CAT_OK;
     }

@@ -37,7 +37,7 @@
 //   e += 2^-24 ||y - mean|| (||w|| + ||V||_F max ||c_k - m||).
 // Several candidates: the same dot products in fp32 from w_k in fp32; for the rows that these leave (one in a thousand) a kernel
 // behind this one forms the projection in fp64 and the distances in the reduced space.  50 000 x 1000, 50 components, K = 64: the projection in fp64, the assignment of
-// the reduced rows and the correction took 377 us.
+// the reduced rows and the correction took 377 us, this takes 235 - 245.
 #include "cat_tc.cuh"
 
 #include <cuda_bf16.h>

@@ -7,7 +7,8 @@
 // inverse iteration with orthogonalisation against all larger pairs, then the reflections are
 // applied to the p vectors.  (Golub & Van Loan, Matrix Computations, ch. 8.)  One-sided Jacobi
 // rotations over all pairs of columns, the earlier form, took 155 ms for D = 1000: about ten sweeps
-// of 999 dependent launches.  This takes 5.1 ms there with p = 50.
+// of 999 dependent launches.  This takes 3.2 ms there with p = 50 (2.5 the reduction, bound by the fp64 latency of its sweeps and one
+// exchange between CTAs a step; 0.7 the eigenvectors); with two exchanges a step and branches in the sweep it took 5.1.
 //
 // Both kernels are cooperative launches; every wait is bounded by TC_TIMEOUT_NS and reports
 // CAT_ERR_DEVICE_TIMEOUT in the control block.  Every sum has a fixed order: results do not vary
