@@ -333,7 +333,7 @@ cat_status_t cat_affine_with_labels(const float *Yq, int64_t N, int32_t D, int32
  * start, `iters` Lloyd rounds, a final assignment), then per cluster the closed-form gamma / beta
  * from the original Yq, Yfp.  centroids_out is [K, p]; gamma_out, beta_out are [K, D].
  * Algorithm 2 as printed (alpha = 1): project, nearest centroid in the reduced space, affine
- * correction in the original space.
+ * correction in the original space.  Y_out [N, D] may be Yq itself; it must not overlap it otherwise.
  */
 size_t cat_fit_pca_workspace_bytes(int64_t N, int32_t D, int32_t K, int32_t p);
 cat_status_t cat_fit_pca(const float *Yq, const float *Yfp, int64_t N, int32_t D, int32_t K,

@@ -727,7 +727,7 @@ __global__ void __launch_bounds__(RES_MAX_THREADS, 1) apply_rows_kernel(ResParam
             load_group<VEC>(p, (int64_t)(grp + g_step) * RR, slots + (slot ^ 1) * slot_floats, bars + (slot ^ 1));
 
         // ---- decide this warp's rows, LPR lanes each
-        int label;   // of row tw + (lane / LPR) TW; -1: beyond the matrix
+        int label;   // of row tw + (lane / LPR) TW; -1: beyond the matrix, or left to the kernel behind this one
         {
             const int r = tw + (lane / LPR) * TW, l = lane % LPR;
             const uint32_t mine = LPR == 32 ? 0xffffffffu : ((1u << (LPR & 31)) - 1u) << (lane / LPR * LPR);
@@ -786,13 +786,16 @@ __global__ void __launch_bounds__(RES_MAX_THREADS, 1) apply_rows_kernel(ResParam
                     uint2 rest;
                     exact = settle_pca<VEC>(rows + ro * p.ldy, mean, reinterpret_cast<const float *>(p.prep + lift_offset(MT, p.nk)), ak, p.D,
                                             make_uint2(mask[0], mask[1]), noise, lane, &rest);
-                    if ((rest.x | rest.y) != 0u && lane == 0)
-                        p.open_rows[atomicAdd(&p.ctl->refine_count, 1)] = make_uint4((uint32_t)(row0 + ro), rest.x, rest.y, 0u);
+                    if ((rest.x | rest.y) != 0u) {
+                        // (left as it is: the kernel behind this one reads the row again, and Y may be the output)
+                        if (lane == 0) p.open_rows[atomicAdd(&p.ctl->refine_count, 1)] = make_uint4((uint32_t)(row0 + ro), rest.x, rest.y, 0u);
+                        exact = -1;
+                    }
                 } else
                     exact = settle<VEC>(rows + ro * p.ldy, p.C, p.D, make_uint4(mask[0], mask[1], mask[2], mask[3]), lane);
                 if (lane / LPR == src / LPR) label = exact;
             }
-            if (l == 0 && live) p.labels[row0 + r] = label;
+            if (l == 0 && live && (!PCA || label >= 0)) p.labels[row0 + r] = label;
             if (!live) label = -1;
         }
 
@@ -873,13 +876,14 @@ __global__ void __launch_bounds__(RES_MAX_THREADS, 1) apply_rows_kernel(ResParam
 }
 
 // The rows that fp32 has not decided, a CTA each: the projection in fp64, rounded to fp32, and the candidates' distances to it
-// in fp64, lowest index on equality; then the correction once more.  A launch of its own: a warp of the kernel above
+// in fp64, lowest index on equality; then the correction.  (Y may be `out`: a row is read before it is written, by the thread
+// that writes it.)  A launch of its own: a warp of the kernel above
 // would be at one such row for as long as it takes its team to go through three groups of rows.
 constexpr int OPEN_THREADS = 256;
-__global__ void __launch_bounds__(OPEN_THREADS) open_rows_kernel(const float *__restrict__ Y, const float *__restrict__ C, int D, int K, int p,
+__global__ void __launch_bounds__(OPEN_THREADS) open_rows_kernel(const float *Y, const float *__restrict__ C, int D, int K, int p,
                                                                  const float *__restrict__ mean, const float *__restrict__ comps,
                                                                  const float *__restrict__ gamma, const float *__restrict__ beta,
-                                                                 float *__restrict__ out, int32_t *__restrict__ labels,
+                                                                 float *out, int32_t *__restrict__ labels,
                                                                  const uint4 *__restrict__ open_rows, const Control *ctl)
 {
     pdl_enter();
@@ -892,7 +896,7 @@ __global__ void __launch_bounds__(OPEN_THREADS) open_rows_kernel(const float *__
     for (int i = blockIdx.x; i < n; i += gridDim.x) {
         const uint4 e = open_rows[i];
         const float *y = Y + (size_t)e.x * D;
-        for (int j = tid; j < D; j += OPEN_THREADS) xs[j] = (double)__ldg(y + j) - (double)__ldg(mean + j);
+        for (int j = tid; j < D; j += OPEN_THREADS) xs[j] = (double)y[j] - (double)__ldg(mean + j);
         __syncthreads();
         // (eight components of a warp side by side, 32 loads in flight per lane)
         for (int r0 = warp * 8; r0 < p; r0 += OPEN_THREADS / 32 * 8) {
@@ -942,7 +946,7 @@ __global__ void __launch_bounds__(OPEN_THREADS) open_rows_kernel(const float *__
         }
         __syncthreads();
         const size_t o = (size_t)s_label * D;
-        for (int j = tid; j < D; j += OPEN_THREADS) out[(size_t)e.x * D + j] = fmaf(__ldg(gamma + o + j), __ldg(y + j), __ldg(beta + o + j));
+        for (int j = tid; j < D; j += OPEN_THREADS) out[(size_t)e.x * D + j] = fmaf(__ldg(gamma + o + j), y[j], __ldg(beta + o + j));
         __syncthreads();
     }
 }

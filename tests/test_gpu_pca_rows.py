@@ -96,3 +96,24 @@ def test_components_that_are_not_unit_vectors_and_rows_out_of_range():
     np.testing.assert_array_equal(got[0][1][rest], got[1][1][rest])
     np.testing.assert_array_equal(got[0][0][rest], got[1][0][rest])
     assert all(0 <= l < 24 for l in got[0][1][[6, 7]])
+
+
+@pytest.mark.parametrize("n,d,k", [(3000, 300, 20), (3001, 301, 20), (4000, 64, 7), (1000, 1001, 40)])
+def test_output_in_the_place_of_the_input(n, d, k):
+    """Rows on bisectors, which the kernel for open rows reads once more, with Y_out = Yq."""
+    rng = np.random.default_rng(n + d)
+    p = 12
+    V = np.linalg.qr(rng.normal(size=(d, p)))[0].T.astype(np.float32)
+    C = rng.normal(size=(k, p)).astype(np.float32)
+    i, j = rng.integers(0, k, size=n), rng.integers(0, k, size=n)
+    Y = ((0.5 * (C[i] + C[j])) @ V + 1e-7 * rng.normal(size=(n, d))).astype(np.float32)
+    g, b = rng.normal(size=(k, d)).astype(np.float32), rng.normal(size=(k, d)).astype(np.float32)
+    mean = np.zeros(d, np.float32)
+    ws = B.pca_workspace("apply_pca", n, d, p, "cuda", k)
+    want, lab = B.cat_apply_pca(dev(Y), dev(mean), dev(V), dev(C), dev(g), dev(b), want_labels=True, ws=ws)
+    np.testing.assert_array_equal(host(want), O.affine_with_labels(Y, host(lab), g, b))
+    assert int(ws[:4].view(torch.int32)) > 100   # (the control block's first word: rows listed for that kernel)
+    y = dev(Y)
+    _, lab2 = B.cat_apply_pca(y, dev(mean), dev(V), dev(C), dev(g), dev(b), out=y, want_labels=True)
+    assert torch.equal(lab, lab2)
+    assert torch.equal(y, want)
