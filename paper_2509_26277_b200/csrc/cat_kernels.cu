@@ -64,6 +64,7 @@ __global__ void centroid_norms_kernel(const float *__restrict__ C, int D, int K,
             ctl->device_status = CAT_OK;
             ctl->refined_total = 0;
             ctl->refined_last = 0;
+            ctl->settled = 0;
         }
     }
     if (warp >= K) return;
@@ -533,6 +534,17 @@ __device__ __forceinline__ void refine_distances(const float *ys, int ld, const 
     else refine_distances<VEC, 1>(ys, ld, C, D, K, dist);
 }
 
+// The counters behind an assignment that has queued `count` rows for the full exact pass (the candidate pass, if any, has
+// already added its rows).  (Behind a fixed point nothing
+// runs: the assignments there would have queued the rows of the one before them.)
+__device__ __forceinline__ void count_refined(Control *ctl, int count)
+{
+    const bool over = ctl->settled;
+    const int64_t last = ctl->refined_last, total = ctl->refined_total;
+    ctl->refined_total = total + (over ? last : count);
+    if (!over) ctl->refined_last = count + ctl->cand_count;
+}
+
 template <bool AFFINE>
 __device__ __forceinline__ void refine_body_grouped(const float *__restrict__ Y, int64_t N, int D, int K,
                                                     const float *__restrict__ C, int32_t *labels,
@@ -541,10 +553,7 @@ __device__ __forceinline__ void refine_body_grouped(const float *__restrict__ Y,
 {
     int count = ctl->refine_count;
     if ((int64_t)count > N) count = (int)N;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        ctl->refined_total += count;
-        ctl->refined_last = count + ctl->cand_count;
-    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) count_refined(ctl, count);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int ld = (D + 3) & ~3;
     float *dist = ys + RG * ld;   // [RG][K]
@@ -620,11 +629,7 @@ __device__ __forceinline__ void refine_body(const float *__restrict__ Y, int64_t
     __shared__ int s_label;
     int count = ctl->refine_count;
     if ((int64_t)count > N) count = (int)N;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        // the candidate pass (if any) ran before this kernel and has already added its rows
-        ctl->refined_total += count;
-        ctl->refined_last = count + ctl->cand_count;
-    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) count_refined(ctl, count);
     const int lane = threadIdx.x & 31;
     const int w = threadIdx.x >> 5;
     for (int it = blockIdx.x; it < count; it += gridDim.x) {

@@ -1171,6 +1171,7 @@ __global__ void __launch_bounds__(256) centroid_prep_kernel(const float *__restr
             ctl->device_status = CAT_OK;
             ctl->refined_total = 0;
             ctl->refined_last = 0;
+            ctl->settled = 0;
         }
     }
     const float *c = C + (size_t)blockIdx.x * D;

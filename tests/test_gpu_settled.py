@@ -43,3 +43,24 @@ def test_rounds_after_a_fixed_point_change_nothing(n, d, k, spread):
     first = O.fit(Yq, Yfp, k, 0)
     assert (got[0][0][3].numpy() != first.labels).mean() < 1e-3
     np.testing.assert_array_equal(counts.cpu().numpy(), np.bincount(got[60][0][3].numpy(), minlength=k))
+
+
+@pytest.mark.parametrize("n,d,k", [(2000, 64, 16), (2001, 100, 5), (1000, 1601, 9), (3000, 30, 3), (3000, 16, 20), (1500, 1000, 8)])
+def test_counters_of_the_exact_pass_do_not_depend_on_the_early_end(n, d, k):
+    """One cloud of rows, some of which are undecided in every round; its labels come to rest within 90 rounds.  With
+    diagnostics every assignment runs, and the counters are those of that fit."""
+    Yq = (np.random.default_rng(4).normal(size=(n, d)) * np.linspace(3.0, 0.3, d)).astype(np.float32)
+    q = torch.from_numpy(Yq).cuda()
+    old = B.cat_get_small_problem_kernels()
+    B.cat_set_small_problem_kernels(0)
+    try:
+        ws = torch.empty(B.lib().cat_fit_workspace_bytes(n, d, k), dtype=torch.uint8, device="cuda")
+        for kw in (dict(), dict(init_centroids=torch.from_numpy(Yq[n - k:]).cuda())):
+            diag = B.cat_fit(q, q, k, 120, want_diag=True, ws=ws, **kw)[-1]
+            B.cat_fit(q, q, k, 120, ws=ws, **kw)
+            rep = B.cat_workspace_report(ws)
+            assert diag["refined_rows_total"] > 0 or k == 3   # (fp32 scores leave hardly a row open)
+            assert rep["refined_rows_last"] == diag["refined_rows_final"]
+            assert rep["refined_rows_total"] == diag["refined_rows_total"]
+    finally:
+        B.cat_set_small_problem_kernels(old)
