@@ -539,6 +539,9 @@ cat_status_t cat_fit_pca(const float *Yq, const float *Yfp, int64_t N, int32_t D
     const size_t need = cat_fit_pca_workspace_bytes(N, D, K, p);
     if (need == 0) return CAT_ERR_UNSUPPORTED;
     if (!workspace || !al16(workspace) || workspace_bytes < need) return CAT_ERR_WORKSPACE;
+    // (gamma and beta are written word by word: any address does)
+    if (!al16(Yq) || !al16(Yfp) || !al16(mean_out) || !al16(components_out) || !al16(centroids_out) || (labels_out && !al16(labels_out)))
+        return CAT_ERR_ALIGN;
     FitPcaWs w = carve_fit_pca(workspace, N, D, K, p);
     int32_t *labels = labels_out ? labels_out : w.labels;
     // Algorithm 1 step 1: the projection; step 2: K-Means on the reduced rows
@@ -548,7 +551,6 @@ cat_status_t cat_fit_pca(const float *Yq, const float *Yfp, int64_t N, int32_t D
     if ((st = fit_clusters(w.Z, N, p, K, iters, centroids_out, labels, w.fit, w.fit_bytes, s)) != CAT_OK) return st;
     CAT_CUDA(launch_absorb_control(reinterpret_cast<Control *>(w.pca), reinterpret_cast<const Control *>(w.fit), s));
     // the loop over the clusters: moments and the closed form in the original space
-    if (!al16(Yfp) || !al16(gamma_out) || !al16(beta_out)) return CAT_ERR_ALIGN;
     return fit_closed_form(Yq, Yfp, N, D, K, labels, gamma_out, beta_out, w.fit, s);
 }
 

@@ -105,6 +105,7 @@ def test_argument_errors_return_before_any_device_work():
     # alignment
     assert L.cat_apply(odd, 8, 4, 2, fake, fake, fake, fake, None, fake, 1 << 20, None) == 3
     assert L.cat_fit(fake, fake, 8, 4, 2, 1, fake, odd, fake, None, fake, 1 << 20, None) == 3
+    assert L.cat_fit_pca(fake, odd, 8, 4, 2, 1, 3, fake, fake, fake, fake, fake, None, fake, 1 << 24, None) == 3
     # workspace
     assert L.cat_apply(fake, 8, 4, 2, fake, fake, fake, fake, None, None, 1 << 20, None) == 4
     assert L.cat_apply(fake, 8, 4, 2, fake, fake, fake, fake, None, fake, 16, None) == 4

@@ -184,3 +184,17 @@ def test_one_control_block_speaks_for_the_composed_calls():
     B.cat_assign(Z, r["centroids"], ws=wz)
     assert rep == B.cat_workspace_report(wz)
     assert rep["device_status"] == 0 and rep["refined_rows_last"] > 0
+
+
+@pytest.mark.parametrize("n,d,k", [(300, 40, 6), (5000, 40, 6)])
+def test_fit_pca_writes_gamma_and_beta_at_any_address(n, d, k):
+    p = 8
+    Y = dev(np.random.default_rng(1).normal(size=(n, d)).astype(np.float32))
+    want = B.cat_fit_pca(Y, Y, k, 3, p)
+    g, b = (torch.empty(k * d + 1, dtype=torch.float32, device="cuda")[1:] for _ in range(2))
+    r = {m: torch.empty_like(want[m]) for m in ("mean", "comps", "centroids")}
+    ws = B.pca_workspace("fit_pca", n, d, p, "cuda", K=k)
+    st = B.lib().cat_fit_pca(Y.data_ptr(), Y.data_ptr(), n, d, k, 3, p, r["mean"].data_ptr(), r["comps"].data_ptr(), r["centroids"].data_ptr(),
+                             g.data_ptr(), b.data_ptr(), None, ws.data_ptr(), ws.numel(), torch.cuda.current_stream().cuda_stream)
+    assert st == 0
+    assert torch.equal(g.view(k, d), want["gamma"]) and torch.equal(b.view(k, d), want["beta"])
