@@ -108,7 +108,7 @@ FitWs carve_fit(void *base, int64_t N, int D, int K)
     w.counts = c.take<int64_t>((size_t)K);
     w.norm_part = c.take<unsigned char>(centroid_update_scratch_bytes(D, K));
     w.arrivals = c.take<uint32_t>((size_t)K);
-    w.moved_flags = c.take<uint64_t>(moved_flag_words());
+    w.moved_state = c.take<uint64_t>(1);
     const size_t tiles = fit_tiles_part_doubles(D, K);   // (by D and K alone: a workspace for more rows serves fewer)
     if (tiles || small_fit_supported(N, D, K)) {
         const size_t a = small_fit_supported(N, D, K) ? small_part_doubles(D, K) : 0, b = small_part_counts(K), t = fit_tiles_counts(K);
@@ -337,12 +337,17 @@ static cat_status_t run_delta_update(const float *Yq, const int32_t *labels, con
     return CAT_OK;
 }
 
-// Rounds whose moved rows are listed instead of sorted: from the fourth on, where a tenth of the rows or fewer moves (262 144 x 1024,
-// K = 256: 45 us a round sorted, 10 listed; in the first rounds, where most rows move, the sort's segments spread them over more CTAs).
-// A cluster's CTAs read the whole list: with fewer than eight clusters too few of them share the sums.
-static bool use_moved_list(int round, int K, bool may_settle)
+// Rounds whose moved rows are listed instead of sorted: from the fourth on (in the first ones nearly all rows move, and the sort's
+// segments spread them over more CTAs).  A cluster's CTAs go through its entries by themselves, so it must not have too many rows;
+// 25 rounds, us sorted / listed (the labels of logits, and of a cloud of points at 600 000 rows, keep moving):
+//   few rows a cluster           20 000 x 300, K = 100 1271 / 1062, K = 8 1051 / 821;  200 000 x 50, K = 128 1865 / 1603
+//   rows a cluster, D % 4 == 0   25 000 (200 000 x 1000) 4598 / 4565, 50 000 (600 000 x 512) 6685 / 6705, 75 000 6582 / 6848
+//   D % 4 != 0                    4 200 (100 000 x 255) 1640 / 1517, 6 250 1582 / 1583, 7 500 (60 000 x 1001) 2412 / 2442,
+//                                25 000 (200 000 x 1001) 4891 / 5761
+// and with fewer than eight clusters too few CTAs share the sums.
+static bool use_moved_list(int round, int64_t N, int D, int K, bool may_settle)
 {
-    return may_settle && round >= 3 && K >= 8;
+    return may_settle && round >= 3 && K >= 8 && N <= (int64_t)(D % 4 == 0 ? 32768 : 6144) * K;
 }
 
 static cat_status_t run_centred(const float *Yq, const float *Yfp, int64_t N, int D, int K, const FitWs &w,
@@ -626,8 +631,8 @@ static cat_status_t cat::fit_from(const float *Yq, const float *Yfp, int64_t N, 
     CAT_CUDA(cudaMemsetAsync(lab[(iters & 1) ^ 1], 0xFF, (size_t)N * sizeof(int32_t), s));
     CAT_CUDA(cudaMemsetAsync(w.sumQ, 0, KD * sizeof(double), s));
     CAT_CUDA(cudaMemsetAsync(w.counts, 0, (size_t)K * sizeof(int64_t), s));
-    // (arrivals, and behind them the flags)
-    CAT_CUDA(cudaMemsetAsync(w.arrivals, 0, (size_t)((char *)(w.moved_flags + moved_flag_words()) - (char *)w.arrivals), s));
+    // (arrivals, and behind them the state)
+    CAT_CUDA(cudaMemsetAsync(w.arrivals, 0, (size_t)((char *)(w.moved_state + 1) - (char *)w.arrivals), s));
     for (int t = 0; t < iters; ++t) {
         int32_t *cur = lab[(iters - t) & 1], *prev = lab[((iters - t) & 1) ^ 1];
         st = run_assign(Yq, N, D, K, C, cur, w.a, nullptr, nullptr, nullptr, s, tc, false, Yh, w.ch, w.hscale,
@@ -636,8 +641,8 @@ static cat_status_t cat::fit_from(const float *Yq, const float *Yfp, int64_t N, 
         if (diag && t < CAT_DIAG_MAX_ROUNDS - 1)
             CAT_CUDA(launch_fit_diag_round(Yq, N, D, K, C, cur, w.a.refine_rows, w.a.cand_rows, w.a.ctl, diag, t,
                                            diag_recorded, s));
-        if (use_moved_list(t, K, settled != nullptr)) {
-            CAT_CUDA(launch_moved_update(Yq, cur, prev, N, D, K, (uint32_t)t, w.order, w.moved_flags, w.counts, w.sumQ, C, w.a.cnorm, w.hscale,
+        if (use_moved_list(t, N, D, K, settled != nullptr)) {
+            CAT_CUDA(launch_moved_update(Yq, cur, prev, N, D, K, w.order, w.blk_hist, w.moved_state, w.counts, w.sumQ, C, w.a.cnorm, w.hscale,
                                          half ? w.ch : nullptr, half ? w.a.mean : nullptr, w.a.cerr, w.norm_part, w.arrivals, w.a.ctl, settled, s));
         } else {
             st = run_delta_update(Yq, cur, prev, N, D, K, w, C, half, s, settled);

@@ -154,7 +154,7 @@ struct FitWs {
     int64_t *counts;       // [K]
     void *norm_part;       // parts of the centroid norms (centroid update)
     uint32_t *arrivals;    // [K] CTAs of a cluster that have left theirs
-    uint64_t *moved_flags; // counts that pass between the CTAs that list moved rows
+    uint64_t *moved_state; // what passes between the CTAs that list moved rows
     double *small_part;    // per-CTA sums of the single-launch fits that keep them in planes (or null)
     int32_t *small_counts; // ... and their counters
     size_t bytes;
@@ -343,11 +343,10 @@ cudaError_t launch_centroid_update(const double *part, const int32_t *seg_start,
                                    const float *mean, float *cerr, void *norm_part, uint32_t *arrivals, Control *ctl,
                                    cudaStream_t s, const int32_t *settled = nullptr);
 size_t centroid_update_scratch_bytes(int D, int K);
-// The same, counts included, straight from two label buffers: for rounds in which few rows move.  list: N 8-byte entries;
-// flags: moved_flag_words() 8-byte words, zero before the first call; tag: not zero, another one for each call on these flags.
-size_t moved_flag_words();
-cudaError_t launch_moved_update(const float *Y, const int32_t *cur, const int32_t *prev, int64_t N, int D, int K, uint32_t tag, void *list,
-                                void *flags, int64_t *counts, double *sums, float *C, float *cnorm, const float *scale, void *Ch,
+// The same, counts included, straight from two label buffers: for rounds in which few rows move.  list: N 8-byte entries; table:
+// 4 (K + 1) bytes for every 2048 rows; state: an 8-byte word, zero before the first call.
+cudaError_t launch_moved_update(const float *Y, const int32_t *cur, const int32_t *prev, int64_t N, int D, int K, void *list, void *table,
+                                void *state, int64_t *counts, double *sums, float *C, float *cnorm, const float *scale, void *Ch,
                                 const float *mean, float *cerr, void *norm_part, uint32_t *arrivals, Control *ctl, int32_t *settled,
                                 cudaStream_t s);
 

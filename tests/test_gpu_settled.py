@@ -6,6 +6,7 @@ import torch
 
 from oracle import cat_oracle as O
 from paper_2509_26277_b200 import binding as B
+from tests.parity import labels_match
 
 pytestmark = pytest.mark.gpu
 
@@ -43,6 +44,33 @@ def test_rounds_after_a_fixed_point_change_nothing(n, d, k, spread):
     first = O.fit(Yq, Yfp, k, 0)
     assert (got[0][0][3].numpy() != first.labels).mean() < 1e-3
     np.testing.assert_array_equal(counts.cpu().numpy(), np.bincount(got[60][0][3].numpy(), minlength=k))
+
+
+# (aligned rows and not; a tile of rows a CTA, several, a last one that is not full; clusters whose entries fill more than a chunk; most
+# clusters and fewest)
+@pytest.mark.parametrize("n,d,k", [(200_000, 1028, 8), (50_003, 33, 512), (303_104, 16, 200), (303_105, 9, 200), (700_001, 12, 200)])
+def test_rounds_in_which_many_rows_move(n, d, k):
+    """One cloud of rows, which keeps moving: from the fourth round on the update follows a list of the moved rows."""
+    Yq = np.random.default_rng(n).normal(size=(n, d)).astype(np.float32)
+    q = torch.from_numpy(Yq).cuda()
+    old = B.cat_get_small_problem_kernels()
+    B.cat_set_small_problem_kernels(0)
+    try:
+        res = {t: [x.cpu().numpy() for x in B.cat_fit(q, q, k, t)] for t in (4, 5, 6)}
+        again = B.cat_fit(q, q, k, 6)
+    finally:
+        B.cat_set_small_problem_kernels(old)
+    assert all(np.array_equal(a, b.cpu().numpy()) for a, b in zip(res[6], again))
+    for t in (4, 5):
+        moved = res[t][3] != res[t + 1][3]
+        entries = np.bincount(np.concatenate([res[t][3][moved], res[t + 1][3][moved]]), minlength=k)
+        assert moved.sum() > n // 200 and (k > 8 or entries.max() > 2048)
+    for t in (4, 5):
+        want, _ = O.update_centroids(Yq, res[t][3], res[t][0])
+        # (both are fp32 roundings of fp64 means)
+        np.testing.assert_allclose(res[t + 1][0], want, rtol=2.0 ** -23, atol=1e-12)
+    lab, best, second = O.assign(Yq, res[6][0])
+    labels_match(res[6][3], lab, best, second, "labels")
 
 
 @pytest.mark.parametrize("n,d,k", [(2000, 64, 16), (2001, 100, 5), (1000, 1601, 9), (3000, 30, 3), (3000, 16, 20), (1500, 1000, 8)])
