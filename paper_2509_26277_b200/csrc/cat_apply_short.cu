@@ -9,6 +9,8 @@
 // The kernel this takes such calls from (csrc/cat_small.cu) passes a tile of 128 rows through five warp roles, whose
 // hand-overs bounded it.  tcgen05 would bring them back: its accumulators are read by other warps than those that
 // wait for its operands; the contraction is small here (K <= 128, D <= 128).
+// Only the tiles of sixteen centroids that exist are formed (all eight from K = 65 on before: 80 000 x 64, K = 80 30.6 us, 26.0 so, 28.1
+// in the persistent kernel; 80 000 x 32, K = 70 22.0, 18.5 and 20.3).
 // The next group's rows are on their way into shared memory (cp.async, every lane what it will read itself) while this one's
 // are worked on.
 //   bound: instruction issue, about 700 instructions a group; 11 us are start, centroids and end.  200 704 x 64, K = 64 (floor
@@ -44,7 +46,7 @@ __host__ __device__ constexpr int short_threads(int nks) { return nks <= 4 ? 512
 __host__ __device__ constexpr int short_ld(int D) { return D % 32 == 0 ? D + 16 : D; }
 size_t short_smem(int D, int K, bool ahead)
 {
-    const size_t nt = K > 64 ? 8 : (K + 15) / 16;
+    const size_t nt = (K + 15) / 16;
     const size_t rows = ahead ? (size_t)short_threads(D / 16) / 32 * 16 * D * 4 : 0;
     return rows + (size_t)3 * K * short_ld(D) * 4 + nt * 16 * D * 2 + nt * 16 * 2 * 4 + (size_t)D * 4;
 }
@@ -516,7 +518,7 @@ cudaError_t launch_apply_short(const float *Y, int64_t N, int D, int K, const fl
                                bool out_bf16, int32_t *labels, Control *ctl, cudaStream_t s)
 {
     if (!apply_short_supported(N, D, K)) return cudaErrorInvalidValue;
-    const int nt = K > 64 ? 8 : (K + 15) / 16;
+    const int nt = (K + 15) / 16;
     const ShortParams p{Y, C, gamma, beta, out, labels, ctl, N, K, nt};
     return out_bf16 ? launch_short_d<true>(D, p, s) : launch_short_d<false>(D, p, s);
 }
