@@ -419,7 +419,7 @@ int32_t cat_get_tensor_core_min_k(void);
  * K <= 128 (K >= a quarter of the threshold; rows up to about 3300 columns for K <= 32, 3000 for K <= 64, 2500 above), in
  * two launches that keep each row in shared memory -- except, for 4096 rows and more with D % 4 == 0 and D <= 1536, where
  * K * D > 32768 (D % 8 == 0) or K > 64 (rows of 128 to 256 columns excepted), and short rows with many centroids: those
- * stay on the tile kernels (cat_kernel_for tells); 8192 and more rows of 32, 48, 64, 96 or 128 columns with K * D small enough for
+ * stay on the tile kernels (cat_kernel_for tells); 8192 and more rows of 32, 48, ... 128 columns (steps of 16) with K * D small enough for
  * shared memory stay in registers in one launch.  mask bit 1: so do the K-Means
  * rounds and the final assignment of cat_fit / cat_fit_from (Algorithm 1, step 2; calls without
  * per-round diagnostics), and of other sets of up to 8192 rows with moderate N * K * D (of those shapes too up to 4096 rows), and

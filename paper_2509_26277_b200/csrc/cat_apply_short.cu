@@ -502,7 +502,9 @@ cudaError_t launch_short_d(int D, const ShortParams &p, cudaStream_t s)
     case 2: return launch_short_nks<2, BF16>(p, s);
     case 3: return launch_short_nks<3, BF16>(p, s);
     case 4: return launch_short_nks<4, BF16>(p, s);
+    case 5: return launch_short_nks<5, BF16>(p, s);
     case 6: return launch_short_nks<6, BF16>(p, s);
+    case 7: return launch_short_nks<7, BF16>(p, s);
     default: return launch_short_nks<8, BF16>(p, s);
     }
 }
@@ -511,7 +513,7 @@ cudaError_t launch_short_d(int D, const ShortParams &p, cudaStream_t s)
 
 bool apply_short_supported(int64_t N, int D, int K)
 {
-    return N >= 1 && K >= 2 && K <= 128 && (D == 32 || D == 48 || D == 64 || D == 96 || D == 128) && short_smem(D, K, false) <= SH_SMEM;
+    return N >= 1 && K >= 2 && K <= 128 && D >= 32 && D <= 128 && D % 16 == 0 && short_smem(D, K, false) <= SH_SMEM;
 }
 
 cudaError_t launch_apply_short(const float *Y, int64_t N, int D, int K, const float *C, const float *gamma, const float *beta, void *out,

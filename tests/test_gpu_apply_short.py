@@ -37,8 +37,8 @@ def _check(Y, C, g, b, alpha=1.0):
 
 
 # every number of column steps, one chunk of centroids and two, tiles of centroids that are not full, a last group of one row
-SHAPES = [(8192, 32, 8), (8193, 32, 128), (8207, 48, 17), (9000, 48, 100), (20_001, 64, 64), (8208, 64, 65), (20_011, 64, 81), (8195, 64, 128), (10_001, 96, 33),
-          (9001, 96, 96), (8197, 32, 113), (8199, 128, 9), (30_005, 128, 64), (8209, 128, 100), (200_704, 64, 64)]
+SHAPES = [(8192, 32, 8), (8193, 32, 128), (8207, 48, 17), (9000, 48, 100), (20_001, 64, 64), (8208, 64, 65), (20_011, 64, 81), (8195, 64, 128), (9003, 80, 8), (8211, 80, 81), (10_001, 96, 33),
+          (9001, 96, 96), (8197, 32, 113), (8193, 112, 64), (20_003, 112, 90), (8199, 128, 9), (30_005, 128, 64), (8209, 128, 100), (200_704, 64, 64)]
 
 
 @pytest.mark.parametrize("n,d,k", SHAPES)
