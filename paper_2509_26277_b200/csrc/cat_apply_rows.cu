@@ -37,7 +37,7 @@
 //   e += 2^-24 ||y - mean|| (||w|| + ||V||_F max ||c_k - m||).
 // Several candidates: the same dot products in fp32 from w_k in fp32; for the rows that these leave (one in a thousand) a kernel
 // behind this one forms the projection in fp64 and the distances in the reduced space.  50 000 x 1000, 50 components, K = 64: the projection in fp64, the assignment of
-// the reduced rows and the correction took 377 us, this takes 235 - 245.
+// the reduced rows and the correction took 377 us, this takes 221.
 #include "cat_tc.cuh"
 
 #include <cuda_bf16.h>
@@ -109,7 +109,7 @@ struct ResParams {
     int T, S;      // teams, row slots per team
     int out_bf16;
     const float *mean;   // PCA: [D]
-    uint4 *open_rows;    // PCA: [N] {row, candidates} that fp32 has not decided
+    uint4 *open_rows;    // PCA: [N] {row, candidates, whether their scores are the same} that fp32 has not decided
     int p;
     ResLayout L;
 };
@@ -312,7 +312,8 @@ __device__ __forceinline__ void dots2(const float *y, const float *mean, const f
     s1 = warp_sum_f(s1);
 }
 
-// Label among the candidates (K <= 64) by the same dot products in fp32; those left are returned where that does not decide.
+// Label among the candidates (K <= 64) by the same dot products in fp32; where that does not decide, those left go to *rest and
+// the result is whether their scores are all the same (those of equal centroids are).
 // noise: bound on the error of a fp32 score here, the rounding of the projected row included.
 template <bool VEC>
 __device__ __noinline__ int settle_pca(const float *y, const float *mean, const float *lift, const float *ak, int D, uint2 mask2, float noise,
@@ -342,14 +343,16 @@ __device__ __noinline__ int settle_pca(const float *y, const float *mean, const 
     }
     const float lim = fmaxf(best, -3.4028235e38f) + 2.f * noise;
     int left = 0;
+    uint32_t others = 0u;   // candidates whose score is not the smallest, bit for bit
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
         mask[i] &= __ballot_sync(0xffffffffu, !(sc[i] > lim));
+        others |= mask[i] & __ballot_sync(0xffffffffu, sc[i] != best);
         left += __popc(mask[i]);
         if (mask[i] && held < 0) held = 32 * i + __ffs(mask[i]) - 1;
     }
     *rest = left == 1 ? make_uint2(0u, 0u) : make_uint2(mask[0], mask[1]);
-    return held < 0 ? 0 : held;
+    return left > 1 ? others == 0u : (held < 0 ? 0 : held);
 }
 
 template <int TW>
@@ -788,7 +791,7 @@ __global__ void __launch_bounds__(RES_MAX_THREADS, 1) apply_rows_kernel(ResParam
                                             make_uint2(mask[0], mask[1]), noise, lane, &rest);
                     if ((rest.x | rest.y) != 0u) {
                         // (left as it is: the kernel behind this one reads the row again, and Y may be the output)
-                        if (lane == 0) p.open_rows[atomicAdd(&p.ctl->refine_count, 1)] = make_uint4((uint32_t)(row0 + ro), rest.x, rest.y, 0u);
+                        if (lane == 0) p.open_rows[atomicAdd(&p.ctl->refine_count, 1)] = make_uint4((uint32_t)(row0 + ro), rest.x, rest.y, (uint32_t)exact);
                         exact = -1;
                     }
                 } else
@@ -876,10 +879,13 @@ __global__ void __launch_bounds__(RES_MAX_THREADS, 1) apply_rows_kernel(ResParam
 }
 
 // The rows that fp32 has not decided, a CTA each: the projection in fp64, rounded to fp32, and the candidates' distances to it
-// in fp64, lowest index on equality; then the correction.  (Y may be `out`: a row is read before it is written, by the thread
+// in fp64, lowest index on equality; then the correction.  Candidates that are equal to the first one have its distance, so a row
+// that has no others needs no projection (50 000 x 1000, 50 components, K = 64 in 32 pairs, which leaves every row to this
+// kernel: 2310 us a call with projections, 541 without).  (Y may be `out`: a row is read before it is written, by the thread
 // that writes it.)  A launch of its own: a warp of the kernel above
 // would be at one such row for as long as it takes its team to go through three groups of rows.
 constexpr int OPEN_THREADS = 256;
+constexpr int OPEN_MAX_D = 1024;
 __global__ void __launch_bounds__(OPEN_THREADS) open_rows_kernel(const float *Y, const float *__restrict__ C, int D, int K, int p,
                                                                  const float *__restrict__ mean, const float *__restrict__ comps,
                                                                  const float *__restrict__ gamma, const float *__restrict__ beta,
@@ -892,61 +898,99 @@ __global__ void __launch_bounds__(OPEN_THREADS) open_rows_kernel(const float *Y,
     __shared__ int s_label;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     float *z = reinterpret_cast<float *>(xs + D);
+    constexpr int PER = OPEN_MAX_D / OPEN_THREADS;   // columns a thread has
     const int n = ctl->refine_count;
     for (int i = blockIdx.x; i < n; i += gridDim.x) {
         const uint4 e = open_rows[i];
         const float *y = Y + (size_t)e.x * D;
-        for (int j = tid; j < D; j += OPEN_THREADS) xs[j] = (double)y[j] - (double)__ldg(mean + j);
-        __syncthreads();
-        // (eight components of a warp side by side, 32 loads in flight per lane)
-        for (int r0 = warp * 8; r0 < p; r0 += OPEN_THREADS / 32 * 8) {
-            double s[8];
-            const float *v[8];
+        const int first = e.y ? __ffs(e.y) - 1 : 31 + __ffs(e.z);
+        float yv[PER], mv[PER];   // (read here and stored from here: a load behind a store that may be to the same place would wait for it)
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                s[q] = 0.0;
-                v[q] = comps + (size_t)(r0 + q < p ? r0 + q : r0) * D;
-            }
-#pragma unroll 4
-            for (int j = lane; j < D; j += 32) {
-                const double x = xs[j];
-#pragma unroll
-                for (int q = 0; q < 8; ++q) s[q] = fma(x, (double)__ldg(v[q] + j), s[q]);
-            }
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
-                if (lane == 0 && r0 + q < p) z[r0 + q] = (float)s[q];
-            }
+        for (int u = 0; u < PER; ++u) {
+            const int j = tid + u * OPEN_THREADS;
+            yv[u] = j < D ? y[j] : 0.f;
+            mv[u] = j < D ? __ldg(mean + j) : 0.f;
         }
-        __syncthreads();
-        for (int k = warp; k < K; k += OPEN_THREADS / 32) {
-            if (!((k < 32 ? e.y >> k : e.z >> (k - 32)) & 1u)) continue;
-            double s = 0.0;
-            for (int r = lane; r < p; r += 32) {
-                const double d = (double)z[r] - (double)__ldg(C + (size_t)k * p + r);
-                s = fma(d, d, s);
+        bool same = e.w != 0u;
+        if (same)
+            for (unsigned long long left = (unsigned long long)e.z << 32 | e.y; left &= left - 1;) {
+                const float *c = C + (size_t)(__ffsll((long long)left) - 1) * p, *c0 = C + (size_t)first * p;
+                for (int r = tid; r < p; r += OPEN_THREADS) same &= __ldg(c + r) == __ldg(c0 + r);
             }
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) s_dist[k] = s;
+        for (int u = 0; u < PER; ++u)
+            if (tid + u * OPEN_THREADS < D) xs[tid + u * OPEN_THREADS] = (double)yv[u] - (double)mv[u];
+        const bool one = __syncthreads_and(same);
+        if (!one) {
+            // (eight components of a warp side by side, 32 loads in flight per lane)
+            for (int r0 = warp * 8; r0 < p; r0 += OPEN_THREADS / 32 * 8) {
+                double s[8];
+                const float *v[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    s[q] = 0.0;
+                    v[q] = comps + (size_t)(r0 + q < p ? r0 + q : r0) * D;
+                }
+                for (int j0 = lane; j0 < D; j0 += 128) {
+                    float c[4][8];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) c[u][q] = j0 + 32 * u < D ? __ldg(v[q] + j0 + 32 * u) : 0.f;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const double x = j0 + 32 * u < D ? xs[j0 + 32 * u] : 0.0;
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) s[q] = fma(x, (double)c[u][q], s[q]);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
+                    if (lane == 0 && r0 + q < p) z[r0 + q] = (float)s[q];
+                }
+            }
+            __syncthreads();
+            for (int k = warp; k < K; k += OPEN_THREADS / 32) {
+                if (!((k < 32 ? e.y >> k : e.z >> (k - 32)) & 1u)) continue;
+                double s = 0.0;
+                for (int r = lane; r < p; r += 32) {
+                    const double d = (double)z[r] - (double)__ldg(C + (size_t)k * p + r);
+                    s = fma(d, d, s);
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                if (lane == 0) s_dist[k] = s;
+            }
+            __syncthreads();
         }
-        __syncthreads();
         if (tid == 0) {
             double best = CUDART_INF;
-            int l = e.y ? __ffs(e.y) - 1 : 31 + __ffs(e.z);   // (when every distance is infinite or NaN)
-            for (int k = 0; k < K; ++k)
-                if (((k < 32 ? e.y >> k : e.z >> (k - 32)) & 1u) && s_dist[k] < best) {
-                    best = s_dist[k];
-                    l = k;
+            int l = first;   // (also when every distance is infinite or NaN)
+            if (!one)
+                for (unsigned long long left = (unsigned long long)e.z << 32 | e.y; left; left &= left - 1) {
+                    const int k = __ffsll((long long)left) - 1;
+                    if (s_dist[k] < best) {
+                        best = s_dist[k];
+                        l = k;
+                    }
                 }
             s_label = l;
             labels[e.x] = l;
         }
         __syncthreads();
         const size_t o = (size_t)s_label * D;
-        for (int j = tid; j < D; j += OPEN_THREADS) out[(size_t)e.x * D + j] = fmaf(__ldg(gamma + o + j), y[j], __ldg(beta + o + j));
+        float gv[PER], bv[PER];
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            const int j = tid + u * OPEN_THREADS;
+            gv[u] = j < D ? __ldg(gamma + o + j) : 0.f;
+            bv[u] = j < D ? __ldg(beta + o + j) : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < PER; ++u)
+            if (tid + u * OPEN_THREADS < D) out[(size_t)e.x * D + tid + u * OPEN_THREADS] = fmaf(gv[u], yv[u], bv[u]);
         __syncthreads();
     }
 }
@@ -1064,7 +1108,7 @@ cudaError_t launch_apply_rows(const float *Y, int64_t N, int D, int K, const flo
 bool apply_rows_pca_supported(int64_t N, int D, int K)
 {
     ResPlan pl;
-    return D <= 1024 && K <= 64 && res_plan(N, D, K, &pl, true);
+    return D <= OPEN_MAX_D && K <= 64 && res_plan(N, D, K, &pl, true);
 }
 
 size_t apply_rows_pca_prep_bytes(int64_t N, int D, int K)

@@ -73,6 +73,26 @@ def test_equal_centroids_and_rows_between_two():
     np.testing.assert_array_equal(host(lab), olab)
 
 
+@pytest.mark.parametrize("n,d,k", [(3000, 300, 40), (3001, 301, 64), (4000, 64, 7), (2003, 100, 33)])
+def test_centroids_that_coincide(n, d, k):
+    """Every row but those of a few clusters is left to the kernel behind; the lowest of the equal centroids has it, and rows on the
+    bisector of two such groups are decided by the projection."""
+    rng = np.random.default_rng(n + k)
+    half = (k + 1) // 2
+    Y, mean, V, C, g, b = _case(n + k, n, d, 12, k, 1.0, 1.0)
+    C[half:] = C[rng.permutation(half)[:k - half]]
+    i, j = rng.integers(0, k, size=n), rng.integers(0, k, size=n)
+    z = np.where((np.arange(n) % 3 == 0)[:, None], 0.5 * (C[i] + C[j]), C[i] + 0.05 * rng.normal(size=(n, 12)))
+    Y = (z @ V + mean + 1e-6 * rng.normal(size=(n, d))).astype(np.float32)
+    ws = B.pca_workspace("apply_pca", n, d, 12, "cuda", k)
+    out, lab = B.cat_apply_pca(dev(Y), dev(mean), dev(V), dev(C), dev(g), dev(b), want_labels=True, ws=ws)
+    assert int(ws[:4].view(torch.int32)) > n // 2   # (the control block's first word: rows listed for that kernel)
+    assert host(lab).max() < half
+    _, olab, best, second = P.apply_pca(Y, mean, V, C[:half], g, b)
+    labels_match(host(lab), olab, best, second, "labels")
+    np.testing.assert_array_equal(host(out), O.affine_with_labels(Y, host(lab), g, b))
+
+
 def test_components_that_are_not_unit_vectors_and_rows_out_of_range():
     rng = np.random.default_rng(6)
     Y, mean, V, C, g, b = _case(6, 1200, 200, 10, 24, 0.0, 1.0)
