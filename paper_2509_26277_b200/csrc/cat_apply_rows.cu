@@ -540,8 +540,8 @@ __global__ void __launch_bounds__(PREP_THREADS) centroid_fragments_kernel(const 
 }
 
 // MT: groups of 16 centroids; VEC: D % 4 == 0; TW: warps per team; BG: the fragments stay in global memory (L2).
-// PCA: the scores are those of the projected rows.
-template <int MT, bool VEC, int TW, bool BG, bool PCA>
+// PCA: the scores are those of the projected rows.  WIDE: see wide_steps.
+template <int MT, bool VEC, int TW, bool BG, bool PCA, bool WIDE>
 __global__ void __launch_bounds__(RES_MAX_THREADS, 1) apply_rows_kernel(ResParams p)
 {
     pdl_enter();
@@ -807,9 +807,8 @@ __global__ void __launch_bounds__(RES_MAX_THREADS, 1) apply_rows_kernel(ResParam
         constexpr int V = Unit<VEC>::N;
         const int DV = p.D / V;
         if (TW >= 4) {
-            // column steps at a time, for each of the warp's rows (scalar loads: eight, 225 us against 245 with four for
-            // 49 999 x 1001, K = 50)
-            constexpr int U = VEC ? (TW == 8 ? 4 : 2) : 8;
+            // column steps at a time, for each of the warp's rows
+            constexpr int U = VEC ? (TW == 8 ? 4 : 2) : (TW == 8 || WIDE ? 8 : 4);
             int lq[RPW];
 #pragma unroll
             for (int q = 0; q < RPW; ++q) lq[q] = __shfl_sync(0xffffffffu, label, q * LPR);
@@ -1031,10 +1030,33 @@ bool res_plan(int64_t N, int D, int K, ResPlan *pl, bool pca = false)
     return false;
 }
 
-template <int MT, bool VEC, int TW, bool BG, bool PCA = false>
+// Eight column steps of gamma and beta in flight in place of four, for scalar rows of 257 to 1024 columns: half as many waits for
+// L2, but registers that spill, in the scores' loops too.  Which weighs more was measured (49 999 rows, us with four / eight):
+//   K to 16     long rows with many centroids gain: 1001, K = 12 143 / 138, K = 16 141 / 134; 1001, K = 4 114 / 118; 513, K = 16
+//               76 / 78; 301, K = 16 45 / 50
+//   K to 32     none: 1001, K = 32 153 / 164; 301 53 / 60
+//   K to 48     777, K = 40 183 / 145; 423 86 / 85; 301 63 / 65
+//   K to 64     1001, K = 64 258 / 238; 777 199 / 188; 641 147 / 158
+//   above       short rows gain: 301, K = 72 114 / 109; 423 182 / 194; 1001, K = 128 394 / 425
+//   with PCA    none: 2 to 18 % longer with eight
+template <int MT>
+bool wide_steps(int D, int K)
+{
+    switch (MT) {
+    case 1: return K >= 12 && D > 700;
+    case 2: return false;
+    case 3: return D > 400;
+    case 4: return D > 700;
+    default: return D <= 384;
+    }
+}
+
+template <int MT, bool VEC, int TW, bool BG, bool PCA = false, bool WIDE = false>
 cudaError_t launch_rows(const ResPlan &pl, const ResParams &p, cudaStream_t s)
 {
-    auto kern = apply_rows_kernel<MT, VEC, TW, BG, PCA>;
+    if constexpr (!VEC && TW == 4 && MT != 2 && !PCA && !WIDE)
+        if (wide_steps<MT>(p.D, p.K)) return launch_rows<MT, VEC, TW, BG, PCA, true>(pl, p, s);
+    auto kern = apply_rows_kernel<MT, VEC, TW, BG, PCA, WIDE>;
     // (the same value whatever the shape: several threads may be launching)
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(RES_SMEM - 1024));
     if (e != cudaSuccess) return e;
