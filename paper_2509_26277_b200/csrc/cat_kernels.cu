@@ -173,7 +173,7 @@ __device__ __forceinline__ void assign_load_tile(AssignSmem<BN> &sm, int stage, 
 template <int BN, bool VEC4, bool AFFINE>
 __global__ void __launch_bounds__(A_THREADS) assign_kernel(AssignParams p)
 {
-    if (p.settled && *p.settled) return;
+    const int over = p.settled ? *p.settled : 0;
     constexpr int TX = BN / 8;
     constexpr int TY = A_THREADS / TX;
     constexpr int TM = A_BM / TY;
@@ -191,6 +191,7 @@ __global__ void __launch_bounds__(A_THREADS) assign_kernel(AssignParams p)
     {
         float m = 0.f;
         for (int k = tid; k < p.K; k += A_THREADS) m = fmaxf(m, p.cnorm[k]);
+        if (over) return;   // (the word and the norms on their way together)
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
         if ((tid & 31) == 0) sm.red[tid >> 5] = m;

@@ -41,15 +41,15 @@ __device__ __forceinline__ int entry_key(const int32_t *__restrict__ cur, const 
                                          int64_t N, int K, int64_t e)
 {
     if (e < N) {
-        const int l = cur[e];
+        const int l = cur[e], was = prev ? prev[e] : -1;   // (both on their way together)
         if (l < 0 || l >= K) return -1;
-        if (prev && prev[e] == l) return -1;
+        if (prev && was == l) return -1;
         return l;
     }
     if (!prev || e >= 2 * N) return -1;
     const int64_t r = e - N;
-    const int o = prev[r];
-    if (o < 0 || o >= K || o == cur[r]) return -1;
+    const int o = prev[r], now = cur[r];
+    if (o < 0 || o >= K || o == now) return -1;
     return K + o;
 }
 
@@ -58,13 +58,14 @@ __global__ void __launch_bounds__(SORT_BLOCK) label_hist_kernel(const int32_t *_
                                                                  int KK, uint32_t *__restrict__ blk_hist,
                                                                  const int32_t *settled)
 {
-    pdl_enter();
-    if (settled && *settled) return;
     extern __shared__ uint32_t hist[];   // [KK]
     for (int k = threadIdx.x; k < KK; k += SORT_BLOCK) hist[k] = 0;
-    __syncthreads();
+    pdl_enter();
+    const int over = settled ? *settled : 0;
     const int64_t e = (int64_t)blockIdx.x * SORT_BLOCK + threadIdx.x;
     const int l = entry_key(cur, prev, N, K, e);
+    if (over) return;
+    __syncthreads();
     if (l >= 0) atomicAdd(&hist[l], 1u);
     __syncthreads();
     for (int k = threadIdx.x; k < KK; k += SORT_BLOCK) blk_hist[(size_t)k * gridDim.x + blockIdx.x] = hist[k];   // [key][block]
@@ -76,14 +77,16 @@ __global__ void __launch_bounds__(256) label_scan_blocks_kernel(uint32_t *__rest
                                                                  uint32_t *__restrict__ key_total, const int32_t *settled)
 {
     pdl_enter();
-    if (settled && *settled) return;
+    const int over = settled ? *settled : 0;
     const int k = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     if (k >= KK) return;
-    uint32_t carry = 0;
+    uint32_t carry = 0, next = lane < nblk ? blk_hist[(size_t)k * nblk + lane] : 0u;
+    if (over) return;
     for (int b0 = 0; b0 < nblk; b0 += 32) {
         const int b = b0 + lane;
-        const uint32_t v = (b < nblk) ? blk_hist[(size_t)k * nblk + b] : 0u;
+        const uint32_t v = next;
+        next = b + 32 < nblk ? blk_hist[(size_t)k * nblk + b + 32] : 0u;
         uint32_t incl = v;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -183,23 +186,24 @@ __global__ void __launch_bounds__(SORT_BLOCK) label_scatter_kernel(const int32_t
                                                                     int32_t *__restrict__ seg_start,
                                                                     int32_t *__restrict__ order, int32_t *settled)
 {
-    pdl_enter();
-    // (one read per CTA: CTA 0 may set the word while others of this launch are here)
-    if (settled && __syncthreads_or(threadIdx.x == 0 && *(volatile int32_t *)settled)) return;
     extern __shared__ uint32_t scatter_smem[];   // [KK] key offsets, then [32][KK] 16-bit warp histograms
     __shared__ uint32_t wsum[33];
     uint32_t *key_off = scatter_smem;
     uint16_t *warp_hist = reinterpret_cast<uint16_t *>(scatter_smem + KK);
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     for (int e = tid; e < 32 * KK; e += SORT_BLOCK) warp_hist[e] = 0;
+    pdl_enter();
+    const int64_t e = (int64_t)blockIdx.x * SORT_BLOCK + tid;
+    const bool over = settled && tid == 0 && *(volatile int32_t *)settled;
+    const int l = entry_key(cur, prev, N, K, e);
+    // (one read per CTA: CTA 0 may set the word while others of this launch are here)
+    if (settled && __syncthreads_or(over)) return;
     {
         const uint32_t ea = scan_keys(key_total, K, KK, seg_rows_max, NE, delta, blockIdx.x == 0, counts, cluster_start,
                                       seg_start, settled, wsum);
         if (tid < KK) key_off[tid] = ea;
     }
     __syncthreads();
-    const int64_t e = (int64_t)blockIdx.x * SORT_BLOCK + tid;
-    const int l = entry_key(cur, prev, N, K, e);
     const unsigned peers = __match_any_sync(0xffffffffu, l);
     const int rank_in_warp = __popc(peers & ((1u << lane) - 1u));
     if (l >= 0 && rank_in_warp == 0) warp_hist[w * KK + l] = (uint16_t)__popc(peers);
@@ -279,10 +283,10 @@ template <int MODE, int VEC>
 __global__ void __launch_bounds__(SEG_THREADS) segment_sums_kernel(SegParams p)
 {
     pdl_enter();
-    if (p.settled && *p.settled) return;
     __shared__ int32_t rows_s[128];
     __shared__ double red_s[SEG_THREADS * VEC];
-    const int nseg_total = p.seg_start[p.K];
+    const int over = p.settled ? *p.settled : 0, nseg_total = p.seg_start[p.K];
+    if (over) return;
     for (int seg = blockIdx.x; seg < nseg_total; seg += gridDim.x) {
     // cluster of this segment: last k with seg_start[k] <= seg
     int lo = 0, hi = p.K;
@@ -608,9 +612,10 @@ __global__ void __launch_bounds__(COMB_THREADS, 4) centroid_update_kernel(const 
         ctl->refine_count = 0;
         ctl->cand_count = 0;
     }
-    if (settled && *settled) return;
+    const int over = settled ? *settled : 0;
     const int j = cb * cols + (threadIdx.x & (cols - 1));
     const int64_t n = counts[k];
+    if (over) return;
     double in[1] = {0.0}, gone[1] = {0.0};
     if (j < D) {
         sum_segments<1>(part + j, seg_start[k] + g, seg_start[k + 1], G, (size_t)2 * D, 0, in);

@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(AFFINE ? TC_THREADS_AFFINE : TC_THREADS_LABELS
 assign_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, TcParams p)
 {
     pdl_enter();
-    if (!AFFINE && p.settled && *p.settled) return;   // (the same word for every CTA: no earlier kernel of the stream runs any more)
+    const int over = !AFFINE && p.settled ? *p.settled : 0;   // (the same word for every CTA: no earlier kernel of the stream runs any more)
     extern __shared__ unsigned char smem_raw[];
     // operand tiles need 1024-byte alignment for the 128-byte swizzle
     const uint32_t raw = smem_u32(smem_raw);
@@ -163,6 +163,7 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
             if (k < p.K) m = fmaxf(m, v);
             if (HALF && k < p.K) me = fmaxf(me, p.cerr[k]);
         }
+        if (!AFFINE && over) return;   // (the word and the norms on their way together)
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
