@@ -135,6 +135,12 @@ def test_teams_that_take_many_groups(n, d, k):
     ("fit", 4096, 1000, 32, "fit_rows_kernel"), ("fit", 8192, 256, 32, "fit_rows_kernel"),
     ("fit", 8192, 256, 64, "assign_tc_kernel, fp16 copies"), ("fit", 6144, 256, 128, "assign_tc_kernel, fp16 copies"),
     ("fit", 8192, 50, 64, "fit_rows_kernel"), ("fit", 5000, 64, 64, "small_kernel"), ("fit", 4096, 64, 64, "fit_rows_kernel"),
+    ("apply", 8191, 64, 64, "small_kernel"), ("apply", 8192, 64, 64, "apply_short_kernel"), ("apply_bf16", 8191, 64, 64, "apply_rows_kernel"),
+    ("apply_bf16", 8192, 112, 64, "apply_short_kernel"), ("apply", 8192, 144, 64, "apply_rows_kernel"),
+    ("apply", 9000, 128, 112, "apply_short_kernel"), ("apply", 9000, 128, 113, "small_kernel"),
+    ("fit", 8192, 64, 64, "small_kernel"), ("fit", 8193, 64, 64, "fit_tiles_kernel"),
+    ("fit", 201_280, 64, 64, "fit_tiles_kernel"), ("fit", 201_281, 64, 64, "small_kernel"),
+    ("fit", 40_256, 256, 32, "fit_tiles_kernel"), ("fit", 40_257, 256, 32, "assign_tc_kernel, fp16 copies"),
 ])
 def test_lines_of_the_dispatch(call, n, d, k, kernel):
     """One shape on each side of the lines; results of either side against the oracle."""

@@ -28,9 +28,13 @@ def test_rounds_after_a_fixed_point_change_nothing(n, d, k, spread):
     try:
         ws = torch.empty(B.lib().cat_fit_workspace_bytes(n, d, k), dtype=torch.uint8, device="cuda")
         want = O.fit(Yq, Yfp, k, 60, near_rel=1e-6)
+        labels = [torch.full((n,), -1, dtype=torch.int32, device="cuda")] + [B.cat_fit(q, f, k, t)[3] for t in range(60)]
+        rounds = next((t for t in range(1, 61) if torch.equal(labels[t], labels[t - 1])), 61)   # the first that moves nothing
         got = {}
         for iters in (60, 59, 12, 0, 60):   # both parities of the label buffers; a fit that settles, then others on its workspace
             C, G, Bt, lab = B.cat_fit(q, f, k, iters, ws=ws)
+            # (the ninth word of the control block: a round has moved nothing)
+            assert bool(ws[32:36].view(torch.int32)) == (iters >= rounds)
             got.setdefault(iters, []).append([t.cpu() for t in (C, G, Bt, lab)])
         sums, counts = B.cat_cluster_sums(q, got[60][0][3].cuda(), k, ws=ws)
     finally:

@@ -88,6 +88,34 @@ def test_fit_matches_the_oracle_and_repeats(n, d, k, small_mask):
         assert (labels0 != labels).float().mean().item() < 1e-3
 
 
+# CTAs that take several tiles of 128 rows (148 of them take 18 944 at a time): stages, phases and accumulators used again.  (Shapes
+# that the kernels for short rows in registers and in shared memory have no room for.)
+@pytest.mark.parametrize("call,n,d,k", [("apply", 40_001, 128, 128), ("apply", 76_000, 128, 120), ("fit", 225_793, 64, 64), ("fit", 110_001, 128, 32),
+                                        ("fit", 420_003, 32, 128)])
+def test_ctas_that_take_many_tiles(call, n, d, k, small_mask):
+    B.cat_set_small_problem_kernels(3)
+    assert B.cat_kernel_for(call, n, d, k) == "small_kernel"
+    Yq, Yfp = _data(n + d + k, n, d)
+    if call == "apply":
+        rng = np.random.default_rng(3)
+        C = Yq[rng.choice(n, size=k, replace=False)].copy()
+        G, Bt = rng.normal(size=(k, d)).astype(np.float32), rng.normal(size=(k, d)).astype(np.float32)
+        lab, best, second = O.assign(Yq, C)
+        out, glab = B.cat_apply(dev(Yq), dev(C), dev(G), dev(Bt), want_labels=True)
+        labels_match(host(glab), lab, best, second, "labels")
+        np.testing.assert_array_equal(host(out), O.affine_with_labels(Yq, host(glab), G, Bt))
+        return
+    C, G, Bt, labels = B.cat_fit(dev(Yq), dev(Yfp), k, 3)
+    assert all(torch.equal(a, b) for a, b in zip((C, G, Bt, labels), B.cat_fit(dev(Yq), dev(Yfp), k, 3)))
+    lab, best, second = O.assign(Yq, host(C))
+    labels_match(host(labels), lab, best, second, "labels")
+    g_want, b_want = O.solve_gamma_beta(Yq, Yfp, host(labels), k)
+    close(host(G), g_want, "gamma")
+    close(host(Bt), b_want, "beta")
+    C1 = B.cat_fit(dev(Yq), dev(Yfp), k, 4)[0]
+    close(host(C1), O.update_centroids(Yq, host(labels), host(C))[0], "centroid update")
+
+
 def test_whole_fit_against_the_oracle(small_mask):
     """Well separated data: the whole trajectory is the oracle's."""
     rng = np.random.default_rng(5)
