@@ -405,6 +405,7 @@ cat_status_t cat_selftest_wait_timeout(void *workspace, size_t workspace_bytes, 
  * columns) a Lloyd round takes half the time on the tensor path and so does inference, except
  * where low-precision scores leave most rows undecided (unimodal data, K = 32: there the fp32
  * pipes are a quarter faster for inference).
+ * The kernels for small problems below have lines of their own; fits of many short rows take theirs whatever K is.
  * This and cat_set_apply_column_split are PROCESS-WIDE tuning and test hooks: they change
  * which kernel every later call of every thread launches (never the results), and they are
  * not meant to be flipped while other threads are inside the library. */

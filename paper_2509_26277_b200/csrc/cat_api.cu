@@ -168,7 +168,9 @@ static bool use_fit_rows(int64_t N, int D, int K)
            (N <= 4096 || !use_small_fit(N, D, K));
 }
 // Rows as fp16 fragments in shared memory for all rounds: more than 8192 rows (200 704 x 64, K = 64 1030 us against 1390 in the
-// persistent kernel, 108 286 x 256, K = 49 1510 against 1790 on the general path).  Up to there the kernels of small sets have the
+// persistent kernel, 40 000 x 256, K = 20 800 against 1100 on the general path; a few centroids and a few columns too: 8193 x 4, K = 3 360
+// against 815, 100 000 x 33, K = 7 630 against 1041, ragged rows 60 000 x 191, K = 8 918 against 1169, so that it does not ask for
+// the tensor-core threshold).  Up to there the kernels of small sets have the
 // shorter rounds (PCA fits with reduced sets of 2048 x 20, K = 10 1314 us against 1358 here, 4096 x 50, K = 32 the same).
 static bool use_fit_tiles(int64_t N, int D, int K)
 {
@@ -179,8 +181,9 @@ static bool use_small_apply(int64_t N, int D, int K)
     return (g_small_kernels.load(std::memory_order_relaxed) & 1) && use_tensor_path(N, D, K) && small_apply_supported(N, D, K);
 }
 
-// Short rows in registers: from 8192 rows on (two groups of sixteen rows for every three warps of the device).  200 704 x 64,
-// K = 64 35 us against 50 in the persistent kernel; 12 155 x 64 and 40 764 x 48 18 - 20 in either; below, launches decide.
+// Short rows in registers: from 8192 rows on, a group of sixteen for every third to fifth warp of the device.  200 704 x 64, K = 64 35 us
+// against 50 in the persistent kernel, 80 000 x 64, K = 80 26 and 28; from 8192 to 40 000 rows a call's launches take the time on the
+// host in either (17 - 18 us), but 20 000 x 96, K = 100 20 us here and 39 in the tile kernels.
 static bool use_apply_short(int64_t N, int D, int K)
 {
     const int min_k = g_tc_min_k.load(std::memory_order_relaxed);

@@ -241,7 +241,8 @@ struct TridiagParams {
 //   y = a - u_1 w0 - w0_1 u needs no sum, so |x|^2 = |y|^2 + 4 h u_1 y'u + 4 h^2 u_1^2 u'u.  Where these cancel by more than
 //   16, the squares are added up in a second exchange.  (u'u is added up with the others: carried over from the step before,
 //   as |x|^2 less one entry, its error would grow by up to 16 a step.)  The mean of the diagonal is taken off the matrix and put back
-//   on the tridiagonal one, which keeps h small: without it nearly every step of a covariance would cancel.
+//   on the tridiagonal one, which makes h smaller: without it nearly every step of a covariance would cancel, with it those whose spectrum
+//   is far from one value still do in most steps (a second summation stays within the CTA).
 //   bound: latency.  A step moves 2 D values between CTAs and does 6 (D - j)^2 / G operations per CTA.
 template <int C>
 __global__ void __launch_bounds__(ET) tridiag_regs_kernel(TridiagParams P)
