@@ -37,8 +37,8 @@
 //   e += 2^-24 ||y - mean|| (||w|| + ||V||_F max ||c_k - m||).
 // Several candidates: the same dot products in fp32 from w_k in fp32; for the rows that these leave (one in a thousand) a kernel
 // behind this one forms the projection in fp64 and the distances in the reduced space.  50 000 x 1000, 50 components, K = 64: the projection in fp64, the assignment of
-// the reduced rows and the correction took 377 us, this takes 221.
-#include "cat_tc.cuh"
+// the reduced rows and the correction took 377 us, this takes 235.
+#include "cat_half.cuh"
 
 #include <cuda_bf16.h>
 
@@ -121,55 +121,11 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_
                  : "memory");
 }
 
-__device__ __forceinline__ void mma_16816(float (&c)[4], const uint4 a, uint32_t b0, uint32_t b1)
-{
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
-}
-
 __device__ __forceinline__ float warp_sum_f(float v)
 {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
-}
-
-// exponent shift that brings m > 0 to [2^13, 2^14), clamped to +-100; 0 for zero or non-finite m
-__device__ __forceinline__ int half_shift(float m)
-{
-    if (!(m > 0.f) || !(m < CUDART_INF_F)) return 0;
-    int s = 13 - ((int)(__float_as_uint(m) >> 23) - 127);
-    s = s > 100 ? 100 : s;
-    return s < -100 ? -100 : s;
-}
-__device__ __forceinline__ float pow2i(int e) { return __uint_as_float((uint32_t)(e + 127) << 23); }
-
-// Pairs of fp32 values in one 64-bit register: one instruction does both.
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2(float a, float b)
-{
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(f32x2 v)
-{
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
-{
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
-{
-    f32x2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
 }
 
 // Two consecutive columns' fp16 roundings and what they leave, squared.
@@ -181,13 +137,6 @@ __device__ __forceinline__ uint32_t round2(f32x2 v, f32x2 &left2)
     const f32x2 d = fma2(pack2(f.x, f.y), pack2(-1.f, -1.f), v);   // (exact)
     left2 = fma2(d, d, left2);
     return *reinterpret_cast<const uint32_t *>(&h);
-}
-
-__device__ __forceinline__ float sqrt_approx(float x)   // (2^-23 relative; callers have slack for more)
-{
-    float r;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
 }
 
 __device__ __forceinline__ float sq_diff(float y, float c, float s)

@@ -21,7 +21,7 @@
 // rounding errors of the fp16 operands are measured.  Rows with several centroids within the bound are settled by the
 // quad of lanes that has the row: direct-form fp32 sums of squares, a lane's D / 4 terms first, and what these leave
 // within their error in fp64, lowest index on equality.
-#include "cat_tc.cuh"
+#include "cat_half.cuh"
 
 #include <cuda_bf16.h>
 
@@ -51,67 +51,6 @@ size_t short_smem(int D, int K, bool ahead)
     return rows + (size_t)3 * K * short_ld(D) * 4 + nt * 16 * D * 2 + nt * 16 * 2 * 4 + (size_t)D * 4;
 }
 
-__device__ __forceinline__ void mma_16816(float (&c)[4], const uint4 a, uint32_t b0, uint32_t b1)
-{
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
-}
-// pairs of fp32 values in one 64-bit register: one instruction does both
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2(float a, float b)
-{
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(f32x2 v)
-{
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
-{
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
-{
-    f32x2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-
-// exponent shift that brings m > 0 to [2^13, 2^14), clamped to +-100; 0 for zero or non-finite m
-__device__ __forceinline__ int half_shift(float m)
-{
-    if (!(m > 0.f) || !(m < CUDART_INF_F)) return 0;
-    int s = 13 - ((int)(__float_as_uint(m) >> 23) - 127);
-    s = s > 100 ? 100 : s;
-    return s < -100 ? -100 : s;
-}
-__device__ __forceinline__ float pow2i(int e) { return __uint_as_float((uint32_t)(e + 127) << 23); }
-// two columns' fp16 roundings and what they leave, squared
-__device__ __forceinline__ uint32_t round_pair(float a, float b, float &left2)
-{
-    const __half2 h = __floats2half2_rn(a, b);
-    const float2 f = __half22float2(h);
-    const float da = a - f.x, db = b - f.y;
-    left2 = fmaf(da, da, fmaf(db, db, left2));
-    return *reinterpret_cast<const uint32_t *>(&h);
-}
-__device__ __forceinline__ float sqrt_approx(float x)   // (2^-23 relative; the slack has room for it)
-{
-    float r;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-__device__ __forceinline__ float max4(float4 a, float m)
-{
-    return fmaxf(fmaxf(m, fmaxf(fabsf(a.x), fabsf(a.y))), fmaxf(fabsf(a.z), fabsf(a.w)));
-}
 __device__ __forceinline__ float dist4(float4 y, float4 c, float s)
 {
     const float a = y.x - c.x, b = y.y - c.y, d = y.z - c.z, e = y.w - c.w;
@@ -121,19 +60,6 @@ __device__ __forceinline__ double dist4(float4 y, float4 c, double s)
 {
     const double a = (double)y.x - (double)c.x, b = (double)y.y - (double)c.y, d = (double)y.z - (double)c.z, e = (double)y.w - (double)c.w;
     return fma(e, e, fma(d, d, fma(b, b, fma(a, a, s))));
-}
-// index of the lowest set bit, which it clears; -1 if none
-template <int W>
-__device__ __forceinline__ int pop_bit(uint32_t (&m)[W])
-{
-#pragma unroll
-    for (int i = 0; i < W; ++i)
-        if (m[i]) {
-            const int k = 32 * i + __ffs(m[i]) - 1;
-            m[i] &= m[i] - 1;
-            return k;
-        }
-    return -1;
 }
 
 // The label of each quad's row among the candidates of its mask (none: `label` stands).  The whole warp calls it.
@@ -380,13 +306,6 @@ __global__ void __launch_bounds__(short_threads(NKS), 1) apply_short_kernel(Shor
                 }
             }
         };
-        // keys: scores with the centroid's index in the low seven bits.  (Those of an infinite or NaN score may get lost, but a
-        // row that has one also has a bound that decides nothing.)
-        auto better = [](float s, int k, float &b1, float &b2) {
-            const float key = __uint_as_float((__float_as_uint(s) & 0xFFFFFF80u) | (uint32_t)k);
-            b2 = fminf(b2, fmaxf(b1, key));
-            b1 = fminf(b1, key);
-        };
         const f32x2 ia2 = pack2(ia, ia), ib2 = pack2(ib, ib);
 #pragma unroll 1
         for (int ch = 0; ch < NC; ++ch) {
@@ -398,21 +317,16 @@ __global__ void __launch_bounds__(short_threads(NKS), 1) apply_short_kernel(Shor
                 const f32x2 n = *reinterpret_cast<const f32x2 *>(ak + k), f = *reinterpret_cast<const f32x2 *>(coef + k);
                 const float2 ua = unpack2(fma2(f, mul2(pack2(acc[i][0], acc[i][1]), ia2), n));
                 const float2 ub = unpack2(fma2(f, mul2(pack2(acc[i][2], acc[i][3]), ib2), n));
-                better(ua.x, k, a1, a2);
-                better(ua.y, k + 1, a1, a2);
-                better(ub.x, k, c1, c2);
-                better(ub.y, k + 1, c1, c2);
+                take_key(ua.x, k, a1, a2);
+                take_key(ua.y, k + 1, a1, a2);
+                take_key(ub.x, k, c1, c2);
+                take_key(ub.y, k + 1, c1, c2);
             }
         }
 #pragma unroll
         for (int o = 1; o < 4; o <<= 1) {
-            float q1 = __shfl_xor_sync(0xffffffffu, a1, o), q2 = __shfl_xor_sync(0xffffffffu, a2, o);
-            a2 = fminf(fminf(a2, q2), fmaxf(a1, q1));
-            a1 = fminf(a1, q1);
-            q1 = __shfl_xor_sync(0xffffffffu, c1, o);
-            q2 = __shfl_xor_sync(0xffffffffu, c2, o);
-            c2 = fminf(fminf(c2, q2), fmaxf(c1, q1));
-            c1 = fminf(c1, q1);
+            merge_keys(o, a1, a2);
+            merge_keys(o, c1, c2);
         }
         int ka = (int)(__float_as_uint(a1) & 0x7Fu), kb = (int)(__float_as_uint(c1) & 0x7Fu);
         if (ka >= K) ka = 0;

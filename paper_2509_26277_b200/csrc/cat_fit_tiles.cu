@@ -22,7 +22,7 @@
 // A round in which no label changes leaves everything as it is, and so would all behind it: the rounds end there.  Sums
 // that follow moves keep what a far larger row rounded off after it has left; where the largest row's exponent is more than
 // X_SPREAD above the rows' average every round adds up all rows afresh (and none ends early).
-#include "cat_tc.cuh"
+#include "cat_half.cuh"
 
 namespace cat {
 
@@ -86,57 +86,6 @@ struct TilesParams {
     TilesLayout L;
 };
 
-__device__ __forceinline__ void mma_16816(float (&c)[4], const uint4 a, uint32_t b0, uint32_t b1)
-{
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
-}
-// pairs of fp32 values in one 64-bit register: one instruction does both
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2(float a, float b)
-{
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(f32x2 v)
-{
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
-{
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
-{
-    f32x2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-
-// exponent shift that brings m > 0 to [2^13, 2^14), clamped to +-100; 0 for zero or non-finite m
-__device__ __forceinline__ int half_shift(float m)
-{
-    if (!(m > 0.f) || !(m < CUDART_INF_F)) return 0;
-    int s = 13 - ((int)(__float_as_uint(m) >> 23) - 127);
-    s = s > 100 ? 100 : s;
-    return s < -100 ? -100 : s;
-}
-__device__ __forceinline__ float pow2i(int e) { return __uint_as_float((uint32_t)(e + 127) << 23); }
-// two columns' fp16 roundings and what they leave, squared
-__device__ __forceinline__ uint32_t round_pair(float a, float b, float &left2)
-{
-    const __half2 h = __floats2half2_rn(a, b);
-    const float2 f = __half22float2(h);
-    const float da = a - f.x, db = b - f.y;
-    left2 = fmaf(da, da, fmaf(db, db, left2));
-    return *reinterpret_cast<const uint32_t *>(&h);
-}
 // upper half of a float that is not below x >= 0
 __device__ __forceinline__ uint32_t ceil_bf16(float x) { return x < CUDART_INF_F ? (__float_as_uint(x) + 0xFFFFu) >> 16 : 0x7F80u; }
 
@@ -155,29 +104,11 @@ __device__ __forceinline__ float4 load4(const float *row, int j, int D)
     }
 }
 __device__ __forceinline__ float4 sub4(float4 a, float4 b) { return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w); }
-__device__ __forceinline__ float max4(float4 a, float m)
-{
-    return fmaxf(fmaxf(m, fmaxf(fabsf(a.x), fabsf(a.y))), fmaxf(fabsf(a.z), fabsf(a.w)));
-}
 __device__ __forceinline__ float sq4(float4 a, float s) { return fmaf(a.x, a.x, fmaf(a.y, a.y, fmaf(a.z, a.z, fmaf(a.w, a.w, s)))); }
 __device__ __forceinline__ double sq4(float4 y, float4 c, double s)
 {
     const double a = (double)y.x - (double)c.x, b = (double)y.y - (double)c.y, d = (double)y.z - (double)c.z, e = (double)y.w - (double)c.w;
     return fma(e, e, fma(d, d, fma(b, b, fma(a, a, s))));
-}
-
-// index of the lowest set bit, which it clears; -1 if none
-template <int W>
-__device__ __forceinline__ int pop_bit(uint32_t (&m)[W])
-{
-#pragma unroll
-    for (int i = 0; i < W; ++i)
-        if (m[i]) {
-            const int k = 32 * i + __ffs(m[i]) - 1;
-            m[i] &= m[i] - 1;
-            return k;
-        }
-    return -1;
 }
 
 // Labels of n <= 4 queued rows, eight lanes a row.
@@ -504,13 +435,6 @@ __global__ void __launch_bounds__(XT, 1) fit_tiles_kernel(TilesParams p)
                     }
                 }
             };
-            // keys: scores with the centroid's index in the low seven bits.  (Those of an infinite or NaN score may get lost, but a
-            // row that has one also has a bound that decides nothing.)
-            auto better = [](float s, int k, float &b1, float &b2) {
-                const float key = __uint_as_float((__float_as_uint(s) & 0xFFFFFF80u) | (uint32_t)k);
-                b2 = fminf(b2, fmaxf(b1, key));
-                b1 = fminf(b1, key);
-            };
             const f32x2 ia2 = pack2(ia, ia), ib2 = pack2(ib, ib);
 #pragma unroll 1
             for (int ch = 0; ch < NC; ++ch) {
@@ -523,21 +447,16 @@ __global__ void __launch_bounds__(XT, 1) fit_tiles_kernel(TilesParams p)
                     const f32x2 n = *reinterpret_cast<const f32x2 *>(cn + k), f = *reinterpret_cast<const f32x2 *>(coef + k);
                     const float2 sa = unpack2(fma2(f, mul2(pack2(acc[i][0], acc[i][1]), ia2), n));
                     const float2 sb = unpack2(fma2(f, mul2(pack2(acc[i][2], acc[i][3]), ib2), n));
-                    better(sa.x, k, a1, a2);
-                    better(sa.y, k + 1, a1, a2);
-                    better(sb.x, k, c1, c2);
-                    better(sb.y, k + 1, c1, c2);
+                    take_key(sa.x, k, a1, a2);
+                    take_key(sa.y, k + 1, a1, a2);
+                    take_key(sb.x, k, c1, c2);
+                    take_key(sb.y, k + 1, c1, c2);
                 }
             }
 #pragma unroll
             for (int o = 1; o < 4; o <<= 1) {
-                float q1 = __shfl_xor_sync(0xffffffffu, a1, o), q2 = __shfl_xor_sync(0xffffffffu, a2, o);
-                a2 = fminf(fminf(a2, q2), fmaxf(a1, q1));
-                a1 = fminf(a1, q1);
-                q1 = __shfl_xor_sync(0xffffffffu, c1, o);
-                q2 = __shfl_xor_sync(0xffffffffu, c2, o);
-                c2 = fminf(fminf(c2, q2), fmaxf(c1, q1));
-                c1 = fminf(c1, q1);
+                merge_keys(o, a1, a2);
+                merge_keys(o, c1, c2);
             }
             const int ka = (int)(__float_as_uint(a1) & 0x7Fu) < K ? (int)(__float_as_uint(a1) & 0x7Fu) : 0;
             const int kb = (int)(__float_as_uint(c1) & 0x7Fu) < K ? (int)(__float_as_uint(c1) & 0x7Fu) : 0;

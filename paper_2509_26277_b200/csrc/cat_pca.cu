@@ -566,7 +566,7 @@ size_t cat_apply_pca_workspace_bytes(int64_t N, int32_t D, int32_t K, int32_t p)
 
 // One kernel that keeps rows in shared memory, where it takes the shape (the selector of cat_apply's kernel of that kind
 // holds here too): against the three steps, 8000 x 777, K = 16, 8 components 30 us and 123, 50 000 x 1000, K = 64, 50
-// components 221 and 372, 50 000 x 100, K = 40 42 and 81, and at the line 656 x 100, K = 2 25 and 31, with 256 components 66 x 1000, K = 16 45
+// components 235 and 372, 50 000 x 100, K = 40 42 and 81, and at the line 656 x 100, K = 2 25 and 31, with 256 components 66 x 1000, K = 16 45
 // and 83.  (Less than a few hundred rows leave either idle.)
 static bool use_apply_rows_pca(int64_t N, int D, int K)
 {
