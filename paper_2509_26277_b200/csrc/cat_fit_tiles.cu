@@ -584,7 +584,10 @@ __global__ void __launch_bounds__(XT, 1) fit_tiles_kernel(TilesParams p)
         }
         if (tid == 0 && total) atomicAdd(moved + (pass & 1), total);
         if (!grid_barrier(&p.ctl->grid_bar, ++bar, p.ctl)) { alive = false; break; }
-        if (__ldcg(moved + (pass & 1)) == 0) break;   // nothing moved: nothing would from here on
+        if (__ldcg(moved + (pass & 1)) == 0) {   // nothing moved: nothing would from here on, and every assignment left would settle these rows
+            if (lane == 0) refined += (long long)refined_pass * (p.passes - 1 - pass);
+            break;
+        }
         // (the first pass has added all rows in either case; the same decision in every CTA)
         afresh = (__ldcg(spread + 2) - X_SPREAD) * (long long)__ldcg(spread + 1) > (long long)__ldcg(spread);
 

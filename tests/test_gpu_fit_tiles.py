@@ -64,6 +64,22 @@ def test_rounds(iters):
     close(host(C), ora.centroids, "centroids")
 
 
+@pytest.mark.parametrize("n,d,k", [(9001, 4, 60), (9000, 10, 100), (20_000, 32, 40)])
+def test_counters_do_not_depend_on_the_early_end(n, d, k):
+    """Labels that come to rest leave the total as if every assignment had run: each one more adds the rows of the last."""
+    Yq = np.random.default_rng(n).normal(size=(1500, d)).astype(np.float32)[np.arange(n) % 1500]   # one cloud of repeated rows
+    ws = B.workspace("fit", n, d, k, "cuda")
+    reps, labels = {}, {}
+    for iters in (150, 151, 165):
+        labels[iters] = B.cat_fit(dev(Yq), dev(Yq), k, iters, ws=ws)[3]
+        reps[iters] = B.cat_workspace_report(ws)
+    assert torch.equal(labels[150], labels[165])
+    last = reps[150]["refined_rows_last"]
+    assert last > 0 and reps[165]["refined_rows_last"] == last
+    assert reps[151]["refined_rows_total"] - reps[150]["refined_rows_total"] == last
+    assert reps[165]["refined_rows_total"] - reps[150]["refined_rows_total"] == 15 * last
+
+
 @pytest.mark.parametrize("k", [2, 9, 70])
 @pytest.mark.parametrize("mag", MAGS)
 def test_magnitudes_at_the_ends_of_fp32(k, mag):
