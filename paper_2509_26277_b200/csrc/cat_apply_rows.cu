@@ -981,8 +981,8 @@ bool res_plan(int64_t N, int D, int K, ResPlan *pl, bool pca = false)
 
 // Eight column steps of gamma and beta in flight in place of four, for scalar rows of 257 to 1024 columns: half as many waits for
 // L2, but registers that spill, in the scores' loops too.  Which weighs more was measured (49 999 rows, us with four / eight):
-//   K to 16     long rows with many centroids gain: 1001, K = 12 143 / 138, K = 16 141 / 134; 1001, K = 4 114 / 118; 513, K = 16
-//               76 / 78; 301, K = 16 45 / 50
+//   K to 16     long rows with many centroids gain: 1001, K = 12 143 / 138, K = 16 141 / 134 (15 000 rows, K = 10 63 / 60); 1001,
+//               K = 4 114 / 118; 513, K = 16 76 / 78; 301, K = 16 45 / 50
 //   K to 32     none: 1001, K = 32 153 / 164; 301 53 / 60
 //   K to 48     777, K = 40 183 / 145; 423 86 / 85; 301 63 / 65
 //   K to 64     1001, K = 64 258 / 238; 777 199 / 188; 641 147 / 158
@@ -992,7 +992,7 @@ template <int MT>
 bool wide_steps(int D, int K)
 {
     switch (MT) {
-    case 1: return K >= 12 && D > 700;
+    case 1: return K > 8 && D > 700;
     case 2: return false;
     case 3: return D > 400;
     case 4: return D > 700;
